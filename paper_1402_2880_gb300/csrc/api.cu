@@ -291,23 +291,17 @@ int build_structure(Ctx& c, const sscf_system* sys) {
             if (c.h_gnb_row[e] <= c.h_gnb_col[e]) c.h_ocolour_blk[f2[col]++] = e;
         }
         // within each colour, blocks between full groups (8 molecules: 32
-        // occupied and 16 virtual MOs) first; FP32 sweeps run them through the
-        // register-resident kernel (occupied passes: A != B only)
-        auto full_first = [&](std::vector<int>& blk, const std::vector<int>& ptr, std::vector<int>& nfull,
-                              bool distinct) {
-            nfull.assign(n_col, 0);
-            for (int k = 0; k < n_col; ++k) {
-                auto b = blk.begin() + ptr[k], en = blk.begin() + ptr[k + 1];
-                auto mid = std::stable_partition(b, en, [&](int e) {
+        // occupied and 16 virtual MOs), the longest ones of a sweep, first
+        auto full_first = [&](std::vector<int>& blk, const std::vector<int>& ptr, bool distinct) {
+            for (int k = 0; k < n_col; ++k)
+                std::stable_partition(blk.begin() + ptr[k], blk.begin() + ptr[k + 1], [&](int e) {
                     const int A = c.h_gnb_row[e], B = c.h_gnb_col[e];
                     return (!distinct || A != B) && c.h_group_nmol[A] == kMaxMolPerGroup &&
                            c.h_group_nmol[B] == kMaxMolPerGroup;
                 });
-                nfull[k] = (int)(mid - b);
-            }
         };
-        full_first(c.h_colour_blk, c.h_colour_ptr, c.h_colour_nfull, false);
-        full_first(c.h_ocolour_blk, c.h_ocolour_ptr, c.h_ocolour_nfull, true);
+        full_first(c.h_colour_blk, c.h_colour_ptr, false);
+        full_first(c.h_ocolour_blk, c.h_ocolour_ptr, true);
     }
 
     // ---- tile pairs of the occupied-virtual transform ----
@@ -861,8 +855,8 @@ int sscf_create(const sscf_system* sys, const sscf_params* prm, void* cuda_strea
     AL(c.d_cci_cnt, (size_t)c.n_tiles * 4);
     AL(c.d_cci_row, (size_t)c.n_mol * c.cap * 4);
     AL(c.d_cci_slot, (size_t)c.n_mol * c.cap * 4);
-    AL(c.d_c_cnz, (size_t)c.n_mol * c.cap);
-    AL(c.d_blk_info, (size_t)std::max(c.n_gnb, 1) * 8 * 4);
+    AL(c.d_c_cnz, sweep_flag_bytes(&c));
+    AL(c.d_blk_info, sweep_info_bytes(&c));
     AL(c.d_y_n, (size_t)c.n_tiles * 4);
     AL(c.d_y_row, (size_t)c.n_tiles * c.capY * 4);
     AL(c.d_y_val, (size_t)c.n_tiles * c.capY * kTileVals * ts);

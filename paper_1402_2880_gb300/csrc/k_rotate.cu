@@ -11,6 +11,7 @@
 // and reads and writes C once.
 #include <math.h>
 
+#include <algorithm>
 #include <vector>
 
 #include "sscf_internal.h"
@@ -452,8 +453,8 @@ struct SweepArgs {
     int* out_tile;
     void* out_val;
     unsigned char* out_nz;   // flags of out: 0 = the tile is all zero (written by the closure, kept by the sweep)
-    unsigned char* col_nz;   // sweeps: the same flags in column-index order (entry p of cci_row / cci_slot)
-    const int4* blk_info;    // FP32 sweeps: per block in colour order, (e, pairs, touch, rows), (pa, pb, rows of B, 0)
+    unsigned char* col_nz;   // sweeps: the same flags in column-index order (flag_base)
+    void* blk_info;          // FP32 sweeps: a BlockInfo per block in colour order
     const unsigned char* in_nz;   // closure: flags of the input (NULL: every listed tile may be nonzero)
     int normalise_pass;      // closure in mode 1: divide by d_i (the first closure of a pass)
     unsigned* err;
@@ -741,35 +742,25 @@ __global__ void __launch_bounds__(256) k_closure(SweepArgs a) {
 }
 
 
-// The tile flags of the sweep's input in column-index order: entry p of tile
-// t's list (row cci_row[p], slot cci_slot[p]) gets the flag of that tile in
-// that row. The sweep kernels then test a block's rows for work with
-// contiguous reads of its tiles' column lists, with no dependence on the slot
-// loads, and raise both copies of a flag together. One CTA per tile.
+// The tile flags of the sweep's input in column-index order: entry k of tile
+// t's list (row cci_row[p], slot cci_slot[p], p = cci_ptr[t] + k) gets the flag
+// of that tile in that row, so that the sweep kernels test a block's rows for
+// work with contiguous reads, and raise both copies of a flag together. Every
+// tile's flags start on a 16-byte boundary and are zero up to the next one.
+__host__ __device__ constexpr size_t flag_bytes(size_t entries, size_t n_tiles) { return entries + 16 * n_tiles + 32; }
+__device__ __forceinline__ int flag_base(int tile, int ptr) { return ((ptr + 15) & ~15) + 16 * tile; }
+
+// One CTA per tile.
 __global__ void __launch_bounds__(256) k_flags_by_column(int cap, const int* __restrict__ cci_ptr,
                                                          const int* __restrict__ cci_row,
                                                          const int* __restrict__ cci_slot,
                                                          const unsigned char* __restrict__ nz,
                                                          unsigned char* __restrict__ col_nz) {
     const int t = blockIdx.x;
-    const int lo = cci_ptr[t], hi = cci_ptr[t + 1];
-    for (int p = lo + threadIdx.x; p < hi; p += blockDim.x) col_nz[p] = nz[(size_t)cci_row[p] * cap + cci_slot[p]];
-}
-
-// What a CTA of k_apply_full needs to start on block q of the pass (colour
-// order), gathered once per sweep so that it costs one load instead of a
-// chain of dependent ones: the block, its pair count and touched tiles, and
-// the column lists of the first tile of each side.
-template <int MODE>
-__global__ void k_block_info(SweepArgs a, int n, int4* __restrict__ info) {
-    const int q = blockIdx.x * blockDim.x + threadIdx.x;
-    if (q >= n) return;
-    const int e = a.blk[q];
-    const int A = a.gnb_row[e], B = a.gnb_col[e];
-    const int ta0 = a.group_ot0[A], tb0 = MODE == 0 ? a.group_vt0[B] : a.group_ot0[B];
-    const int pa = a.cci_ptr[ta0], pb = a.cci_ptr[tb0];
-    info[2 * q] = make_int4(e, a.pr_n[e], a.pr_touch[e], a.cci_ptr[ta0 + 1] - pa);
-    info[2 * q + 1] = make_int4(pa, pb, a.cci_ptr[tb0 + 1] - pb, 0);
+    const int lo = cci_ptr[t], n = cci_ptr[t + 1] - lo;
+    unsigned char* f = col_nz + flag_base(t, lo);
+    for (int k = threadIdx.x; k < ((n + 15) & ~15); k += blockDim.x)
+        f[k] = k < n ? nz[(size_t)cci_row[lo + k] * cap + cci_slot[lo + k]] : 0;
 }
 
 // side tiles of a block: up to 3 per side, as (first tile of a run, offset)
@@ -848,7 +839,7 @@ __global__ void __launch_bounds__(apply_threads<T>()) k_apply_colour(SweepArgs a
     __shared__ int s_lvl[kMaxSub + 1];
     __shared__ int s_row[CH];
     __shared__ int s_slot[CH][NT];
-    __shared__ int s_cp[NT];   // start of each panel tile's column list (-1: not held)
+    __shared__ int s_cp[NT];   // start of each panel tile's flags (-1: not held)
     // side A occupies panel tiles [0, kSideA), side B [kSideA, NT)
     constexpr int kSideA = MODE == 0 ? 2 : NT / 2;
     if (*a.err & (kErrCapacity | kErrSortSize)) return;
@@ -897,7 +888,7 @@ __global__ void __launch_bounds__(apply_threads<T>()) k_apply_colour(SweepArgs a
             if (i < sb.nrun0) tile = sb.run0 + i;
             else if (i < sb.n) tile = sb.run1 + (i - sb.nrun0);
         }
-        s_cp[p] = tile >= 0 ? a.cci_ptr[tile] : -1;
+        s_cp[p] = tile >= 0 ? flag_base(tile, a.cci_ptr[tile]) : -1;
     }
     __syncthreads();
     // a chunk whose held tiles are all flagged zero in all its rows stays as it
@@ -1070,41 +1061,78 @@ __global__ void __launch_bounds__(apply_threads<T>()) k_apply_colour(SweepArgs a
     }
 }
 
-// Blocks between full groups (8 molecules: 32 occupied and 16 virtual MOs per
-// group) in FP32 storage: rotations (MODE 0, A occupied x B virtual) and
-// occupied-pass combinations (MODE 1, A occupied x B occupied, A != B). The
-// in-block colour of such a block is (i + j) mod 32. Same updates, order and
-// truncation as k_apply_colour, laid out for fewer shared-memory round trips:
-// each thread owns a pair of adjacent AO rows; the 32 A-side values of those rows
-// stay in registers (the index i is static once the slot loop is unrolled),
-// the NB B-side values sit in a thread-private shared-memory panel indexed by
-// j = (level - i) mod 32. The block's pairs are expanded into a dense
-// [level][i] coefficient table with a selection mask per level. The level loop
-// needs no barrier: a thread reads back only the panel rows it wrote.
-// Row pairs whose touched tiles are all flagged zero (per-tile flags written by
-// the closure and raised by the sweep) are skipped: the updates would leave
-// those zeros as they are. The others are collected over several row chunks so
-// that the level loop runs in full warps.
-constexpr int kFullDenseMin = 12;                 // pairs in a level from which MODE 1 runs it without branches
-constexpr int kFullBatch = 8;                     // slots loaded ahead in a branch-free level (multiple of 4)
-constexpr int kFusedBatch = 4;                    // slots loaded ahead when two levels share a pass (even)
-constexpr int kFullMinCtas[2] = {6, 5};          // resident CTAs per SM the register budget is cut for
-constexpr int kFullWaves[2] = {16, 4};            // resident-CTA multiples per launch (fewer: more row chunks per CTA to collect from)
-constexpr int kFullCH = 32;                       // row blocks per CTA
-constexpr int kFullNR = kFullCH * kAoPerMol;      // AO rows per CTA (panel stride, floats)
-constexpr int kFullThreads = kFullNR / 2;         // one pair of adjacent AO rows per thread (two pairs measured slower)
-template <int MODE> struct FullShape;
-template <> struct FullShape<0> {   // rotations: B = one virtual tile, coefficients (c, c, s, s)
-    static constexpr int nb = 16;
-    using Coef = float4;
+// FP32 sweeps, one warp at a time. Same updates, order and truncation as
+// k_apply_colour; what differs is where the values sit and who waits for whom.
+//
+// A CTA serves a block (A, B) of the colour. It reads the tile flags of all the
+// block's rows: one bit per row block with work (where every touched tile is
+// flagged all-zero, the updates would leave the zeros as they are). The AO rows
+// of the row blocks with work, six each, are the block's work, in runs of 32
+// entries; CTA s of the block takes the s-th share of the runs, and its warps
+// take run after run from it and work on them alone, so only a block's last run
+// is not full. (A warp that listed its own chunk of the rows ran half-empty:
+// 68.9 -> 45.8 ms for an occupied pass at 4096 molecules. CTAs that stay and
+// take runs of other blocks when theirs are done were slower: 55 ms.)
+//
+// Two ways to run the updates of a block, by its number of pairs:
+//   dense   both sides of an entry's AO rows in registers (two adjacent rows
+//           packed in occupied passes, one in passes over all MOs). At level l
+//           slot i pairs x_i with y_((l - i) mod n); y is held in slot order and
+//           the value slot i has updated is the partner of slot i + 1 at the next
+//           level, so writing it to register i + 1 rotates y without a move. A
+//           slot without a pair has (c, t) = (0, 0), which leaves both values as
+//           they are. Per slot two FMAs, a compare and a multiply per value, and
+//           half a coefficient load: 7.6 clocks of an SM quarter per slot and row
+//           packed, 8.2 unpacked, in a loop of its own; the FMA and ALU pipes
+//           would take 4, the operand reads of the register file bound it.
+//   list    the block's pairs one after the other in schedule order, both sides
+//           in a shared-memory panel [column][lane], one AO row per lane. Self
+//           blocks, rotations, and combination blocks with few pairs.
+// n = max(MOs of A, MOs of B) is the modulus of the in-block colour; the dense
+// loop exists for every n a pair of groups can have, so blocks of partly filled
+// groups run it as well (their missing MOs are zero columns without pairs).
+// Measured (one pass or sweep, FP32; before: full groups in a kernel with one
+// side in registers, the others staged for the generic kernel): occupied pass
+// at 4096 molecules 68.9 -> 41.9 ms, at 997 9.9 -> 5.3; four passes over all
+// MOs at 512 18.6 -> 5.2; rotations at 4096 14.8 -> 9.6, at 997 3.2 -> 1.7.
+constexpr int kWsWarps = 4;
+constexpr int kWsThreads = 32 * kWsWarps;
+constexpr int kFullCH = 32;                  // row blocks per word of the bits of rows with work
+constexpr int kFullBatch = 8;                // 16-byte pieces of a tile per lane and run of 32 row pairs, all in flight
+// runs a CTA takes at least: one per warp, or two where a launch could have more than kWsManyRuns
+// runs per resident CTA (at 4096 molecules most shares are empty, and fewer of them are launched:
+// 43.0 -> 41.9 ms; at 997 one per warp spreads better, 5.8 -> 5.3)
+constexpr int kWsManyRuns = 32;
+// rotations: CTAs of a launch as a multiple of the resident ones (2, 4, 8, 16: 13.8, 10.8, 9.6, 9.5 ms
+// at 4096 molecules, 1.91, 1.88, 1.74, 1.74 at 997)
+constexpr int kWsRotWaves = 8;
+constexpr int kWsPad = 34;                   // floats per panel column: 16-byte pieces scatter over all banks
+// pairs from which a combination block runs dense, as a divisor of n^2: the dense loop costs
+// ~8 n^2 clocks per row whatever the number of pairs, the list ~15 per pair with more latency (3, 4,
+// 8: 5.7, 5.35, 5.2 ms for the passes over all MOs at 512 molecules; few blocks lie in between later)
+constexpr int kWsDenseDiv = 8;
+// MODE 0 rotations, MODE 1 combinations of occupied MOs (ALL = false) or of all MOs
+template <int MODE, bool ALL> struct WarpShape {
+    static constexpr int nta = ALL ? 3 : 2;                    // side tiles
+    static constexpr int ntb = MODE == 0 ? 1 : nta;
+    static constexpr int nmax = ALL ? 48 : 32;                 // largest modulus
+    static constexpr int gstep = ALL ? 6 : 4;                  // MOs per molecule and side
+    static constexpr int halves = MODE == 1 && !ALL ? 2 : 1;   // AO rows a lane holds in the dense loop
+    // bytes of the block's coefficients or pairs: MODE 0 at most kRotCap pairs of 16; MODE 1 a dense
+    // table of n^2 (c, t), or 8-byte pairs (fewer than n^2 / kWsDenseDiv, or n (n - 1) / 2 of a self
+    // block), and four ending the list
+    static constexpr int table = MODE == 0 ? (kRotCap + 4) * 16 : nmax * nmax * 8;
+    static_assert(MODE == 0 || (nmax * (nmax - 1) / 2 + 4) * 8 <= nmax * nmax * 8, "");
+    // bytes per warp: the list's panel; the dense loop's: one side of 32 row pairs (occupied passes),
+    // or a run's tiles as they lie in memory and the next run's (passes over all MOs)
+    static constexpr int raw = ALL ? (nta + ntb) * 32 * 64 : 0;
+    static constexpr int panel = (nta + ntb) * 16 * kWsPad * 4;
+    static constexpr int per_warp = 2 * raw > panel ? 2 * raw : panel;
+    static_assert(MODE == 0 || ALL || per_warp >= nta * 16 * 64 * 4, "");
+    static constexpr size_t smem = (size_t)table + (size_t)kWsWarps * per_warp;   // + row bits
+    // resident CTAs the register budget is cut for: the dense loop holds 2 n values per row
+    static constexpr int min_ctas = MODE == 0 ? 6 : (ALL ? 2 : 3);
 };
-template <> struct FullShape<1> {   // combinations: B = two occupied tiles, (-c, truncation threshold)
-    static constexpr int nb = 32;
-    using Coef = float2;
-};
-template <int MODE> __host__ __device__ constexpr size_t full_apply_smem() {
-    return (size_t)FullShape<MODE>::nb * kFullNR * 4 + (size_t)32 * 32 * sizeof(typename FullShape<MODE>::Coef);
-}
 
 // 1.0 where |v| >= t, 0.0 below (and for NaN): one compare that writes the
 // factor itself
@@ -1114,350 +1142,560 @@ __device__ __forceinline__ float ge_abs_factor(float v, float t) {
     return k;
 }
 
-// x with the values below t in magnitude set to zero, as a product with 0/1
-// factors: two compares on the ALU pipe and one packed multiply on the FMA
-// pipe instead of two compares and two selects (a value set to zero may come
-// out as -0, which every later test treats as zero)
-__device__ __forceinline__ float2 trunc2_mul(float2 v, float t) {
+// v with a value below t in magnitude set to zero, as a product with a 0/1
+// factor: a compare on the ALU pipe and a multiply on the FMA pipe instead of a
+// compare and a select on the ALU pipe, which has half the rate (a value set to
+// zero may come out as -0, which every later test treats as zero)
+__device__ __forceinline__ float trunc_mul(float v, float t) { return __fmul_rn(v, ge_abs_factor(v, t)); }
+__device__ __forceinline__ float fma_s(float c, float a, float b) { return __fmaf_rn(c, a, b); }
+
+__device__ __forceinline__ float2 trunc_mul(float2 v, float t) {
     return __fmul2_rn(v, make_float2(ge_abs_factor(v.x, t), ge_abs_factor(v.y, t)));
 }
+__device__ __forceinline__ float2 fma_s(float c, float2 a, float2 b) { return __ffma2_rn(make_float2(c, c), a, b); }
 
-__device__ __forceinline__ void load_pair_rows(const float* src, float4 (&r0)[4], float4 (&r1)[4]) {
-    const float4* s = (const float4*)src;
+// The NS levels of a block on a lane's AO rows (V: one, or two packed). Slots
+// run downwards: the updated partner of slot i goes to register i + 1, whose old
+// value slot i + 1 has already used; slot NS - 1's goes to register 0 at the end
+// of the level.
+template <int NS, typename V>
+__device__ __forceinline__ void dense_levels(V (&x)[NS], V (&ys)[NS], const float2* coef) {
+    static_assert(NS % 2 == 0, "");
+#pragma unroll 1
+    for (int lv = 0; lv < NS; ++lv) {
+        const float4* c4 = (const float4*)(coef + lv * NS);
+        V carry;
 #pragma unroll
-    for (int v = 0; v < 4; ++v) {
-        r0[v] = s[v];
-        r1[v] = s[4 + v];   // next AO row: 16 floats on
+        for (int h = NS / 2 - 1; h >= 0; --h) {
+            const float4 q = c4[h];
+#pragma unroll
+            for (int u = 1; u >= 0; --u) {
+                const int i = 2 * h + u;
+                const float c = u ? q.z : q.x, t = u ? q.w : q.y;
+                const V xn = fma_s(c, ys[i], x[i]);
+                const V yn = fma_s(c, x[i], ys[i]);
+                x[i] = trunc_mul(xn, t);
+                const V yt = trunc_mul(yn, t);
+                if (i == NS - 1) carry = yt;
+                else ys[i + 1] = yt;
+            }
+        }
+        ys[0] = carry;
     }
 }
 
-template <int MODE>
-__global__ void __launch_bounds__(kFullThreads, kFullMinCtas[MODE]) k_apply_full(SweepArgs a, int p0) {
-    constexpr int NB = FullShape<MODE>::nb;
-    using Coef = typename FullShape<MODE>::Coef;
+__device__ __forceinline__ void cp_async16(void* dst, const void* src, bool in) {   // zeros where !in
+    const unsigned d = (unsigned)__cvta_generic_to_shared(dst);
+    const int n = in ? 16 : 0;
+    asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(d), "l"(src), "r"(n) : "memory");
+}
+
+// What a CTA of k_apply_warp needs to start on block q of the pass (colour
+// order), gathered once per sweep so that it costs one load instead of a chain
+// of dependent ones: (block, pairs, touched tiles, rows), (column lists of the
+// sides' first tiles, rows of B, molecules of A and of B), (column lists of the
+// sides' virtual tiles in passes over all MOs), (flags of each side's tiles).
+struct BlockInfo {
+    int4 i0, i1, i2;
+    int flagA[3], flagB[3];
+};
+template <int MODE, bool ALL>
+__global__ void k_block_info(SweepArgs a, int n, BlockInfo* __restrict__ info) {
+    const int q = blockIdx.x * blockDim.x + threadIdx.x;
+    if (q >= n) return;
+    const int e = a.blk[q];
+    const int A = a.gnb_row[e], B = a.gnb_col[e];
+    const int ta0 = a.group_ot0[A], tb0 = MODE == 0 ? a.group_vt0[B] : a.group_ot0[B];
+    const int pa = a.cci_ptr[ta0], pb = a.cci_ptr[tb0];
+    int touch = a.pr_touch[e];
+    const bool same = MODE == 1 && A == B;
+    if (same) touch |= touch >> 3;   // one set of tiles, held as side A
+    BlockInfo b;
+    b.i0 = make_int4(e, a.pr_n[e], touch, a.cci_ptr[ta0 + 1] - pa);
+    b.i1 = make_int4(pa, pb, a.cci_ptr[tb0 + 1] - pb, a.group_nmol[A] | (a.group_nmol[B] << 8) | ((int)same << 16));
+    b.i2 = make_int4(ALL ? a.cci_ptr[a.group_vt0[A]] : 0, ALL ? a.cci_ptr[a.group_vt0[B]] : 0, 0, 0);
+    for (int t = 0; t < 3; ++t) {
+        const int ta = t < a.group_not[A] ? ta0 + t : a.group_vt0[A];
+        const int tb = MODE == 0 ? tb0 : (t < a.group_not[B] ? tb0 + t : a.group_vt0[B]);
+        b.flagA[t] = flag_base(ta, a.cci_ptr[ta]);
+        b.flagB[t] = flag_base(tb, a.cci_ptr[tb]);
+    }
+    info[q] = b;
+    // the 2x2 row updates the algorithm defines, rows proven unchanged and skipped included
+    const int col = a.gnb_colour[e];
+    if (b.i0.y && col >= a.col_lo && col < a.col_hi)
+        atomicAdd(a.upd, (unsigned long long)b.i0.y * (unsigned long long)(b.i0.w * kAoPerMol));
+}
+
+template <int MODE, bool ALL>
+__global__ void __launch_bounds__(kWsThreads, (WarpShape<MODE, ALL>::min_ctas))
+k_apply_warp(SweepArgs a, int p0, int nb, int min_runs) {
+    using Sh = WarpShape<MODE, ALL>;
+    constexpr int NTA = Sh::nta, NTB = Sh::ntb;
     extern __shared__ __align__(16) unsigned char smraw[];
-    float* panel = (float*)smraw;                           // [NB B columns][kFullNR rows]
-    Coef* coef = (Coef*)(panel + NB * kFullNR);             // [32 levels][32 i]
-    __shared__ unsigned s_mask[32];
+    __shared__ int s_wsum[kWsWarps], s_next;
     if (*a.err & (kErrCapacity | kErrSortSize)) return;
-    const int4 i0 = a.blk_info[2 * (p0 + blockIdx.y)], i1 = a.blk_info[2 * (p0 + blockIdx.y) + 1];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const BlockInfo& info = ((const BlockInfo*)a.blk_info)[p0 + blockIdx.x % nb];
+    const int4 i0 = info.i0, i1 = info.i1, i2 = info.i2;
     const int e = i0.x, np = i0.y, touch = i0.z, n_rows = i0.w;
-    const int pa = i1.x, pb = i1.y;
     if (np == 0) return;
-    // CTA x takes row chunks x, x + gridDim.x, ... of the block, so its
-    // coefficient table serves several chunks
-    const int k_first = blockIdx.x * kFullCH;
-    if (k_first >= n_rows) return;
+    const int pa = i1.x, pb = i1.y;
     if (i1.z != n_rows) {
         if (threadIdx.x == 0) atomicOr(a.err, kErrCapacity);
         return;
     }
-    // rotations read only the slots that hold a pair (the mask's bits); the
-    // dense levels of occupied passes read every slot, so those start at zero
-    if constexpr (MODE == 1)
-        for (int i = threadIdx.x; i < 32 * 32; i += blockDim.x) coef[i] = make_float2(0.f, 0.f);
-    if (threadIdx.x < 32) s_mask[threadIdx.x] = 0u;
-    __syncthreads();
-    const float* cs = (const float*)a.pr_cs + (size_t)e * kOrthoCap * 2;
-    const uint16_t* ij = a.pr_ij + (size_t)e * kOrthoCap;
-    for (int q = threadIdx.x; q < np; q += blockDim.x) {
-        const unsigned w = ij[q];
-        const int il = w & 255, jl = w >> 8, lv = (il + jl) & 31;
-        const float c = cs[2 * q];
-        if constexpr (MODE == 0) {
-            const float sn = cs[2 * q + 1];
-            coef[lv * 32 + il] = make_float4(c, c, sn, sn);
-        } else {
-            coef[lv * 32 + il] = make_float2(-c, a.trunc_f);   // a slot without a pair keeps (0, 0)
+    const int mA = i1.w & 255, mB = (i1.w >> 8) & 255;
+    const bool same = (i1.w >> 16) & 1;
+    // occupied MOs and tiles of both sides, MOs of the pass on each side
+    const int noA = 4 * mA, noB = MODE == 0 ? 0 : 4 * mB;
+    const int otA = (noA + 15) >> 4, otB = MODE == 0 ? 0 : (noB + 15) >> 4;
+    const int nA = MODE == 0 ? noA : Sh::gstep * mA, nB = MODE == 0 ? 2 * mB : Sh::gstep * mB;
+    const int n = max(nA, nB);
+    // bits of the row blocks with work, 16 flags per load (a tile's flags start on 16 bytes and are
+    // zero past its last row), then the bits before each word
+    unsigned* bits = (unsigned*)(smraw + Sh::smem);
+    const int nw = (n_rows + kFullCH - 1) / kFullCH;
+    int* wpre = (int*)(bits + nw);
+    for (int hw = threadIdx.x; hw < 2 * nw; hw += kWsThreads) {
+        uint4 f = make_uint4(0u, 0u, 0u, 0u);
+        if (16 * hw < n_rows) {
+#pragma unroll
+            for (int t = 0; t < NTA + NTB; ++t) {
+                const bool sideB = t >= NTA;
+                const int tt = sideB ? t - NTA : t;
+                if (!(touch >> (sideB ? 3 + tt : tt) & 1)) continue;
+                const uint4 v = *(const uint4*)(a.col_nz + (sideB ? info.flagB[tt] : info.flagA[tt]) + 16 * (size_t)hw);
+                f.x |= v.x;
+                f.y |= v.y;
+                f.z |= v.z;
+                f.w |= v.w;
+            }
         }
-        atomicOr(&s_mask[lv], 1u << il);
+        // four 0/1 bytes of a word to four bits: byte i lands on bit 24 + i
+        constexpr unsigned kGather = 0x01020408u;
+        ((unsigned short*)bits)[hw] = (unsigned short)((f.x * kGather >> 24 & 15u) | (f.y * kGather >> 24 & 15u) << 4 |
+                                                       (f.z * kGather >> 24 & 15u) << 8 | (f.w * kGather >> 24 & 15u) << 12);
     }
     __syncthreads();
-    // tiles no selected pair touches (touch bits clear) keep their values:
-    // neither loaded nor stored
-    float* val = (float*)a.out_val;   // in place
-    // The side tiles of a unit are consecutive tile ids with equal column
-    // lists, so side tile t's list starts t * n_rows after the first one's.
-    // Each row chunk first tells, per row pair, whether it has work: a row pair
-    // whose touched tiles are all flagged zero stays zero under the block's
-    // updates (x - c y and c x + s y of zeros, truncation keeps zeros), and so
-    // does a flagged row pair of zeros that runs through them. The row pairs
-    // with work are appended to a shared list; once it holds a CTA's worth,
-    // every thread takes one, loads both sides and runs the updates, so that the
-    // level loop runs in full warps. The rest runs at the end. The flags are
-    // read in column-index order (contiguous for consecutive rows of the
-    // block), together with the rows and slots the run needs.
-    __shared__ int s_list[2 * kFullThreads];   // row pairs with work, not yet run
-    __shared__ int s_lrow[2 * kFullThreads];   // their row block and the slots of both sides there
-    __shared__ int s_lsa[2 * kFullThreads];
-    __shared__ int s_lsb[2 * kFullThreads];
-    __shared__ int s_wcnt[kFullThreads / 32];
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    const int rb = threadIdx.x / 3;   // own row block (of the chunk)
-    // the updates of one row pair with work: entry = (row block in the block's
-    // row list) * 3 + pair
-    auto run = [&](const int ent, const int row, const int slA, const int slB) {
-        const int kr = ent / 3, k2s = 2 * (ent - 3 * kr);
-        const size_t baseA = ((size_t)row * a.cap + slA) * kTileVals + k2s * kTileW;
-        const size_t baseB = ((size_t)row * a.cap + slB) * kTileVals + k2s * kTileW;
-        // the B side goes to the thread's own panel rows (consecutive threads,
-        // consecutive 8-byte words: no bank conflicts in the level loop)
-        float* ps = panel + 2 * threadIdx.x;
+    const int wper = (nw + kWsThreads - 1) / kWsThreads;
+    const int wlo = min(nw, (int)threadIdx.x * wper), whi = min(nw, wlo + wper);
+    int cnt = 0;
+    for (int w = wlo; w < whi; ++w) cnt += __popc(bits[w]);
+    int inc = cnt;
 #pragma unroll
-        for (int t = 0; t < NB / 16; ++t) {
-            float4 v0[4], v1[4];
-            if (touch >> (3 + t) & 1) {
-                load_pair_rows(val + baseB + (size_t)t * kTileVals, v0, v1);
-            } else {
+    for (int o = 1; o < 32; o <<= 1) {
+        const int v = __shfl_up_sync(0xffffffffu, inc, o);
+        if (lane >= o) inc += v;
+    }
+    if (lane == 31) s_wsum[warp] = inc;
+    __syncthreads();
+    int n_work = 0, before = inc - cnt;
 #pragma unroll
-                for (int v = 0; v < 4; ++v) v0[v] = v1[v] = make_float4(0.f, 0.f, 0.f, 0.f);
-            }
+    for (int w = 0; w < kWsWarps; ++w) {
+        before += w < warp ? s_wsum[w] : 0;
+        n_work += s_wsum[w];
+    }
+    const bool dense = MODE == 1 && !same && np * kWsDenseDiv >= n * n;
+    const int hh = dense ? Sh::halves : 1;   // AO rows of a lane's entry (adjacent ones)
+    const int n_ent = kAoPerMol / hh * n_work, n_run = (n_ent + 31) / 32;
+    const int share = blockIdx.x / nb, shares = gridDim.x / nb;
+    const int per = max(min_runs, (n_run + shares - 1) / shares);
+    const int run_lo = share * per, run_hi = min(n_run, run_lo + per);
+    if (run_lo >= run_hi) return;
+    if (threadIdx.x == 0) s_next = run_lo;
+    for (int w = wlo; w < whi; ++w) {
+        wpre[w] = before;
+        before += __popc(bits[w]);
+    }
+    // panel column of a side's local MO: occupied MOs from column 0, virtual ones (passes over
+    // all MOs) from the tile after the occupied ones
+    auto colA = [&](int i) { return MODE == 0 || !ALL || i < noA ? i : 16 * otA + i - noA; };
+    auto colB = [&](int j) { return MODE == 0 || !ALL || j < noB ? j : 16 * otB + j - noB; };
+    // table (dense) or list of the block's pairs
+    const float* cs = (const float*)a.pr_cs + (size_t)e * kOrthoCap * 2;
+    const uint16_t* ij = a.pr_ij + (size_t)e * kOrthoCap;
+    float2* table = (float2*)smraw;
+    float2* pair2 = (float2*)smraw;
+    float4* pair4 = (float4*)smraw;
+    if (dense) {
+        for (int i = threadIdx.x; i < n * n; i += kWsThreads) table[i] = make_float2(0.f, 0.f);
+        __syncthreads();
+    }
+    for (int q = threadIdx.x; q < np; q += kWsThreads) {
+        const int w = ij[q], il = w & 255, jl = w >> 8;
+        const int s = il + jl, lv = s >= n ? s - n : s;
+        const float2 c = ((const float2*)cs)[q];
+        // list: panel offsets of both sides (12 bits each) and, between them, the level
+        const unsigned off = (unsigned)(colA(il) * kWsPad) | (unsigned)lv << 12 |
+                             ((unsigned)(((same ? 0 : 16 * NTA) + colB(jl)) * kWsPad) << 18);
+        if constexpr (MODE == 0) pair4[q] = make_float4(__uint_as_float(off), c.x, c.y, 0.f);
+        else if (dense) table[lv * n + il] = make_float2(-c.x, a.trunc_f);
+        else pair2[q] = make_float2(__uint_as_float(off), -c.x);
+    }
+    if (!dense && threadIdx.x < 4) {   // ends the list: a level of its own
+        if constexpr (MODE == 0) pair4[np + threadIdx.x] = make_float4(__uint_as_float(63u << 12), 0.f, 0.f, 0.f);
+        else pair2[np + threadIdx.x] = make_float2(__uint_as_float(63u << 12), 0.f);
+    }
+    __syncthreads();
+    float* const mem = (float*)(smraw + Sh::table + (size_t)warp * Sh::per_warp);   // the warp's
+    float* const val = (float*)a.out_val;                                           // in place
+    // the block's pairs on the panel, in schedule order (lanes hold different rows)
+    auto run_list = [&](bool active) {
+        // pairs of one level touch different columns: up to four of them in flight
+        if (active) {
+            auto upd = [&](int q, auto width) {
+                constexpr int N = decltype(width)::value;
+                float *px[N], *py[N], xv[N], yv[N], c0[N], c1[N];
 #pragma unroll
-            for (int v = 0; v < 4; ++v) {
-                *(float2*)(ps + (t * 16 + 4 * v + 0) * kFullNR) = make_float2(v0[v].x, v1[v].x);
-                *(float2*)(ps + (t * 16 + 4 * v + 1) * kFullNR) = make_float2(v0[v].y, v1[v].y);
-                *(float2*)(ps + (t * 16 + 4 * v + 2) * kFullNR) = make_float2(v0[v].z, v1[v].z);
-                *(float2*)(ps + (t * 16 + 4 * v + 3) * kFullNR) = make_float2(v0[v].w, v1[v].w);
-            }
-        }
-        float2 x[32];
-#pragma unroll
-        for (int t = 0; t < 2; ++t) {
-            float4 u0[4], u1[4];
-            if (touch >> t & 1) {
-                load_pair_rows(val + baseA + (size_t)t * kTileVals, u0, u1);
-            } else {
-#pragma unroll
-                for (int v = 0; v < 4; ++v) u0[v] = u1[v] = make_float4(0.f, 0.f, 0.f, 0.f);
-            }
-#pragma unroll
-            for (int v = 0; v < 4; ++v) {
-                x[t * 16 + 4 * v + 0] = make_float2(u0[v].x, u1[v].x);
-                x[t * 16 + 4 * v + 1] = make_float2(u0[v].y, u1[v].y);
-                x[t * 16 + 4 * v + 2] = make_float2(u0[v].z, u1[v].z);
-                x[t * 16 + 4 * v + 3] = make_float2(u0[v].w, u1[v].w);
-            }
-        }
-        const float tf = a.trunc_f;
-        for (int lv = 0; lv < 32; ++lv) {
-            const unsigned m = s_mask[lv];
-            if (m == 0u) continue;
-            const Coef* cl = coef + lv * 32;
-            if constexpr (MODE == 1) {
-                if (__popc(m) >= kFullDenseMin) {
-                    // Most slots of the level hold a pair: all 32 run without a
-                    // branch; a slot without a pair (c = 0, threshold 0) leaves
-                    // both of its values as they are. Each slot reads (c, t) from
-                    // the table, two slots per 16-byte load.
-                    if (lv + 1 < 32 && __popc(s_mask[lv + 1]) >= kFullDenseMin) {
-                        // Two dense levels in one pass over the slots. Slot i of
-                        // level lv+1 pairs x_i with y_(lv+1-i), the value slot i-1
-                        // has just updated at level lv: it stays in a register for
-                        // its second update and is stored once. Slot 0's level-lv+1
-                        // partner, y_(lv+1), is last updated at level lv by slot 31,
-                        // so that update comes after the pass. Every value sees its
-                        // updates in level order, as in the one-level pass.
-                        const float4* ca4 = (const float4*)cl;
-                        const float4* cb4 = (const float4*)(cl + 32);
-                        float2 yprev = make_float2(0.f, 0.f);
-#pragma unroll
-                        for (int i0 = 0; i0 < 32; i0 += kFusedBatch) {
-                            float2 yv[kFusedBatch];
-                            float4 ca[kFusedBatch / 2], cb[kFusedBatch / 2];
-#pragma unroll
-                            for (int u = 0; u < kFusedBatch / 2; ++u) {
-                                ca[u] = ca4[i0 / 2 + u];
-                                cb[u] = cb4[i0 / 2 + u];
-                            }
-#pragma unroll
-                            for (int u = 0; u < kFusedBatch; ++u)
-                                yv[u] = *(const float2*)(ps + ((lv - i0 - u) & 31) * kFullNR);
-#pragma unroll
-                            for (int u = 0; u < kFusedBatch; ++u) {
-                                const int i = i0 + u;
-                                const float c0 = (u & 1) ? ca[u / 2].z : ca[u / 2].x;
-                                const float t0 = (u & 1) ? ca[u / 2].w : ca[u / 2].y;
-                                const float2 cc0 = make_float2(c0, c0);
-                                const float2 xn = __ffma2_rn(cc0, yv[u], x[i]);
-                                const float2 yn = __ffma2_rn(cc0, x[i], yv[u]);
-                                x[i] = trunc2_mul(xn, t0);
-                                const float2 ynew = trunc2_mul(yn, t0);
-                                if (i > 0) {
-                                    const float c1 = (u & 1) ? cb[u / 2].z : cb[u / 2].x;
-                                    const float t1 = (u & 1) ? cb[u / 2].w : cb[u / 2].y;
-                                    const float2 cc1 = make_float2(c1, c1);
-                                    const float2 xn1 = __ffma2_rn(cc1, yprev, x[i]);
-                                    const float2 yn1 = __ffma2_rn(cc1, x[i], yprev);
-                                    x[i] = trunc2_mul(xn1, t1);
-                                    *(float2*)(ps + ((lv + 1 - i) & 31) * kFullNR) = trunc2_mul(yn1, t1);
-                                }
-                                yprev = ynew;
-                            }
-                        }
-                        {   // slot 0 of level lv+1 with y_(lv+1)
-                            const float2 ct = cl[32];
-                            const float2 cc1 = make_float2(ct.x, ct.x);
-                            const float2 xn1 = __ffma2_rn(cc1, yprev, x[0]);
-                            const float2 yn1 = __ffma2_rn(cc1, x[0], yprev);
-                            x[0] = trunc2_mul(xn1, ct.y);
-                            *(float2*)(ps + ((lv + 1) & 31) * kFullNR) = trunc2_mul(yn1, ct.y);
-                        }
-                        ++lv;
-                        continue;
-                    }
-                    const float4* cl4 = (const float4*)cl;
-#pragma unroll
-                    for (int i0 = 0; i0 < 32; i0 += kFullBatch) {
-                        float2 yv[kFullBatch];
-                        float4 cv[kFullBatch / 2];
-#pragma unroll
-                        for (int u = 0; u < kFullBatch / 2; ++u) cv[u] = cl4[i0 / 2 + u];
-#pragma unroll
-                        for (int u = 0; u < kFullBatch; ++u)
-                            yv[u] = *(const float2*)(ps + ((lv - i0 - u) & 31) * kFullNR);
-#pragma unroll
-                        for (int u = 0; u < kFullBatch; ++u) {
-                            const int i = i0 + u;
-                            const float c = (u & 1) ? cv[u / 2].z : cv[u / 2].x;
-                            const float t = (u & 1) ? cv[u / 2].w : cv[u / 2].y;
-                            const float2 cc = make_float2(c, c);
-                            const float2 xn = __ffma2_rn(cc, yv[u], x[i]);
-                            const float2 yn = __ffma2_rn(cc, x[i], yv[u]);
-                            x[i] = trunc2_mul(xn, t);
-                            *(float2*)(ps + ((lv - i) & 31) * kFullNR) = trunc2_mul(yn, t);
-                        }
-                    }
-                    continue;
-                }
-            }
-#pragma unroll
-            for (int i = 0; i < 32; ++i) {
-                if (m & (1u << i)) {
-                    float2* py = (float2*)(ps + ((lv - i) & 31) * kFullNR);
-                    const Coef c4 = cl[i];
-                    const float2 y = *py;
-                    float2 xn, yn;
+                for (int u = 0; u < N; ++u) {
+                    unsigned off;
                     if constexpr (MODE == 0) {
-                        const float2 cc = make_float2(c4.x, c4.y);
-                        xn = __ffma2_rn(cc, x[i], __fmul2_rn(make_float2(c4.z, c4.w), y));
-                        yn = __ffma2_rn(cc, y, __fmul2_rn(make_float2(-c4.z, -c4.w), x[i]));
+                        const float4 c = pair4[q + u];
+                        off = __float_as_uint(c.x);
+                        c0[u] = c.y;
+                        c1[u] = c.z;
                     } else {
-                        const float2 cc = make_float2(c4.x, c4.x);
-                        xn = __ffma2_rn(cc, y, x[i]);
-                        yn = __ffma2_rn(cc, x[i], y);
+                        const float2 c = pair2[q + u];
+                        off = __float_as_uint(c.x);
+                        c0[u] = c.y;
+                        c1[u] = 0.f;
                     }
-                    x[i] = trunc2(xn, tf);
-                    *py = trunc2(yn, tf);
+                    px[u] = mem + (off & 0xfffu) + lane;
+                    py[u] = mem + (off >> 18) + lane;
+                    xv[u] = *px[u];
+                    yv[u] = *py[u];
                 }
-            }
-        }
-        // store, and mark the tiles that hold a nonzero value now (a flag is
-        // never cleared during the sweep: 1 only means "may be nonzero")
-        unsigned char* f = a.out_nz + (size_t)row * a.cap;
 #pragma unroll
-        for (int t = 0; t < 2; ++t) {
-            if (!(touch >> t & 1)) continue;
-            float4* d0 = (float4*)(val + baseA + (size_t)t * kTileVals);
-            bool any = false;
-#pragma unroll
-            for (int v = 0; v < 4; ++v) {
-                const float2 a0 = x[t * 16 + 4 * v], a1 = x[t * 16 + 4 * v + 1];
-                const float2 a2 = x[t * 16 + 4 * v + 2], a3 = x[t * 16 + 4 * v + 3];
-                d0[v] = make_float4(a0.x, a1.x, a2.x, a3.x);
-                d0[4 + v] = make_float4(a0.y, a1.y, a2.y, a3.y);
-                any |= a0.x != 0.f || a0.y != 0.f || a1.x != 0.f || a1.y != 0.f || a2.x != 0.f ||
-                       a2.y != 0.f || a3.x != 0.f || a3.y != 0.f;
-            }
-            if (any) {
-                f[slA + t] = 1;
-                a.col_nz[pa + t * n_rows + kr] = 1;
-            }
-        }
-#pragma unroll
-        for (int t = 0; t < NB / 16; ++t) {
-            if (!(touch >> (3 + t) & 1)) continue;
-            float4* d1 = (float4*)(val + baseB + (size_t)t * kTileVals);
-            bool any = false;
-#pragma unroll
-            for (int v = 0; v < 4; ++v) {
-                const float2 b0 = *(const float2*)(ps + (t * 16 + 4 * v + 0) * kFullNR);
-                const float2 b1 = *(const float2*)(ps + (t * 16 + 4 * v + 1) * kFullNR);
-                const float2 b2 = *(const float2*)(ps + (t * 16 + 4 * v + 2) * kFullNR);
-                const float2 b3 = *(const float2*)(ps + (t * 16 + 4 * v + 3) * kFullNR);
-                d1[v] = make_float4(b0.x, b1.x, b2.x, b3.x);
-                d1[4 + v] = make_float4(b0.y, b1.y, b2.y, b3.y);
-                any |= b0.x != 0.f || b0.y != 0.f || b1.x != 0.f || b1.y != 0.f || b2.x != 0.f ||
-                       b2.y != 0.f || b3.x != 0.f || b3.y != 0.f;
-            }
-            if (any) {
-                f[slB + t] = 1;
-                a.col_nz[pb + t * n_rows + kr] = 1;
+                for (int u = 0; u < N; ++u) {
+                    float xn, yn;
+                    if constexpr (MODE == 0) {
+                        xn = __fmaf_rn(c0[u], xv[u], __fmul_rn(c1[u], yv[u]));
+                        yn = __fmaf_rn(c0[u], yv[u], __fmul_rn(-c1[u], xv[u]));
+                    } else {
+                        xn = __fmaf_rn(c0[u], yv[u], xv[u]);
+                        yn = __fmaf_rn(c0[u], xv[u], yv[u]);
+                    }
+                    *px[u] = below(xn, a) ? 0.f : xn;
+                    *py[u] = below(yn, a) ? 0.f : yn;
+                }
+            };
+            auto level = [&](int q) {
+                unsigned off;
+                if constexpr (MODE == 0) off = __float_as_uint(pair4[q].x);
+                else off = __float_as_uint(pair2[q].x);
+                return off >> 12 & 63u;
+            };
+            for (int q = 0; q < np;) {
+                const unsigned l = level(q);
+                if (level(q + 3) == l) {
+                    upd(q, std::integral_constant<int, 4>());
+                    q += 4;
+                } else if (level(q + 1) == l) {
+                    upd(q, std::integral_constant<int, 2>());
+                    q += 2;
+                } else {
+                    upd(q, std::integral_constant<int, 1>());
+                    q += 1;
+                }
             }
         }
     };
-    int n_acc = 0;   // entries in s_list (the same in every thread)
-    int k0 = k_first;
-    // one call site of the update code (it is large): collect row pairs until
-    // a CTA's worth is listed or the block's rows run out, then run them
-    for (;;) {
-        while (n_acc < kFullThreads && k0 < n_rows) {
-            const int nk = min(kFullCH, n_rows - k0);
-            // the counter holds the 2x2 row updates the algorithm defines, rows proven
-            // unchanged and skipped included
-            if (threadIdx.x == 0) atomicAdd(a.upd, (unsigned long long)np * (unsigned long long)(nk * 6));
-            bool work = false;
-            int row = 0, slA = 0, slB = 0;
-            if (rb < nk) {
-                const int k = k0 + rb;
-                row = a.cci_row[pa + k];
-                slA = a.cci_slot[pa + k];
-                slB = a.cci_slot[pb + k];
-#pragma unroll
-                for (int t = 0; t < 2; ++t) work |= (touch >> t & 1) && a.col_nz[pa + t * n_rows + k];
-#pragma unroll
-                for (int t = 0; t < NB / 16; ++t) work |= (touch >> (3 + t) & 1) && a.col_nz[pb + t * n_rows + k];
-            }
-            // pack the row pairs with work to the first threads
-            const unsigned bal = __ballot_sync(0xffffffffu, work);
-            if (lane == 0) s_wcnt[warp] = __popc(bal);
-            __syncthreads();
-            int before = 0, n_work = 0;
-#pragma unroll
-            for (int w = 0; w < kFullThreads / 32; ++w) {
-                before += w < warp ? s_wcnt[w] : 0;
-                n_work += s_wcnt[w];
-            }
-            if (work) {
-                const int i = n_acc + before + __popc(bal & ((1u << lane) - 1u));
-                s_list[i] = 3 * k0 + threadIdx.x;
-                s_lrow[i] = row;
-                s_lsa[i] = slA;
-                s_lsb[i] = slB;
-            }
-            n_acc += n_work;
-            k0 += gridDim.x * kFullCH;
-            __syncthreads();
+    const int qe = lane >> 2, qp = lane & 3;   // row (mod 8) and 16-byte piece of it that a lane moves
+    // an AO row of a run: the tiles (row block * cap + slot) its first occupied tile and its virtual
+    // one have on either side, and 8 * position in the block's row list + AO row of the row block
+    struct Row {
+        unsigned a, b, av, bv;
+        int k;
+    };
+    auto look_up = [&](int run) {
+        Row r{0, 0, 0, 0, 0};
+        const int idx = 32 * run + lane, per_mol = kAoPerMol / hh;
+        if (idx >= n_ent) return r;
+        const int rank = hh == 2 ? idx / 3 : idx / kAoPerMol;   // its row block is the rank-th set bit
+        int lo = 0, hi = nw;                // last word with wpre <= rank
+        while (hi - lo > 1) {
+            const int mid = (lo + hi) >> 1;
+            if (wpre[mid] <= rank) lo = mid;
+            else hi = mid;
         }
-        if (n_acc == 0) break;
-        const int take = min(n_acc, kFullThreads);
-        const bool mine = (int)threadIdx.x < take;
-        int ent = 0, erow = 0, esa = 0, esb = 0;
-        if (mine) {
-            ent = s_list[threadIdx.x];
-            erow = s_lrow[threadIdx.x];
-            esa = s_lsa[threadIdx.x];
-            esb = s_lsb[threadIdx.x];
+        unsigned w = bits[lo];
+        int left = rank - wpre[lo], pos = 0;
+#pragma unroll
+        for (int half = 16; half > 0; half >>= 1) {
+            const unsigned low = w & ((1u << half) - 1u);
+            const int c = __popc(low);
+            if (left >= c) {
+                left -= c;
+                pos += half;
+                w >>= half;
+            } else {
+                w = low;
+            }
         }
-        __syncthreads();   // entries read: move the rest (fewer than a CTA's worth) to the front
-        for (int i = threadIdx.x; i < n_acc - take; i += blockDim.x) {
-            s_list[i] = s_list[take + i];
-            s_lrow[i] = s_lrow[take + i];
-            s_lsa[i] = s_lsa[take + i];
-            s_lsb[i] = s_lsb[take + i];
+        const int k = 32 * lo + pos;
+        const unsigned row0 = (unsigned)a.cci_row[pa + k] * (unsigned)a.cap;
+        r.a = row0 + (unsigned)a.cci_slot[pa + k];
+        r.b = row0 + (unsigned)a.cci_slot[pb + k];
+        if constexpr (ALL) {
+            r.av = row0 + (unsigned)a.cci_slot[i2.x + k];
+            r.bv = row0 + (unsigned)a.cci_slot[i2.y + k];
         }
-        n_acc -= take;
-        if (mine) run(ent, erow, esa, esb);
-        __syncthreads();   // the list is rewritten by the next chunk
+        r.k = 8 * k + (idx - per_mol * rank) * hh;
+        return r;
+    };
+    auto touched = [&](int t) { return (touch >> (t >= NTA ? 3 + t - NTA : t) & 1) && !(t >= NTA && same); };
+    // panel tile t of a row, and the row's 16 values there
+    auto tile_of = [&](const Row& r, int t) {
+        const bool sideB = t >= NTA;
+        const int tt = sideB ? t - NTA : t;
+        if (ALL && tt >= (sideB ? otB : otA)) return sideB ? r.bv : r.av;
+        return (sideB ? r.b : r.a) + (unsigned)tt;
+    };
+    auto values = [&](const Row& r, unsigned tile) { return val + (size_t)tile * kTileVals + (r.k & 7) * kTileW; };
+    // of a value written nonzero: the tile's flags (1 only means "may be nonzero")
+    auto raise = [&](const Row& r, int t, unsigned tile) {
+        a.out_nz[tile] = 1;
+        a.col_nz[(t >= NTA ? info.flagB[t - NTA] : info.flagA[t]) + (r.k >> 3)] = 1;
+    };
+    auto row_from = [&](const Row& r, int src) {   // lane src's row
+        Row o{0, 0, 0, 0, 0};
+        o.a = __shfl_sync(0xffffffffu, r.a, src);
+        o.b = __shfl_sync(0xffffffffu, r.b, src);
+        if constexpr (ALL) {
+            o.av = __shfl_sync(0xffffffffu, r.av, src);
+            o.bv = __shfl_sync(0xffffffffu, r.bv, src);
+        }
+        o.k = __shfl_sync(0xffffffffu, r.k, src);
+        return o;
+    };
+    auto grab = [&]() { return lane == 0 ? atomicAdd(&s_next, 1) : 0; };
+    int run = __shfl_sync(0xffffffffu, grab(), 0);
+    if (run >= run_hi) return;
+    if (MODE == 0 || !dense) {
+        float* const pq = mem + 4 * qp * kWsPad + qe;
+        while (run < run_hi) {
+            const Row r = look_up(run);
+            const int grabbed = grab();
+            const int take = min(32, n_ent - 32 * run);
+            float4 v[NTA + NTB][4];
+#pragma unroll
+            for (int u = 0; u < 4; ++u) {
+                const Row o = row_from(r, 8 * u + qe);
+#pragma unroll
+                for (int t = 0; t < NTA + NTB; ++t) {
+                    v[t][u] = make_float4(0.f, 0.f, 0.f, 0.f);
+                    if (8 * u + qe < take && touched(t)) v[t][u] = *((const float4*)values(o, tile_of(o, t)) + qp);
+                }
+            }
+#pragma unroll
+            for (int t = 0; t < NTA + NTB; ++t)
+#pragma unroll
+                for (int u = 0; u < 4; ++u) {
+                    float* d = pq + t * 16 * kWsPad + 8 * u;
+                    d[0] = v[t][u].x;
+                    d[kWsPad] = v[t][u].y;
+                    d[2 * kWsPad] = v[t][u].z;
+                    d[3 * kWsPad] = v[t][u].w;
+                }
+            __syncwarp();
+            run_list(lane < take);
+            __syncwarp();
+#pragma unroll
+            for (int u = 0; u < 4; ++u) {
+                const Row o = row_from(r, 8 * u + qe);
+                if (8 * u + qe >= take) continue;
+#pragma unroll
+                for (int t = 0; t < NTA + NTB; ++t) {
+                    if (!touched(t)) continue;
+                    const float* d = pq + t * 16 * kWsPad + 8 * u;
+                    const float4 f = make_float4(d[0], d[kWsPad], d[2 * kWsPad], d[3 * kWsPad]);
+                    const unsigned tile = tile_of(o, t);
+                    *((float4*)values(o, tile) + qp) = f;
+                    if (f.x != 0.f || f.y != 0.f || f.z != 0.f || f.w != 0.f) raise(o, t, tile);
+                }
+            }
+            __syncwarp();
+            run = __shfl_sync(0xffffffffu, grabbed, 0);
+        }
+        return;
+    }
+    // an occupied pass: 32 row pairs per run. Eight lanes move one contiguous 128-byte row pair of a
+    // tile; a per-warp panel [column][lane] of packed rows, one side at a time, turns it around.
+    if constexpr (MODE == 1 && !ALL) {
+        float2* const panel = (float2*)mem;
+        const int le = lane >> 3, lp = lane & 7;            // entry (mod 4) and 16-byte piece a lane moves
+        const int prow = lp >> 2, pcol = 4 * (lp & 3);      // the piece's row of the pair and first column
+        // a column's entries are rotated by its quarter of the tile: the pieces of eight lanes, and a
+        // column of all lanes, hit all banks
+        auto at = [&](int col) { return panel + col * 32 + ((lane + (col & 12)) & 31); };
+        auto part = [&](int t, int u) {
+            return (float*)panel + ((16 * t + pcol) * 32 + ((4 * u + le + pcol) & 31)) * 2 + prow;
+        };
+        auto one_run = [&](auto ns) {
+            constexpr int NS = decltype(ns)::value;
+            const int take = n_ent - 32 * run;
+            const Row r = look_up(run);
+            float4 v[NTA + NTB][kFullBatch];
+#pragma unroll
+            for (int u = 0; u < kFullBatch; ++u) {
+                const Row o = row_from(r, 4 * u + le);
+#pragma unroll
+                for (int t = 0; t < NTA + NTB; ++t) {
+                    v[t][u] = make_float4(0.f, 0.f, 0.f, 0.f);
+                    if (4 * u + le < take && touched(t)) v[t][u] = *((const float4*)values(o, tile_of(o, t)) + lp);
+                }
+            }
+            auto put = [&](int t0) {
+#pragma unroll
+                for (int t = 0; t < NTA; ++t)
+#pragma unroll
+                    for (int u = 0; u < kFullBatch; ++u) {
+                        float* d = part(t, u);
+                        d[0] = v[t0 + t][u].x;
+                        d[64] = v[t0 + t][u].y;
+                        d[128] = v[t0 + t][u].z;
+                        d[192] = v[t0 + t][u].w;
+                    }
+                __syncwarp();
+            };
+            // y in slot order: level 0 pairs slot i with y_(-i mod n), and after n levels the order is
+            // the same again
+            float2 x[NS], ys[NS];
+            put(0);
+#pragma unroll
+            for (int i = 0; i < NS; ++i) x[i] = i < nA ? *at(i) : make_float2(0.f, 0.f);
+            __syncwarp();
+            put(NTA);
+#pragma unroll
+            for (int i = 0; i < NS; ++i) ys[i] = (NS - i) % NS < nB ? *at((NS - i) % NS) : make_float2(0.f, 0.f);
+            dense_levels<NS>(x, ys, table);
+            // panel -> tiles, up to the side's last MO (four per molecule: a piece is never cut)
+            auto store = [&](bool sideB) {
+                __syncwarp();
+#pragma unroll
+                for (int u = 0; u < kFullBatch; ++u) {
+                    const Row o = row_from(r, 4 * u + le);
+                    if (4 * u + le >= take) continue;
+#pragma unroll
+                    for (int t = 0; t < NTA; ++t) {
+                        const int pt = sideB ? NTA + t : t;
+                        if (!touched(pt) || 16 * t + pcol >= (sideB ? noB : noA)) continue;
+                        const float* d = part(t, u);
+                        const float4 f = make_float4(d[0], d[64], d[128], d[192]);
+                        const unsigned tile = tile_of(o, pt);
+                        *((float4*)values(o, tile) + lp) = f;
+                        if (f.x != 0.f || f.y != 0.f || f.z != 0.f || f.w != 0.f) raise(o, pt, tile);
+                    }
+                }
+                __syncwarp();
+            };
+            __syncwarp();
+#pragma unroll
+            for (int i = 0; i < NS; ++i)
+                if ((NS - i) % NS < nB) *at((NS - i) % NS) = ys[i];
+            store(true);
+#pragma unroll
+            for (int i = 0; i < NS; ++i)
+                if (i < nA) *at(i) = x[i];
+            store(false);
+        };
+        while (run < run_hi) {
+            switch (n / Sh::gstep) {
+                case 1: one_run(std::integral_constant<int, 1 * Sh::gstep>()); break;
+                case 2: one_run(std::integral_constant<int, 2 * Sh::gstep>()); break;
+                case 3: one_run(std::integral_constant<int, 3 * Sh::gstep>()); break;
+                case 4: one_run(std::integral_constant<int, 4 * Sh::gstep>()); break;
+                case 5: one_run(std::integral_constant<int, 5 * Sh::gstep>()); break;
+                case 6: one_run(std::integral_constant<int, 6 * Sh::gstep>()); break;
+                case 7: one_run(std::integral_constant<int, 7 * Sh::gstep>()); break;
+                default: one_run(std::integral_constant<int, 8 * Sh::gstep>()); break;
+            }
+            run = __shfl_sync(0xffffffffu, grab(), 0);
+        }
+    }
+    // a pass over all MOs: 32 AO rows per run, whose tiles come in by cp.async while the run before
+    // computes
+    if constexpr (MODE == 1 && ALL) {
+        // where piece p (columns 4p .. 4p + 3) of panel tile t of the run's row e lies: eight lanes
+        // reading the same piece of consecutive rows hit all banks
+        auto at = [&](int buf, int t, int e, int p) {
+            return mem + buf * (Sh::raw / 4) + ((t * 32 + e) * 16 + 4 * (p ^ ((e >> 1) & 3)));
+        };
+        auto fetch = [&](int buf, int run_) {
+            const int take = n_ent - 32 * run_;
+            const Row r = look_up(run_);
+#pragma unroll
+            for (int u = 0; u < 4; ++u) {
+                const Row o = row_from(r, 8 * u + qe);
+                const int e = 8 * u + qe;
+#pragma unroll
+                for (int t = 0; t < NTA + NTB; ++t)
+                    cp_async16(at(buf, t, e, qp), values(o, tile_of(o, t)) + 4 * qp, e < take && touched(t));
+            }
+            asm volatile("cp.async.commit_group;" ::: "memory");
+        };
+        fetch(0, run);
+        int run2 = __shfl_sync(0xffffffffu, grab(), 0);
+        int buf = 0;
+        auto one_run = [&](auto ns) {
+            constexpr int NS = decltype(ns)::value;
+            const int take = n_ent - 32 * run;
+            float x[NS], ys[NS];
+            asm volatile("cp.async.wait_group 0;" ::: "memory");
+            __syncwarp();
+            // column of a panel side in a lane's own row (scalar accesses: virtual MOs may follow a
+            // partly filled occupied tile)
+            auto column = [&](int t0, int col) {
+                return at(buf, t0 + (col >> 4), lane, (col >> 2) & 3) + (col & 3);
+            };
+#pragma unroll
+            for (int i = 0; i < NS; ++i) {
+                x[i] = i < nA ? *column(0, colA(i)) : 0.f;
+                ys[i] = (NS - i) % NS < nB ? *column(NTA, colB((NS - i) % NS)) : 0.f;
+            }
+            if (run2 < run_hi) fetch(1 - buf, run2);
+            dense_levels<NS>(x, ys, table);
+            // back to the run's buffer (columns without an MO still hold what they held), then four
+            // lanes per 64-byte row
+#pragma unroll
+            for (int i = 0; i < NS; ++i) {
+                if (i < nA) *column(0, colA(i)) = x[i];
+                if ((NS - i) % NS < nB) *column(NTA, colB((NS - i) % NS)) = ys[i];
+            }
+            const Row r = look_up(run);
+            __syncwarp();
+#pragma unroll
+            for (int u = 0; u < 4; ++u) {
+                const Row o = row_from(r, 8 * u + qe);
+                if (8 * u + qe >= take) continue;
+#pragma unroll
+                for (int t = 0; t < NTA + NTB; ++t) {
+                    if (!touched(t)) continue;
+                    const float4 f = *(const float4*)at(buf, t, 8 * u + qe, qp);
+                    const unsigned tile = tile_of(o, t);
+                    *((float4*)values(o, tile) + qp) = f;
+                    if (f.x != 0.f || f.y != 0.f || f.z != 0.f || f.w != 0.f) raise(o, t, tile);
+                }
+            }
+            __syncwarp();
+        };
+        while (run < run_hi) {
+            const int grabbed = grab();   // the run after the next one
+            switch (n / Sh::gstep) {
+                case 1: one_run(std::integral_constant<int, 1 * Sh::gstep>()); break;
+                case 2: one_run(std::integral_constant<int, 2 * Sh::gstep>()); break;
+                case 3: one_run(std::integral_constant<int, 3 * Sh::gstep>()); break;
+                case 4: one_run(std::integral_constant<int, 4 * Sh::gstep>()); break;
+                case 5: one_run(std::integral_constant<int, 5 * Sh::gstep>()); break;
+                case 6: one_run(std::integral_constant<int, 6 * Sh::gstep>()); break;
+                case 7: one_run(std::integral_constant<int, 7 * Sh::gstep>()); break;
+                default: one_run(std::integral_constant<int, 8 * Sh::gstep>()); break;
+            }
+            buf ^= 1;
+            run = run2;
+            run2 = __shfl_sync(0xffffffffu, grabbed, 0);
+        }
     }
 }
 
@@ -1518,6 +1756,9 @@ __global__ void __launch_bounds__(256) k_compact(int cap, const int* __restrict_
 }
 
 }  // namespace
+
+size_t sweep_flag_bytes(const Ctx* c) { return flag_bytes((size_t)c->n_mol * c->cap, c->n_tiles); }
+size_t sweep_info_bytes(const Ctx* c) { return (size_t)std::max(c->n_gnb, 1) * sizeof(BlockInfo); }
 
 size_t closure_smem_bytes(const Ctx* c) {
     const size_t uw = (size_t)(2 * c->max_cl_groups + 31) / 32;
@@ -1679,6 +1920,57 @@ static cudaError_t closure_t(Ctx* c, int mode, int which, int col_lo, int col_hi
     return cudaGetLastError();
 }
 
+// The generic kernel for every block: FP64 storage, and FP32 on request (apply_variant 1).
+template <typename T, int MODE, int NT, int PCAP>
+static cudaError_t apply_generic_t(Ctx* c, const SweepArgs& a, int col_lo, int col_hi) {
+    const size_t smem = (size_t)NT * 16 * apply_nrp<T>() * sizeof(T) + (size_t)2 * PCAP * sizeof(T) + (size_t)PCAP * 4;
+    cudaError_t e = cudaFuncSetAttribute(k_apply_colour<T, MODE, NT, PCAP>,
+                                         cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    if (e != cudaSuccess) return e;
+    const std::vector<int>& ptr = MODE == 0 ? c->h_colour_ptr : c->h_ocolour_ptr;
+    constexpr int CH = ApplyShape<T>::chunk;
+    const int gx = (c->n_mol + CH - 1) / CH;
+    for (int col = col_lo; col < col_hi; ++col) {
+        const int nb = ptr[col + 1] - ptr[col];
+        if (nb == 0) continue;
+        k_apply_colour<T, MODE, NT, PCAP><<<dim3(gx, nb), apply_threads<T>(), smem, c->stream>>>(a, ptr[col]);
+        c->n_launch += 1;
+    }
+    return cudaGetLastError();
+}
+
+// FP32 storage: the warp-at-a-time kernel, one launch per colour.
+template <int MODE, bool ALL>
+static cudaError_t apply_warp_t(Ctx* c, SweepArgs& a, int col_lo, int col_hi) {
+    using Sh = WarpShape<MODE, ALL>;
+    // the bits of a block's rows (a cluster's at most) and the counts before each word
+    const int chunks = (c->n_mol + kFullCH - 1) / kFullCH;
+    const size_t smem = Sh::smem + (size_t)std::min(chunks, (c->max_cl_mol + kFullCH - 1) / kFullCH) * 8;
+    if (smem > (size_t)kMaxDynSmem) return cudaErrorInvalidValue;
+    cudaError_t e = cudaFuncSetAttribute(k_apply_warp<MODE, ALL>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    if (e != cudaSuccess) return e;
+    if (a.n_blk == 0) return cudaSuccess;
+    a.blk_info = c->d_blk_info;
+    k_block_info<MODE, ALL><<<(a.n_blk + 127) / 128, 128, 0, c->stream>>>(a, a.n_blk, (BlockInfo*)c->d_blk_info);
+    c->n_launch += 1;
+    const std::vector<int>& ptr = MODE == 0 ? c->h_colour_ptr : c->h_ocolour_ptr;
+    // CTAs per block: shares of `per` runs for as many runs as the largest cluster's rows can give
+    // (variant 2: one CTA takes all runs of its block; same results)
+    const int full = c->n_sm * Sh::min_ctas;
+    for (int col = col_lo; col < col_hi; ++col) {
+        const int nb = ptr[col + 1] - ptr[col];
+        if (nb == 0) continue;
+        const int runs = (kAoPerMol / Sh::halves * c->max_cl_mol + 31) / 32;   // at most, of a block
+        const int per = MODE == 1 && (long long)nb * runs > kWsManyRuns * full ? 2 * kWsWarps : kWsWarps;
+        int gx = (runs + per - 1) / per;
+        if (MODE == 0) gx = std::min(gx, (kWsRotWaves * full + nb - 1) / nb);
+        if (c->apply_variant == 2) gx = 1;
+        k_apply_warp<MODE, ALL><<<nb * gx, kWsThreads, smem, c->stream>>>(a, ptr[col], nb, per);
+        c->n_launch += 1;
+    }
+    return cudaGetLastError();
+}
+
 template <typename T, int MODE, int NT, int PCAP>
 static cudaError_t apply_mode_t(Ctx* c, int which, int col_lo, int col_hi) {
     SweepArgs a;
@@ -1688,58 +1980,15 @@ static cudaError_t apply_mode_t(Ctx* c, int which, int col_lo, int col_hi) {
     a.in_val = a.out_val = c->d_c_val[c->cur];
     a.out_nz = c->d_c_nz[c->cur];
     a.col_nz = c->d_c_cnz;
-    const size_t smem = (size_t)NT * 16 * apply_nrp<T>() * sizeof(T) + (size_t)2 * PCAP * sizeof(T) + (size_t)PCAP * 4;
-    cudaError_t e = cudaFuncSetAttribute(k_apply_colour<T, MODE, NT, PCAP>,
-                                         cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    if (e != cudaSuccess) return e;
-    const std::vector<int>& ptr = MODE == 0 ? c->h_colour_ptr : c->h_ocolour_ptr;
-    constexpr int CH = ApplyShape<T>::chunk;
-    const int gx = (c->n_mol + CH - 1) / CH;
-    // FP32 rotations and occupied passes: blocks between full groups take the register-resident kernel
-    const bool full = std::is_same<T, float>::value && (MODE == 0 || which == 1) && c->apply_variant != 1;
-    if (full) {
-        e = cudaFuncSetAttribute(k_apply_full<MODE>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                 (int)full_apply_smem<MODE>());
-        if (e != cudaSuccess) return e;
-    }
-    const std::vector<int>& nfull = MODE == 0 ? c->h_colour_nfull : c->h_ocolour_nfull;
-    // row chunks per block in x: enough CTAs to fill the GPU a few times over,
-    // each looping over its chunks with one coefficient table
-    static int full_occ[2] = {0, 0};
-    if (full && full_occ[MODE] == 0) {
-        e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&full_occ[MODE], k_apply_full<MODE>, kFullThreads,
-                                                              full_apply_smem<MODE>());
-        if (e != cudaSuccess) return e;
-        full_occ[MODE] = std::max(full_occ[MODE], 1);
-    }
-    const int chunks = (c->n_mol + kFullCH - 1) / kFullCH;
+    a.col_lo = col_lo;
+    a.col_hi = col_hi;
     k_flags_by_column<<<c->n_tiles, 256, 0, c->stream>>>(c->cap, c->d_cci_ptr, c->d_cci_row, c->d_cci_slot,
                                                          a.out_nz, a.col_nz);
     c->n_launch += 1;
-    if (full && a.n_blk > 0) {
-        a.blk_info = (const int4*)c->d_blk_info;
-        k_block_info<MODE><<<(a.n_blk + 127) / 128, 128, 0, c->stream>>>(a, a.n_blk, (int4*)c->d_blk_info);
-        c->n_launch += 1;
-    }
-    for (int col = col_lo; col < col_hi; ++col) {
-        const int nf = full ? nfull[col] : 0;
-        if (nf > 0) {
-            // variant 2: one CTA takes all row chunks of its block (the longest
-            // collection of row pairs; same results)
-            const int gxf = c->apply_variant == 2
-                                ? 1
-                                : std::min(chunks, std::max(1, (kFullWaves[MODE] * c->n_sm * full_occ[MODE]) /
-                                                                   std::max(nf, 1) + 1));
-            k_apply_full<MODE><<<dim3(gxf, nf), kFullThreads, full_apply_smem<MODE>(), c->stream>>>(a, ptr[col]);
-            c->n_launch += 1;
-        }
-        const int nb = ptr[col + 1] - ptr[col] - nf;
-        if (nb == 0) continue;
-        dim3 grid(gx, nb);
-        k_apply_colour<T, MODE, NT, PCAP><<<grid, apply_threads<T>(), smem, c->stream>>>(a, ptr[col] + nf);
-        c->n_launch += 1;
-    }
-    return cudaGetLastError();
+    if constexpr (std::is_same<T, float>::value)
+        if (c->apply_variant != 1)
+            return apply_warp_t<MODE, NT == 6>(c, a, col_lo, col_hi);
+    return apply_generic_t<T, MODE, NT, PCAP>(c, a, col_lo, col_hi);
 }
 
 // side tiles and pair capacity per pass: rotations 2 occupied + 1 virtual

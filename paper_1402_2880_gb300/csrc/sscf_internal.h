@@ -112,7 +112,6 @@ struct Ctx {
     std::vector<int> h_gnb_ptr, h_gnb_col, h_gnb_row, h_gnb_colour;
     std::vector<int> h_colour_ptr, h_colour_blk;        // all directed blocks by colour
     std::vector<int> h_ocolour_ptr, h_ocolour_blk;      // blocks with A <= B by colour
-    std::vector<int> h_colour_nfull, h_ocolour_nfull;   // leading blocks of each colour between full groups
     // tile-pair lists of the transforms
     std::vector<int> h_rot_tp_ptr;   // per a-tile CSR into (b, out) for the F_ov blocks
     std::vector<int> h_rot_tp_b, h_rot_tp_out;
@@ -191,7 +190,7 @@ struct Ctx {
     void* d_c_val[2] = {nullptr, nullptr};
     unsigned char* d_c_nz[2] = {nullptr, nullptr};   // per (row block, slot): 0 = tile known all-zero during a sweep
     unsigned char* d_c_cnz = nullptr;   // the current sweep's flags in column-index order
-    int* d_blk_info = nullptr;          // per block of a sweep in colour order: 8 ints the FP32 sweep kernel starts from
+    void* d_blk_info = nullptr;         // per block of a sweep in colour order: what the FP32 sweep kernel starts from
     int cur = 0;
     int* d_cci_ptr = nullptr;     // n_tiles + 1
     int* d_cci_cnt = nullptr;     // n_tiles
@@ -307,6 +306,8 @@ cudaError_t launch_select_rot(Ctx* c);
 cudaError_t launch_ortho_prepare(Ctx* c, int which, double tol);
 // structural fill of the sweep's colours [col_lo, col_hi) (col_hi < 0: all); cur <- other
 cudaError_t launch_closure(Ctx* c, int mode, int which, int col_lo = 0, int col_hi = -1, bool first = true);
+size_t sweep_flag_bytes(const Ctx* c);   // d_c_cnz
+size_t sweep_info_bytes(const Ctx* c);   // d_blk_info
 size_t closure_smem_bytes(const Ctx* c);
 size_t closure_labels_smem_bytes(const Ctx* c);
 // mode 0 rotations, 1 combinations, colours [col_lo, col_hi) (col_hi < 0: all); in place
