@@ -134,7 +134,8 @@ typedef struct {
  *   n_link: 1 .. 8 molecules per group
  *   group_of_mol: host, n_atoms / 3, written; n_groups_out, iters_out may be NULL
  * Device memory comes from the allocator of sscf_set_allocator, if set, and is
- * freed before the call returns. Errors: INVALID_ARG, NONFINITE, OOM, CUDA. */
+ * freed before the call returns. Errors: INVALID_ARG, NONFINITE, OOM, CUDA, TIMEOUT
+ * (a bounded wait on the device gave up). */
 int sscf_group_molecules(int n_atoms, const double* xyz, int n_link, int max_iter, double tol,
                          void* cuda_stream, int* group_of_mol, int* n_groups_out, int* iters_out);
 

@@ -8,14 +8,15 @@
 //
 // The paper links atoms in list order (one OpenMP lock per centre) and evens
 // out the order dependence by shuffling the centres at every iteration. Here
-// the link step is the molecule-proposing deferred-acceptance matching: in
-// rounds, every unlinked molecule proposes to its next centre in increasing
-// (distance^2, centre index); every centre keeps the n_link candidates (its
-// members and the new proposers) with the smallest (distance^2, molecule
-// index). The result does not depend on any processing order, so one thread
-// per molecule and one per centre compute it without locks, bit for bit the
-// same on every run. Squared distances are (dx*dx + dy*dy) + dz*dz with
-// explicitly rounded operations (no fused multiply-add).
+// the link step is the molecule-proposing deferred-acceptance matching: an
+// unlinked molecule proposes to its next centre in increasing (distance^2,
+// centre index); a centre keeps the n_link proposers with the smallest
+// (distance^2, molecule index), and one it rejects or displaces proposes on.
+// The matching that comes out does not depend on the order of the proposals
+// (preferences are strict), so warps make them concurrently, one molecule and
+// the chain of molecules it displaces per warp, with a lock per centre. Squared
+// distances are (dx*dx + dy*dy) + dz*dz with explicitly rounded operations (no
+// fused multiply-add).
 #include <algorithm>
 #include <cmath>
 #include <vector>
@@ -33,88 +34,155 @@ __device__ __forceinline__ double d2_rn(const double* a, const double* b) {
 // (d, i) < (e, j) lexicographically
 __device__ __forceinline__ bool lex_less(double d, int i, double e, int j) { return d < e || (d == e && i < j); }
 
-// Every unlinked molecule proposes to its next centre: the smallest
-// (distance^2, centre) above the last one it proposed to.
-__global__ void k_km_propose(int n, int nc, const double* __restrict__ pos, const double* __restrict__ cen,
-                             const int* __restrict__ holder, int* __restrict__ prop, double* __restrict__ last_d,
-                             int* __restrict__ last_c, int* __restrict__ n_free) {
-    const int m = blockIdx.x * blockDim.x + threadIdx.x;
-    if (m >= n) return;
-    if (holder[m] >= 0) {
-        prop[m] = -1;
-        return;
-    }
-    const double ld = last_d[m];
-    const int lc = last_c[m];
-    double bd = INFINITY;
-    int bc = -1;
-    for (int c = 0; c < nc; ++c) {
-        const double d = d2_rn(pos + 3 * m, cen + 3 * c);
-        if (lc >= 0 && !lex_less(ld, lc, d, c)) continue;   // at or before the last proposal
-        if (bc < 0 || lex_less(d, c, bd, bc)) {
-            bd = d;
-            bc = c;
-        }
-    }
-    prop[m] = bc;
-    last_d[m] = bd;
-    last_c[m] = bc;
-    atomicAdd(n_free, 1);
+// Squared distances of all (molecule, centre) pairs, molecule-major.
+__global__ void k_km_dist(int n, int nc, const double* __restrict__ pos, const double* __restrict__ cen,
+                          double* __restrict__ D) {
+    const long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x;
+    if (i >= (long long)n * nc) return;
+    const int m = (int)(i / nc), c = (int)(i - (long long)m * nc);
+    D[i] = d2_rn(pos + 3 * (size_t)m, cen + 3 * (size_t)c);
 }
 
-// Every centre keeps its n_link best candidates (members and new proposers).
-template <int kMaxLink>
-__global__ void k_km_accept(int n, int nc, int n_link, const double* __restrict__ pos, const double* __restrict__ cen,
-                            int* __restrict__ holder, const int* __restrict__ prop) {
-    const int c = blockIdx.x * blockDim.x + threadIdx.x;
-    if (c >= nc) return;
-    double kd[kMaxLink];
-    int km[kMaxLink];
-    int nk = 0;
-    for (int m = 0; m < n; ++m) {
-        if (holder[m] != c && prop[m] != c) continue;
-        const double d = d2_rn(pos + 3 * m, cen + 3 * c);
-        if (nk == n_link && !lex_less(d, m, kd[nk - 1], km[nk - 1])) {
-            holder[m] = -1;   // rejected (or displaced)
-            continue;
+// What a centre holds: its members sorted by (distance^2, molecule).
+struct KmCentre {
+    double d[kMaxMolPerGroup];
+    int m[kMaxMolPerGroup];
+    int n, lock;
+};
+constexpr int kKmSpin = 1 << 22;   // polls of a centre's lock before a warp gives up
+
+// The matching. A warp takes an unlinked molecule, finds its next centre (lanes
+// over the centres, a lexicographic minimum), and inserts it under the centre's
+// lock; a displaced molecule is the warp's next one and goes on after the centre
+// that let it go, so that nothing but the centres' lists is kept. A step is a
+// row of distances and a few hundred clocks in a list, and chains of steps are
+// serial: the lists sit in shared memory where they fit one CTA (IN_SMEM), in
+// global memory with many CTAs else. D = NULL: distances from the positions
+// (more pairs than are worth storing). No warp waits while it holds a lock.
+// 1000 molecules, 150 centres, 101 matchings: 34 ms; with a pair of launches and
+// a host round trip per round of proposals, each centre scanning all molecules,
+// 219-318 ms (1000 molecules of a strongly disordered liquid, 48 matchings: 21
+// against 950 ms).
+template <bool IN_SMEM>
+__global__ void __launch_bounds__(1024) k_km_match(int n, int nc, int n_link, const double* __restrict__ pos,
+                                                   const double* __restrict__ cen, const double* __restrict__ D,
+                                                   KmCentre* __restrict__ lists, int* __restrict__ next,
+                                                   int* __restrict__ failed) {
+    extern __shared__ __align__(16) unsigned char kmraw[];
+    KmCentre* const L = IN_SMEM ? (KmCentre*)kmraw : lists;
+    if (IN_SMEM) {
+        for (int c = threadIdx.x; c < nc; c += blockDim.x) L[c].n = L[c].lock = 0;
+        __syncthreads();
+    }
+    const int lane = threadIdx.x & 31;
+    for (;;) {
+        int m = 0;
+        if (lane == 0) m = atomicAdd(next, 1);
+        m = __shfl_sync(0xffffffffu, m, 0);
+        if (m >= n) break;
+        double ld = -1.0;   // the last proposal of m: everything after (ld, lc) is open
+        int lc = -1;
+        while (m >= 0) {
+            double bd = INFINITY;
+            int bc = 0x7fffffff;
+            for (int c = lane; c < nc; c += 32) {
+                const double d = D ? D[(size_t)m * nc + c] : d2_rn(pos + 3 * (size_t)m, cen + 3 * (size_t)c);
+                if (lex_less(ld, lc, d, c) && lex_less(d, c, bd, bc)) {
+                    bd = d;
+                    bc = c;
+                }
+            }
+#pragma unroll
+            for (int o = 16; o > 0; o >>= 1) {
+                const double od = __shfl_xor_sync(0xffffffffu, bd, o);
+                const int oc = __shfl_xor_sync(0xffffffffu, bc, o);
+                if (lex_less(od, oc, bd, bc)) {
+                    bd = od;
+                    bc = oc;
+                }
+            }
+            int out = -1;   // the molecule to go on with, and its last proposal's distance
+            double out_d = 0.0;
+            if (lane == 0) {
+                if (bc >= nc) {   // no centre left: cannot happen while there is room for every molecule
+                    atomicExch(failed, 1);
+                } else {
+                    volatile KmCentre& k = L[bc];
+                    int spins = 0;
+                    while (atomicCAS(&L[bc].lock, 0, 1) != 0)
+                        if (++spins > kKmSpin) break;
+                    if (spins > kKmSpin) {
+                        atomicExch(failed, 1);
+                    } else {
+                        __threadfence();
+                        const int held = k.n;
+                        int p = held;
+                        if (held == n_link) {
+                            const double wd = k.d[held - 1];
+                            const int wm = k.m[held - 1];
+                            if (lex_less(bd, m, wd, wm)) {   // the worst member is displaced
+                                out = wm;
+                                out_d = wd;
+                                p = held - 1;
+                            } else {                         // m is rejected
+                                out = m;
+                                out_d = bd;
+                                p = -1;
+                            }
+                        }
+                        if (p >= 0) {
+                            for (; p > 0; --p) {
+                                const double qd = k.d[p - 1];
+                                const int qm = k.m[p - 1];
+                                if (!lex_less(bd, m, qd, qm)) break;
+                                k.d[p] = qd;
+                                k.m[p] = qm;
+                            }
+                            k.d[p] = bd;
+                            k.m[p] = m;
+                            if (held < n_link) k.n = held + 1;
+                        }
+                        __threadfence();
+                        atomicExch(&L[bc].lock, 0);
+                    }
+                }
+            }
+            m = __shfl_sync(0xffffffffu, out, 0);
+            ld = __shfl_sync(0xffffffffu, out_d, 0);
+            lc = bc;
         }
-        if (nk == n_link) holder[km[nk - 1]] = -1;   // the worst kept one is displaced
-        int p = nk < n_link ? nk++ : nk - 1;
-        while (p > 0 && lex_less(d, m, kd[p - 1], km[p - 1])) {
-            kd[p] = kd[p - 1];
-            km[p] = km[p - 1];
-            --p;
-        }
-        kd[p] = d;
-        km[p] = m;
-        holder[m] = c;
+    }
+    if (IN_SMEM) {
+        __syncthreads();
+        for (int c = threadIdx.x; c < nc; c += blockDim.x) lists[c] = L[c];
     }
 }
 
-// Centroid of every centre's members, summed in increasing molecule index; a
-// centre without members keeps its place.
-__global__ void k_km_centroids(int n, int nc, const double* __restrict__ pos, const int* __restrict__ holder,
-                               const double* __restrict__ cen, double* __restrict__ cen_new) {
+// Every centre's members as holders, and the centroid of the members summed in
+// increasing molecule index; a centre without members keeps its place.
+__global__ void k_km_centroids(int nc, const double* __restrict__ pos, const KmCentre* __restrict__ lists,
+                               const double* __restrict__ cen, double* __restrict__ cen_new,
+                               int* __restrict__ holder) {
     const int c = blockIdx.x * blockDim.x + threadIdx.x;
     if (c >= nc) return;
+    const int k = lists[c].n;
     double s0 = 0.0, s1 = 0.0, s2 = 0.0;
-    int k = 0;
-    for (int m = 0; m < n; ++m) {
-        if (holder[m] != c) continue;
-        s0 = __dadd_rn(s0, pos[3 * m]);
-        s1 = __dadd_rn(s1, pos[3 * m + 1]);
-        s2 = __dadd_rn(s2, pos[3 * m + 2]);
-        ++k;
+    int last = -1;
+    for (int i = 0; i < k; ++i) {
+        int m = 0x7fffffff;   // the next member by index
+        for (int j = 0; j < k; ++j) {
+            const int q = lists[c].m[j];
+            if (q > last && q < m) m = q;
+        }
+        last = m;
+        holder[m] = c;
+        s0 = __dadd_rn(s0, pos[3 * (size_t)m]);
+        s1 = __dadd_rn(s1, pos[3 * (size_t)m + 1]);
+        s2 = __dadd_rn(s2, pos[3 * (size_t)m + 2]);
     }
-    if (k == 0) {
-        cen_new[3 * c] = cen[3 * c];
-        cen_new[3 * c + 1] = cen[3 * c + 1];
-        cen_new[3 * c + 2] = cen[3 * c + 2];
-    } else {
-        cen_new[3 * c] = __ddiv_rn(s0, (double)k);
-        cen_new[3 * c + 1] = __ddiv_rn(s1, (double)k);
-        cen_new[3 * c + 2] = __ddiv_rn(s2, (double)k);
-    }
+    cen_new[3 * c] = k == 0 ? cen[3 * c] : __ddiv_rn(s0, (double)k);
+    cen_new[3 * c + 1] = k == 0 ? cen[3 * c + 1] : __ddiv_rn(s1, (double)k);
+    cen_new[3 * c + 2] = k == 0 ? cen[3 * c + 2] : __ddiv_rn(s2, (double)k);
 }
 
 struct Buf {
@@ -138,25 +206,36 @@ struct Buf {
         }                                           \
     } while (0)
 
-// Deferred acceptance on the device: every molecule linked, at most n_link per centre.
-int link_all(cudaStream_t st, int n, int nc, int n_link, const double* d_pos, const double* d_cen, int* d_holder,
-             int* d_prop, double* d_last_d, int* d_last_c, int* d_free) {
-    KM_CK(cudaMemsetAsync(d_holder, 0xff, (size_t)n * 4, st));   // -1: unlinked
-    KM_CK(cudaMemsetAsync(d_last_c, 0xff, (size_t)n * 4, st));
-    const int th = 128;
-    // each round links or moves at least one molecule a step down its list: at most n * nc rounds
-    for (long long round = 0; round <= (long long)n * nc; ++round) {
-        KM_CK(cudaMemsetAsync(d_free, 0, 4, st));
-        k_km_propose<<<(n + th - 1) / th, th, 0, st>>>(n, nc, d_pos, d_cen, d_holder, d_prop, d_last_d, d_last_c,
-                                                       d_free);
-        int n_free = 0;
-        KM_CK(cudaMemcpyAsync(&n_free, d_free, 4, cudaMemcpyDeviceToHost, st));
-        KM_CK(cudaStreamSynchronize(st));
-        if (n_free == 0) return SSCF_OK;
-        k_km_accept<kMaxMolPerGroup><<<(nc + th - 1) / th, th, 0, st>>>(n, nc, n_link, d_pos, d_cen, d_holder, d_prop);
-        KM_CK(cudaGetLastError());
+struct KmState {
+    int n, nc, n_link;
+    double *pos, *D;
+    KmCentre* lists;
+    int *holder, *next;   // next: [0] first molecule not taken, [1] a warp gave up
+};
+constexpr long long kKmMaxPairs = 1ll << 27;           // distances stored up to here (1 GB)
+constexpr size_t kKmMaxSmem = 200 * 1024;
+
+// The links of the centres `cen` (in st.lists) and the centroids they give.
+int link_all(cudaStream_t s, const KmState& st, const double* cen, double* cen_new) {
+    const int th = 256;
+    KM_CK(cudaMemsetAsync(st.next, 0, 8, s));
+    if (st.D) {
+        const long long pairs = (long long)st.n * st.nc;
+        k_km_dist<<<(unsigned)((pairs + th - 1) / th), th, 0, s>>>(st.n, st.nc, st.pos, cen, st.D);
     }
-    return SSCF_ERR_STATE;
+    const size_t smem = (size_t)st.nc * sizeof(KmCentre);
+    if (smem <= kKmMaxSmem) {
+        KM_CK(cudaFuncSetAttribute(k_km_match<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+        k_km_match<true><<<1, 1024, smem, s>>>(st.n, st.nc, st.n_link, st.pos, cen, st.D, st.lists, st.next,
+                                               st.next + 1);
+    } else {
+        KM_CK(cudaMemsetAsync(st.lists, 0, smem, s));
+        k_km_match<false><<<128, th, 0, s>>>(st.n, st.nc, st.n_link, st.pos, cen, st.D, st.lists, st.next,
+                                             st.next + 1);
+    }
+    k_km_centroids<<<(st.nc + th - 1) / th, th, 0, s>>>(st.nc, st.pos, st.lists, cen, cen_new, st.holder);
+    KM_CK(cudaGetLastError());
+    return SSCF_OK;
 }
 
 }  // namespace
@@ -209,27 +288,30 @@ extern "C" int sscf_group_molecules(int n_atoms, const double* xyz, int n_link, 
     }
     cudaStream_t st = (cudaStream_t)cuda_stream;
     Buf buf;
-    double* d_pos = buf.get<double>(3 * (size_t)n);
+    KmState km;
+    km.n = n;
+    km.nc = nc;
+    km.n_link = n_link;
+    km.pos = buf.get<double>(3 * (size_t)n);
     double* d_cen = buf.get<double>(3 * (size_t)nc);
     double* d_cen_new = buf.get<double>(3 * (size_t)nc);
-    int* d_holder = buf.get<int>(n);
-    int* d_prop = buf.get<int>(n);
-    double* d_last_d = buf.get<double>(n);
-    int* d_last_c = buf.get<int>(n);
-    int* d_free = buf.get<int>(1);
-    if (!d_pos || !d_cen || !d_cen_new || !d_holder || !d_prop || !d_last_d || !d_last_c || !d_free)
-        return SSCF_ERR_OOM;
-    KM_CK(cudaMemcpyAsync(d_pos, pos.data(), pos.size() * 8, cudaMemcpyHostToDevice, st));
+    km.lists = buf.get<KmCentre>(nc);
+    km.holder = buf.get<int>(n);
+    km.next = buf.get<int>(2);
+    if (!km.pos || !d_cen || !d_cen_new || !km.lists || !km.holder || !km.next) return SSCF_ERR_OOM;
+    // (without room for the distances the matching computes them as it goes)
+    km.D = (long long)n * nc <= kKmMaxPairs ? buf.get<double>((size_t)n * nc) : nullptr;
+    KM_CK(cudaMemcpyAsync(km.pos, pos.data(), pos.size() * 8, cudaMemcpyHostToDevice, st));
     KM_CK(cudaMemcpyAsync(d_cen, cen.data(), cen.size() * 8, cudaMemcpyHostToDevice, st));
-    int s = link_all(st, n, nc, n_link, d_pos, d_cen, d_holder, d_prop, d_last_d, d_last_c, d_free);
+    int s = link_all(st, km, d_cen, d_cen_new);
     if (s != SSCF_OK) return s;
     int it = 0;
-    const int th = 128;
+    int given_up[2] = {0, 0};
     for (it = 1; it <= max_iter; ++it) {
-        k_km_centroids<<<(nc + th - 1) / th, th, 0, st>>>(n, nc, d_pos, d_holder, d_cen, d_cen_new);
-        KM_CK(cudaGetLastError());
         KM_CK(cudaMemcpyAsync(cen_new.data(), d_cen_new, cen_new.size() * 8, cudaMemcpyDeviceToHost, st));
+        KM_CK(cudaMemcpyAsync(given_up, km.next, 8, cudaMemcpyDeviceToHost, st));
         KM_CK(cudaStreamSynchronize(st));
+        if (given_up[1]) return SSCF_ERR_TIMEOUT;
         double moved = 0.0;
         for (int c = 0; c < nc; ++c) {
             const double dx = cen_new[3 * c] - cen[3 * c], dy = cen_new[3 * c + 1] - cen[3 * c + 1],
@@ -240,14 +322,16 @@ extern "C" int sscf_group_molecules(int n_atoms, const double* xyz, int n_link, 
         }
         std::swap(cen, cen_new);
         std::swap(d_cen, d_cen_new);
-        s = link_all(st, n, nc, n_link, d_pos, d_cen, d_holder, d_prop, d_last_d, d_last_c, d_free);
+        s = link_all(st, km, d_cen, d_cen_new);
         if (s != SSCF_OK) return s;
         if (moved / nc < tol) break;
     }
     if (it > max_iter) it = max_iter;
     std::vector<int> holder(n);
-    KM_CK(cudaMemcpyAsync(holder.data(), d_holder, (size_t)n * 4, cudaMemcpyDeviceToHost, st));
+    KM_CK(cudaMemcpyAsync(holder.data(), km.holder, (size_t)n * 4, cudaMemcpyDeviceToHost, st));
+    KM_CK(cudaMemcpyAsync(given_up, km.next, 8, cudaMemcpyDeviceToHost, st));
     KM_CK(cudaStreamSynchronize(st));
+    if (given_up[1]) return SSCF_ERR_TIMEOUT;
     std::vector<int> remap(nc, -1);
     for (int m = 0; m < n; ++m) {
         if (holder[m] < 0 || holder[m] >= nc) return SSCF_ERR_STATE;
