@@ -7,6 +7,7 @@
 #include <numeric>
 #include <new>
 
+#include "shares.h"
 #include "sscf_internal.h"
 
 using namespace sscf;
@@ -801,6 +802,21 @@ int sscf_create(const sscf_system* sys, const sscf_params* prm, void* cuda_strea
     UP(c.d_gnb_row, c.h_gnb_row);
     UP(c.d_gnb_col, c.h_gnb_col);
     UP(c.d_gnb_colour, c.h_gnb_colour);
+    {
+        std::vector<int> rev(c.n_gnb), mp(c.n_groups + 1, 0), mol(c.n_mol);
+        for (int e = 0; e < c.n_gnb; ++e) {
+            const int A = c.h_gnb_row[e], B = c.h_gnb_col[e];
+            const auto b = c.h_gnb_col.begin();
+            rev[e] = (int)(std::lower_bound(b + c.h_gnb_ptr[B], b + c.h_gnb_ptr[B + 1], A) - b);
+        }
+        UP(c.d_gnb_rev, rev);
+        for (int m = 0; m < c.n_mol; ++m) mp[c.h_mol_group[m] + 1]++;
+        for (int g = 0; g < c.n_groups; ++g) mp[g + 1] += mp[g];
+        std::vector<int> f(mp.begin(), mp.end() - 1);
+        for (int m = 0; m < c.n_mol; ++m) mol[f[c.h_mol_group[m]]++] = m;
+        UP(c.d_grp_mol_ptr, mp);
+        UP(c.d_grp_mol, mol);
+    }
     UP(c.d_colour_ptr, c.h_colour_ptr);
     UP(c.d_colour_blk, c.h_colour_blk);
     UP(c.d_ocolour_ptr, c.h_ocolour_ptr);
@@ -877,7 +893,8 @@ int sscf_create(const sscf_system* sys, const sscf_params* prm, void* cuda_strea
     AL(c.d_dq, (size_t)c.n_atoms * 8);
     AL(c.d_Q, (size_t)c.n_atoms * 8);
     AL(c.d_e_mol, (size_t)c.n_mol * 8);
-    AL(c.d_red, (size_t)(c.n_mol + 4096) * 8);
+    c.n_shares = std::min(kMaxShares, (3 * c.max_cl_mol + kShareAtoms - 1) / kShareAtoms);
+    AL(c.d_share, (size_t)c.n_shares * c.n_atoms * 3 * 8);
     AL(c.d_cl_E, (size_t)c.n_clusters * 8);
     AL(c.d_cl_sel, (size_t)c.n_clusters * 6 * 8);
     AL(c.d_cl_hist, (size_t)c.n_clusters * 256 * 8);
@@ -1299,6 +1316,7 @@ int sscf_gradients(sscf_ctx* h, double* dE_dxyz, double* dE_dparams) {
     if (!h) return SSCF_ERR_INVALID_ARG;
     Ctx& c = h->c;
     if (!c.have_guess) return SSCF_ERR_STATE;
+    if (!c.d_adj) CKS(dalloc(&c, &c.d_adj, adjoint_scratch_values(&c)));
     CK(cudaMemsetAsync(c.d_sc, 0, offsetof(DeviceScalars, hist), c.stream));
     // charges of the current MOs (they become the SCC input), H without threshold
     CKS(density_async(c, false));

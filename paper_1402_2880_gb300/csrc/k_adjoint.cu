@@ -12,104 +12,41 @@
 // derivatives of the Slater-Koster blocks.
 #include <math.h>
 
+#include <algorithm>
+
+#include <type_traits>
+
+#include "shares.h"
 #include "sscf_internal.h"
 
 namespace sscf {
 
 namespace {
 
-template <typename T> struct AccA;
-template <> struct AccA<double> { using type = double; };
-template <> struct AccA<float> { using type = float; };
-
-// group-graph entry (g1, g2) with g1 <= g2, or -1
-__device__ __forceinline__ int gnb_entry(const int* __restrict__ gnb_ptr, const int* __restrict__ gnb_col, int g1,
-                                         int g2) {
-    int lo = gnb_ptr[g1], hi = gnb_ptr[g1 + 1] - 1;
-    while (lo <= hi) {
-        const int mid = (lo + hi) >> 1;
-        const int v = gnb_col[mid];
-        if (v == g2) return mid;
-        if (v < g2) lo = mid + 1;
-        else hi = mid - 1;
-    }
-    return -1;
-}
-
-// F_oo[tB, tA] element (i, j) address inside the occupied tile-pair storage
-// (blocks A <= B, inside one group a <= b); transposed when stored the other way
-struct FRef {
-    int tp;
-    bool transposed;
-};
-
-__device__ __forceinline__ FRef f_ref(const int* gnb_ptr, const int* gnb_col, const int* self_blk,
-                                      const int* blk_tp, const int* group_ot0, int gB, int tB, int gA, int tA) {
-    const int posB = tB - group_ot0[gB], posA = tA - group_ot0[gA];
-    FRef f{-1, false};
-    if (gB < gA) {
-        const int e = gnb_entry(gnb_ptr, gnb_col, gB, gA);
-        if (e >= 0) f.tp = blk_tp[e * 9 + posB * 3 + posA];
-    } else if (gB > gA) {
-        const int e = gnb_entry(gnb_ptr, gnb_col, gA, gB);
-        if (e >= 0) {
-            f.tp = blk_tp[e * 9 + posA * 3 + posB];
-            f.transposed = true;
-        }
-    } else {
-        const int e = self_blk[gA];
-        if (posB <= posA) {
-            f.tp = blk_tp[e * 9 + posB * 3 + posA];
-        } else {
-            f.tp = blk_tp[e * 9 + posA * 3 + posB];
-            f.transposed = true;
-        }
-    }
-    return f;
-}
-
-// Z = C_o F_oo, row-major like C. Row block r gets the occupied tiles of every
-// group adjacent (or equal) to a group whose occupied tiles it holds; one warp
-// per output tile sums C[r, tB] F_oo[tB, tA] over r's tiles tB of adjacent groups.
-template <typename T>
-__global__ void __launch_bounds__(256) k_zmul(int n_tiles, int n_occ_tiles, int n_groups, int cap,
-                                              const int* __restrict__ c_nt, const int* __restrict__ c_tile,
-                                              const T* __restrict__ c_val, const int* __restrict__ tile_group,
-                                              const int* __restrict__ group_ot0, const int* __restrict__ group_not,
-                                              const int* __restrict__ gnb_ptr, const int* __restrict__ gnb_col,
-                                              const int* __restrict__ self_blk, const int* __restrict__ blk_tp,
-                                              const T* __restrict__ F, int* __restrict__ z_nt,
-                                              int* __restrict__ z_tile, T* __restrict__ z_val,
-                                              unsigned* __restrict__ err) {
+// Z = C_o F_oo, row-major like C: row block r gets the occupied tiles of every
+// group adjacent (or equal) to a group whose occupied tiles it holds.
+//
+// k_zlists writes the rows' tile lists; k_zmul the values.
+__global__ void __launch_bounds__(256) k_zlists(int n_occ_tiles, int n_groups, int cap, const int* __restrict__ c_nt,
+                                                const int* __restrict__ c_tile, const int* __restrict__ tile_group,
+                                                const int* __restrict__ group_ot0, const int* __restrict__ group_not,
+                                                const int* __restrict__ gnb_ptr, const int* __restrict__ gnb_col,
+                                                int* __restrict__ z_nt, int* __restrict__ z_tile,
+                                                unsigned* __restrict__ err) {
     extern __shared__ __align__(16) unsigned char smraw[];
     const int gw = (n_groups + 31) >> 5;
     unsigned* pres = (unsigned*)smraw;          // gw: groups with occupied tiles in row r
     unsigned* outg = pres + gw;                 // gw: groups of Z's tiles
-    int* in_t = (int*)(outg + gw);              // cap: r's occupied tiles
-    int* in_s = in_t + cap;                     // cap: their slots
-    int* out_t = in_s + cap;                    // cap: Z's tiles
     __shared__ int part[256];
-    __shared__ int s_nin, s_nout;
+    __shared__ int s_nout;
     const int r = blockIdx.x;
     for (int i = threadIdx.x; i < gw; i += blockDim.x) pres[i] = outg[i] = 0u;
-    if (threadIdx.x == 0) s_nin = 0;
     __syncthreads();
     const int n0 = c_nt[r];
-    if (threadIdx.x == 0) {
-        int k = 0;
-        for (int s = 0; s < n0; ++s) {
-            const int t = c_tile[(size_t)r * cap + s];
-            if (t >= n_occ_tiles) break;
-            in_t[k] = t;
-            in_s[k] = s;
-            ++k;
-        }
-        s_nin = k;
-    }
-    __syncthreads();
-    const int nin = s_nin;
-    for (int k = threadIdx.x; k < nin; k += blockDim.x) {
-        const int g = tile_group[in_t[k]];
+    for (int s = threadIdx.x; s < n0; s += blockDim.x) {
+        const int t = c_tile[(size_t)r * cap + s];
+        if (t >= n_occ_tiles) continue;
+        const int g = tile_group[t];
         atomicOr(&pres[g >> 5], 1u << (g & 31));
     }
     __syncthreads();
@@ -139,8 +76,7 @@ __global__ void __launch_bounds__(256) k_zmul(int n_tiles, int n_occ_tiles, int 
         s_nout = run;
     }
     __syncthreads();
-    const int nout = s_nout;
-    if (nout > cap) {
+    if (s_nout > cap) {
         if (threadIdx.x == 0) {
             atomicOr(err, kErrCapacity);
             z_nt[r] = 0;
@@ -150,36 +86,152 @@ __global__ void __launch_bounds__(256) k_zmul(int n_tiles, int n_occ_tiles, int 
     int pos = part[threadIdx.x];
     for (int g = g0; g < g1; ++g)
         if ((outg[g >> 5] >> (g & 31)) & 1)
-            for (int i = 0; i < group_not[g]; ++i) out_t[pos++] = group_ot0[g] + i;
+            for (int i = 0; i < group_not[g]; ++i) z_tile[(size_t)r * cap + pos++] = group_ot0[g] + i;
+    if (threadIdx.x == 0) z_nt[r] = s_nout;
+}
+
+// first position of the sorted list with a tile >= t
+__device__ __forceinline__ int first_at(const int* __restrict__ list, int n, int t) {
+    int lo = 0, hi = n;
+    while (lo < hi) {
+        const int mid = (lo + hi) >> 1;
+        if (list[mid] < t) lo = mid + 1;
+        else hi = mid;
+    }
+    return lo;
+}
+
+// Z's values. A CTA makes the 48 x 32 outputs of one MO group's molecules (48 AO
+// rows) and one out group A (two tiles), over the in groups B adjacent to A that
+// any of the rows holds: per B it stages the rows' 48 x 32 values and the 32 x 32
+// block F[B, A], so that a block of F is read once per group of molecules, and
+// each of 96 threads keeps 4 x 4 outputs. Terms are added in the order of the
+// row's tiles and of the MOs inside a tile, one product at a time; a tile that a
+// row does not hold contributes zeros. (One warp per row and out tile read a
+// block of F for six rows of work and looked it up by a binary search:
+// 27.6 ms at 2000 molecules; now 6.6.)
+constexpr int kZThreads = 96;
+constexpr int kZRows = kMaxMolPerGroup * kAoPerMol;   // 48
+constexpr int kZStride = kZRows + 4;                  // values per staged MO (16-byte aligned, bank-spread)
+template <typename T> __host__ __device__ constexpr size_t zmul_smem(int max_nb) {
+    return (size_t)32 * kZStride * sizeof(T) + (size_t)32 * 32 * sizeof(T) +
+           (size_t)max_nb * kMaxMolPerGroup * sizeof(int2) + (size_t)max_nb * sizeof(int);
+}
+template <typename T>
+__global__ void __launch_bounds__(kZThreads)
+k_zmul(int g_lo, int max_nb, int cap, const int* __restrict__ group_cl, const int* __restrict__ cl_g0,
+       const int* __restrict__ grp_mol_ptr, const int* __restrict__ grp_mol,
+       const int* __restrict__ c_nt, const int* __restrict__ c_tile, const T* __restrict__ c_val,
+       const int* __restrict__ group_ot0, const int* __restrict__ group_not, const int* __restrict__ gnb_ptr,
+       const int* __restrict__ gnb_col, const int* __restrict__ blk_tp, const int* __restrict__ gnb_rev,
+       const T* __restrict__ F, const int* __restrict__ z_nt, const int* __restrict__ z_tile, T* __restrict__ z_val) {
+    extern __shared__ __align__(16) unsigned char smraw[];
+    T* sc = (T*)smraw;                                // [32 MOs of B][kZStride]: the rows' values
+    T* sf = sc + 32 * kZStride;                       // [32 MOs of B][32 MOs of A]
+    int2* slot = (int2*)(sf + 32 * 32);               // [neighbour of A][molecule]: slots of B's two tiles, or -1
+    int* any = (int*)(slot + (size_t)max_nb * kMaxMolPerGroup);   // [neighbour of A]: some row holds a tile of B
+    __shared__ int s_mol[kMaxMolPerGroup], s_z[kMaxMolPerGroup];
+    const int G = g_lo + blockIdx.y, cl = group_cl[G], A = cl_g0[cl] + blockIdx.x;
+    if (A >= cl_g0[cl + 1]) return;
+    const int m0 = grp_mol_ptr[G], nm = grp_mol_ptr[G + 1] - m0;
+    const int e0 = gnb_ptr[A], nb = gnb_ptr[A + 1] - e0;
+    const int otA = group_ot0[A], ntA = group_not[A];
+    // the rows with tiles of A in Z, and their first slot there
+    bool mine = false;
+    if ((int)threadIdx.x < nm) {
+        const int r = grp_mol[m0 + threadIdx.x];
+        const int n = z_nt[r];
+        const int* zt = z_tile + (size_t)r * cap;
+        const int p = first_at(zt, n, otA);
+        mine = p < n && zt[p] == otA;
+        s_mol[threadIdx.x] = r;
+        s_z[threadIdx.x] = mine ? p : -1;
+    }
+    if (!__syncthreads_or(mine)) return;
+    for (int i = threadIdx.x; i < nb; i += kZThreads) any[i] = 0;
     __syncthreads();
-    if (threadIdx.x == 0) z_nt[r] = nout;
-    for (int s = threadIdx.x; s < nout; s += blockDim.x) z_tile[(size_t)r * cap + s] = out_t[s];
-    using A = typename AccA<T>::type;
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nwarps = blockDim.x >> 5;
-    const int j = lane & 15, kh = lane >> 4;
-    for (int s = warp; s < nout; s += nwarps) {
-        const int tA = out_t[s];
-        const int gA = tile_group[tA];
-        A acc[3] = {0, 0, 0};
-        for (int k = 0; k < nin; ++k) {
-            const int tB = in_t[k];
-            const int gB = tile_group[tB];
-            const FRef f = f_ref(gnb_ptr, gnb_col, self_blk, blk_tp, group_ot0, gB, tB, gA, tA);
-            if (f.tp < 0) continue;
-            const T* cv = c_val + ((size_t)r * cap + in_s[k]) * kTileVals;
-            const T* fv = F + (size_t)f.tp * 256;
-#pragma unroll 4
-            for (int i = 0; i < 16; ++i) {
-                const A fij = (A)(f.transposed ? fv[j * 16 + i] : fv[i * 16 + j]);
-                acc[0] += (A)cv[(kh)*16 + i] * fij;
-                acc[1] += (A)cv[(kh + 2) * 16 + i] * fij;
-                acc[2] += (A)cv[(kh + 4) * 16 + i] * fij;
-            }
+    for (int i = threadIdx.x; i < nb * nm; i += kZThreads) {
+        const int k = i / nm, q = i - k * nm;
+        const int B = gnb_col[e0 + k], t = group_ot0[B];
+        const int* ct = c_tile + (size_t)s_mol[q] * cap;
+        const int n = c_nt[s_mol[q]];
+        const int p = first_at(ct, n, t);
+        int2 s = make_int2(-1, -1);
+        if (p < n && ct[p] == t) {
+            s.x = p;
+            if (group_not[B] > 1 && p + 1 < n && ct[p + 1] == t + 1) s.y = p + 1;
+        } else if (group_not[B] > 1 && p < n && ct[p] == t + 1) {
+            s.y = p;
         }
-        T* zv = z_val + ((size_t)r * cap + s) * kTileVals;
-        zv[(kh)*16 + j] = (T)acc[0];
-        zv[(kh + 2) * 16 + j] = (T)acc[1];
-        zv[(kh + 4) * 16 + j] = (T)acc[2];
+        slot[k * kMaxMolPerGroup + q] = s;
+        if (s.x >= 0 || s.y >= 0) any[k] = 1;
+    }
+    __syncthreads();
+    const int ti = threadIdx.x >> 3, tj = threadIdx.x & 7;   // rows 4 ti .. 4 ti + 3, MOs 4 tj .. 4 tj + 3 of A
+    T acc[4][4];
+#pragma unroll
+    for (int i = 0; i < 4; ++i)
+#pragma unroll
+        for (int j = 0; j < 4; ++j) acc[i][j] = (T)0;
+    using V = typename std::conditional<sizeof(T) == 4, float4, double2>::type;
+    constexpr int kV = 16 / (int)sizeof(T);
+    for (int k = 0; k < nb; ++k) {
+        if (!any[k]) continue;
+        const int e = e0 + k, B = gnb_col[e];
+        __syncthreads();   // the buffers are free
+        // rows: 16-byte pieces along the MOs, turned to [MO][row]
+        constexpr int kPer = 16 / kV;   // pieces per tile row
+        for (int i = threadIdx.x; i < kZRows * 2 * kPer; i += kZThreads) {
+            const int row = i / (2 * kPer), rem = i - row * (2 * kPer), t = rem / kPer, p = rem - t * kPer;
+            const int q = row / kAoPerMol;
+            const int s = q < nm ? (t ? slot[k * kMaxMolPerGroup + q].y : slot[k * kMaxMolPerGroup + q].x) : -1;
+            T v[kV];
+#pragma unroll
+            for (int u = 0; u < kV; ++u) v[u] = (T)0;
+            if (s >= 0)
+                *(V*)v = *(const V*)(c_val + ((size_t)s_mol[q] * cap + s) * kTileVals + (row - q * kAoPerMol) * kTileW +
+                                     p * kV);
+#pragma unroll
+            for (int u = 0; u < kV; ++u) sc[(t * 16 + p * kV + u) * kZStride + row] = v[u];
+        }
+        // F[B, A]: tile pairs are stored for blocks (lower group, upper group), inside a group for
+        // positions a <= b; transposed when stored the other way
+        const int eb = B <= A ? gnb_rev[e] : e;   // entry (min, max)
+        for (int i = threadIdx.x; i < 32 * 32; i += kZThreads) {
+            const int ib = i >> 5, ja = i & 31;           // MO of B, MO of A
+            const int pB = ib >> 4, pA = ja >> 4;
+            T v = (T)0;
+            if (pB < group_not[B] && pA < ntA) {
+                const bool straight = B < A || (B == A && pB <= pA);   // stored as [B][A]
+                const int tp = straight ? blk_tp[(size_t)eb * 9 + pB * 3 + pA] : blk_tp[(size_t)eb * 9 + pA * 3 + pB];
+                const T* f = F + (size_t)tp * 256;
+                v = straight ? f[(ib & 15) * 16 + (ja & 15)] : f[(ja & 15) * 16 + (ib & 15)];
+            }
+            sf[i] = v;
+        }
+        __syncthreads();
+#pragma unroll 8
+        for (int q = 0; q < 32; ++q) {
+            T c[4], f[4];
+#pragma unroll
+            for (int u = 0; u < 4; u += kV) {
+                *(V*)(c + u) = *(const V*)(sc + q * kZStride + 4 * ti + u);
+                *(V*)(f + u) = *(const V*)(sf + q * 32 + 4 * tj + u);
+            }
+#pragma unroll
+            for (int i = 0; i < 4; ++i)
+#pragma unroll
+                for (int j = 0; j < 4; ++j) acc[i][j] += c[i] * f[j];
+        }
+    }
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+        const int row = 4 * ti + i, q = row / kAoPerMol;
+        if (q >= nm || s_z[q] < 0 || (tj >> 2) >= ntA) continue;
+        T* z = z_val + ((size_t)s_mol[q] * cap + s_z[q] + (tj >> 2)) * kTileVals + (row - q * kAoPerMol) * kTileW +
+               4 * (tj & 3);
+#pragma unroll
+        for (int u = 0; u < 4; u += kV) *(V*)(z + u) = *(const V*)(acc[i] + u);
     }
 }
 
@@ -200,8 +252,8 @@ __device__ __forceinline__ int ao_off(int k) { return k == 0 ? 0 : 3 + k; }
 // Contribution of the ordered atom pair (a in m, b in n) to dE: the force on
 // atom a (-2 g, g = sum P dH/dR + GS dS/dR, R = x_b - x_a; the pair (b, a)
 // gives the same on a) and the parameter partials sum P H0^(k) and GS S^(k).
-__device__ void pair_terms(const SKd& P, const double* xa, const double* xb, int na, int nb, int oa, int ob,
-                           const double* Pm, const double* GS, double* fa, double* dpar) {
+__device__ __forceinline__ void pair_terms(const SKd& P, const double* xa, const double* xb, int na, int nb,
+                                           const double* Pm, const double* GS, double* fa, double* dpar) {
     double d2 = dist2_rn(xa, xb);
     if (!(d2 <= P.rc2)) return;
     const double r = sqrt(d2);
@@ -221,9 +273,12 @@ __device__ void pair_terms(const SKd& P, const double* xa, const double* xb, int
         }
         double g[3] = {0, 0, 0};
         double par[4] = {0, 0, 0, 0};
-        for (int i = 0; i < na; ++i)
-            for (int jj = 0; jj < nb; ++jj) {
-                const double w = Wt[(oa + i) * 6 + ob + jj];
+#pragma unroll
+        for (int i = 0; i < 4; ++i)
+#pragma unroll
+            for (int jj = 0; jj < 4; ++jj) {
+                if (i >= na || jj >= nb) continue;
+                const double w = Wt[i * 4 + jj];
                 if (w == 0.0) continue;
                 for (int k = 0; k < 3; ++k) {
                     double v;
@@ -260,20 +315,56 @@ __device__ void pair_terms(const SKd& P, const double* xa, const double* xb, int
     }
 }
 
-// One CTA per row block m, one warp per pattern neighbour n: P_mn and
-// W_mn = 2 sum_t C[m,t] Z[n,t]^T on the tiles both rows hold, then the pair
-// terms of the 9 atom pairs; per-molecule partials summed in neighbour order.
+// s + e = a + b exactly
+__device__ __forceinline__ void two_sum(float a, float b, float& s, float& e) {
+    s = __fadd_rn(a, b);
+    const float t = __fsub_rn(s, a);
+    e = __fadd_rn(__fsub_rn(a, __fsub_rn(s, t)), __fsub_rn(b, t));
+}
+
+// One CTA per row block m, one warp per pattern neighbour n: P_mn (n >= m only,
+// P_nm = P_mn^T) and W_mn = 2 sum_t C[m,t] Z[n,t]^T on the tiles both rows hold,
+// written as 6 x 6 blocks. Products of FP32 values are rounded to FP32 and
+// summed without further error worth the name: FP64 sums in FP64 storage, pairs
+// of floats (the running sum and what its roundings dropped, 48 bits) in FP32
+// storage. FP64 additions bounded the kernel (two lanes per clock and SM; 72 of
+// them per shared tile and lane): 34.2 ms at 2000 molecules with the pair terms; now 2.5, and 0.33 for those.
 constexpr int kGradWarps = 8;
+template <typename T> struct SumOf;
+template <> struct SumOf<double> {
+    double v;
+    __device__ __forceinline__ void zero() { v = 0.0; }
+    __device__ __forceinline__ void add_product(double a, double b) { v += a * b; }
+    __device__ __forceinline__ void add(const SumOf& o) { v += o.v; }
+    __device__ __forceinline__ double value() const { return v; }
+};
+template <> struct SumOf<float> {
+    float hi, lo;
+    __device__ __forceinline__ void zero() { hi = lo = 0.f; }
+    __device__ __forceinline__ void add_product(float a, float b) {
+        float e;
+        two_sum(hi, __fmul_rn(a, b), hi, e);
+        lo = __fadd_rn(lo, e);
+    }
+    __device__ __forceinline__ void add(const SumOf& o) {
+        float e;
+        two_sum(hi, o.hi, hi, e);
+        lo = __fadd_rn(lo, __fadd_rn(e, o.lo));
+    }
+    __device__ __forceinline__ double value() const { return (double)hi + (double)lo; }
+};
+template <typename T> __host__ __device__ constexpr size_t grad_smem(int map_n) {
+    return (size_t)((map_n + 3) & ~3) * 4 + (size_t)kGradWarps * 36 * 33 * sizeof(SumOf<T>);
+}
 template <typename T>
-__global__ void __launch_bounds__(kGradWarps * 32)
+__global__ void __launch_bounds__(kGradWarps * 32, 2)
 k_grad_blocks(int n_occ_tiles, int map_n, const int* __restrict__ mol_ot0, int cap, const int* __restrict__ c_nt,
-              const int* __restrict__ c_tile,
-              const T* __restrict__ c_val, const int* __restrict__ z_nt, const int* __restrict__ z_tile,
-              const T* __restrict__ z_val, const int* __restrict__ mp_ptr, const int* __restrict__ mp_col,
-              const double* __restrict__ xyz, const double* __restrict__ Q, SKd P, double* __restrict__ gmol,
-              double* __restrict__ pmol) {
-    extern __shared__ int smap[];   // map_n: slot in C row m of each occupied tile of m's cluster, or -1
-    __shared__ double part[kGradWarps][17];
+              const int* __restrict__ c_tile, const T* __restrict__ c_val, const int* __restrict__ z_nt,
+              const int* __restrict__ z_tile, const T* __restrict__ z_val, const int* __restrict__ mp_ptr,
+              const int* __restrict__ mp_col, const int* __restrict__ mp_rev, double* __restrict__ Pb,
+              double* __restrict__ Wb) {
+    extern __shared__ __align__(16) int smap[];   // map_n: slot in C row m of each occupied tile of m's cluster, or -1
+    SumOf<T>* sums = (SumOf<T>*)(smap + ((map_n + 3) & ~3));   // [warp][36][33]: the lanes' sums
     const int m = blockIdx.x;
     const int t0 = mol_ot0[m];
     for (int i = threadIdx.x; i < map_n; i += blockDim.x) smap[i] = -1;
@@ -287,124 +378,171 @@ k_grad_blocks(int n_occ_tiles, int map_n, const int* __restrict__ mol_ot0, int c
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int e0 = mp_ptr[m], ne = mp_ptr[m + 1] - e0;
     const int col = lane & 15, half = lane >> 4;
-    using A = typename AccA<T>::type;
-    double wsum[17];
-    for (int u = 0; u < 17; ++u) wsum[u] = 0.0;
-    for (int w = warp; w < ne; w += kGradWarps) {
-        const int n = mp_col[e0 + w];
-        double accP[36], accW[36];
-        for (int u = 0; u < 36; ++u) accP[u] = accW[u] = 0.0;
-        const int ntn = c_nt[n];
-        for (int s = half; s < ntn; s += 2) {
-            const int t = c_tile[(size_t)n * cap + s];
-            if (t >= n_occ_tiles) break;
-            const int sm_ = smap[t - t0];
-            if (sm_ < 0) continue;
-            const T* cm = c_val + ((size_t)m * cap + sm_) * kTileVals + col;
-            const T* cn = c_val + ((size_t)n * cap + s) * kTileVals + col;
-            A a6[6], b6[6];
-            for (int k = 0; k < 6; ++k) {
-                a6[k] = (A)cm[k * kTileW];
-                b6[k] = (A)cn[k * kTileW];
-            }
-            for (int k = 0; k < 6; ++k)
-                for (int l = 0; l < 6; ++l) accP[k * 6 + l] += (double)(a6[k] * b6[l]);
-        }
-        const int nzn = z_nt[n];
-        for (int s = half; s < nzn; s += 2) {
-            const int t = z_tile[(size_t)n * cap + s];
-            const int sm_ = smap[t - t0];
-            if (sm_ < 0) continue;
-            const T* cm = c_val + ((size_t)m * cap + sm_) * kTileVals + col;
-            const T* zn = z_val + ((size_t)n * cap + s) * kTileVals + col;
-            A a6[6], b6[6];
-            for (int k = 0; k < 6; ++k) {
-                a6[k] = (A)cm[k * kTileW];
-                b6[k] = (A)zn[k * kTileW];
-            }
-            for (int k = 0; k < 6; ++k)
-                for (int l = 0; l < 6; ++l) accW[k * 6 + l] += (double)(a6[k] * b6[l]);
-        }
-        for (int u = 0; u < 36; ++u) {
-            for (int off = 16; off > 0; off >>= 1) {
-                accP[u] += __shfl_xor_sync(0xffffffffu, accP[u], off);
-                accW[u] += __shfl_xor_sync(0xffffffffu, accW[u], off);
-            }
-        }
-        // lanes 0..8: atom pair (a in m, b in n)
-        double fa[3] = {0, 0, 0}, dp[8] = {0, 0, 0, 0, 0, 0, 0, 0};
-        if (lane < 9) {
-            const int ia = lane / 3, ib = lane % 3;
-            const int a = 3 * m + ia, b = 3 * n + ib;
-            if (a != b) {
-                double Pm[36], GS[36];
-                for (int u = 0; u < 36; ++u) {
-                    const int k = u / 6, l = u % 6;
-                    const int at_k = 3 * m + (k < 4 ? 0 : k - 3), at_l = 3 * n + (l < 4 ? 0 : l - 3);
-                    Pm[u] = 2.0 * accP[u];
-                    GS[u] = 0.5 * Pm[u] * (Q[at_k] + Q[at_l]) - 2.0 * accW[u];
+    SumOf<T>* mys = sums + (size_t)warp * 36 * 33;
+    // 2 sum_t C[m,t] B[n,t]^T over the occupied tiles of row n's list that row m holds
+    auto block = [&](int n, const int* __restrict__ b_nt, const int* __restrict__ b_tile, const T* __restrict__ b_val,
+                     double* out, double* out_t) {
+        SumOf<T> acc[36];
+#pragma unroll
+        for (int u = 0; u < 36; ++u) acc[u].zero();
+        const int nt = b_nt[n];
+        // 32 of n's tiles at a time, the shared ones found with one ballot; the halves of the warp
+        // take them in turn
+        for (int base = 0; base < nt; base += 32) {
+            const int s = base + lane;
+            const int t = s < nt ? b_tile[(size_t)n * cap + s] : n_occ_tiles;
+            const int sm_ = t < n_occ_tiles ? smap[t - t0] : -1;
+            unsigned mm = __ballot_sync(0xffffffffu, sm_ >= 0);
+            const bool past = __any_sync(0xffffffffu, s < nt && t >= n_occ_tiles);
+            while (mm) {
+                const int b0 = __ffs(mm) - 1;
+                mm &= mm - 1;
+                int b1 = -1;
+                if (mm) {
+                    b1 = __ffs(mm) - 1;
+                    mm &= mm - 1;
                 }
-                pair_terms(P, xyz + 3 * a, xyz + 3 * b, ia == 0 ? 4 : 1, ib == 0 ? 4 : 1, ao_off(ia), ao_off(ib), Pm,
-                           GS, fa, dp);
+                const int src = half ? b1 : b0;
+                const int sl = __shfl_sync(0xffffffffu, sm_, src < 0 ? 0 : src);
+                if (src < 0) continue;
+                const T* cm = c_val + ((size_t)m * cap + sl) * kTileVals + col;
+                const T* bn = b_val + ((size_t)n * cap + base + src) * kTileVals + col;
+                T a6[6], b6[6];
+#pragma unroll
+                for (int k = 0; k < 6; ++k) {
+                    a6[k] = cm[k * kTileW];
+                    b6[k] = bn[k * kTileW];
+                }
+#pragma unroll
+                for (int k = 0; k < 6; ++k)
+#pragma unroll
+                    for (int l = 0; l < 6; ++l) acc[k * 6 + l].add_product(a6[k], b6[l]);
             }
+            if (past) break;   // tiles are sorted: occupied tiles first
         }
-        // gather the 9 pair results into lane 0 (fixed order)
-        for (int src = 0; src < 9; ++src) {
-            const double f0 = __shfl_sync(0xffffffffu, fa[0], src), f1 = __shfl_sync(0xffffffffu, fa[1], src),
-                         f2 = __shfl_sync(0xffffffffu, fa[2], src);
-            double pp[8];
-            for (int q = 0; q < 8; ++q) pp[q] = __shfl_sync(0xffffffffu, dp[q], src);
-            const int ia = src / 3;
-            wsum[ia * 3 + 0] += f0;
-            wsum[ia * 3 + 1] += f1;
-            wsum[ia * 3 + 2] += f2;
-            for (int q = 0; q < 8; ++q) wsum[9 + q] += pp[q];
+#pragma unroll
+        for (int u = 0; u < 36; ++u) mys[u * 33 + lane] = acc[u];
+        __syncwarp();
+        for (int u = lane; u < 36; u += 32) {
+            SumOf<T> v = mys[u * 33];
+            for (int j = 1; j < 32; ++j) v.add(mys[u * 33 + j]);
+            const double x = 2.0 * v.value();
+            out[u] = x;
+            if (out_t) out_t[(u % 6) * 6 + u / 6] = x;
         }
-    }
-    if (lane == 0)
-        for (int u = 0; u < 17; ++u) part[warp][u] = wsum[u];
-    __syncthreads();
-    if (threadIdx.x < 17) {
-        double s = 0.0;
-        for (int w = 0; w < kGradWarps; ++w) s += part[w][threadIdx.x];
-        if (threadIdx.x < 9)
-            gmol[(size_t)m * 9 + threadIdx.x] = s;
-        else
-            pmol[(size_t)m * 8 + threadIdx.x - 9] = s;
+        __syncwarp();
+    };
+    for (int w = warp; w < ne; w += kGradWarps) {
+        const int e = e0 + w, n = mp_col[e];
+        if (n >= m)
+            block(n, c_nt, c_tile, c_val, Pb + (size_t)e * 36, n > m ? Pb + (size_t)mp_rev[e] * 36 : nullptr);
+        block(n, z_nt, z_tile, z_val, Wb + (size_t)e * 36, nullptr);
     }
 }
 
-// dE/dx_a of dq^T gamma dq / 2: -dq_a sum_b dq_b gamma_ab^3 (x_a - x_b)
-__global__ void k_gamma_force(int n, const double* __restrict__ xyz, const int* __restrict__ species,
-                              const int* __restrict__ atom_lo, const int* __restrict__ atom_hi,
-                              const double* __restrict__ dq, double invU0, double invU1, double* __restrict__ out) {
-    const int a = blockIdx.x * blockDim.x + threadIdx.x;
-    if (a >= n) return;
-    const int b_lo = atom_lo[a], b_hi = atom_hi[a];   // gamma couples atoms of one cluster only
+// The pair terms of the molecule pairs: one thread per ordered atom pair (kind k
+// of the nine: O-O first, then the pairs of O and H, then H-H, each for all
+// molecule pairs, so that the threads of a warp run the same loops). Nine
+// threads per warp did them at the end of each pair's block before, and the FP64
+// pipe spends the same time on nine lanes as on 32.
+constexpr int kPairOut = 11;   // force on a, parameter partials
+__global__ void __launch_bounds__(128) k_pair_terms(int n_mp, const int* __restrict__ mp_row,
+                                                    const int* __restrict__ mp_col, const double* __restrict__ xyz,
+                                                    const double* __restrict__ Q, SKd P, const double* __restrict__ Pb,
+                                                    const double* __restrict__ Wb, double* __restrict__ out) {
+    const int e = blockIdx.x * blockDim.x + threadIdx.x;
+    if (e >= n_mp) return;
+    const int ia = blockIdx.y / 3, ib = blockIdx.y % 3;
+    const int m = mp_row[e], n = mp_col[e];
+    const int a = 3 * m + ia, b = 3 * n + ib;
+    double fa[3] = {0, 0, 0}, dp[8] = {0, 0, 0, 0, 0, 0, 0, 0};
+    if (a != b) {
+        const int na = ia == 0 ? 4 : 1, nb = ib == 0 ? 4 : 1, oa = ao_off(ia), ob = ao_off(ib);
+        const double h = 0.5 * (Q[a] + Q[b]);
+        double Pm[16], GS[16];   // the atom pair's na x nb values
+#pragma unroll
+        for (int i = 0; i < 4; ++i)
+#pragma unroll
+            for (int j = 0; j < 4; ++j) {
+                const bool in = i < na && j < nb;
+                const size_t u = (size_t)e * 36 + (in ? (oa + i) * 6 + ob + j : 0);
+                Pm[i * 4 + j] = in ? Pb[u] : 0.0;
+                GS[i * 4 + j] = in ? h * Pb[u] - Wb[u] : 0.0;
+            }
+        pair_terms(P, xyz + 3 * a, xyz + 3 * b, na, nb, Pm, GS, fa, dp);
+    }
+    double* o = out + (size_t)blockIdx.y * kPairOut * n_mp + e;
+#pragma unroll
+    for (int k = 0; k < 3; ++k) o[(size_t)k * n_mp] = fa[k];
+#pragma unroll
+    for (int q = 0; q < 8; ++q) o[(size_t)(3 + q) * n_mp] = dp[q];
+}
+
+// Per molecule, in neighbour order: the forces on its atoms and the parameter
+// partials of its pairs. One thread per molecule and output.
+__global__ void k_pair_sum(int n_mol, int n_mp, const int* __restrict__ mp_ptr, const double* __restrict__ pt,
+                           double* __restrict__ gmol, double* __restrict__ pmol) {
+    const int i = blockIdx.x * blockDim.x + threadIdx.x;
+    if (i >= 17 * n_mol) return;
+    const int m = i / 17, u = i - 17 * m;
+    double s = 0.0;
+    for (int e = mp_ptr[m]; e < mp_ptr[m + 1]; ++e) {
+        if (u < 9) {   // atom u / 3, component u % 3
+            for (int ib = 0; ib < 3; ++ib) s += pt[((size_t)(u / 3 * 3 + ib) * kPairOut + u % 3) * n_mp + e];
+        } else {
+            for (int k = 0; k < 9; ++k) s += pt[((size_t)k * kPairOut + 3 + u - 9) * n_mp + e];
+        }
+    }
+    if (u < 9) gmol[(size_t)m * 9 + u] = s;
+    else pmol[(size_t)m * 8 + u - 9] = s;
+}
+
+// dE/dx_a of dq^T gamma dq / 2: -dq_a sum_b dq_b gamma_ab^3 (x_a - x_b), one
+// warp per 32 atoms a and share of the atoms b (the FP64 pipe bounds it: one
+// thread per atom over all b kept a third of the SMs busy, 7.3 ms at 6000
+// atoms; now 1.3).
+__global__ void __launch_bounds__(32) k_gamma_force(int n, const double* __restrict__ xyz,
+                                                    const int* __restrict__ species, const int* __restrict__ atom_lo,
+                                                    const int* __restrict__ atom_hi, const double* __restrict__ dq,
+                                                    double invU0, double invU1, double* __restrict__ part) {
+    const int a0 = blockIdx.x * 32, a = min(a0 + (int)threadIdx.x, n - 1);
+    const int lo = atom_lo[a], hi = atom_hi[a];   // gamma couples atoms of one cluster only
     const double xa = xyz[3 * a], ya = xyz[3 * a + 1], za = xyz[3 * a + 2];
     const double ia = species[a] == 0 ? invU0 : invU1;
+    int b0, b1;
+    share_range(atom_lo[a0], atom_hi[min(a0 + 31, n - 1)], b0, b1);
     double f[3] = {0, 0, 0};
-    for (int b = b_lo; b < b_hi; ++b) {
-        if (b == a) continue;
+    for (int b = b0; b < b1; ++b) {
         const double dx = xa - xyz[3 * b], dy = ya - xyz[3 * b + 1], dz = za - xyz[3 * b + 2];
         const double h = 0.5 * (ia + (species[b] == 0 ? invU0 : invU1));
-        const double g = 1.0 / sqrt(dx * dx + dy * dy + dz * dz + h * h);
-        const double w = dq[b] * g * g * g;
+        const double g = rsqrt(dx * dx + dy * dy + dz * dz + h * h);
+        const double w = b != a && b >= lo && b < hi ? dq[b] * g * g * g : 0.0;
         f[0] += w * dx;
         f[1] += w * dy;
         f[2] += w * dz;
     }
-    for (int d = 0; d < 3; ++d) out[3 * a + d] = -dq[a] * f[d];
+    if (a0 + (int)threadIdx.x >= n) return;
+    for (int d = 0; d < 3; ++d) part[(size_t)blockIdx.y * 3 * n + 3 * a + d] = f[d];
 }
 
-__global__ void k_grad_finish(int n_mol, const double* __restrict__ gmol, const double* __restrict__ pmol,
-                              double* __restrict__ grad, double* __restrict__ dpar) {
-    for (int i = threadIdx.x; i < 9 * n_mol; i += blockDim.x) grad[i] += gmol[i];
-    if (threadIdx.x < 8) {
-        double s = 0.0;
-        for (int m = 0; m < n_mol; ++m) s += pmol[(size_t)m * 8 + threadIdx.x];
-        dpar[threadIdx.x] = s;
-    }
+// dE/dxyz: the gamma forces' shares and the molecules' pair forces
+__global__ void k_grad_finish(int n_atoms, int n_shares, const double* __restrict__ part,
+                              const double* __restrict__ dq, const double* __restrict__ gmol,
+                              double* __restrict__ grad) {
+    const int i = blockIdx.x * blockDim.x + threadIdx.x;
+    if (i >= 3 * n_atoms) return;
+    double s = 0.0;
+    for (int y = 0; y < n_shares; ++y) s += part[(size_t)y * 3 * n_atoms + i];
+    grad[i] = gmol[i] - dq[i / 3] * s;
+}
+
+// parameter gradients: one warp per parameter
+__global__ void k_par_finish(int n_mol, const double* __restrict__ pmol, double* __restrict__ dpar) {
+    const int lane = threadIdx.x & 31, p = threadIdx.x >> 5;
+    double s = 0.0;
+    for (int m = lane; m < n_mol; m += 32) s += pmol[(size_t)m * 8 + p];
+    for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+    if (lane == 0) dpar[p] = s;
 }
 
 }  // namespace
@@ -413,14 +551,27 @@ template <typename T>
 static cudaError_t adjoint_t(Ctx* c, double* d_grad, double* d_par, double* d_gmol, double* d_pmol) {
     const int in = c->cur, zb = 1 - c->cur;
     const int gw = (c->n_groups + 31) / 32;
-    const size_t smem_z = (size_t)2 * gw * 4 + (size_t)3 * c->cap * 4;
-    if (smem_z > 200 * 1024) return cudaErrorInvalidValue;
-    cudaError_t e = cudaFuncSetAttribute(k_zmul<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem_z);
+    const size_t smem_l = (size_t)2 * gw * 4;
+    int max_nb = 1;
+    for (int g = 0; g < c->n_groups; ++g) max_nb = std::max(max_nb, c->h_gnb_ptr[g + 1] - c->h_gnb_ptr[g]);
+    const size_t smem_z = zmul_smem<T>(max_nb), smem_g = grad_smem<T>(c->max_cl_otiles);
+    if (smem_l > 200 * 1024 || smem_z > 200 * 1024 || smem_g > 200 * 1024) return cudaErrorInvalidValue;
+    cudaError_t e = cudaFuncSetAttribute(k_zlists, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem_l);
     if (e != cudaSuccess) return e;
-    k_zmul<T><<<c->n_mol, 256, smem_z, c->stream>>>(
-        c->n_tiles, c->n_occ_tiles, c->n_groups, c->cap, c->d_c_nt[in], c->d_c_tile[in], (const T*)c->d_c_val[in],
-        c->d_tile_group, c->d_group_ot0, c->d_group_not, c->d_gnb_ptr, c->d_gnb_col, c->d_self_blk,
-        c->d_ort_blk_tp[1], (const T*)c->d_sig, c->d_c_nt[zb], c->d_c_tile[zb], (T*)c->d_c_val[zb], &c->d_sc->err);
+    k_zlists<<<c->n_mol, 256, smem_l, c->stream>>>(
+        c->n_occ_tiles, c->n_groups, c->cap, c->d_c_nt[in], c->d_c_tile[in], c->d_tile_group, c->d_group_ot0,
+        c->d_group_not, c->d_gnb_ptr, c->d_gnb_col, c->d_c_nt[zb], c->d_c_tile[zb], &c->d_sc->err);
+    e = cudaFuncSetAttribute(k_zmul<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem_z);
+    if (e != cudaSuccess) return e;
+    // groups of molecules on grid y (65535 at most), out groups of their cluster on grid x
+    for (int g0 = 0; g0 < c->n_groups; g0 += 65535) {
+        const int ng = std::min(65535, c->n_groups - g0);
+        k_zmul<T><<<dim3(c->max_cl_groups, ng), kZThreads, smem_z, c->stream>>>(
+            g0, max_nb, c->cap, c->d_group_cl, c->d_cl_g0, c->d_grp_mol_ptr, c->d_grp_mol, c->d_c_nt[in], c->d_c_tile[in],
+            (const T*)c->d_c_val[in], c->d_group_ot0, c->d_group_not, c->d_gnb_ptr, c->d_gnb_col, c->d_ort_blk_tp[1],
+            c->d_gnb_rev, (const T*)c->d_sig, c->d_c_nt[zb], c->d_c_tile[zb], (T*)c->d_c_val[zb]);
+        c->n_launch += 1;
+    }
     SKd P;
     for (int i = 0; i < 4; ++i) {
         P.V0[i] = c->prm.V0[i];
@@ -428,19 +579,29 @@ static cudaError_t adjoint_t(Ctx* c, double* d_grad, double* d_par, double* d_gm
     }
     P.r_decay = c->prm.r_decay;
     P.rc2 = c->prm.r_cut * c->prm.r_cut;
-    const size_t smem_g = (size_t)c->max_cl_otiles * 4;
+    double* Pb = c->d_adj;
+    double* Wb = Pb + (size_t)c->n_mp * 36;
+    double* pt = Wb + (size_t)c->n_mp * 36;
     e = cudaFuncSetAttribute(k_grad_blocks<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem_g);
     if (e != cudaSuccess) return e;
     k_grad_blocks<T><<<c->n_mol, kGradWarps * 32, smem_g, c->stream>>>(
-        c->n_occ_tiles, c->max_cl_otiles, c->d_mol_ot0, c->cap, c->d_c_nt[in], c->d_c_tile[in], (const T*)c->d_c_val[in], c->d_c_nt[zb],
-        c->d_c_tile[zb], (const T*)c->d_c_val[zb], c->d_mp_ptr, c->d_mp_col, c->d_xyz, c->d_Q, P, d_gmol, d_pmol);
-    k_gamma_force<<<(c->n_atoms + 127) / 128, 128, 0, c->stream>>>(c->n_atoms, c->d_xyz, c->d_species, c->d_atom_lo,
-                                                                  c->d_atom_hi, c->d_dq,
-                                                                  1.0 / c->prm.U[0], 1.0 / c->prm.U[1], d_grad);
-    k_grad_finish<<<1, 1024, 0, c->stream>>>(c->n_mol, d_gmol, d_pmol, d_grad, d_par);
-    c->n_launch += 4;
+        c->n_occ_tiles, c->max_cl_otiles, c->d_mol_ot0, c->cap, c->d_c_nt[in], c->d_c_tile[in],
+        (const T*)c->d_c_val[in], c->d_c_nt[zb], c->d_c_tile[zb], (const T*)c->d_c_val[zb], c->d_mp_ptr, c->d_mp_col,
+        c->d_mp_rev, Pb, Wb);
+    k_pair_terms<<<dim3((c->n_mp + 127) / 128, 9), 128, 0, c->stream>>>(c->n_mp, c->d_mp_row, c->d_mp_col, c->d_xyz,
+                                                                       c->d_Q, P, Pb, Wb, pt);
+    k_pair_sum<<<(17 * c->n_mol + 127) / 128, 128, 0, c->stream>>>(c->n_mol, c->n_mp, c->d_mp_ptr, pt, d_gmol, d_pmol);
+    k_gamma_force<<<dim3((c->n_atoms + 31) / 32, c->n_shares), 32, 0, c->stream>>>(
+        c->n_atoms, c->d_xyz, c->d_species, c->d_atom_lo, c->d_atom_hi, c->d_dq, 1.0 / c->prm.U[0],
+        1.0 / c->prm.U[1], c->d_share);
+    k_grad_finish<<<(3 * c->n_atoms + 127) / 128, 128, 0, c->stream>>>(c->n_atoms, c->n_shares, c->d_share, c->d_dq,
+                                                                      d_gmol, d_grad);
+    k_par_finish<<<1, 8 * 32, 0, c->stream>>>(c->n_mol, d_pmol, d_par);
+    c->n_launch += 7;
     return cudaGetLastError();
 }
+
+size_t adjoint_scratch_values(const Ctx* c) { return (size_t)c->n_mp * (36 + 36 + 9 * kPairOut); }
 
 cudaError_t launch_adjoint(Ctx* c, double* d_grad, double* d_par, double* d_gmol, double* d_pmol) {
     return c->prec == SSCF_FP64 ? adjoint_t<double>(c, d_grad, d_par, d_gmol, d_pmol)

@@ -2,6 +2,7 @@
 // the DFTB Hamiltonian of Eq. (H_dftb2) and the per-molecule initial guess.
 #include <math.h>
 
+#include "shares.h"
 #include "sscf_internal.h"
 
 namespace sscf {
@@ -90,71 +91,85 @@ __global__ void k_sk_blocks(int n_mp, const int* __restrict__ mp_row, const int*
 
 // Q_a = sum_b gamma_ab dq_b over all atom pairs (unscreened, Section
 // "Specific implementation for DFTB"), gamma_ab = 1/sqrt(r^2 + a^2),
-// a = (1/U_a + 1/U_b)/2. One thread per atom a, atoms b staged in smem.
-// P = double: every pair term in FP64. P = float (mixed precision): pair
-// terms in FP32, summed in FP32 over one smem tile of 256 atoms, tile sums
-// accumulated in FP64.
+// a = (1/U_a + 1/U_b)/2; atoms of one cluster only.
+//
+// Mixed precision: pair terms in FP32, summed in FP32 over tiles of 256 atoms b
+// (from the first atom that the 256 atoms around a couple to), tile sums added
+// in FP64 in tile order. A CTA takes 32 atoms, one per lane, and its warps the
+// tiles; a square root and a division per pair bound it, so it needs every SM:
+// with 256 atoms and all tiles per CTA it ran on 48 of them at 12,288 atoms
+// and on 24 at 6,000 (0.56 ms; now 0.10).
 constexpr int kGammaTile = 256;
-template <typename P>
-__global__ void k_gamma(int n, const double* __restrict__ xyz, const int* __restrict__ species,
-                        const int* __restrict__ atom_lo, const int* __restrict__ atom_hi,
-                        const double* __restrict__ dq, double invU0, double invU1, double* __restrict__ Q) {
-    __shared__ P sx[kGammaTile * 3];
-    __shared__ P sq[kGammaTile];
-    __shared__ P si[kGammaTile];
-    __shared__ int s_lo, s_hi;
-    const int a = blockIdx.x * blockDim.x + threadIdx.x;
-    double xa_d[3] = {0, 0, 0}, ia_d = invU0;
-    int lo = 1 << 30, hi = -1;   // gamma couples atoms of one cluster only
-    if (a < n) {
-        xa_d[0] = xyz[3 * a];
-        xa_d[1] = xyz[3 * a + 1];
-        xa_d[2] = xyz[3 * a + 2];
-        ia_d = species[a] == 0 ? invU0 : invU1;
-        lo = atom_lo[a];
-        hi = atom_hi[a];
-    }
-    if (threadIdx.x == 0) {
-        s_lo = 1 << 30;
-        s_hi = -1;
-    }
-    __syncthreads();
-    atomicMin(&s_lo, lo);
-    atomicMax(&s_hi, hi);
-    __syncthreads();
-    const P xa[3] = {(P)xa_d[0], (P)xa_d[1], (P)xa_d[2]};
-    const P ia = (P)ia_d;
+constexpr int kGammaWarps = 8;
+__global__ void __launch_bounds__(32 * kGammaWarps)
+k_gamma_mixed(int n, const double* __restrict__ xyz, const int* __restrict__ species,
+              const int* __restrict__ atom_lo, const int* __restrict__ atom_hi, const double* __restrict__ dq,
+              double invU0, double invU1, double* __restrict__ Q) {
+    __shared__ float4 s_b[kGammaWarps][kGammaTile];   // x, y, z, dq
+    __shared__ float s_i[kGammaWarps][kGammaTile];
+    __shared__ double s_part[kGammaWarps][32];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int a0 = blockIdx.x * 32, a = min(a0 + lane, n - 1);
+    const float xa[3] = {(float)xyz[3 * a], (float)xyz[3 * a + 1], (float)xyz[3 * a + 2]};
+    const float ia = (float)(species[a] == 0 ? invU0 : invU1);
+    const int lo = atom_lo[a], hi = atom_hi[a];
+    const int blo = atom_lo[a0 & ~(kGammaTile - 1)], bhi = atom_hi[min(a0 + 31, n - 1)];
+    const int n_tile = (bhi - blo + kGammaTile - 1) / kGammaTile;
     double acc = 0.0;
-    const int blo = s_lo, bhi = s_hi;
-    for (int b0 = blo; b0 < bhi; b0 += kGammaTile) {
-        __syncthreads();
-        for (int t = threadIdx.x; t < kGammaTile; t += blockDim.x) {
-            int b = b0 + t;
-            if (b < bhi) {
-                sx[3 * t] = (P)xyz[3 * b];
-                sx[3 * t + 1] = (P)xyz[3 * b + 1];
-                sx[3 * t + 2] = (P)xyz[3 * b + 2];
-                sq[t] = (P)dq[b];
-                si[t] = (P)(species[b] == 0 ? invU0 : invU1);
-            } else {
-                sx[3 * t] = sx[3 * t + 1] = sx[3 * t + 2] = (P)0;
-                sq[t] = (P)0;
-                si[t] = (P)invU0;
+    for (int t0 = 0; t0 < n_tile; t0 += kGammaWarps) {
+        const int b0 = blo + (t0 + warp) * kGammaTile;
+        float part = 0.f;
+        if (t0 + warp < n_tile) {
+            for (int t = lane; t < kGammaTile; t += 32) {
+                const int b = min(b0 + t, bhi - 1);
+                s_b[warp][t] = make_float4((float)xyz[3 * b], (float)xyz[3 * b + 1], (float)xyz[3 * b + 2], (float)dq[b]);
+                s_i[warp][t] = (float)(species[b] == 0 ? invU0 : invU1);
+            }
+            __syncwarp();
+            const int t_lo = max(0, lo - b0), t_hi = min(kGammaTile, hi - b0);
+            // (lanes of different clusters run to the last of their ranges together)
+            const int w_lo = __reduce_min_sync(0xffffffffu, t_lo), w_hi = __reduce_max_sync(0xffffffffu, t_hi);
+#pragma unroll 4
+            for (int t = w_lo; t < w_hi; ++t) {
+                const float4 b = s_b[warp][t];
+                const float dx = b.x - xa[0], dy = b.y - xa[1], dz = b.z - xa[2];
+                const float d2 = dx * dx + dy * dy + dz * dz;
+                const float h = 0.5f * (ia + s_i[warp][t]);
+                const float term = b.w / sqrtf(d2 + h * h);
+                if (t >= t_lo && t < t_hi) part += term;
             }
         }
+        s_part[warp][lane] = (double)part;
         __syncthreads();
-        const int nb = min(kGammaTile, bhi - b0);
-        P part = 0;
-        const int t_lo = max(0, lo - b0), t_hi = min(nb, hi - b0);
-        for (int t = t_lo; t < t_hi; ++t) {
-            const P dx = sx[3 * t] - xa[0], dy = sx[3 * t + 1] - xa[1], dz = sx[3 * t + 2] - xa[2];
-            const P d2 = dx * dx + dy * dy + dz * dz;
-            const P h = (P)0.5 * (ia + si[t]);
-            part += sq[t] / sqrt(d2 + h * h);
-        }
-        acc += (double)part;
+        if (warp == 0)
+            for (int w = 0; w < min(kGammaWarps, n_tile - t0); ++w) acc += s_part[w][lane];
+        __syncthreads();
     }
-    if (a < n) Q[a] = acc;
+    if (warp == 0 && a0 + lane < n) Q[a0 + lane] = acc;
+}
+
+// FP64: one warp per 32 atoms a and share y of the atoms b; the shares are
+// summed in order by k_sum_shares. The FP64 pipe (2 lanes per clock and SM)
+// bounds it: every SM has to take part, and the term is a product with
+// 1/sqrt instead of a square root and a division (648 atoms: 1.17 -> 0.04 ms).
+__global__ void __launch_bounds__(32) k_gamma_fp64(int n, const double* __restrict__ xyz,
+                                                   const int* __restrict__ species, const int* __restrict__ atom_lo,
+                                                   const int* __restrict__ atom_hi, const double* __restrict__ dq,
+                                                   double invU0, double invU1, double* __restrict__ part) {
+    const int a0 = blockIdx.x * 32, a = min(a0 + (int)threadIdx.x, n - 1);
+    const double x = xyz[3 * a], y = xyz[3 * a + 1], z = xyz[3 * a + 2];
+    const double ia = species[a] == 0 ? invU0 : invU1;
+    const int lo = atom_lo[a], hi = atom_hi[a];
+    int b0, b1;
+    share_range(atom_lo[a0], atom_hi[min(a0 + 31, n - 1)], b0, b1);
+    double acc = 0.0;
+    for (int b = b0; b < b1; ++b) {
+        const double dx = xyz[3 * b] - x, dy = xyz[3 * b + 1] - y, dz = xyz[3 * b + 2] - z;
+        const double h = 0.5 * (ia + (species[b] == 0 ? invU0 : invU1));
+        const double term = dq[b] * rsqrt(dx * dx + dy * dy + dz * dz + h * h);
+        if (b >= lo && b < hi) acc += term;
+    }
+    if (a0 + (int)threadIdx.x < n) part[(size_t)blockIdx.y * n + a] = acc;
 }
 
 // H = H0 + 1/2 S (Q_a + Q_b) on every molecule-pair block (Eq. H_dftb2);
@@ -353,16 +368,18 @@ cudaError_t launch_sk_blocks(Ctx* c) {
 }
 
 cudaError_t launch_gamma(Ctx* c, const double* dq, double* Q) {
-    c->n_launch += 1;
-    const int th = 256;
-    if (c->prec == SSCF_FP64)
-        k_gamma<double><<<(c->n_atoms + th - 1) / th, th, 0, c->stream>>>(c->n_atoms, c->d_xyz, c->d_species,
-                                                                          c->d_atom_lo, c->d_atom_hi, dq,
-                                                                          1.0 / c->prm.U[0], 1.0 / c->prm.U[1], Q);
-    else
-        k_gamma<float><<<(c->n_atoms + th - 1) / th, th, 0, c->stream>>>(c->n_atoms, c->d_xyz, c->d_species,
-                                                                         c->d_atom_lo, c->d_atom_hi, dq,
-                                                                         1.0 / c->prm.U[0], 1.0 / c->prm.U[1], Q);
+    const double i0 = 1.0 / c->prm.U[0], i1 = 1.0 / c->prm.U[1];
+    const int blocks = (c->n_atoms + 31) / 32;
+    if (c->prec == SSCF_FP64) {
+        k_gamma_fp64<<<dim3(blocks, c->n_shares), 32, 0, c->stream>>>(c->n_atoms, c->d_xyz, c->d_species, c->d_atom_lo,
+                                                                      c->d_atom_hi, dq, i0, i1, c->d_share);
+        k_sum_shares<<<(c->n_atoms + 127) / 128, 128, 0, c->stream>>>(c->n_atoms, c->n_shares, c->d_share, Q);
+        c->n_launch += 2;
+    } else {
+        k_gamma_mixed<<<blocks, 32 * kGammaWarps, 0, c->stream>>>(c->n_atoms, c->d_xyz, c->d_species, c->d_atom_lo,
+                                                                  c->d_atom_hi, dq, i0, i1, Q);
+        c->n_launch += 1;
+    }
     return cudaGetLastError();
 }
 

@@ -1,0 +1,28 @@
+// Sums over all atom pairs of a cluster, split for the FP64 pipe: one warp takes
+// 32 atoms (blockIdx.x) and share blockIdx.y of gridDim.y of the atoms they
+// couple to; the shares are added in order afterwards.
+#pragma once
+
+namespace sscf {
+
+// atoms of a share (at least, so that small clusters do not get empty warps) and shares (at most)
+constexpr int kShareAtoms = 64;
+constexpr int kMaxShares = 64;
+
+// the atoms [b0, b1) of this CTA's share of [lo, hi)
+__device__ __forceinline__ void share_range(int lo, int hi, int& b0, int& b1) {
+    const int per = (hi - lo + (int)gridDim.y - 1) / (int)gridDim.y;
+    b0 = min(hi, lo + (int)blockIdx.y * per);
+    b1 = min(hi, b0 + per);
+}
+
+// out[i] = sum over the shares, in order
+static __global__ void k_sum_shares(int n, int n_shares, const double* __restrict__ part, double* __restrict__ out) {
+    const int i = blockIdx.x * blockDim.x + threadIdx.x;
+    if (i >= n) return;
+    double s = 0.0;
+    for (int y = 0; y < n_shares; ++y) s += part[(size_t)y * n + i];
+    out[i] = s;
+}
+
+}  // namespace sscf

@@ -179,6 +179,9 @@ struct Ctx {
     int* d_gnb_row = nullptr;
     int* d_gnb_col = nullptr;
     int* d_gnb_colour = nullptr;
+    int* d_gnb_rev = nullptr;         // n_gnb: the entry (B, A) of the entry (A, B)
+    int* d_grp_mol_ptr = nullptr;     // n_groups + 1, n_mol: the molecules of every group
+    int* d_grp_mol = nullptr;
     int* d_colour_ptr = nullptr;
     int* d_colour_blk = nullptr;
     int* d_ocolour_ptr = nullptr;
@@ -242,7 +245,9 @@ struct Ctx {
     double* d_P = nullptr;        // n_mp * 36: density blocks (allocated by the first sscf_get_density_blocks)
     unsigned char* d_stage = nullptr;   // staging of sscf_set_C_tiles (grown as needed)
     size_t stage_bytes = 0;
-    double* d_red = nullptr;      // reduction scratch (n_mol + 1024)
+    int n_shares = 1;             // shares of a sum over the atom pairs of a cluster
+    double* d_share = nullptr;    // n_shares x 3 n_atoms: their partial sums
+    double* d_adj = nullptr;      // adjoint: P and W blocks, terms of the atom pairs (allocated by the first sscf_gradients)
     double* d_grad = nullptr;     // 3 n_atoms: dE/dxyz
     double* d_par = nullptr;      // 8: dE/d(V0, S0)
     double* d_gmol = nullptr;     // 9 n_mol: per-molecule force partials
@@ -317,6 +322,7 @@ cudaError_t launch_compact(Ctx* c);                      // drop all-zero tiles;
 cudaError_t launch_charges_finish(Ctx* c, bool mix);
 cudaError_t launch_count_tiles(Ctx* c, unsigned long long* out);
 // adjoint
+size_t adjoint_scratch_values(const Ctx* c);   // d_adj
 cudaError_t launch_adjoint(Ctx* c, double* d_grad, double* d_par, double* d_gmol, double* d_pmol);
 
 }  // namespace sscf
