@@ -194,110 +194,158 @@ __global__ void k_build_h(int n_mp, const int* __restrict__ mp_row, const int* _
 }
 
 // ---- per-molecule generalised eigensolve (step II) --------------------------
-// Cholesky S = L L^T, A = L^-1 H L^-T, cyclic Jacobi on A, x = L^-T v.
-__device__ bool small_geneig6(const double* Hm, const double* Sm, double* w, double* X) {
-    double L[36];
-    for (int i = 0; i < 36; ++i) L[i] = 0.0;
-    for (int j = 0; j < 6; ++j) {
-        double d = Sm[j * 6 + j];
-        for (int k = 0; k < j; ++k) d -= L[j * 6 + k] * L[j * 6 + k];
-        if (!(d > 0.0)) return false;
-        d = sqrt(d);
-        L[j * 6 + j] = d;
-        for (int i = j + 1; i < 6; ++i) {
-            double v = Sm[i * 6 + j];
-            for (int k = 0; k < j; ++k) v -= L[i * 6 + k] * L[j * 6 + k];
-            L[i * 6 + j] = v / d;
+// Cholesky S = L L^T, A = L^-1 H L^-T, cyclic Jacobi on A, x = L^-T v. Every
+// index is a constant once the loops are unrolled, so that the 6x6 matrices are
+// registers. Jacobi converges quadratically: the sweep that starts with the
+// off-diagonal part below 1e-12 of the matrix ends with it below rounding and is
+// the last (running until it was below 1e-17 took most of 60 sweeps of rounding
+// noise). 5.0 ms before, with indexed matrices in local memory, for any number
+// of molecules up to the GPU's threads; now 0.43.
+__device__ __forceinline__ bool small_geneig6(const double* __restrict__ Hm, const double* __restrict__ Sm, double* X) {
+    double Li[36];   // L, then its inverse (lower triangles)
+    {
+        double L[36];
+#pragma unroll
+        for (int j = 0; j < 6; ++j) {
+            double d = Sm[j * 6 + j];
+#pragma unroll
+            for (int k = 0; k < j; ++k) d -= L[j * 6 + k] * L[j * 6 + k];
+            if (!(d > 0.0)) return false;
+            d = sqrt(d);
+            L[j * 6 + j] = d;
+#pragma unroll
+            for (int i = j + 1; i < 6; ++i) {
+                double v = Sm[i * 6 + j];
+#pragma unroll
+                for (int k = 0; k < j; ++k) v -= L[i * 6 + k] * L[j * 6 + k];
+                L[i * 6 + j] = v / d;
+            }
+        }
+#pragma unroll
+        for (int j = 0; j < 6; ++j) {
+            Li[j * 6 + j] = 1.0 / L[j * 6 + j];
+#pragma unroll
+            for (int i = j + 1; i < 6; ++i) {
+                double v = 0.0;
+#pragma unroll
+                for (int k = j; k < i; ++k) v -= L[i * 6 + k] * Li[k * 6 + j];
+                Li[i * 6 + j] = v / L[i * 6 + i];
+            }
         }
     }
-    // Linv (lower triangular inverse)
-    double Li[36];
-    for (int i = 0; i < 36; ++i) Li[i] = 0.0;
-    for (int j = 0; j < 6; ++j) {
-        Li[j * 6 + j] = 1.0 / L[j * 6 + j];
-        for (int i = j + 1; i < 6; ++i) {
-            double v = 0.0;
-            for (int k = j; k < i; ++k) v -= L[i * 6 + k] * Li[k * 6 + j];
-            Li[i * 6 + j] = v / L[i * 6 + i];
-        }
+    double A[36], V[36];
+    {
+        double T1[36];
+#pragma unroll
+        for (int i = 0; i < 6; ++i)
+#pragma unroll
+            for (int j = 0; j < 6; ++j) {
+                double v = 0.0;
+#pragma unroll
+                for (int k = 0; k <= i; ++k) v += Li[i * 6 + k] * Hm[k * 6 + j];
+                T1[i * 6 + j] = v;
+            }
+#pragma unroll
+        for (int i = 0; i < 6; ++i)
+#pragma unroll
+            for (int j = 0; j < 6; ++j) {
+                double v = 0.0;
+#pragma unroll
+                for (int k = 0; k <= j; ++k) v += T1[i * 6 + k] * Li[j * 6 + k];
+                A[i * 6 + j] = v;
+            }
     }
-    double A[36], T1[36];
+#pragma unroll
     for (int i = 0; i < 6; ++i)
-        for (int j = 0; j < 6; ++j) {
-            double v = 0.0;
-            for (int k = 0; k < 6; ++k) v += Li[i * 6 + k] * Hm[k * 6 + j];
-            T1[i * 6 + j] = v;
-        }
-    for (int i = 0; i < 6; ++i)
-        for (int j = 0; j < 6; ++j) {
-            double v = 0.0;
-            for (int k = 0; k < 6; ++k) v += T1[i * 6 + k] * Li[j * 6 + k];
-            A[i * 6 + j] = v;
-        }
-    for (int i = 0; i < 6; ++i)
+#pragma unroll
         for (int j = 0; j < i; ++j) A[i * 6 + j] = A[j * 6 + i] = 0.5 * (A[i * 6 + j] + A[j * 6 + i]);
-    double V[36];
+#pragma unroll
     for (int i = 0; i < 36; ++i) V[i] = (i % 7 == 0) ? 1.0 : 0.0;
+#pragma unroll 1
     for (int sweep = 0; sweep < 60; ++sweep) {
         double off = 0.0, tot = 0.0;
+#pragma unroll
         for (int i = 0; i < 6; ++i)
+#pragma unroll
             for (int j = 0; j < 6; ++j) {
                 tot += A[i * 6 + j] * A[i * 6 + j];
                 if (i != j) off += A[i * 6 + j] * A[i * 6 + j];
             }
-        if (off <= 1e-34 * tot) break;
+        if (off == 0.0) break;
+        const bool last = off <= 1e-24 * tot;
+#pragma unroll
         for (int p = 0; p < 5; ++p)
+#pragma unroll
             for (int q = p + 1; q < 6; ++q) {
-                double apq = A[p * 6 + q];
+                const double apq = A[p * 6 + q];
                 if (apq == 0.0) continue;
-                double theta = (A[q * 6 + q] - A[p * 6 + p]) / (2.0 * apq);
-                double t = (theta >= 0 ? 1.0 : -1.0) / (fabs(theta) + sqrt(theta * theta + 1.0));
-                double cs = 1.0 / sqrt(t * t + 1.0), sn = t * cs;
+                const double theta = (A[q * 6 + q] - A[p * 6 + p]) / (2.0 * apq);
+                const double t = (theta >= 0 ? 1.0 : -1.0) / (fabs(theta) + sqrt(theta * theta + 1.0));
+                const double cs = 1.0 / sqrt(t * t + 1.0), sn = t * cs;
+#pragma unroll
                 for (int k = 0; k < 6; ++k) {
-                    double akp = A[k * 6 + p], akq = A[k * 6 + q];
+                    const double akp = A[k * 6 + p], akq = A[k * 6 + q];
                     A[k * 6 + p] = cs * akp - sn * akq;
                     A[k * 6 + q] = sn * akp + cs * akq;
                 }
+#pragma unroll
                 for (int k = 0; k < 6; ++k) {
-                    double apk = A[p * 6 + k], aqk = A[q * 6 + k];
+                    const double apk = A[p * 6 + k], aqk = A[q * 6 + k];
                     A[p * 6 + k] = cs * apk - sn * aqk;
                     A[q * 6 + k] = sn * apk + cs * aqk;
                 }
+#pragma unroll
                 for (int k = 0; k < 6; ++k) {
-                    double vkp = V[k * 6 + p], vkq = V[k * 6 + q];
+                    const double vkp = V[k * 6 + p], vkq = V[k * 6 + q];
                     V[k * 6 + p] = cs * vkp - sn * vkq;
                     V[k * 6 + q] = sn * vkp + cs * vkq;
                 }
             }
+        if (last) break;
     }
-    // sort ascending
-    int ord[6];
-    for (int i = 0; i < 6; ++i) ord[i] = i;
+    // sort ascending (insertion: later ones move down past strictly larger ones)
+    double w[6];
+#pragma unroll
+    for (int i = 0; i < 6; ++i) w[i] = A[i * 7];
+#pragma unroll
     for (int i = 1; i < 6; ++i)
-        for (int j = i; j > 0 && A[ord[j] * 7] < A[ord[j - 1] * 7]; --j) {
-            int t = ord[j];
-            ord[j] = ord[j - 1];
-            ord[j - 1] = t;
+#pragma unroll
+        for (int j = i; j > 0; --j) {
+            const bool sw = w[j] < w[j - 1];
+            const double a = w[j], b = w[j - 1];
+            w[j] = sw ? b : a;
+            w[j - 1] = sw ? a : b;
+#pragma unroll
+            for (int k = 0; k < 6; ++k) {
+                const double x = V[k * 6 + j], y = V[k * 6 + j - 1];
+                V[k * 6 + j] = sw ? y : x;
+                V[k * 6 + j - 1] = sw ? x : y;
+            }
         }
+#pragma unroll
     for (int n = 0; n < 6; ++n) {
-        const int src = ord[n];
-        w[n] = A[src * 7];
         // x = L^-T v
         double x[6];
+#pragma unroll
         for (int i = 0; i < 6; ++i) {
             double v = 0.0;
-            for (int k = 0; k < 6; ++k) v += Li[k * 6 + i] * V[k * 6 + src];
+#pragma unroll
+            for (int k = i; k < 6; ++k) v += Li[k * 6 + i] * V[k * 6 + n];
             x[i] = v;
         }
         double amax = 0.0;
+#pragma unroll
         for (int i = 0; i < 6; ++i) amax = fmax(amax, fabs(x[i]));
-        int kk = 0;
-        for (int i = 0; i < 6; ++i)
-            if (fabs(x[i]) >= amax * (1.0 - 1e-9)) {
-                kk = i;
-                break;
-            }
-        double sg = x[kk] > 0 ? 1.0 : -1.0;
+        double first = 0.0;   // the first coefficient within 1e-9 of the largest
+        bool found = false;
+#pragma unroll
+        for (int i = 0; i < 6; ++i) {
+            const bool is = !found && fabs(x[i]) >= amax * (1.0 - 1e-9);
+            first = is ? x[i] : first;
+            found |= is;
+        }
+        const double sg = (found ? first : x[0]) > 0 ? 1.0 : -1.0;
+#pragma unroll
         for (int i = 0; i < 6; ++i) X[i * 6 + n] = sg * x[i];
     }
     return true;
@@ -318,8 +366,8 @@ __global__ void k_guess(int n_mol, const int* __restrict__ mp_ptr, const int* __
     int kd = -1;
     for (int k = mp_ptr[m]; k < mp_ptr[m + 1]; ++k)
         if (mp_col[k] == m) kd = k;
-    double w[6], X[36];
-    bool ok = kd >= 0 && small_geneig6(H0b + (size_t)kd * 36, Sb + (size_t)kd * 36, w, X);
+    double X[36];
+    bool ok = kd >= 0 && small_geneig6(H0b + (size_t)kd * 36, Sb + (size_t)kd * 36, X);
     if (!ok) {
         atomicOr(err, kErrGuess);
         c_nt[m] = 0;
@@ -337,8 +385,11 @@ __global__ void k_guess(int n_mol, const int* __restrict__ mp_ptr, const int* __
         vo[i] = (T)0;
         vv[i] = (T)0;
     }
+#pragma unroll
     for (int r = 0; r < 6; ++r) {
+#pragma unroll
         for (int n = 0; n < 4; ++n) vo[r * kTileW + co + n] = (T)X[r * 6 + n];
+#pragma unroll
         for (int n = 0; n < 2; ++n) vv[r * kTileW + cv + n] = (T)X[r * 6 + 4 + n];
     }
 }
@@ -400,7 +451,7 @@ cudaError_t launch_build_h(Ctx* c, double eps_threshold) {
 
 cudaError_t launch_guess(Ctx* c) {
     c->n_launch += 1;
-    const int th = 64;
+    const int th = 32;
     c->cur = 0;
     if (c->prec == SSCF_FP64)
         k_guess<double><<<(c->n_mol + th - 1) / th, th, 0, c->stream>>>(
