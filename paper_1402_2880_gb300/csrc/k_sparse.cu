@@ -8,6 +8,7 @@
 // reduced over the row blocks the two columns share.
 #include "sscf_internal.h"
 
+#include <algorithm>
 #include <type_traits>
 
 namespace sscf {
@@ -133,16 +134,76 @@ __global__ void __launch_bounds__(kSortThreads) k_ci_sort(const int* __restrict_
     }
 }
 
+// The whole column index in one CTA, for small systems (kCiSmallEntries): a bit
+// per (tile, row block) in shared memory; the set bits before a row are its
+// place in the tile's list, so that nothing is sorted. Four launches and two
+// memsets of a few microseconds each otherwise: 20 us of kernels and the gaps
+// between them a call at 8 molecules, now 4.6; at 343 (54,880 entries) one CTA
+// took 65 us, the launches 32.
+constexpr long long kCiSmallEntries = 12288;      // rows x capacity
+constexpr size_t kCiSmallSmem = 96 * 1024;
+__global__ void __launch_bounds__(1024) k_ci_small(int n_mol, int n_tiles, int cap, const int* __restrict__ c_nt,
+                                                   const int* __restrict__ c_tile, int* __restrict__ ptr,
+                                                   int* __restrict__ row, int* __restrict__ slot) {
+    extern __shared__ unsigned cbits[];               // [n_tiles][words], then the tiles' starts
+    const int words = (n_mol + 31) >> 5;
+    int* start = (int*)(cbits + (size_t)n_tiles * words);
+    __shared__ int s_w[32];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    for (int i = threadIdx.x; i < n_tiles * words; i += blockDim.x) cbits[i] = 0u;
+    __syncthreads();
+    for (int r = warp; r < n_mol; r += 32)
+        for (int s = lane; s < c_nt[r]; s += 32)
+            atomicOr(&cbits[(size_t)c_tile[(size_t)r * cap + s] * words + (r >> 5)], 1u << (r & 31));
+    __syncthreads();
+    int base = 0;   // entries of the tiles before this round's 1024
+    for (int t0 = 0; t0 < n_tiles; t0 += 1024) {
+        const int t = t0 + threadIdx.x;
+        int cnt = 0;
+        if (t < n_tiles)
+            for (int w = 0; w < words; ++w) cnt += __popc(cbits[(size_t)t * words + w]);
+        int inc = cnt;
+        for (int o = 1; o < 32; o <<= 1) {
+            const int v = __shfl_up_sync(0xffffffffu, inc, o);
+            if (lane >= o) inc += v;
+        }
+        if (lane == 31) s_w[warp] = inc;
+        __syncthreads();
+        int before = base, total = base;
+        for (int w = 0; w < 32; ++w) {
+            before += w < warp ? s_w[w] : 0;
+            total += s_w[w];
+        }
+        if (t < n_tiles) start[t] = ptr[t] = before + inc - cnt;
+        base = total;
+        __syncthreads();
+    }
+    if (threadIdx.x == 0) ptr[n_tiles] = base;
+    for (int r = warp; r < n_mol; r += 32)
+        for (int s = lane; s < c_nt[r]; s += 32) {
+            const int t = c_tile[(size_t)r * cap + s];
+            const unsigned* b = cbits + (size_t)t * words;
+            int pos = start[t] + __popc(b[r >> 5] & ((1u << (r & 31)) - 1u));
+            for (int w = 0; w < (r >> 5); ++w) pos += __popc(b[w]);
+            row[pos] = r;
+            slot[pos] = s;
+        }
+}
+
 // ---------------------------------------------------------------------------
 // Y[:, t] = X C[:, t] for tiles t in [tile_lo, tile_hi), column-major output.
 // One CTA per tile: mark the row blocks reachable from the tile's rows
 // through the molecule-pair pattern (tiles below own_below: the tile's own
-// rows only), then one warp per output row block sums X[r, n] (6x6)
+// rows only; n_share CTAs per tile do that each and share the rows, so that a
+// few tiles fill the GPU), then one warp per output row block sums X[r, n] (6x6)
 // C[n, t] (6x16) over the pattern neighbours n holding t.
 // ---------------------------------------------------------------------------
+// CTAs per SM that a launch aims at (FP32, one CTA per tile: 4.4 ms at 4096 molecules, 1.18 at 997;
+// 8: 4.4 and 0.73; 32: 3.7 and 0.68; FP64 at 343: 1.86 -> 0.99)
+constexpr int kXcCtas = 32;
 constexpr int kXcBatch = 4;   // matched neighbours whose loads are in flight together
 template <typename T>
-__global__ void k_xc(int tile_lo, int n_rows, int own_below, int cap, int capY, const int* __restrict__ tile_row0,
+__global__ void k_xc(int tile_lo, int n_t, int n_share, int n_rows, int own_below, int cap, int capY, const int* __restrict__ tile_row0,
                      const int* __restrict__ cci_ptr, const int* __restrict__ cci_row,
                      const int* __restrict__ cci_slot, const T* __restrict__ c_val, const int* __restrict__ mp_ptr,
                      const int* __restrict__ mp_col, const T* __restrict__ Xb, int* __restrict__ y_n,
@@ -155,7 +216,8 @@ __global__ void k_xc(int tile_lo, int n_rows, int own_below, int cap, int capY, 
     short* rowpos = (short*)(wpre + nw);          // n_rows: index into the tile's column list or -1
     __shared__ int s_total;
     // tiles from own_below on (the longer ones: every reachable row) first
-    const int t = tile_lo + (int)((blockIdx.x + (unsigned)max(own_below - tile_lo, 0)) % gridDim.x);
+    const int t = tile_lo + (int)((blockIdx.x / n_share + (unsigned)max(own_below - tile_lo, 0)) % n_t);
+    const int share = blockIdx.x % n_share;   // of the tile's rows of Y
     const int r0 = tile_row0[t];
     const int lo = cci_ptr[t], nc = cci_ptr[t + 1] - lo;
     if (nc > 32767) {   // the 16-bit row map cannot index this column
@@ -199,8 +261,8 @@ __global__ void k_xc(int tile_lo, int n_rows, int own_below, int cap, int capY, 
         }
         return;
     }
-    if (threadIdx.x == 0) y_n[t] = ny;
-    // write sorted row list
+    if (threadIdx.x == 0 && share == 0) y_n[t] = ny;
+    // write sorted row list (every share writes the same and reads its own rows)
     for (int w = threadIdx.x; w < nw; w += blockDim.x) {
         unsigned b = bits[w];
         int p = wpre[w];
@@ -214,7 +276,7 @@ __global__ void k_xc(int tile_lo, int n_rows, int own_below, int cap, int capY, 
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nwarps = blockDim.x >> 5;
     const int col = lane & 15, q0 = lane >> 4;   // AO rows q0, q0+2, q0+4
     using A = typename Acc<T>::type;
-    for (int k = warp; k < ny; k += nwarps) {
+    for (int k = share * nwarps + warp; k < ny; k += n_share * nwarps) {
         const int r = y_row[(size_t)t * capY + k];
         A acc0 = 0, acc1 = 0, acc2 = 0;
         // 32 pattern neighbours at a time: their ids, positions and slots are
@@ -745,10 +807,17 @@ __global__ void k_density_sum(int n_mol, const int* __restrict__ mp_ptr, const d
 static cudaError_t ensure_attrs();
 
 cudaError_t launch_colindex(Ctx* c) {
-    c->n_launch += 4;
     cudaError_t ea = ensure_attrs();
     if (ea != cudaSuccess) return ea;
     const int b = c->cur;
+    const size_t small = (size_t)c->n_tiles * ((c->n_mol + 31) / 32 + 1) * 4;
+    if ((long long)c->n_mol * c->cap <= kCiSmallEntries && small <= kCiSmallSmem) {
+        c->n_launch += 1;
+        k_ci_small<<<1, 1024, small, c->stream>>>(c->n_mol, c->n_tiles, c->cap, c->d_c_nt[b], c->d_c_tile[b],
+                                                  c->d_cci_ptr, c->d_cci_row, c->d_cci_slot);
+        return cudaGetLastError();
+    }
+    c->n_launch += 4;
     cudaMemsetAsync(c->d_cci_cnt, 0, (size_t)c->n_tiles * 4, c->stream);
     k_ci_count<<<c->n_mol, 128, 0, c->stream>>>(c->n_mol, c->cap, c->d_c_nt[b], c->d_c_tile[b], c->d_cci_cnt);
     k_scan<<<1, 1024, 0, c->stream>>>(c->n_tiles, c->d_cci_cnt, c->d_cci_ptr);
@@ -781,6 +850,8 @@ static cudaError_t ensure_attrs() {
     cudaError_t e = cudaGetDevice(&dev);
     if (e != cudaSuccess) return e;
     if (dev >= 0 && dev < 64 && g_attr_done[dev]) return cudaSuccess;
+    e = cudaFuncSetAttribute(k_ci_small, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kCiSmallSmem);
+    if (e != cudaSuccess) return e;
     e = set_attrs<double>();
     if (e != cudaSuccess) return e;
     e = set_attrs<float>();
@@ -798,13 +869,15 @@ cudaError_t launch_xc(Ctx* c, bool use_h, int tile_lo, int tile_hi, int own_belo
     const int nr = c->max_cl_mol;
     const size_t smem = (size_t)((nr + 31) / 32) * 8 + (size_t)nr * 2 + 64;
     if (smem > 200 * 1024) return cudaErrorInvalidValue;
+    // CTAs per tile: enough for kXcCtas per SM
+    const int sh = std::min(8, std::max(1, (kXcCtas * c->n_sm + n - 1) / n));
     if (c->prec == SSCF_FP64)
-        k_xc<double><<<n, 256, smem, c->stream>>>(tile_lo, nr, own_below, c->cap, c->capY, c->d_tile_row0, c->d_cci_ptr, c->d_cci_row,
+        k_xc<double><<<n * sh, 256, smem, c->stream>>>(tile_lo, n, sh, nr, own_below, c->cap, c->capY, c->d_tile_row0, c->d_cci_ptr, c->d_cci_row,
                                                   c->d_cci_slot, (const double*)c->d_c_val[b], c->d_mp_ptr,
                                                   c->d_mp_col, (const double*)(use_h ? c->d_Hb : c->d_Sbt),
                                                   c->d_y_n, c->d_y_row, (double*)c->d_y_val, &c->d_sc->err);
     else
-        k_xc<float><<<n, 256, smem, c->stream>>>(tile_lo, nr, own_below, c->cap, c->capY, c->d_tile_row0, c->d_cci_ptr, c->d_cci_row,
+        k_xc<float><<<n * sh, 256, smem, c->stream>>>(tile_lo, n, sh, nr, own_below, c->cap, c->capY, c->d_tile_row0, c->d_cci_ptr, c->d_cci_row,
                                                  c->d_cci_slot, (const float*)c->d_c_val[b], c->d_mp_ptr,
                                                  c->d_mp_col, (const float*)(use_h ? c->d_Hb : c->d_Sbt),
                                                  c->d_y_n, c->d_y_row, (float*)c->d_y_val, &c->d_sc->err);
@@ -818,12 +891,23 @@ cudaError_t launch_xc_rot(Ctx* c) {
     return launch_xc(c, true, 0, c->n_tiles, c->n_occ_tiles);
 }
 
+// CTAs sharing one occupied tile's pairs: what sscf_autotune chose, or enough
+// for kTfCtas per SM, at least 8 (four for every size before: FP64 at 343
+// molecules 5.1 + 3.3 ms, with 24 3.9 + 2.2, as the SMs share the work more
+// evenly; FP32 at 997 1.58 + 1.33 ms, with 10 1.50 + 1.09, with 20 1.97 + 1.45)
+constexpr int kTfCtas = 16;
+static int transform_split(const Ctx* c) {
+    if (c->tf_split > 0) return c->tf_split;
+    return std::min(32, std::max(8, (kTfCtas * c->n_sm + c->n_occ_tiles - 1) / c->n_occ_tiles));
+}
+
 template <typename T>
 static cudaError_t transform_t(Ctx* c, const int* ptr, const int* bl, const int* outl, void* out) {
     const size_t smem = (size_t)kTfWarps * tf_stage_vals<T>() * sizeof(T) + (size_t)c->max_cl_mol * 2;
     auto kern = c->tf_regs == 1 ? k_transform<T, 4> : k_transform<T, 1>;
-    kern<<<c->n_tiles * c->tf_split, kTfWarps * 32, smem, c->stream>>>(
-        c->tf_split, c->max_cl_mol, c->d_tile_row0, c->cap, c->capY, ptr, bl, outl, c->d_cci_ptr, c->d_cci_row,
+    const int split = transform_split(c);
+    kern<<<c->n_tiles * split, kTfWarps * 32, smem, c->stream>>>(
+        split, c->max_cl_mol, c->d_tile_row0, c->cap, c->capY, ptr, bl, outl, c->d_cci_ptr, c->d_cci_row,
         c->d_cci_slot, (const T*)c->d_c_val[c->cur], c->d_y_n, c->d_y_row, (const T*)c->d_y_val, (T*)out);
     return cudaGetLastError();
 }

@@ -86,7 +86,7 @@ struct Ctx {
     int closure_window = 0;  // colours per closure (bounded fill); 0: one closure per sweep
     int apply_variant = 0;   // 0 specialised sweep kernels where they apply, 1 generic only,
                              // 2 specialised with one CTA per block
-    int tf_split = 4;        // CTAs sharing one occupied tile's pairs in the transform (sscf_autotune)
+    int tf_split = 0;        // CTAs sharing one occupied tile's pairs in the transform (sscf_autotune; 0: by size)
     int tf_regs = 0;         // transform register budget: 0 uncut, 1 cut for 4 CTAs per SM (sscf_autotune)
     int n_sm = 152;          // multiprocessors of the context's device
     bool have_guess = false;
@@ -193,7 +193,7 @@ struct Ctx {
     void* d_c_val[2] = {nullptr, nullptr};
     unsigned char* d_c_nz[2] = {nullptr, nullptr};   // per (row block, slot): 0 = tile known all-zero during a sweep
     unsigned char* d_c_cnz = nullptr;   // the current sweep's flags in column-index order
-    void* d_blk_info = nullptr;         // per block of a sweep in colour order: what the FP32 sweep kernel starts from
+    void* d_blk_info = nullptr;         // per block of a sweep in colour order: what the sweep kernel starts from
     int cur = 0;
     int* d_cci_ptr = nullptr;     // n_tiles + 1
     int* d_cci_cnt = nullptr;     // n_tiles
