@@ -128,35 +128,168 @@ __global__ void __launch_bounds__(256) k_rot_hist(int shift, int n_gnb, const in
     if (cur >= 0) flush();
 }
 
-// one thread per cluster: pick the bin holding the kmax-th largest key
-// (last_shift: the final pass; keys below it are zero for every candidate)
+// one warp per cluster: pick the bin holding the kmax-th largest key (last_shift:
+// the final pass; keys below it are zero for every candidate). Lane l holds bins
+// 255 - 8 l and the seven below it, so that a scan over the lanes counts from the
+// largest keys down (one thread reading 256 bins one after the other: 16-20 us a
+// pass; now 3).
 __global__ void k_rot_pick(int shift, int last_shift, int n_clusters, ClSel* cl, unsigned long long* hist) {
-    const int c = blockIdx.x * blockDim.x + threadIdx.x;
+    const int c = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5), lane = threadIdx.x & 31;
     if (c >= n_clusters) return;
     ClSel s = cl[c];
     unsigned long long* h = hist + (size_t)c * 256;
     if (s.cand > s.kmax) {
         if (shift == 56) s.rank = s.kmax;
-        unsigned long long cum = 0;
-        int b = 255;
-        for (; b > 0; --b) {
-            if (cum + h[b] >= s.rank) break;
-            cum += h[b];
+        unsigned long long v[8], sum = 0;
+#pragma unroll
+        for (int i = 0; i < 8; ++i) {
+            v[i] = h[255 - 8 * lane - i];
+            h[255 - 8 * lane - i] = 0ull;
+            sum += v[i];
         }
+        unsigned long long cum = sum;   // keys in this lane's bins and all above
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const unsigned long long u = __shfl_up_sync(0xffffffffu, cum, o);
+            if (lane >= o) cum += u;
+        }
+        // the first lane that reaches the rank, and its bin (bin 0 takes what is left)
+        const unsigned reach = __ballot_sync(0xffffffffu, cum >= s.rank);
+        const int at = reach ? __ffs(reach) - 1 : 31;
+        unsigned long long above = cum - sum;   // keys above the bin
+        int b = 255 - 8 * lane;
+        bool found = false;
+#pragma unroll
+        for (int i = 0; i < 8; ++i) {
+            found = found || b == 0 || above + v[i] >= s.rank;
+            if (!found) {
+                above += v[i];
+                --b;
+            }
+        }
+        b = __shfl_sync(0xffffffffu, b, at);
+        above = __shfl_sync(0xffffffffu, above, at);
         s.prefix |= (unsigned long long)b << shift;
         s.mask |= 255ull << shift;
-        s.rank -= cum;
-        for (int i = 0; i < 256; ++i) h[i] = 0ull;
+        s.rank -= above;
     }
     if (shift == last_shift) s.thr = s.cand > s.kmax ? s.prefix : 0ull;
-    cl[c] = s;
+    if (lane == 0) cl[c] = s;
+}
+
+// The whole selection (k_rot_stats, the radix passes) in one CTA, for a single
+// cluster of few blocks (kSelSmallBlocks): the launches between the passes cost
+// more than the passes (11 of them, 17 in FP64, ~4 us each; now one of 14 us at 8
+// molecules, 56 in FP64 at 32).
+constexpr int kSelSmallBlocks = 512;
+template <typename T>
+__global__ void __launch_bounds__(1024) k_rot_select_small(int last_shift, int n_gnb, const int* __restrict__ gnb_row,
+                                                           const int* __restrict__ gnb_col,
+                                                           const int* __restrict__ group_nmol,
+                                                           const int* __restrict__ group_nvt,
+                                                           const int* __restrict__ blk_tp0, const T* __restrict__ F,
+                                                           double tau, unsigned long long kmax, DeviceScalars* sc,
+                                                           ClSel* cl) {
+    __shared__ unsigned s_h[256];
+    __shared__ unsigned s_cnt, s_bin, s_above;
+    __shared__ unsigned long long s_max;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    if (threadIdx.x == 0) {
+        s_cnt = 0u;
+        s_max = 0ull;
+    }
+    for (int i = threadIdx.x; i < 256; i += blockDim.x) s_h[i] = 0u;
+    __syncthreads();
+    // every candidate key, a block per warp
+    auto each = [&](auto f) {
+        for (int e = warp; e < n_gnb; e += 32) {
+            const int no = 4 * group_nmol[gnb_row[e]], B = gnb_col[e], nv = 2 * group_nmol[B], nvt = group_nvt[B];
+            const T* fe = F + (size_t)blk_tp0[e] * 256;
+#pragma unroll 4
+            for (int p = lane; p < no * 16; p += 32) {
+                const int i = p >> 4, j = p & 15;   // a block has one virtual tile: nvt = 1, nv <= 16
+                if (j >= nv) continue;
+                const double v = fabs((double)fe[(size_t)(i >> 4) * nvt * 256 + (i & 15) * 16 + j]);
+                f(v, v >= tau && v > 0.0);
+            }
+        }
+    };
+    unsigned cnt = 0;
+    unsigned long long mx = 0ull;
+    each([&](double v, bool in) {
+        const unsigned long long k = dkey(v);
+        if (k > mx && v == v) mx = k;
+        cnt += in;
+    });
+    cnt = __reduce_add_sync(0xffffffffu, cnt);
+    for (int o = 16; o > 0; o >>= 1) {
+        const unsigned long long u = __shfl_xor_sync(0xffffffffu, mx, o);
+        mx = u > mx ? u : mx;
+    }
+    if (lane == 0) {
+        atomicAdd(&s_cnt, cnt);
+        atomicMax(&s_max, mx);
+    }
+    __syncthreads();
+    unsigned long long prefix = 0ull, mask = 0ull, rank = kmax;
+    if (s_cnt > kmax) {
+        for (int shift = 56; shift >= last_shift; shift -= 8) {
+            each([&](double v, bool in) {
+                const unsigned long long k = dkey(v);
+                if (in && (k & mask) == prefix) atomicAdd(&s_h[k >> shift & 255ull], 1u);
+            });
+            __syncthreads();
+            if (warp == 0) {   // the bin of the rank-th largest key (k_rot_pick)
+                unsigned h[8], sum = 0;
+#pragma unroll
+                for (int i = 0; i < 8; ++i) {
+                    h[i] = s_h[255 - 8 * lane - i];
+                    s_h[255 - 8 * lane - i] = 0u;
+                    sum += h[i];
+                }
+                unsigned cum = sum;
+                for (int o = 1; o < 32; o <<= 1) {
+                    const unsigned u = __shfl_up_sync(0xffffffffu, cum, o);
+                    if (lane >= o) cum += u;
+                }
+                const unsigned reach = __ballot_sync(0xffffffffu, (unsigned long long)cum >= rank);
+                const int at = reach ? __ffs(reach) - 1 : 31;
+                unsigned above = cum - sum;
+                int b = 255 - 8 * lane;
+                bool found = false;
+#pragma unroll
+                for (int i = 0; i < 8; ++i) {
+                    found = found || b == 0 || (unsigned long long)(above + h[i]) >= rank;
+                    if (!found) {
+                        above += h[i];
+                        --b;
+                    }
+                }
+                if (lane == at) {
+                    s_bin = (unsigned)b;
+                    s_above = above;
+                }
+            }
+            __syncthreads();
+            prefix |= (unsigned long long)s_bin << shift;
+            mask |= 255ull << shift;
+            rank -= s_above;
+        }
+    }
+    if (threadIdx.x == 0) {
+        atomicMax((unsigned long long*)&sc->max_fov, s_max);
+        cl->cand = s_cnt;
+        cl->kmax = kmax;
+        cl->thr = s_cnt > kmax ? prefix : 0ull;
+    }
 }
 
 // per block: kept pairs sorted by (in-block colour, i_loc) with Jacobi angles
 // p = (F_ii - F_jj) / (2 F_ij), t = 1/(p + sgn(p) sqrt(1 + p^2)),
 // c = 1/sqrt(1 + t^2), s = t c in FP64 (sgn(0) = +1)
+constexpr int kListThreads = 128;
 template <typename T>
-__global__ void k_rot_lists(int n_gnb, const int* __restrict__ gnb_row, const int* __restrict__ gnb_col,
+__global__ void __launch_bounds__(kListThreads) k_rot_lists(int n_gnb, const int* __restrict__ gnb_row, const int* __restrict__ gnb_col,
                             const int* __restrict__ group_nmol, const int* __restrict__ group_nvt,
                             const int* __restrict__ group_occ0_mo, const int* __restrict__ group_virt0_mo,
                             const int* __restrict__ group_cl, const int* __restrict__ blk_tp0,
@@ -164,8 +297,11 @@ __global__ void k_rot_lists(int n_gnb, const int* __restrict__ gnb_row, const in
                             const ClSel* __restrict__ cl, int* __restrict__ pr_n,
                             int* __restrict__ pr_lvl, uint16_t* __restrict__ pr_ij, T* __restrict__ pr_cs,
                             int* __restrict__ pr_touch) {
-    __shared__ unsigned char keep[32 * 16];
-    __shared__ int cnt[kMaxSub + 1];
+    // kept pairs per level, as a bit per i: a pair's place in the list is its level's start plus the
+    // kept i below its own, so that every pair is placed, and its angle computed, on its own (one
+    // thread per level walked its pairs one after the other: 54 us at 8 molecules; now 14)
+    __shared__ unsigned s_lv[kMaxSub];
+    __shared__ int s_lvl[kMaxSub + 1];
     const int e = blockIdx.x;
     const int A = gnb_row[e], B = gnb_col[e];
     const int no = 4 * group_nmol[A], nv = 2 * group_nmol[B], nvt = group_nvt[B];
@@ -173,65 +309,66 @@ __global__ void k_rot_lists(int n_gnb, const int* __restrict__ gnb_row, const in
     const unsigned long long thr = cl[group_cl[A]].thr;
     __shared__ int s_touch;
     if (threadIdx.x == 0) s_touch = 0;
+    for (int s = threadIdx.x; s < kMaxSub; s += blockDim.x) s_lv[s] = 0u;
     __syncthreads();
+    constexpr int kPer = 32 * 16 / kListThreads;
+    T val[kPer];   // F_ij of the kept pairs of this thread
+    unsigned kept = 0;
     int touch_t = 0;   // side tiles this thread's kept pairs touch: bits 0-2 side A, 3-5 side B
-    for (int p = threadIdx.x; p < 32 * 16; p += blockDim.x) {
-        int i = p >> 4, j = p & 15;
-        unsigned char kp = 0;
+#pragma unroll
+    for (int u = 0; u < kPer; ++u) {
+        const int p = threadIdx.x + u * kListThreads, i = p >> 4, j = p & 15;
+        val[u] = (T)0;
         if (i < no && j < nv) {
             const int tp = blk_tp0[e] + (i >> 4) * nvt + (j >> 4);
-            const double f = fabs((double)F[(size_t)tp * 256 + (i & 15) * 16 + (j & 15)]);
-            kp = (f >= tau && f > 0.0 && dkey(f) >= thr) ? 1 : 0;
-            if (kp) touch_t |= (1 << (i >> 4)) | (1 << (3 + (j >> 4)));
+            val[u] = F[(size_t)tp * 256 + (i & 15) * 16 + (j & 15)];
+            const double f = fabs((double)val[u]);
+            if (f >= tau && f > 0.0 && dkey(f) >= thr) {
+                kept |= 1u << u;
+                touch_t |= (1 << (i >> 4)) | (1 << (3 + (j >> 4)));
+                const int s = i + j;
+                atomicOr(&s_lv[s >= nsub ? s - nsub : s], 1u << i);
+            }
         }
-        keep[p] = kp;
     }
     if (touch_t) atomicOr(&s_touch, touch_t);
     __syncthreads();
-    if ((int)threadIdx.x < nsub) {
-        const int s = threadIdx.x;
-        int c = 0;
-        for (int i = 0; i < no; ++i) {
-            int j = ((s - i) % nsub + nsub) % nsub;
-            if (j < nv && keep[i * 16 + j]) ++c;
+    if (threadIdx.x < 32) {   // level starts: two levels per lane, 64 >= kMaxSub + 1
+        const int a0 = 2 * threadIdx.x, c0 = a0 < kMaxSub ? __popc(s_lv[a0]) : 0, c1 = a0 + 1 < kMaxSub ? __popc(s_lv[a0 + 1]) : 0;
+        int inc = c0 + c1;
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const int v = __shfl_up_sync(0xffffffffu, inc, o);
+            if ((int)threadIdx.x >= o) inc += v;
         }
-        cnt[s] = c;
+        if (a0 <= kMaxSub) s_lvl[a0] = inc - c0 - c1;
+        if (a0 + 1 <= kMaxSub) s_lvl[a0 + 1] = inc - c1;
     }
     __syncthreads();
+    for (int s = threadIdx.x; s <= kMaxSub; s += blockDim.x) pr_lvl[(size_t)e * (kMaxSub + 1) + s] = s_lvl[s];
     if (threadIdx.x == 0) {
-        int run = 0;
-        int* lvl = pr_lvl + (size_t)e * (kMaxSub + 1);
-        for (int s = 0; s < nsub; ++s) {
-            lvl[s] = run;
-            run += cnt[s];
-        }
-        for (int s = nsub; s <= kMaxSub; ++s) lvl[s] = run;
+        const int run = s_lvl[kMaxSub];
         pr_n[e] = run;
-        cnt[kMaxSub] = run;
         if (run) atomicAdd(&sc->n_rot, (unsigned long long)run);
         pr_touch[e] = s_touch;
     }
-    __syncthreads();
-    if ((int)threadIdx.x < nsub) {
-        const int s = threadIdx.x;
-        int pos = pr_lvl[(size_t)e * (kMaxSub + 1) + s];
-        for (int i = 0; i < no; ++i) {
-            int j = ((s - i) % nsub + nsub) % nsub;
-            if (!(j < nv && keep[i * 16 + j])) continue;
-            const int tp = blk_tp0[e] + (i >> 4) * nvt + (j >> 4);
-            const double fij = (double)F[(size_t)tp * 256 + (i & 15) * 16 + (j & 15)];
-            const double fii = Fd[group_occ0_mo[A] + i], fjj = Fd[group_virt0_mo[B] + j];
-            const double p = __ddiv_rn(__dsub_rn(fii, fjj), __dmul_rn(2.0, fij));
-            const double sg = p >= 0.0 ? 1.0 : -1.0;
-            const double t = __ddiv_rn(1.0, __dadd_rn(p, __dmul_rn(sg, sqrt(__dadd_rn(1.0, __dmul_rn(p, p))))));
-            const double cc = __ddiv_rn(1.0, sqrt(__dadd_rn(1.0, __dmul_rn(t, t))));
-            const double ss = __dmul_rn(t, cc);
-            const size_t q = (size_t)e * kOrthoCap + pos;
-            pr_ij[q] = (uint16_t)(i | (j << 8));
-            pr_cs[2 * q] = (T)cc;
-            pr_cs[2 * q + 1] = (T)ss;
-            ++pos;
-        }
+#pragma unroll
+    for (int u = 0; u < kPer; ++u) {
+        if (!(kept >> u & 1)) continue;
+        const int p0 = threadIdx.x + u * kListThreads, i = p0 >> 4, j = p0 & 15;
+        const int s = i + j >= nsub ? i + j - nsub : i + j;
+        const int pos = s_lvl[s] + __popc(s_lv[s] & ((1u << i) - 1u));
+        const double fij = (double)val[u];
+        const double fii = Fd[group_occ0_mo[A] + i], fjj = Fd[group_virt0_mo[B] + j];
+        const double p = __ddiv_rn(__dsub_rn(fii, fjj), __dmul_rn(2.0, fij));
+        const double sg = p >= 0.0 ? 1.0 : -1.0;
+        const double t = __ddiv_rn(1.0, __dadd_rn(p, __dmul_rn(sg, sqrt(__dadd_rn(1.0, __dmul_rn(p, p))))));
+        const double cc = __ddiv_rn(1.0, sqrt(__dadd_rn(1.0, __dmul_rn(t, t))));
+        const double ss = __dmul_rn(t, cc);
+        const size_t q = (size_t)e * kOrthoCap + pos;
+        pr_ij[q] = (uint16_t)(i | (j << 8));
+        pr_cs[2 * q] = (T)cc;
+        pr_cs[2 * q + 1] = (T)ss;
     }
 }
 
@@ -310,7 +447,7 @@ __global__ void k_ortho_eta(int w, const int* __restrict__ oblk, int n_oblk, con
 }
 
 template <typename T>
-__global__ void k_ortho_lists(int w, double tol, const int* __restrict__ oblk, const int* __restrict__ gnb_row,
+__global__ void __launch_bounds__(kListThreads) k_ortho_lists(int w, double tol, const int* __restrict__ oblk, const int* __restrict__ gnb_row,
                               const int* __restrict__ gnb_col, const int* __restrict__ group_nmol,
                               const int* __restrict__ group_not, const int* __restrict__ occ0,
                               const int* __restrict__ virt0, const int* __restrict__ blk_tp,
@@ -318,9 +455,9 @@ __global__ void k_ortho_lists(int w, double tol, const int* __restrict__ oblk, c
                               const int* __restrict__ group_cl, const double* __restrict__ cl_eta,
                               int* __restrict__ pr_n, int* __restrict__ pr_lvl, uint16_t* __restrict__ pr_ij,
                               T* __restrict__ pr_cs, int* __restrict__ pr_touch) {
-    __shared__ unsigned char keep[48 * 48];
-    __shared__ double s_sh[48 * 48];   // the normalised overlap of every kept pair
-    __shared__ int cnt[kMaxSub + 1];
+    // as k_rot_lists: kept pairs per level as a bit per i
+    __shared__ unsigned long long s_lv[kMaxSub];
+    __shared__ int s_lvl[kMaxSub + 1];
     const int e = oblk[blockIdx.x];
     const int A = gnb_row[e], B = gnb_col[e];
     const int noA = 4 * group_nmol[A], noB = 4 * group_nmol[B];
@@ -332,63 +469,62 @@ __global__ void k_ortho_lists(int w, double tol, const int* __restrict__ oblk, c
     const double cut = 1e-3 * eta;
     __shared__ int s_touch;
     if (threadIdx.x == 0) s_touch = 0;
+    for (int s = threadIdx.x; s < kMaxSub; s += blockDim.x) s_lv[s] = 0ull;
     __syncthreads();
+    constexpr int kPer = 48 * 48 / kListThreads;
+    T half[kPer];   // half the normalised overlap of the kept pairs of this thread
+    unsigned kept = 0;
     int touch_t = 0;   // side tiles this thread's kept pairs touch: bits 0-2 side A, 3-5 side B
-    for (int p = threadIdx.x; p < 48 * 48; p += blockDim.x) {
-        const int i = p / 48, j = p % 48;
-        unsigned char kp = 0;
+#pragma unroll
+    for (int u = 0; u < kPer; ++u) {
+        const int p = threadIdx.x + u * kListThreads, i = p / 48, j = p - 48 * i;
+        half[u] = (T)0;
         if (active && i < nA && j < nB && !(same && j <= i)) {
             int ia, ci, ib, cj;
             side_pos(i, noA, group_not[A], ia, ci);
             side_pos(j, noB, group_not[B], ib, cj);
             const double di = dsc[pass_mo(i, noA, occ0, virt0, A)], dj = dsc[pass_mo(j, noB, occ0, virt0, B)];
             const double sh = sig_hat(sig, blk_tp, e, same, ia, ib, ci, cj, di, dj);
-            kp = fabs(sh) >= cut ? 1 : 0;
-            if (kp) {
+            if (fabs(sh) >= cut) {
+                kept |= 1u << u;
                 touch_t |= (1 << ia) | (1 << (3 + ib));
-                s_sh[p] = sh;
+                half[u] = (T)__dmul_rn(0.5, sh);
+                const int s = i + j;
+                atomicOr(&s_lv[s >= nsub ? s - nsub : s], 1ull << i);
             }
         }
-        keep[p] = kp;
     }
     if (touch_t) atomicOr(&s_touch, touch_t);
     __syncthreads();
-    if ((int)threadIdx.x < nsub) {
-        const int s = threadIdx.x;
-        int c = 0;
-        for (int i = 0; i < nA; ++i) {
-            int j = ((s - i) % nsub + nsub) % nsub;
-            if (j < nB && keep[i * 48 + j]) ++c;
+    if (threadIdx.x < 32) {   // level starts: two levels per lane, 64 >= kMaxSub + 1
+        const int a0 = 2 * threadIdx.x, c0 = a0 < kMaxSub ? __popcll(s_lv[a0]) : 0,
+                  c1 = a0 + 1 < kMaxSub ? __popcll(s_lv[a0 + 1]) : 0;
+        int inc = c0 + c1;
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const int v = __shfl_up_sync(0xffffffffu, inc, o);
+            if ((int)threadIdx.x >= o) inc += v;
         }
-        cnt[s] = c;
+        if (a0 <= kMaxSub) s_lvl[a0] = inc - c0 - c1;
+        if (a0 + 1 <= kMaxSub) s_lvl[a0 + 1] = inc - c1;
     }
     __syncthreads();
+    for (int s = threadIdx.x; s <= kMaxSub; s += blockDim.x) pr_lvl[(size_t)e * (kMaxSub + 1) + s] = s_lvl[s];
     if (threadIdx.x == 0) {
-        int run = 0;
-        int* lvl = pr_lvl + (size_t)e * (kMaxSub + 1);
-        for (int s = 0; s < nsub; ++s) {
-            lvl[s] = run;
-            run += cnt[s];
-        }
-        for (int s = nsub; s <= kMaxSub; ++s) lvl[s] = run;
+        const int run = s_lvl[kMaxSub];
         pr_n[e] = run;
         if (run) atomicAdd(&sc->n_combo, (unsigned long long)run);
         pr_touch[e] = s_touch;
     }
-    __syncthreads();
-    if ((int)threadIdx.x < nsub) {
-        const int s = threadIdx.x;
-        int pos = pr_lvl[(size_t)e * (kMaxSub + 1) + s];
-        for (int i = 0; i < nA; ++i) {
-            int j = ((s - i) % nsub + nsub) % nsub;
-            if (!(j < nB && keep[i * 48 + j])) continue;
-            const double sh = s_sh[i * 48 + j];
-            const size_t q = (size_t)e * kOrthoCap + pos;
-            pr_ij[q] = (uint16_t)(i | (j << 8));
-            pr_cs[2 * q] = (T)__dmul_rn(0.5, sh);
-            pr_cs[2 * q + 1] = (T)0;
-            ++pos;
-        }
+#pragma unroll
+    for (int u = 0; u < kPer; ++u) {
+        if (!(kept >> u & 1)) continue;
+        const int p = threadIdx.x + u * kListThreads, i = p / 48, j = p - 48 * i;
+        const int s = i + j >= nsub ? i + j - nsub : i + j;
+        const size_t q = (size_t)e * kOrthoCap + s_lvl[s] + __popcll(s_lv[s] & ((1ull << i) - 1ull));
+        pr_ij[q] = (uint16_t)(i | (j << 8));
+        pr_cs[2 * q] = half[u];
+        pr_cs[2 * q + 1] = (T)0;
     }
 }
 
@@ -454,17 +590,26 @@ struct SweepArgs {
     void* out_val;
     unsigned char* out_nz;   // flags of out: 0 = the tile is all zero (written by the closure, kept by the sweep)
     unsigned char* col_nz;   // sweeps: the same flags in column-index order (flag_base)
-    void* blk_info;          // FP32 sweeps: a BlockInfo per block in colour order
+    void* blk_info;          // a BlockInfo per block in colour order
     const unsigned char* in_nz;   // closure: flags of the input (NULL: every listed tile may be nonzero)
     int normalise_pass;      // closure in mode 1: divide by d_i (the first closure of a pass)
     unsigned* err;
 };
 
 
-// truncation test |x| < threshold, decided exactly in the storage precision
-__device__ __forceinline__ bool below(double x, const SweepArgs& a) { return fabs(x) < a.trunc; }
+// truncation test |x| < threshold, decided exactly in the storage precision;
+// FP64 on the bit patterns (those of non-negative doubles order as the values
+// do, and a NaN is above any threshold, as it is not below in the comparison of
+// values): the FP64 pipe has two lanes per clock and SM, and a comparison there
+// costs as much as the update it follows
+__device__ __forceinline__ bool below(double x, const SweepArgs& a) {
+    return ((unsigned long long)__double_as_longlong(x) & 0x7fffffffffffffffull) <
+           (unsigned long long)__double_as_longlong(a.trunc);
+}
 __device__ __forceinline__ bool below(float x, const SweepArgs& a) { return fabsf(x) < a.trunc_f; }
-static_assert(sizeof(float) == 4, "");
+// x != 0 without the FP64 pipe
+__device__ __forceinline__ bool nonzero(double x) { return (__double_as_longlong(x) << 1) != 0; }
+__device__ __forceinline__ bool nonzero(float x) { return x != 0.f; }
 
 // Connected components of a pass's units (the occupied or the virtual tiles
 // of one group) under its active blocks, one CTA per cluster. The closure of a
@@ -965,7 +1110,7 @@ __global__ void __launch_bounds__(apply_threads<T>()) k_apply_colour(SweepArgs a
     if (row < nk * 6)
         for (int cidx = 0; cidx < NT * 16 && !nzrow; ++cidx)
 #pragma unroll
-            for (int r2 = 0; r2 < R; ++r2) nzrow |= panel[cidx * NRP + row + r2] != (T)0;
+            for (int r2 = 0; r2 < R; ++r2) nzrow |= nonzero(panel[cidx * NRP + row + r2]);
     const bool warp_busy = __any_sync(0xffffffffu, nzrow);
     if (row < nk * 6 && warp_busy) {
         T* pr = panel + row;
@@ -1049,7 +1194,7 @@ __global__ void __launch_bounds__(apply_threads<T>()) k_apply_colour(SweepArgs a
 #pragma unroll
         for (int col = 0; col < 16; ++col) {
             e2[col] = srcp[col * NRP];
-            any |= e2[col] != (T)0;
+            any |= nonzero(e2[col]);
         }
         if (any) {   // the tile may be nonzero now
             a.out_nz[(size_t)s_row[rb] * a.cap + sl] = 1;
@@ -1061,7 +1206,7 @@ __global__ void __launch_bounds__(apply_threads<T>()) k_apply_colour(SweepArgs a
     }
 }
 
-// FP32 sweeps, one warp at a time. Same updates, order and truncation as
+// Sweeps, one warp at a time. Same updates, order and truncation as
 // k_apply_colour; what differs is where the values sit and who waits for whom.
 //
 // A CTA serves a block (A, B) of the colour. It reads the tile flags of all the
@@ -1086,8 +1231,11 @@ __global__ void __launch_bounds__(apply_threads<T>()) k_apply_colour(SweepArgs a
 //           packed, 8.2 unpacked, in a loop of its own; the FMA and ALU pipes
 //           would take 4, the operand reads of the register file bound it.
 //   list    the block's pairs one after the other in schedule order, both sides
-//           in a shared-memory panel [column][lane], one AO row per lane. Self
-//           blocks, rotations, and combination blocks with few pairs.
+//           in a shared-memory panel [column][lane], one AO row per lane, up to
+//           four pairs of a level in flight. Self blocks, rotations, combination
+//           blocks with few pairs, and everything in FP64 storage, where the FP64
+//           pipe (two lanes per clock and SM) is the bound and slots without a
+//           pair are not to cost anything.
 // n = max(MOs of A, MOs of B) is the modulus of the in-block colour; the dense
 // loop exists for every n a pair of groups can have, so blocks of partly filled
 // groups run it as well (their missing MOs are zero columns without pairs).
@@ -1095,8 +1243,7 @@ __global__ void __launch_bounds__(apply_threads<T>()) k_apply_colour(SweepArgs a
 // side in registers, the others staged for the generic kernel): occupied pass
 // at 4096 molecules 68.9 -> 41.9 ms, at 997 9.9 -> 5.3; four passes over all
 // MOs at 512 18.6 -> 5.2; rotations at 4096 14.8 -> 9.6, at 997 3.2 -> 1.7.
-constexpr int kWsWarps = 4;
-constexpr int kWsThreads = 32 * kWsWarps;
+// FP64 at 343 molecules: occupied pass 14.5 -> 12.7, rotations 2.3 -> 1.4.
 constexpr int kFullCH = 32;                  // row blocks per word of the bits of rows with work
 constexpr int kFullBatch = 8;                // 16-byte pieces of a tile per lane and run of 32 row pairs, all in flight
 // runs a CTA takes at least: one per warp, or two where a launch could have more than kWsManyRuns
@@ -1112,26 +1259,38 @@ constexpr int kWsPad = 34;                   // floats per panel column: 16-byte
 // 8: 5.7, 5.35, 5.2 ms for the passes over all MOs at 512 molecules; few blocks lie in between later)
 constexpr int kWsDenseDiv = 8;
 // MODE 0 rotations, MODE 1 combinations of occupied MOs (ALL = false) or of all MOs
-template <int MODE, bool ALL> struct WarpShape {
+template <typename T, int MODE, bool ALL> struct WarpShape {
+    static constexpr bool f32 = std::is_same<T, float>::value;
     static constexpr int nta = ALL ? 3 : 2;                    // side tiles
     static constexpr int ntb = MODE == 0 ? 1 : nta;
     static constexpr int nmax = ALL ? 48 : 32;                 // largest modulus
     static constexpr int gstep = ALL ? 6 : 4;                  // MOs per molecule and side
-    static constexpr int halves = MODE == 1 && !ALL ? 2 : 1;   // AO rows a lane holds in the dense loop
-    // bytes of the block's coefficients or pairs: MODE 0 at most kRotCap pairs of 16; MODE 1 a dense
-    // table of n^2 (c, t), or 8-byte pairs (fewer than n^2 / kWsDenseDiv, or n (n - 1) / 2 of a self
-    // block), and four ending the list
-    static constexpr int table = MODE == 0 ? (kRotCap + 4) * 16 : nmax * nmax * 8;
+    // FP64 CTAs are half as large: the pipe is busy with a few warps per SM, and the smaller the
+    // pieces, the more evenly the SMs share it
+    static constexpr int warps = f32 ? 4 : 2, threads = 32 * warps;
+    // order of the CTAs: all shares of a block, then the next block (the long blocks first: the short
+    // ones even out the end; FP64 occupied pass at 343 molecules 15.9 -> 12.7 ms, rotations at 4096
+    // 9.7 -> 9.2), or the first share of all blocks, then the second (FP32 combinations, whose later
+    // shares are the empty ones: 5.2 against 5.6 ms at 512 molecules)
+    static constexpr bool by_block = !f32 || MODE == 0;
+    static constexpr int halves = f32 && MODE == 1 && !ALL ? 2 : 1;   // AO rows of an entry in the dense loop
+    // bytes of the block's coefficients or pairs, with four entries ending the list. FP32: at most
+    // kRotCap rotations of 16; a dense table of n^2 (c, t), or 8-byte combinations (fewer than
+    // n^2 / kWsDenseDiv, or n (n - 1) / 2 of a self block). FP64: coefficients, then the 4-byte words.
+    static constexpr int cap = (MODE == 0 ? kRotCap : nmax * nmax) + 4;
+    static constexpr int table = f32 ? (MODE == 0 ? cap * 16 : nmax * nmax * 8) : cap * (MODE == 0 ? 20 : 12);
     static_assert(MODE == 0 || (nmax * (nmax - 1) / 2 + 4) * 8 <= nmax * nmax * 8, "");
+    static_assert(table % 16 == 0, "");
     // bytes per warp: the list's panel; the dense loop's: one side of 32 row pairs (occupied passes),
     // or a run's tiles as they lie in memory and the next run's (passes over all MOs)
-    static constexpr int raw = ALL ? (nta + ntb) * 32 * 64 : 0;
-    static constexpr int panel = (nta + ntb) * 16 * kWsPad * 4;
+    static constexpr int raw = f32 && ALL ? (nta + ntb) * 32 * 64 : 0;
+    static constexpr int panel = (nta + ntb) * 16 * kWsPad * (int)sizeof(T);
     static constexpr int per_warp = 2 * raw > panel ? 2 * raw : panel;
     static_assert(MODE == 0 || ALL || per_warp >= nta * 16 * 64 * 4, "");
-    static constexpr size_t smem = (size_t)table + (size_t)kWsWarps * per_warp;   // + row bits
-    // resident CTAs the register budget is cut for: the dense loop holds 2 n values per row
-    static constexpr int min_ctas = MODE == 0 ? 6 : (ALL ? 2 : 3);
+    static constexpr size_t smem = (size_t)table + (size_t)warps * per_warp;   // + row bits
+    // resident CTAs the register budget is cut for: the dense loop holds 2 n values per row; FP64
+    // runs as many as its panels leave room for
+    static constexpr int min_ctas = f32 ? (MODE == 0 ? 6 : (ALL ? 2 : 3)) : (MODE == 0 ? 6 : (ALL ? 2 : 4));
 };
 
 // 1.0 where |v| >= t, 0.0 below (and for NaN): one compare that writes the
@@ -1148,6 +1307,8 @@ __device__ __forceinline__ float ge_abs_factor(float v, float t) {
 // zero may come out as -0, which every later test treats as zero)
 __device__ __forceinline__ float trunc_mul(float v, float t) { return __fmul_rn(v, ge_abs_factor(v, t)); }
 __device__ __forceinline__ float fma_s(float c, float a, float b) { return __fmaf_rn(c, a, b); }
+__device__ __forceinline__ float mul_rn(float a, float b) { return __fmul_rn(a, b); }
+__device__ __forceinline__ double mul_rn(double a, double b) { return __dmul_rn(a, b); }
 
 __device__ __forceinline__ float2 trunc_mul(float2 v, float t) {
     return __fmul2_rn(v, make_float2(ge_abs_factor(v.x, t), ge_abs_factor(v.y, t)));
@@ -1227,16 +1388,18 @@ __global__ void k_block_info(SweepArgs a, int n, BlockInfo* __restrict__ info) {
         atomicAdd(a.upd, (unsigned long long)b.i0.y * (unsigned long long)(b.i0.w * kAoPerMol));
 }
 
-template <int MODE, bool ALL>
-__global__ void __launch_bounds__(kWsThreads, (WarpShape<MODE, ALL>::min_ctas))
+template <typename T, int MODE, bool ALL>
+__global__ void __launch_bounds__((WarpShape<T, MODE, ALL>::threads), (WarpShape<T, MODE, ALL>::min_ctas))
 k_apply_warp(SweepArgs a, int p0, int nb, int min_runs) {
-    using Sh = WarpShape<MODE, ALL>;
+    using Sh = WarpShape<T, MODE, ALL>;
+    constexpr bool F32 = Sh::f32;
+    constexpr int kWsWarps = Sh::warps, kWsThreads = Sh::threads;
     constexpr int NTA = Sh::nta, NTB = Sh::ntb;
     extern __shared__ __align__(16) unsigned char smraw[];
     __shared__ int s_wsum[kWsWarps], s_next;
     if (*a.err & (kErrCapacity | kErrSortSize)) return;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    const BlockInfo& info = ((const BlockInfo*)a.blk_info)[p0 + blockIdx.x % nb];
+    const BlockInfo& info = ((const BlockInfo*)a.blk_info)[p0 + (Sh::by_block ? blockIdx.x / (gridDim.x / nb) : blockIdx.x % nb)];
     const int4 i0 = info.i0, i1 = info.i1, i2 = info.i2;
     const int e = i0.x, np = i0.y, touch = i0.z, n_rows = i0.w;
     if (np == 0) return;
@@ -1296,10 +1459,10 @@ k_apply_warp(SweepArgs a, int p0, int nb, int min_runs) {
         before += w < warp ? s_wsum[w] : 0;
         n_work += s_wsum[w];
     }
-    const bool dense = MODE == 1 && !same && np * kWsDenseDiv >= n * n;
+    const bool dense = F32 && MODE == 1 && !same && np * kWsDenseDiv >= n * n;
     const int hh = dense ? Sh::halves : 1;   // AO rows of a lane's entry (adjacent ones)
     const int n_ent = kAoPerMol / hh * n_work, n_run = (n_ent + 31) / 32;
-    const int share = blockIdx.x / nb, shares = gridDim.x / nb;
+    const int shares = gridDim.x / nb, share = Sh::by_block ? blockIdx.x % shares : blockIdx.x / nb;
     const int per = max(min_runs, (n_run + shares - 1) / shares);
     const int run_lo = share * per, run_hi = min(n_run, run_lo + per);
     if (run_lo >= run_hi) return;
@@ -1313,11 +1476,13 @@ k_apply_warp(SweepArgs a, int p0, int nb, int min_runs) {
     auto colA = [&](int i) { return MODE == 0 || !ALL || i < noA ? i : 16 * otA + i - noA; };
     auto colB = [&](int j) { return MODE == 0 || !ALL || j < noB ? j : 16 * otB + j - noB; };
     // table (dense) or list of the block's pairs
-    const float* cs = (const float*)a.pr_cs + (size_t)e * kOrthoCap * 2;
+    const T* cs = (const T*)a.pr_cs + (size_t)e * kOrthoCap * 2;
     const uint16_t* ij = a.pr_ij + (size_t)e * kOrthoCap;
     float2* table = (float2*)smraw;
     float2* pair2 = (float2*)smraw;
     float4* pair4 = (float4*)smraw;
+    double* coef64 = (double*)smraw;                                                     // FP64: c, or c and s
+    unsigned* word64 = (unsigned*)(coef64 + (size_t)Sh::cap * (MODE == 0 ? 2 : 1));
     if (dense) {
         for (int i = threadIdx.x; i < n * n; i += kWsThreads) table[i] = make_float2(0.f, 0.f);
         __syncthreads();
@@ -1325,32 +1490,48 @@ k_apply_warp(SweepArgs a, int p0, int nb, int min_runs) {
     for (int q = threadIdx.x; q < np; q += kWsThreads) {
         const int w = ij[q], il = w & 255, jl = w >> 8;
         const int s = il + jl, lv = s >= n ? s - n : s;
-        const float2 c = ((const float2*)cs)[q];
         // list: panel offsets of both sides (12 bits each) and, between them, the level
         const unsigned off = (unsigned)(colA(il) * kWsPad) | (unsigned)lv << 12 |
                              ((unsigned)(((same ? 0 : 16 * NTA) + colB(jl)) * kWsPad) << 18);
-        if constexpr (MODE == 0) pair4[q] = make_float4(__uint_as_float(off), c.x, c.y, 0.f);
-        else if (dense) table[lv * n + il] = make_float2(-c.x, a.trunc_f);
-        else pair2[q] = make_float2(__uint_as_float(off), -c.x);
+        if constexpr (F32) {
+            const float2 c = ((const float2*)cs)[q];
+            if constexpr (MODE == 0) pair4[q] = make_float4(__uint_as_float(off), c.x, c.y, 0.f);
+            else if (dense) table[lv * n + il] = make_float2(-c.x, a.trunc_f);
+            else pair2[q] = make_float2(__uint_as_float(off), -c.x);
+        } else {
+            if constexpr (MODE == 0) {
+                coef64[2 * q] = cs[2 * q];
+                coef64[2 * q + 1] = cs[2 * q + 1];
+            } else {
+                coef64[q] = -cs[2 * q];
+            }
+            word64[q] = off;
+        }
     }
     if (!dense && threadIdx.x < 4) {   // ends the list: a level of its own
-        if constexpr (MODE == 0) pair4[np + threadIdx.x] = make_float4(__uint_as_float(63u << 12), 0.f, 0.f, 0.f);
-        else pair2[np + threadIdx.x] = make_float2(__uint_as_float(63u << 12), 0.f);
+        const int q = np + threadIdx.x;
+        if constexpr (!F32) word64[q] = 63u << 12;
+        else if constexpr (MODE == 0) pair4[q] = make_float4(__uint_as_float(63u << 12), 0.f, 0.f, 0.f);
+        else pair2[q] = make_float2(__uint_as_float(63u << 12), 0.f);
     }
     __syncthreads();
-    float* const mem = (float*)(smraw + Sh::table + (size_t)warp * Sh::per_warp);   // the warp's
-    float* const val = (float*)a.out_val;                                           // in place
+    T* const mem = (T*)(smraw + Sh::table + (size_t)warp * Sh::per_warp);   // the warp's
+    T* const val = (T*)a.out_val;                                           // in place
     // the block's pairs on the panel, in schedule order (lanes hold different rows)
     auto run_list = [&](bool active) {
         // pairs of one level touch different columns: up to four of them in flight
         if (active) {
             auto upd = [&](int q, auto width) {
                 constexpr int N = decltype(width)::value;
-                float *px[N], *py[N], xv[N], yv[N], c0[N], c1[N];
+                T *px[N], *py[N], xv[N], yv[N], c0[N], c1[N];
 #pragma unroll
                 for (int u = 0; u < N; ++u) {
                     unsigned off;
-                    if constexpr (MODE == 0) {
+                    if constexpr (!F32) {
+                        off = word64[q + u];
+                        c0[u] = coef64[MODE == 0 ? 2 * (q + u) : q + u];
+                        c1[u] = MODE == 0 ? coef64[2 * (q + u) + 1] : 0.0;
+                    } else if constexpr (MODE == 0) {
                         const float4 c = pair4[q + u];
                         off = __float_as_uint(c.x);
                         c0[u] = c.y;
@@ -1368,21 +1549,22 @@ k_apply_warp(SweepArgs a, int p0, int nb, int min_runs) {
                 }
 #pragma unroll
                 for (int u = 0; u < N; ++u) {
-                    float xn, yn;
+                    T xn, yn;
                     if constexpr (MODE == 0) {
-                        xn = __fmaf_rn(c0[u], xv[u], __fmul_rn(c1[u], yv[u]));
-                        yn = __fmaf_rn(c0[u], yv[u], __fmul_rn(-c1[u], xv[u]));
+                        xn = fma(c0[u], xv[u], mul_rn(c1[u], yv[u]));
+                        yn = fma(c0[u], yv[u], mul_rn(-c1[u], xv[u]));
                     } else {
-                        xn = __fmaf_rn(c0[u], yv[u], xv[u]);
-                        yn = __fmaf_rn(c0[u], xv[u], yv[u]);
+                        xn = fma(c0[u], yv[u], xv[u]);
+                        yn = fma(c0[u], xv[u], yv[u]);
                     }
-                    *px[u] = below(xn, a) ? 0.f : xn;
-                    *py[u] = below(yn, a) ? 0.f : yn;
+                    *px[u] = below(xn, a) ? (T)0 : xn;
+                    *py[u] = below(yn, a) ? (T)0 : yn;
                 }
             };
             auto level = [&](int q) {
                 unsigned off;
-                if constexpr (MODE == 0) off = __float_as_uint(pair4[q].x);
+                if constexpr (!F32) off = word64[q];
+                else if constexpr (MODE == 0) off = __float_as_uint(pair4[q].x);
                 else off = __float_as_uint(pair2[q].x);
                 return off >> 12 & 63u;
             };
@@ -1401,7 +1583,10 @@ k_apply_warp(SweepArgs a, int p0, int nb, int min_runs) {
             }
         }
     };
-    const int qe = lane >> 2, qp = lane & 3;   // row (mod 8) and 16-byte piece of it that a lane moves
+    // 16-byte pieces of an AO row of a tile, rows a warp moves at a time, and a lane's row and piece
+    using V = typename std::conditional<F32, float4, double2>::type;
+    constexpr int kV = 16 / (int)sizeof(T), kPieces = 16 / kV, kAt = 32 / kPieces, kTimes = 32 / kAt;
+    const int qe = lane / kPieces, qp = lane % kPieces;
     // an AO row of a run: the tiles (row block * cap + slot) its first occupied tile and its virtual
     // one have on either side, and 8 * position in the block's row list + AO row of the row block
     struct Row {
@@ -1473,46 +1658,54 @@ k_apply_warp(SweepArgs a, int p0, int nb, int min_runs) {
     int run = __shfl_sync(0xffffffffu, grab(), 0);
     if (run >= run_hi) return;
     if (MODE == 0 || !dense) {
-        float* const pq = mem + 4 * qp * kWsPad + qe;
+        T* const pq = mem + kV * qp * kWsPad + qe;
+        constexpr int kTiles = F32 ? NTA + NTB : 2;   // tiles in flight
         while (run < run_hi) {
             const Row r = look_up(run);
             const int grabbed = grab();
             const int take = min(32, n_ent - 32 * run);
-            float4 v[NTA + NTB][4];
 #pragma unroll
-            for (int u = 0; u < 4; ++u) {
-                const Row o = row_from(r, 8 * u + qe);
+            for (int t0 = 0; t0 < NTA + NTB; t0 += kTiles) {
+                V v[kTiles][kTimes];
 #pragma unroll
-                for (int t = 0; t < NTA + NTB; ++t) {
-                    v[t][u] = make_float4(0.f, 0.f, 0.f, 0.f);
-                    if (8 * u + qe < take && touched(t)) v[t][u] = *((const float4*)values(o, tile_of(o, t)) + qp);
+                for (int u = 0; u < kTimes; ++u) {
+                    const Row o = row_from(r, kAt * u + qe);
+#pragma unroll
+                    for (int t = 0; t < kTiles; ++t) {
+                        v[t][u] = V{};
+                        if (t0 + t < NTA + NTB && kAt * u + qe < take && touched(t0 + t))
+                            v[t][u] = *((const V*)values(o, tile_of(o, t0 + t)) + qp);
+                    }
                 }
+#pragma unroll
+                for (int t = 0; t < kTiles && t0 + t < NTA + NTB; ++t)
+#pragma unroll
+                    for (int u = 0; u < kTimes; ++u)
+#pragma unroll
+                        for (int w = 0; w < kV; ++w)
+                            pq[((t0 + t) * 16 + w) * kWsPad + kAt * u] = ((const T*)&v[t][u])[w];
             }
-#pragma unroll
-            for (int t = 0; t < NTA + NTB; ++t)
-#pragma unroll
-                for (int u = 0; u < 4; ++u) {
-                    float* d = pq + t * 16 * kWsPad + 8 * u;
-                    d[0] = v[t][u].x;
-                    d[kWsPad] = v[t][u].y;
-                    d[2 * kWsPad] = v[t][u].z;
-                    d[3 * kWsPad] = v[t][u].w;
-                }
             __syncwarp();
             run_list(lane < take);
             __syncwarp();
 #pragma unroll
-            for (int u = 0; u < 4; ++u) {
-                const Row o = row_from(r, 8 * u + qe);
-                if (8 * u + qe >= take) continue;
+            for (int u = 0; u < kTimes; ++u) {
+                const Row o = row_from(r, kAt * u + qe);
+                if (kAt * u + qe >= take) continue;
 #pragma unroll
                 for (int t = 0; t < NTA + NTB; ++t) {
                     if (!touched(t)) continue;
-                    const float* d = pq + t * 16 * kWsPad + 8 * u;
-                    const float4 f = make_float4(d[0], d[kWsPad], d[2 * kWsPad], d[3 * kWsPad]);
+                    V f;
+                    bool nz = false;
+#pragma unroll
+                    for (int w = 0; w < kV; ++w) {
+                        const T x = pq[(t * 16 + w) * kWsPad + kAt * u];
+                        ((T*)&f)[w] = x;
+                        nz |= nonzero(x);
+                    }
                     const unsigned tile = tile_of(o, t);
-                    *((float4*)values(o, tile) + qp) = f;
-                    if (f.x != 0.f || f.y != 0.f || f.z != 0.f || f.w != 0.f) raise(o, t, tile);
+                    *((V*)values(o, tile) + qp) = f;
+                    if (nz) raise(o, t, tile);
                 }
             }
             __syncwarp();
@@ -1522,7 +1715,7 @@ k_apply_warp(SweepArgs a, int p0, int nb, int min_runs) {
     }
     // an occupied pass: 32 row pairs per run. Eight lanes move one contiguous 128-byte row pair of a
     // tile; a per-warp panel [column][lane] of packed rows, one side at a time, turns it around.
-    if constexpr (MODE == 1 && !ALL) {
+    if constexpr (F32 && MODE == 1 && !ALL) {
         float2* const panel = (float2*)mem;
         const int le = lane >> 3, lp = lane & 7;            // entry (mod 4) and 16-byte piece a lane moves
         const int prow = lp >> 2, pcol = 4 * (lp & 3);      // the piece's row of the pair and first column
@@ -1616,7 +1809,7 @@ k_apply_warp(SweepArgs a, int p0, int nb, int min_runs) {
     }
     // a pass over all MOs: 32 AO rows per run, whose tiles come in by cp.async while the run before
     // computes
-    if constexpr (MODE == 1 && ALL) {
+    if constexpr (F32 && MODE == 1 && ALL) {
         // where piece p (columns 4p .. 4p + 3) of panel tile t of the run's row e lies: eight lanes
         // reading the same piece of consecutive rows hit all banks
         auto at = [&](int buf, int t, int e, int p) {
@@ -1730,7 +1923,7 @@ __global__ void __launch_bounds__(256) k_compact(int cap, const int* __restrict_
             if constexpr (sizeof(T) == 4)
                 nz |= x.x != 0.f || x.y != 0.f || x.z != 0.f || x.w != 0.f;
             else
-                nz |= x.x != 0.0 || x.y != 0.0;
+                nz |= nonzero(x.x) || nonzero(x.y);
         }
         if (__any_sync(0xffffffffu, nz) && lane == 0) atomicOr(&s_bits[s >> 5], 1u << (s & 31));
     }
@@ -1774,25 +1967,34 @@ template <typename T>
 static cudaError_t select_rot_t(Ctx* c) {
     const double tau = c->prm.eps;
     ClSel* cl = (ClSel*)c->d_cl_sel;
-    // per-cluster state: counts and prefixes zero, kmax = rot_cap_factor * N_occ(cluster)
-    cudaError_t e = cudaMemcpyAsync(c->d_cl_sel, c->d_cl_sel_init, c->h_cl_sel_init.size() * 8,
-                                    cudaMemcpyDeviceToDevice, c->stream);
-    if (e != cudaSuccess) return e;
-    k_rot_stats<T><<<c->n_gnb, 256, 0, c->stream>>>(c->n_gnb, c->d_gnb_row, c->d_gnb_col, c->d_group_nmol,
-                                                    c->d_group_nvt, c->d_group_cl, c->d_rot_blk_tp0, (const T*)c->d_F,
-                                                    tau, c->d_sc, cl);
-    const int hb = std::min(c->n_gnb, 1024);
     // the keys are the bit patterns of |F| as doubles; a float widened to double
     // has its 29 lowest mantissa bits zero, so for FP32 storage the radix passes
     // below bit 24 would only ever pick bin 0 and are left out
     const int last = std::is_same<T, float>::value ? 24 : 0;
-    for (int shift = 56; shift >= last; shift -= 8) {
-        k_rot_hist<T><<<hb, 256, 0, c->stream>>>(shift, c->n_gnb, c->d_gnb_row, c->d_gnb_col, c->d_group_nmol,
-                                                 c->d_group_nvt, c->d_group_cl, c->d_rot_blk_tp0, (const T*)c->d_F,
-                                                 tau, cl, c->d_cl_hist);
-        k_rot_pick<<<(c->n_clusters + 127) / 128, 128, 0, c->stream>>>(shift, last, c->n_clusters, cl, c->d_cl_hist);
+    if (c->n_clusters == 1 && c->n_gnb <= kSelSmallBlocks) {
+        k_rot_select_small<T><<<1, 1024, 0, c->stream>>>(last, c->n_gnb, c->d_gnb_row, c->d_gnb_col, c->d_group_nmol,
+                                                         c->d_group_nvt, c->d_rot_blk_tp0, (const T*)c->d_F, tau,
+                                                         c->h_cl_sel_init[5], c->d_sc, cl);
+        c->n_launch += 1;
+    } else {
+        // per-cluster state: counts and prefixes zero, kmax = rot_cap_factor * N_occ(cluster)
+        cudaError_t e = cudaMemcpyAsync(c->d_cl_sel, c->d_cl_sel_init, c->h_cl_sel_init.size() * 8,
+                                        cudaMemcpyDeviceToDevice, c->stream);
+        if (e != cudaSuccess) return e;
+        k_rot_stats<T><<<c->n_gnb, 256, 0, c->stream>>>(c->n_gnb, c->d_gnb_row, c->d_gnb_col, c->d_group_nmol,
+                                                        c->d_group_nvt, c->d_group_cl, c->d_rot_blk_tp0,
+                                                        (const T*)c->d_F, tau, c->d_sc, cl);
+        const int hb = std::min(c->n_gnb, 1024);
+        for (int shift = 56; shift >= last; shift -= 8) {
+            k_rot_hist<T><<<hb, 256, 0, c->stream>>>(shift, c->n_gnb, c->d_gnb_row, c->d_gnb_col, c->d_group_nmol,
+                                                     c->d_group_nvt, c->d_group_cl, c->d_rot_blk_tp0, (const T*)c->d_F,
+                                                     tau, cl, c->d_cl_hist);
+            k_rot_pick<<<(c->n_clusters + 3) / 4, 128, 0, c->stream>>>(shift, last, c->n_clusters, cl, c->d_cl_hist);
+        }
+        c->n_launch += std::is_same<T, double>::value ? 1 + 2 * 8 : 1 + 2 * 5;
     }
-    k_rot_lists<T><<<c->n_gnb, 128, 0, c->stream>>>(
+    c->n_launch += 1;
+    k_rot_lists<T><<<c->n_gnb, kListThreads, 0, c->stream>>>(
         c->n_gnb, c->d_gnb_row, c->d_gnb_col, c->d_group_nmol, c->d_group_nvt, c->d_group_occ0_mo,
         c->d_group_virt0_mo, c->d_group_cl, c->d_rot_blk_tp0, (const T*)c->d_F, c->d_Fd, tau, c->d_sc, cl, c->d_pr_n,
         c->d_pr_lvl, c->d_pr_ij, (T*)c->d_pr_cs, c->d_pr_touch);
@@ -1800,7 +2002,6 @@ static cudaError_t select_rot_t(Ctx* c) {
 }
 
 cudaError_t launch_select_rot(Ctx* c) {
-    c->n_launch += c->prec == SSCF_FP64 ? 2 + 2 * 8 : 2 + 2 * 5;   // stats, lists, radix passes (hist + pick)
     return c->prec == SSCF_FP64 ? select_rot_t<double>(c) : select_rot_t<float>(c);
 }
 
@@ -1817,7 +2018,7 @@ static cudaError_t ortho_prepare_t(Ctx* c, int w, double tol) {
                                               c->d_group_nmol, c->d_group_not, c->d_group_occ0_mo,
                                               c->d_group_virt0_mo, c->d_ort_blk_tp[w], (const T*)c->d_sig,
                                               c->d_scale, c->d_sc, c->d_group_cl, c->d_cl_eta);
-    k_ortho_lists<T><<<nob, 128, 0, c->stream>>>(w, tol, c->d_ocolour_blk, c->d_gnb_row, c->d_gnb_col,
+    k_ortho_lists<T><<<nob, kListThreads, 0, c->stream>>>(w, tol, c->d_ocolour_blk, c->d_gnb_row, c->d_gnb_col,
                                                 c->d_group_nmol, c->d_group_not, c->d_group_occ0_mo,
                                                 c->d_group_virt0_mo, c->d_ort_blk_tp[w], (const T*)c->d_sig,
                                                 c->d_scale, c->d_sc, c->d_group_cl, c->d_cl_eta, c->d_pr_n,
@@ -1920,7 +2121,7 @@ static cudaError_t closure_t(Ctx* c, int mode, int which, int col_lo, int col_hi
     return cudaGetLastError();
 }
 
-// The generic kernel for every block: FP64 storage, and FP32 on request (apply_variant 1).
+// The generic kernel for every block, on request (apply_variant 1).
 template <typename T, int MODE, int NT, int PCAP>
 static cudaError_t apply_generic_t(Ctx* c, const SweepArgs& a, int col_lo, int col_hi) {
     const size_t smem = (size_t)NT * 16 * apply_nrp<T>() * sizeof(T) + (size_t)2 * PCAP * sizeof(T) + (size_t)PCAP * 4;
@@ -1939,15 +2140,16 @@ static cudaError_t apply_generic_t(Ctx* c, const SweepArgs& a, int col_lo, int c
     return cudaGetLastError();
 }
 
-// FP32 storage: the warp-at-a-time kernel, one launch per colour.
-template <int MODE, bool ALL>
+// The warp-at-a-time kernel, one launch per colour.
+template <typename T, int MODE, bool ALL>
 static cudaError_t apply_warp_t(Ctx* c, SweepArgs& a, int col_lo, int col_hi) {
-    using Sh = WarpShape<MODE, ALL>;
+    using Sh = WarpShape<T, MODE, ALL>;
     // the bits of a block's rows (a cluster's at most) and the counts before each word
     const int chunks = (c->n_mol + kFullCH - 1) / kFullCH;
     const size_t smem = Sh::smem + (size_t)std::min(chunks, (c->max_cl_mol + kFullCH - 1) / kFullCH) * 8;
     if (smem > (size_t)kMaxDynSmem) return cudaErrorInvalidValue;
-    cudaError_t e = cudaFuncSetAttribute(k_apply_warp<MODE, ALL>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    cudaError_t e = cudaFuncSetAttribute(k_apply_warp<T, MODE, ALL>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                         (int)smem);
     if (e != cudaSuccess) return e;
     if (a.n_blk == 0) return cudaSuccess;
     a.blk_info = c->d_blk_info;
@@ -1961,11 +2163,11 @@ static cudaError_t apply_warp_t(Ctx* c, SweepArgs& a, int col_lo, int col_hi) {
         const int nb = ptr[col + 1] - ptr[col];
         if (nb == 0) continue;
         const int runs = (kAoPerMol / Sh::halves * c->max_cl_mol + 31) / 32;   // at most, of a block
-        const int per = MODE == 1 && (long long)nb * runs > kWsManyRuns * full ? 2 * kWsWarps : kWsWarps;
+        const int per = MODE == 1 && (long long)nb * runs > kWsManyRuns * full ? 2 * Sh::warps : Sh::warps;
         int gx = (runs + per - 1) / per;
         if (MODE == 0) gx = std::min(gx, (kWsRotWaves * full + nb - 1) / nb);
         if (c->apply_variant == 2) gx = 1;
-        k_apply_warp<MODE, ALL><<<nb * gx, kWsThreads, smem, c->stream>>>(a, ptr[col], nb, per);
+        k_apply_warp<T, MODE, ALL><<<nb * gx, Sh::threads, smem, c->stream>>>(a, ptr[col], nb, per);
         c->n_launch += 1;
     }
     return cudaGetLastError();
@@ -1985,9 +2187,7 @@ static cudaError_t apply_mode_t(Ctx* c, int which, int col_lo, int col_hi) {
     k_flags_by_column<<<c->n_tiles, 256, 0, c->stream>>>(c->cap, c->d_cci_ptr, c->d_cci_row, c->d_cci_slot,
                                                          a.out_nz, a.col_nz);
     c->n_launch += 1;
-    if constexpr (std::is_same<T, float>::value)
-        if (c->apply_variant != 1)
-            return apply_warp_t<MODE, NT == 6>(c, a, col_lo, col_hi);
+    if (c->apply_variant != 1) return apply_warp_t<T, MODE, NT == 6>(c, a, col_lo, col_hi);
     return apply_generic_t<T, MODE, NT, PCAP>(c, a, col_lo, col_hi);
 }
 

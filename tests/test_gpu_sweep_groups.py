@@ -48,3 +48,24 @@ def test_sweeps_of_partly_filled_groups_match_the_generic_kernel(n, kind, closur
     for a, b in zip(i0, i1):
         for k in ("energy", "n_rot", "n_combo", "upd_rot", "upd_combo", "eta"):
             assert a[k] == b[k], k
+
+
+@pytest.mark.parametrize("n,kind", [(1, "ramp"), (37, "ramp"), (97, "ramp"), (131, "sevens")])
+def test_fp64_sweeps_match_the_generic_kernel(n, kind):
+    """FP64 storage: one sweep and one pass of each kind. The products of a rotation may be
+    contracted differently (an ulp of 1 per update, 200 updates of a value at most: 1e-13)."""
+    library()
+    from paper_1402_2880_gb300 import Context
+    s = water(n)
+    out = []
+    for variant in (0, 1):
+        ctx = Context(s.species, s.xyz, _groups(n, kind), P, precision=0, apply_variant=variant)
+        ctx.set_thresholds(1e-4, 1e-3, 1e-8)
+        ctx.guess()
+        ctx.orthonormalise(0, max_pass=1)
+        ctx.orthonormalise(1, max_pass=1)
+        ctx.build_fock()
+        ctx.rotate_sweep()
+        out.append(ctx.get_C())
+        ctx.close()
+    assert np.abs(out[0] - out[1]).max() <= 1e-13
