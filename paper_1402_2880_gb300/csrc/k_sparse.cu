@@ -274,11 +274,17 @@ __global__ void k_xc(int tile_lo, int n_t, int n_share, int n_rows, int own_belo
     }
     __syncthreads();
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nwarps = blockDim.x >> 5;
-    const int col = lane & 15, q0 = lane >> 4;   // AO rows q0, q0+2, q0+4
-    using A = typename Acc<T>::type;
+    // A lane's outputs: FP64 three AO rows of one column; FP32 two AO rows of two columns, which
+    // takes 6 loads of C and 3 of X a neighbour where the other needs 6 and 9 (and leaves a quarter of
+    // the lanes idle): the loads bound the FP32 kernel (4096 molecules, H and S: 3.7 + 2.7 ms, now 3.5 + 2.4)
+    constexpr bool kWide = std::is_same<T, float>::value;
+    const int col = kWide ? 2 * (lane & 7) : lane & 15;
+    const int q0 = kWide ? 2 * min(lane >> 3, 2) : lane >> 4;   // FP64: AO rows q0, q0 + 2, q0 + 4
+    const bool idle = kWide && lane >= 24;
     for (int k = share * nwarps + warp; k < ny; k += n_share * nwarps) {
         const int r = y_row[(size_t)t * capY + k];
-        A acc0 = 0, acc1 = 0, acc2 = 0;
+        T acc0 = 0, acc1 = 0, acc2 = 0;
+        float2 acc[2] = {make_float2(0.f, 0.f), make_float2(0.f, 0.f)};
         // 32 pattern neighbours at a time: their ids, positions and slots are
         // looked up in parallel, one per lane; the matched ones are then summed
         // in pattern order with their data broadcast from the owning lane
@@ -300,50 +306,83 @@ __global__ void k_xc(int tile_lo, int n_t, int n_share, int n_rows, int own_belo
                     src[u] = mm ? __ffs(mm) - 1 : -1;
                     if (mm) mm &= mm - 1;
                 }
-                A c6[kXcBatch][6];
-                const T* xb[kXcBatch];
+                if constexpr (kWide) {
+                    float2 c6[kXcBatch][6];
+                    float x[kXcBatch][12];   // AO rows q0, q0 + 1 of the 6x6 block
 #pragma unroll
-                for (int u = 0; u < kXcBatch; ++u) {
-                    const int sv = src[u] < 0 ? 0 : src[u];
-                    const int n = __shfl_sync(0xffffffffu, nl, sv);
-                    const int ss = __shfl_sync(0xffffffffu, sl, sv);
-                    xb[u] = Xb + (size_t)(eb + sv) * 36;
-                    if (src[u] >= 0) {
-                        const T* cv = c_val + ((size_t)n * cap + ss) * kTileVals + col;
+                    for (int u = 0; u < kXcBatch; ++u) {
+                        const int sv = src[u] < 0 ? 0 : src[u];
+                        const int n = __shfl_sync(0xffffffffu, nl, sv);
+                        const int ss = __shfl_sync(0xffffffffu, sl, sv);
+                        if (src[u] >= 0) {
+                            const T* cv = c_val + ((size_t)n * cap + ss) * kTileVals + col;
+                            const float4* xb = (const float4*)(Xb + (size_t)(eb + sv) * 36 + q0 * 6);
 #pragma unroll
-                        for (int q = 0; q < 6; ++q) c6[u][q] = (A)cv[q * kTileW];
-                    }
-                }
+                            for (int q = 0; q < 6; ++q) c6[u][q] = *(const float2*)(cv + q * kTileW);
 #pragma unroll
-                for (int u = 0; u < kXcBatch; ++u) {
-                    if (src[u] < 0) continue;
-                    // the lane's three rows of the 6x6 block, two values per load
-                    // (rows start 6 values apart: 8-byte aligned for FP32, 16 for FP64)
-                    using V2 = typename std::conditional<sizeof(T) == 4, float2, double2>::type;
-                    A xr[3][6];
-#pragma unroll
-                    for (int rr = 0; rr < 3; ++rr) {
-                        const V2* x2 = (const V2*)(xb[u] + (q0 + 2 * rr) * 6);
-#pragma unroll
-                        for (int h = 0; h < 3; ++h) {
-                            const V2 v = x2[h];
-                            xr[rr][2 * h] = (A)v.x;
-                            xr[rr][2 * h + 1] = (A)v.y;
+                            for (int h = 0; h < 3; ++h) *(float4*)&x[u][4 * h] = xb[h];
                         }
                     }
 #pragma unroll
-                    for (int q = 0; q < 6; ++q) {
-                        acc0 += xr[0][q] * c6[u][q];
-                        acc1 += xr[1][q] * c6[u][q];
-                        acc2 += xr[2][q] * c6[u][q];
+                    for (int u = 0; u < kXcBatch; ++u) {
+                        if (src[u] < 0) continue;
+#pragma unroll
+                        for (int q = 0; q < 6; ++q) {
+                            acc[0] = __ffma2_rn(make_float2(x[u][q], x[u][q]), c6[u][q], acc[0]);
+                            acc[1] = __ffma2_rn(make_float2(x[u][6 + q], x[u][6 + q]), c6[u][q], acc[1]);
+                        }
+                    }
+                } else {
+                    T c6[kXcBatch][6];
+                    const T* xb[kXcBatch];
+#pragma unroll
+                    for (int u = 0; u < kXcBatch; ++u) {
+                        const int sv = src[u] < 0 ? 0 : src[u];
+                        const int n = __shfl_sync(0xffffffffu, nl, sv);
+                        const int ss = __shfl_sync(0xffffffffu, sl, sv);
+                        xb[u] = Xb + (size_t)(eb + sv) * 36;
+                        if (src[u] >= 0) {
+                            const T* cv = c_val + ((size_t)n * cap + ss) * kTileVals + col;
+#pragma unroll
+                            for (int q = 0; q < 6; ++q) c6[u][q] = cv[q * kTileW];
+                        }
+                    }
+#pragma unroll
+                    for (int u = 0; u < kXcBatch; ++u) {
+                        if (src[u] < 0) continue;
+                        // the lane's three rows of the 6x6 block, two values per load
+                        double xr[3][6];
+#pragma unroll
+                        for (int rr = 0; rr < 3; ++rr) {
+                            const double2* x2 = (const double2*)(xb[u] + (q0 + 2 * rr) * 6);
+#pragma unroll
+                            for (int h = 0; h < 3; ++h) {
+                                const double2 v = x2[h];
+                                xr[rr][2 * h] = v.x;
+                                xr[rr][2 * h + 1] = v.y;
+                            }
+                        }
+#pragma unroll
+                        for (int q = 0; q < 6; ++q) {
+                            acc0 += xr[0][q] * c6[u][q];
+                            acc1 += xr[1][q] * c6[u][q];
+                            acc2 += xr[2][q] * c6[u][q];
+                        }
                     }
                 }
             }
         }
         T* yv = y_val + ((size_t)t * capY + k) * kTileVals;
-        yv[(q0)*kTileW + col] = (T)acc0;
-        yv[(q0 + 2) * kTileW + col] = (T)acc1;
-        yv[(q0 + 4) * kTileW + col] = (T)acc2;
+        if constexpr (kWide) {
+            if (!idle) {
+                *(float2*)(yv + q0 * kTileW + col) = acc[0];
+                *(float2*)(yv + (q0 + 1) * kTileW + col) = acc[1];
+            }
+        } else {
+            yv[(q0)*kTileW + col] = acc0;
+            yv[(q0 + 2) * kTileW + col] = acc1;
+            yv[(q0 + 4) * kTileW + col] = acc2;
+        }
     }
 }
 
