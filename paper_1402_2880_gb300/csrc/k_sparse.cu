@@ -6,6 +6,8 @@
 // tile column (column-major, only the row blocks reachable through X), and
 // every kept block of C^T X C is one output-stationary 16x16 tile pair
 // reduced over the row blocks the two columns share.
+#include <cuda_bf16.h>
+
 #include "sscf_internal.h"
 
 #include <algorithm>
@@ -641,6 +643,13 @@ k_transform(int n_split, int n_rows, const int* __restrict__ tile_row0, int cap,
     }
 }
 
+// s + e = a + b exactly, s the rounded sum
+__device__ __forceinline__ void two_sum(float a, float b, float& s, float& e) {
+    s = __fadd_rn(a, b);
+    const float t = __fsub_rn(s, a);
+    e = __fadd_rn(__fsub_rn(a, __fsub_rn(s, t)), __fsub_rn(b, t));
+}
+
 // diag(F) per MO from the diagonal tile pairs
 template <typename T>
 __global__ void k_extract_diag(int n_tiles, const int* __restrict__ tile_mo0, const int* __restrict__ tile_nmo,
@@ -660,9 +669,60 @@ __global__ void k_extract_diag(int n_tiles, const int* __restrict__ tile_mo0, co
 // molecule in neighbour order.
 // ---------------------------------------------------------------------------
 constexpr int kDensWarps = 8;
-constexpr int kDensFlush = 32;  // tiles per lane between FP64 flushes (FP32 sums of at most 32 products)
+constexpr int kDensFlush = 32;  // tiles per lane in one FP32 sum
 constexpr int kDensUnroll = 1;  // shared tiles per half-warp and round (2 measured no faster)
 constexpr int kDensMinBlocks = 2;   // resident CTAs per SM the register budget aims at
+// A sum of floats in three, each the roundings dropped by the one before: 70 bits.
+// FP32 storage adds its partial sums of 32 products so (where FP64 carried 53): the
+// FP64 pipe, two lanes per clock and SM, was two thirds busy with them and with
+// the sums over a warp (density at 997 and 4096 molecules 0.55 and 3.60 ms, now 0.43
+// and 2.83). A lane keeps two floats in shared memory and the third, 2^-48 of the sum,
+// as eight bits of bf16 in a register (as floats: 0.47 and 3.14 ms).
+struct Sum3 {
+    float h, l, m;
+    __device__ __forceinline__ void add(float v) {
+        float e, d;
+        two_sum(h, v, h, e);
+        two_sum(l, e, l, d);
+        m = __fadd_rn(m, d);
+    }
+    __device__ __forceinline__ void add(float2 v) {
+        float d;
+        add(v.x);
+        two_sum(l, v.y, l, d);
+        m = __fadd_rn(m, d);
+    }
+    __device__ __forceinline__ double value() const {
+        return isfinite(h) ? ((double)h + (double)l) + (double)m : (double)h;
+    }
+};
+
+// s += v; lost: what the two floats of s drop of it
+__device__ __forceinline__ void sum_add(float2& s, float v, float& lost) {
+    float h, l, e;
+    two_sum(s.x, v, h, e);
+    two_sum(s.y, e, l, lost);
+    s = make_float2(h, l);
+}
+
+// The sums of a pair's 36 products over its 32 lanes: lane u sums product u (32
+// entries, from entry u on around: no bank conflicts) and four entries of one of
+// the last four products, which the eight lanes that share it then add up.
+__device__ __forceinline__ void pair_sums(const double* acc, int lane, double& p0, double& p1) {
+    const double *row0 = acc + lane * 32, *row1 = acc + (32 + (lane >> 3)) * 32 + 4 * (lane & 7);
+    p0 = p1 = 0.0;
+    for (int j = 0; j < 32; ++j) p0 += row0[(j + lane) & 31];
+    for (int j = 0; j < 4; ++j) p1 += row1[j];
+}
+__device__ __forceinline__ void pair_sums(const float2* acc, int lane, double& p0, double& p1) {
+    const float2 *row0 = acc + lane * 32, *row1 = acc + (32 + (lane >> 3)) * 32 + 4 * (lane & 7);
+    Sum3 s0 = {0.f, 0.f, 0.f}, s1 = {0.f, 0.f, 0.f};
+    for (int j = 0; j < 32; ++j) s0.add(row0[(j + lane) & 31]);
+    for (int j = 0; j < 4; ++j) s1.add(row1[(j + (lane >> 3)) & 3]);
+    p0 = s0.value();
+    p1 = s1.value();
+}
+
 template <typename T>
 __global__ void __launch_bounds__(kDensWarps * 32, kDensMinBlocks)
 k_density(int n_occ_tiles, int map_n, const int* __restrict__ mol_ot0, int cap, const int* __restrict__ c_nt,
@@ -670,11 +730,11 @@ k_density(int n_occ_tiles, int map_n, const int* __restrict__ mol_ot0, int cap, 
           const int* __restrict__ mp_col, const double* __restrict__ H0b, const double* __restrict__ Sb,
           const int* __restrict__ mp_rev, double2* __restrict__ dpart, double* __restrict__ P_out) {
     // slot of every occupied tile of m's cluster in row m, or -1 (map_n = largest cluster);
-    // then, in mixed precision, the FP64 sums of each lane's 36 products (flushed
-    // from FP32 every kDensFlush tiles), kept in shared memory to save registers
+    // then the sums of each lane's 36 products (in mixed precision of FP32 sums of
+    // kDensFlush tiles each), kept in shared memory to save registers
     extern __shared__ int smap[];
-    constexpr bool kSplit = !std::is_same<typename Acc<T>::type, double>::value;
-    double* sacc = (double*)(smap + ((map_n + 1) & ~1));   // [warp][36][32]: per-lane FP64 sums
+    constexpr bool kSplit = !std::is_same<typename Acc<T>::type, double>::value;   // FP32 storage
+    double* sacc = (double*)(smap + ((map_n + 1) & ~1));   // [warp][36][32]: the lanes' sums
     const int m = blockIdx.x;
     const int t0 = mol_ot0[m];
     // P_nm = P_mn^T: this CTA takes the pairs with n >= m (neighbour lists are
@@ -696,12 +756,46 @@ k_density(int n_occ_tiles, int map_n, const int* __restrict__ mol_ot0, int cap, 
     const int e0 = mp_ptr[m], ne = mp_ptr[m + 1] - e0;
     using A = typename Acc<T>::type;
     const int col = lane & 15, half = lane >> 4;
+    double* wsum = sacc + (size_t)warp * 36 * 32;
+    using L = typename std::conditional<kSplit, float2, double>::type;
+    __nv_bfloat162 low[18];
+    // a lane's next partial sums
+    auto flush = [&](A* acc, int part) {
+        L* d = (L*)wsum + lane;
+#pragma unroll
+        for (int u = 0; u < 36; u += 2) {
+            if constexpr (kSplit) {
+                if (part == 0) {
+                    d[u * 32] = make_float2(acc[u], 0.f);
+                    d[u * 32 + 32] = make_float2(acc[u + 1], 0.f);
+                } else {
+                    float l0, l1;
+                    sum_add(d[u * 32], acc[u], l0);
+                    sum_add(d[u * 32 + 32], acc[u + 1], l1);
+                    low[u / 2] = __hadd2(low[u / 2], __floats2bfloat162_rn(l0, l1));
+                }
+            } else {
+                d[u * 32] = acc[u];
+                d[u * 32 + 32] = acc[u + 1];
+            }
+            acc[u] = acc[u + 1] = 0;
+        }
+    };
+    // sum_id: atoms of m, atoms of n, energy; take: which of its nine products the lane adds
+    const int sum_id = lane >> 2;
+    unsigned take = 0;
+    for (int j = 0; j < 9; ++j) {
+        const int u = 9 * (lane & 3) + j, ao = sum_id < 3 ? u / 6 : u % 6, atom = max(ao - 3, 0);
+        if (sum_id == 6 || atom == sum_id % 3) take |= 1u << j;
+    }
     for (int w = s_jlo + warp; w < ne; w += kDensWarps) {
         const int e = e0 + w;
         const int n = mp_col[e];
         A acc[36];
-        double* wacc = sacc + (size_t)warp * 36 * 32 + lane;
-        bool flushed = false;   // the first flush stores instead of adding
+        int n_part = 0;   // partial sums of this lane so far
+        if constexpr (kSplit)
+#pragma unroll
+            for (int u = 0; u < 18; ++u) low[u] = __floats2bfloat162_rn(0.f, 0.f);
 #pragma unroll
         for (int u = 0; u < 36; ++u) acc[u] = 0;
         const int ntn = c_nt[n];
@@ -756,65 +850,70 @@ k_density(int n_occ_tiles, int map_n, const int* __restrict__ mol_ot0, int cap, 
                     if constexpr (kSplit) {
                         if (++since == kDensFlush) {
                             since = 0;
-#pragma unroll
-                            for (int v = 0; v < 36; ++v) {
-                                wacc[v * 32] = flushed ? wacc[v * 32] + (double)acc[v] : (double)acc[v];
-                                acc[v] = 0;
-                            }
-                            flushed = true;
+                            flush(acc, n_part++);
                         }
                     }
                 }
             }
             if (virt_seen) break;   // tiles are sorted: occupied tiles first
         }
-        // lane sums to shared memory, then lane u < 36 adds up entry u over the
-        // 32 lanes (rotated start: no bank conflicts) and weights it by S and H0
-#pragma unroll
-        for (int u = 0; u < 36; ++u) wacc[u * 32] = flushed ? wacc[u * 32] + (double)acc[u] : (double)acc[u];
+        flush(acc, n_part++);
         __syncwarp();
-        // row sums of P o S by the atoms of m, column sums by the atoms of n
-        // (AOs: O s, p, p, p, then H1 s, H2 s), and sum P o H0
+        double p[2];
+        pair_sums((const L*)wsum, lane, p[0], p[1]);
+        if constexpr (kSplit) {
+            unsigned any = 0;
+#pragma unroll
+            for (int u = 0; u < 18; ++u) any |= *(const unsigned*)&low[u] & 0x7fff7fffu;
+            if (__any_sync(0xffffffffu, any != 0)) {   // the third parts, in the same way
+                __syncwarp();
+                float2* f = (float2*)wsum + lane;
+#pragma unroll
+                for (int u = 0; u < 36; ++u)
+                    f[u * 32] = make_float2(u & 1 ? __high2float(low[u / 2]) : __low2float(low[u / 2]), 0.f);
+                __syncwarp();
+                double l0, l1;
+                pair_sums((const L*)wsum, lane, l0, l1);
+                p[0] += l0;
+                p[1] += l1;
+            }
+        }
+#pragma unroll
+        for (int off = 4; off > 0; off >>= 1) p[1] += __shfl_xor_sync(0xffffffffu, p[1], off);
+        __syncwarp();
+        // the products weighted by S (36) and by H0 (36) back to shared memory, then four lanes
+        // each for the sums of P o S over the atoms of m and of n (AOs: O s, p, p, p, then H1 s,
+        // H2 s) and of P o H0
         const bool self = n == m;
         const int er = self ? e : mp_rev[e];
-        double qr[3] = {0, 0, 0}, qc[3] = {0, 0, 0}, eb = 0.0;
-        for (int u = lane; u < 36; u += 32) {
-            const double* row = sacc + ((size_t)warp * 36 + u) * 32;
-            double v = 0.0;
-            for (int j = 0; j < 32; ++j) v += row[(j + lane) & 31];
-            const double P = 2.0 * v;
-            const int k = u / 6, l = u - 6 * k;   // AO of m, AO of n
+#pragma unroll
+        for (int i = 0; i < 2; ++i) {
+            if (i && (lane & 7)) break;
+            const int u = i ? 32 + (lane >> 3) : lane;
+            const double P = 2.0 * p[i];
             if (P_out) {
                 P_out[(size_t)e * 36 + u] = P;
+                const int k = u / 6, l = u - 6 * k;   // AO of m, AO of n
                 if (!self) P_out[(size_t)er * 36 + l * 6 + k] = P;
             }
-            const double pq = P * Sb[(size_t)e * 36 + u];
-            qr[0] += k < 4 ? pq : 0.0;
-            qr[1] += k == 4 ? pq : 0.0;
-            qr[2] += k == 5 ? pq : 0.0;
-            qc[0] += l < 4 ? pq : 0.0;
-            qc[1] += l == 4 ? pq : 0.0;
-            qc[2] += l == 5 ? pq : 0.0;
-            eb += P * H0b[(size_t)e * 36 + u];
-        }
-#pragma unroll
-        for (int off = 16; off > 0; off >>= 1) {
-#pragma unroll
-            for (int i = 0; i < 3; ++i) {
-                qr[i] += __shfl_xor_sync(0xffffffffu, qr[i], off);
-                qc[i] += __shfl_xor_sync(0xffffffffu, qc[i], off);
-            }
-            eb += __shfl_xor_sync(0xffffffffu, eb, off);
+            wsum[u] = P * Sb[(size_t)e * 36 + u];
+            wsum[36 + u] = P * H0b[(size_t)e * 36 + u];
         }
         __syncwarp();
-        if (lane == 0) {
-            dpart[2 * (size_t)e] = make_double2(qr[0], qr[1]);
-            dpart[2 * (size_t)e + 1] = make_double2(qr[2], eb);
-            if (!self) {
-                dpart[2 * (size_t)er] = make_double2(qc[0], qc[1]);
-                dpart[2 * (size_t)er + 1] = make_double2(qc[2], eb);
+        if (lane < 28) {
+            const double* w9 = wsum + (sum_id == 6 ? 36 : 0) + 9 * (lane & 3);
+            double v = 0.0;
+#pragma unroll
+            for (int j = 0; j < 9; ++j) v += (take >> j) & 1 ? w9[j] : 0.0;
+            v += __shfl_xor_sync(0x0fffffffu, v, 1);
+            v += __shfl_xor_sync(0x0fffffffu, v, 2);
+            if ((lane & 3) == 0) {
+                double* out = (double*)dpart;   // per entry: atoms O, H1, H2 and the energy
+                if (sum_id < 3 || sum_id == 6) out[4 * (size_t)e + min(sum_id, 3)] = v;
+                if (sum_id >= 3 && !self) out[4 * (size_t)er + sum_id - 3] = v;
             }
         }
+        __syncwarp();
     }
 }
 
