@@ -395,55 +395,23 @@ __global__ void k_xc(int tile_lo, int n_t, int n_share, int n_rows, int own_belo
 // a it stages the two 6x16 tiles (C[r, a] and Y[r, b]) in a per-warp buffer
 // with 16-byte loads, kStage row blocks at a time; every lane then owns a 2x4
 // block of the 16x16 result and does 8 FMAs per K step from one 8-byte and
-// one 16-byte shared load. Rows are summed in ascending order (fixed order);
-// mixed precision flushes the FP32 partial sums to FP64 every 32 rows.
+// two 16-byte shared loads. Rows are summed in ascending order (fixed order),
+// 32 of b's rows at a time. FP64 storage; FP32 storage: k_transform_tc.
 // ---------------------------------------------------------------------------
 constexpr int kTfWarps = 4;
-constexpr int kStage = 4;   // row blocks staged per warp at a time
-constexpr int kTcStride = 24;   // floats per staged AO row in the tensor-core path (bank-conflict-free fragments)
-constexpr int kTcRows = kStage * kAoPerMol;   // staged AO rows (K) per round: 24 = 3 k-steps of 8
-
-// x = hi + lo with hi, lo in TF32 (10 explicit mantissa bits each): hi by
-// round-to-nearest, lo the rounded remainder, so hi + lo carries ~21 bits.
-__device__ __forceinline__ void split_tf32(float x, uint32_t& hi, uint32_t& lo) {
-    uint32_t h, l;
-    asm("cvt.rna.tf32.f32 %0, %1;" : "=r"(h) : "f"(x));
-    const float r = x - __uint_as_float(h);
-    asm("cvt.rna.tf32.f32 %0, %1;" : "=r"(l) : "f"(r));
-    hi = h;
-    lo = l;
-}
-
-// D (16x8, FP32) += A (16x8, TF32, row-major) x B (8x8, TF32, column-major)
-__device__ __forceinline__ void mma_tf32(float (&d)[4], const uint32_t (&a)[4], const uint32_t (&b)[2]) {
-    asm volatile(
-        "mma.sync.aligned.m16n8k8.row.col.f32.tf32.tf32.f32 {%0, %1, %2, %3}, {%4, %5, %6, %7}, {%8, %9}, "
-        "{%0, %1, %2, %3};"
-        : "+f"(d[0]), "+f"(d[1]), "+f"(d[2]), "+f"(d[3])
-        : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b[0]), "r"(b[1]));
-}
-
-template <typename T> struct V4;
-template <> struct V4<float> { using type = float4; };
-template <> struct V4<double> { using type = double2; };
-
-// Staged values per warp: FP64 [kStage][2][96]; FP32 (tensor cores) C rows
-// then Y rows, kTcRows rows of kTcStride floats each.
-template <typename T> __host__ __device__ constexpr int tf_stage_vals() {
-    return std::is_same<T, float>::value ? 2 * kTcRows * kTcStride : kStage * 2 * kTileVals;
-}
-
+constexpr int kStage = 4;   // row blocks taken per warp at a time
+constexpr int kTfStageVals = kStage * 2 * kTileVals;   // staged values per warp: [kStage][2][96]
 // MINB: resident CTAs per SM the register budget is cut for (1: no cut)
-template <typename T, int MINB>
+template <int MINB>
 __global__ void __launch_bounds__(kTfWarps * 32, MINB)
 k_transform(int n_split, int n_rows, const int* __restrict__ tile_row0, int cap, int capY, const int* __restrict__ tp_ptr,
             const int* __restrict__ tp_b,
             const int* __restrict__ tp_out, const int* __restrict__ cci_ptr, const int* __restrict__ cci_row,
-            const int* __restrict__ cci_slot, const T* __restrict__ c_val, const int* __restrict__ y_n,
-            const int* __restrict__ y_row, const T* __restrict__ y_val, T* __restrict__ out) {
+            const int* __restrict__ cci_slot, const double* __restrict__ c_val, const int* __restrict__ y_n,
+            const int* __restrict__ y_row, const double* __restrict__ y_val, double* __restrict__ out) {
     extern __shared__ __align__(16) unsigned char sraw[];
-    T* stage = (T*)sraw;                                        // [warps][tf_stage_vals]
-    short* slot_of = (short*)(stage + (size_t)kTfWarps * tf_stage_vals<T>());   // n_rows (cluster-local)
+    double* stage = (double*)sraw;                                        // [warps][kTfStageVals]
+    short* slot_of = (short*)(stage + (size_t)kTfWarps * kTfStageVals);   // n_rows (cluster-local)
     // CTA (a, s) takes the pairs of tile a with index = s (mod n_split)
     const int a = blockIdx.x / n_split, split = blockIdx.x % n_split;
     const int p0 = tp_ptr[a], p1 = tp_ptr[a + 1];
@@ -455,120 +423,15 @@ k_transform(int n_split, int n_rows, const int* __restrict__ tile_row0, int cap,
     for (int k = threadIdx.x; k < nc; k += blockDim.x) slot_of[cci_row[lo + k] - r0] = (short)cci_slot[lo + k];
     __syncthreads();
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    T* buf = stage + (size_t)warp * tf_stage_vals<T>();
-    if constexpr (std::is_same<T, float>::value) {
-        // FP32 storage: the 16x16 block is two m16n8 tensor-core tiles, K = the
-        // staged AO rows (up to 4 matched row blocks = 24 rows = 3 k-steps of 8).
-        // Each product is split into TF32 hi + lo parts and summed as
-        // hi*hi + hi*lo + lo*hi (the lo*lo term is below FP32 rounding), into
-        // FP32 fragments flushed to FP64 every 32 of b's rows, as the FP64 path.
-        float* bc = buf;                          // [kTcRows][kTcStride]: C[r, a] rows
-        float* by = buf + kTcRows * kTcStride;    // [kTcRows][kTcStride]: Y[r, b] rows
-        const int gq = lane >> 2, tq = lane & 3;
-        for (int p = p0 + split + warp * n_split; p < p1; p += kTfWarps * n_split) {
-            const int b = tp_b[p];
-            const int nb = y_n[b];
-            const int* yr = y_row + (size_t)b * capY;
-            float acc[2][4];
-            double accd[2][4];
-#pragma unroll
-            for (int h = 0; h < 2; ++h)
-#pragma unroll
-                for (int q = 0; q < 4; ++q) {
-                    acc[h][q] = 0.f;
-                    accd[h][q] = 0.0;
-                }
-            for (int k0 = 0; k0 < nb; k0 += 32) {
-                const int k = k0 + lane;
-                const int rr = k < nb ? yr[k] : 0;
-                const int sl = k < nb ? slot_of[rr - r0] : -1;
-                unsigned m = __ballot_sync(0xffffffffu, sl >= 0);
-                while (m) {
-                    // up to kStage matched row blocks: their row, a's slot and b's position
-                    int nst = 0, rowv[kStage], ssv[kStage], kkv[kStage];
-#pragma unroll
-                    for (int g = 0; g < kStage; ++g) {
-                        const int src_lane = m ? __ffs(m) - 1 : 0;
-                        if (m) {
-                            m &= m - 1;
-                            ++nst;
-                        }
-                        rowv[g] = __shfl_sync(0xffffffffu, rr, src_lane);
-                        ssv[g] = __shfl_sync(0xffffffffu, sl, src_lane);
-                        kkv[g] = k0 + src_lane;
-                    }
-                    // stage: lane q*4 + part (< 24) copies 16 bytes of AO row q of
-                    // C[r, a] and of Y[r, b] for every staged row block, loads first
-                    if (lane < 24) {
-                        const int q = lane >> 2, part = lane & 3;
-                        float4 cv[kStage], yv[kStage];
-#pragma unroll
-                        for (int g = 0; g < kStage; ++g)
-                            if (g < nst) {
-                                cv[g] = *((const float4*)(c_val + ((size_t)rowv[g] * cap + ssv[g]) * kTileVals +
-                                                          q * 16) + part);
-                                yv[g] = *((const float4*)(y_val + ((size_t)b * capY + kkv[g]) * kTileVals + q * 16) +
-                                          part);
-                            }
-#pragma unroll
-                        for (int g = 0; g < kStage; ++g)
-                            if (g < nst) {
-                                *(float4*)(bc + (g * kAoPerMol + q) * kTcStride + 4 * part) = cv[g];
-                                *(float4*)(by + (g * kAoPerMol + q) * kTcStride + 4 * part) = yv[g];
-                            }
-                    }
-                    __syncwarp();
-                    const int nkr = nst * kAoPerMol;
-                    for (int ks = 0; ks < nkr; ks += 8) {
-                        const int ka = ks + tq, kb = ks + tq + 4;
-                        const bool va = ka < nkr, vb = kb < nkr;
-                        uint32_t ah[4], al[4];
-                        split_tf32(va ? bc[ka * kTcStride + gq] : 0.f, ah[0], al[0]);
-                        split_tf32(va ? bc[ka * kTcStride + gq + 8] : 0.f, ah[1], al[1]);
-                        split_tf32(vb ? bc[kb * kTcStride + gq] : 0.f, ah[2], al[2]);
-                        split_tf32(vb ? bc[kb * kTcStride + gq + 8] : 0.f, ah[3], al[3]);
-#pragma unroll
-                        for (int h = 0; h < 2; ++h) {
-                            uint32_t bh[2], bl[2];
-                            split_tf32(va ? by[ka * kTcStride + 8 * h + gq] : 0.f, bh[0], bl[0]);
-                            split_tf32(vb ? by[kb * kTcStride + 8 * h + gq] : 0.f, bh[1], bl[1]);
-                            mma_tf32(acc[h], al, bh);
-                            mma_tf32(acc[h], ah, bl);
-                            mma_tf32(acc[h], ah, bh);
-                        }
-                    }
-                    __syncwarp();
-                }
-#pragma unroll
-                for (int h = 0; h < 2; ++h)
-#pragma unroll
-                    for (int q = 0; q < 4; ++q) {
-                        accd[h][q] += (double)acc[h][q];
-                        acc[h][q] = 0.f;
-                    }
-            }
-            T* o = out + (size_t)tp_out[p] * 256;
-#pragma unroll
-            for (int h = 0; h < 2; ++h) {
-                o[gq * 16 + 8 * h + 2 * tq] = (T)accd[h][0];
-                o[gq * 16 + 8 * h + 2 * tq + 1] = (T)accd[h][1];
-                o[(gq + 8) * 16 + 8 * h + 2 * tq] = (T)accd[h][2];
-                o[(gq + 8) * 16 + 8 * h + 2 * tq + 1] = (T)accd[h][3];
-            }
-        }
-        return;
-    }
+    double* buf = stage + (size_t)warp * kTfStageVals;
     const int i0 = 2 * (lane >> 2), j0 = 4 * (lane & 3);
-    using A = typename Acc<T>::type;
-    using VT = typename V4<T>::type;
-    constexpr int kVec = sizeof(VT) / sizeof(T);          // values per 16-byte load
-    constexpr int kPerTile = kTileVals / kVec;            // 16-byte loads per tile
+    constexpr int kPerTile = kTileVals / 2;   // 16-byte loads per tile
     for (int p = p0 + split + warp * n_split; p < p1; p += kTfWarps * n_split) {
         const int b = tp_b[p];
         const int nb = y_n[b];
         const int* yr = y_row + (size_t)b * capY;
         double accd[8];
-        A acc[8];
+        double acc[8];
 #pragma unroll
         for (int q = 0; q < 8; ++q) {
             acc[q] = 0;
@@ -598,10 +461,10 @@ k_transform(int n_split, int n_rows, const int* __restrict__ tile_row0, int cap,
                     const int ss = __shfl_sync(0xffffffffu, s, rows[g]);
                     const int kk = k0 + rows[g];
                     const int r = yr[kk];
-                    const VT* cs = (const VT*)(c_val + ((size_t)r * cap + ss) * kTileVals);
-                    const VT* ys = (const VT*)(y_val + ((size_t)b * capY + kk) * kTileVals);
-                    VT* bc = (VT*)(buf + (size_t)g * 2 * kTileVals);
-                    VT* by = (VT*)(buf + (size_t)g * 2 * kTileVals + kTileVals);
+                    const double2* cs = (const double2*)(c_val + ((size_t)r * cap + ss) * kTileVals);
+                    const double2* ys = (const double2*)(y_val + ((size_t)b * capY + kk) * kTileVals);
+                    double2* bc = (double2*)(buf + (size_t)g * 2 * kTileVals);
+                    double2* by = (double2*)(buf + (size_t)g * 2 * kTileVals + kTileVals);
                     for (int v = lane; v < kPerTile; v += 32) {
                         bc[v] = cs[v];
                         by[v] = ys[v];
@@ -609,13 +472,13 @@ k_transform(int n_split, int n_rows, const int* __restrict__ tile_row0, int cap,
                 }
                 __syncwarp();
                 for (int g = 0; g < nst; ++g) {
-                    const T* bc = buf + (size_t)g * 2 * kTileVals;
-                    const T* by = bc + kTileVals;
+                    const double* bc = buf + (size_t)g * 2 * kTileVals;
+                    const double* by = bc + kTileVals;
 #pragma unroll
                     for (int q = 0; q < 6; ++q) {
-                        const A c0 = (A)bc[q * 16 + i0], c1 = (A)bc[q * 16 + i0 + 1];
-                        const A y0 = (A)by[q * 16 + j0], y1 = (A)by[q * 16 + j0 + 1];
-                        const A y2 = (A)by[q * 16 + j0 + 2], y3 = (A)by[q * 16 + j0 + 3];
+                        const double c0 = bc[q * 16 + i0], c1 = bc[q * 16 + i0 + 1];
+                        const double y0 = by[q * 16 + j0], y1 = by[q * 16 + j0 + 1];
+                        const double y2 = by[q * 16 + j0 + 2], y3 = by[q * 16 + j0 + 3];
                         acc[0] += c0 * y0;
                         acc[1] += c0 * y1;
                         acc[2] += c0 * y2;
@@ -630,15 +493,15 @@ k_transform(int n_split, int n_rows, const int* __restrict__ tile_row0, int cap,
             }
 #pragma unroll
             for (int q = 0; q < 8; ++q) {
-                accd[q] += (double)acc[q];
+                accd[q] += acc[q];
                 acc[q] = 0;
             }
         }
-        T* o = out + (size_t)tp_out[p] * 256;
+        double* o = out + (size_t)tp_out[p] * 256;
 #pragma unroll
         for (int u = 0; u < 4; ++u) {
-            o[i0 * 16 + j0 + u] = (T)accd[u];
-            o[(i0 + 1) * 16 + j0 + u] = (T)accd[4 + u];
+            o[i0 * 16 + j0 + u] = accd[u];
+            o[(i0 + 1) * 16 + j0 + u] = accd[4 + u];
         }
     }
 }
@@ -648,6 +511,171 @@ __device__ __forceinline__ void two_sum(float a, float b, float& s, float& e) {
     s = __fadd_rn(a, b);
     const float t = __fsub_rn(s, a);
     e = __fadd_rn(__fsub_rn(a, __fsub_rn(s, t)), __fsub_rn(b, t));
+}
+// Sum of partial sums to be rounded to FP32: a float and what its roundings
+// dropped (exact unless the terms are 24 binary orders apart, then to 2^-48).
+__device__ __forceinline__ void sum_add(float2& s, float v) {
+    float h, e;
+    two_sum(s.x, v, h, e);
+    s = make_float2(h, __fadd_rn(s.y, e));
+}
+__device__ __forceinline__ float sum_value(float2 s) { return isfinite(s.x) ? __fadd_rn(s.x, s.y) : s.x; }
+
+// x = hi + lo with hi, lo in TF32 (10 explicit mantissa bits each): hi by
+// round-to-nearest, ties away, lo the rounded remainder, so hi + lo carries ~21
+// bits. Rounded in the bits, as cvt.rna.tf32 rounds (the kernel ran 5 % longer
+// with that instruction). The last step keeps a NaN, which the bits would lose;
+// an infinite x has a NaN remainder.
+__device__ __forceinline__ uint32_t round_tf32(float x) { return (__float_as_uint(x) + 0x1000u) & 0xffffe000u; }
+__device__ __forceinline__ void split_tf32(float x, uint32_t& hi, uint32_t& lo) {
+    hi = round_tf32(x);
+    const float r = x - __uint_as_float(hi);
+    lo = __float_as_uint(__fmaf_rn(r, 0.f, __uint_as_float(round_tf32(r))));
+}
+
+// D (16x8, FP32) += A (16x8, TF32, row-major) x B (8x8, TF32, column-major)
+__device__ __forceinline__ void mma_tf32(float (&d)[4], const uint32_t (&a)[4], const uint32_t (&b)[2]) {
+    asm volatile(
+        "mma.sync.aligned.m16n8k8.row.col.f32.tf32.tf32.f32 {%0, %1, %2, %3}, {%4, %5, %6, %7}, {%8, %9}, "
+        "{%0, %1, %2, %3};"
+        : "+f"(d[0]), "+f"(d[1]), "+f"(d[2]), "+f"(d[3])
+        : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b[0]), "r"(b[1]));
+}
+
+// FP32 storage: the 16x16 block of a pair as two m16n8 tensor-core tiles, K = the
+// AO rows of up to four matched row blocks (24 rows, 3 k-steps of 8) at a time.
+// Each product is split into TF32 hi + lo parts and summed as hi*hi + hi*lo +
+// lo*hi (the lo*lo term is below FP32 rounding), into FP32 fragments that are
+// added up in two floats every 32 of b's rows.
+// A row of a 6x16 tile is 64 bytes, so a warp reads a fragment's four rows of two
+// columns per lane straight from memory: no staging, no shared-memory traffic, and
+// a's tiles are found in L1 by the CTA's other warps (b's pass it by). Bound by the
+// splits (48 of ~75 instructions a k-step) and the L2 latency that three CTAs'
+// 80-register warps leave uncovered (issue slots 55 % used); four CTAs spill, two
+// are 20 % slower. Staged through shared memory, with cvt.rna.tf32 and sums in
+// FP64 (a quarter of the FP64 pipe's time): 8.0 + 6.3 ms for the two
+// transforms at 4096 molecules, now 6.2 + 4.8; at 997 1.48 + 1.07, now 1.23 + 0.90.
+constexpr int kTcWarps = 8, kTcCtas = 3;
+__device__ __forceinline__ float2 load_stream(const float* p) {
+    float2 v;
+    asm volatile("ld.global.L1::no_allocate.v2.f32 {%0, %1}, [%2];" : "=f"(v.x), "=f"(v.y) : "l"(p));
+    return v;
+}
+__global__ void __launch_bounds__(kTcWarps * 32, kTcCtas)
+k_transform_tc(int n_split, int n_rows, const int* __restrict__ tile_row0, int cap, int capY,
+               const int* __restrict__ tp_ptr, const int* __restrict__ tp_b, const int* __restrict__ tp_out,
+               const int* __restrict__ cci_ptr, const int* __restrict__ cci_row, const int* __restrict__ cci_slot,
+               const float* __restrict__ c_val, const int* __restrict__ y_n, const int* __restrict__ y_row,
+               const float* __restrict__ y_val, float* __restrict__ out) {
+    extern __shared__ __align__(16) unsigned char sraw[];
+    int2* lists = (int2*)sraw;                       // [warps][32]: matched row blocks (tile of C, b's position)
+    short* slot_of = (short*)(lists + kTcWarps * 32);   // n_rows (cluster-local)
+    // CTA (a, s) takes the pairs of tile a with index = s (mod n_split)
+    const int a = blockIdx.x / n_split, split = blockIdx.x % n_split;
+    const int p0 = tp_ptr[a], p1 = tp_ptr[a + 1];
+    if (p0 + split >= p1) return;
+    const int r0 = tile_row0[a];
+    const int lo = cci_ptr[a], nc = cci_ptr[a + 1] - lo;
+    for (int i = threadIdx.x; i < n_rows; i += blockDim.x) slot_of[i] = -1;
+    __syncthreads();
+    for (int k = threadIdx.x; k < nc; k += blockDim.x) slot_of[cci_row[lo + k] - r0] = (short)cci_slot[lo + k];
+    __syncthreads();
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    int2* list = lists + warp * 32;
+    const int gq = lane >> 2, tq = lane & 3;
+    // A k-step's fragments are rows tq and tq + 4 of its eight. Over the 24 rows of four blocks these are
+    // rows tq | lowhi, tq+2, tq | lowhi, tq+2 of blocks 0, 0|1, 1, 2, 2|3, 3, where lowhi is row tq + 4 of the
+    // one block or row tq - 2 of the next. A fragment's columns gq and gq + 8 are columns 2gq and 2gq + 1.
+    const bool early = tq < 2;
+    const int o0 = tq * 16 + 2 * gq, o1 = (early ? tq + 4 : tq - 2) * 16 + 2 * gq, o2 = (tq + 2) * 16 + 2 * gq;
+    // the next pair's tile, row count and first rows, and the next 32 rows of this one, are read ahead
+    const int step = kTcWarps * n_split;
+    int p = p0 + split + warp * n_split;
+    int b = p < p1 ? tp_b[p] : 0, nb = p < p1 ? y_n[b] : 0;
+    int r = lane < nb ? y_row[(size_t)b * capY + lane] : -1;
+    int b_next = p + step < p1 ? tp_b[p + step] : 0;
+    for (; p < p1; p += step) {
+        const int nb_next = p + step < p1 ? y_n[b_next] : 0;
+        const int b_after = p + 2 * step < p1 ? tp_b[p + 2 * step] : 0;
+        const int* yr = y_row + (size_t)b * capY;
+        const float* yb = y_val + (size_t)b * capY * kTileVals;
+        float acc[2][4];
+        float2 sum[2][4];
+#pragma unroll
+        for (int h = 0; h < 2; ++h)
+#pragma unroll
+            for (int q = 0; q < 4; ++q) {
+                acc[h][q] = 0.f;
+                sum[h][q] = make_float2(0.f, 0.f);
+            }
+        for (int k0 = 0; k0 < nb; k0 += 32) {
+            const int k = k0 + lane;
+            int at = -1;   // index of the tile C[r, a]
+            if (r >= 0) {
+                const int sl = slot_of[r - r0];
+                if (sl >= 0) at = r * cap + sl;
+            }
+            if (k0 + 32 < nb)
+                r = k + 32 < nb ? yr[k + 32] : -1;
+            else
+                r = lane < nb_next ? y_row[(size_t)b_next * capY + lane] : -1;
+            const unsigned m = __ballot_sync(0xffffffffu, at >= 0);
+            if (!m) continue;   // nothing to add, nothing to flush
+            if (at >= 0) list[__popc(m & ((1u << lane) - 1u))] = make_int2(at, k);
+            __syncwarp();
+            const int n = __popc(m);
+            for (int g = 0; g < n; g += kStage) {
+                const int rows = min(n - g, kStage) * kAoPerMol;
+                float2 cv[6], yv[6];
+#pragma unroll
+                for (int u = 0; u < 6; ++u) {
+                    // blocks 0, 0|1, 1, 2, 2|3, 3
+                    const int blk = u == 0 ? 0 : u == 1 ? (early ? 0 : 1) : u == 2 ? 1 : u == 3 ? 2 : u == 4 ? (early ? 2 : 3) : 3;
+                    const int off = u % 3 == 0 ? o0 : u % 3 == 1 ? o1 : o2;
+                    cv[u] = yv[u] = make_float2(0.f, 0.f);
+                    if (4 * u + tq < rows) {
+                        const int2 e = list[g + blk];
+                        cv[u] = *(const float2*)(c_val + (size_t)e.x * kTileVals + off);
+                        yv[u] = load_stream(yb + (size_t)e.y * kTileVals + off);
+                    }
+                }
+#pragma unroll
+                for (int u = 0; u < 3; ++u) {
+                    if (8 * u >= rows) break;
+                    uint32_t ah[4], al[4];
+                    split_tf32(cv[2 * u].x, ah[0], al[0]);
+                    split_tf32(cv[2 * u].y, ah[1], al[1]);
+                    split_tf32(cv[2 * u + 1].x, ah[2], al[2]);
+                    split_tf32(cv[2 * u + 1].y, ah[3], al[3]);
+#pragma unroll
+                    for (int h = 0; h < 2; ++h) {
+                        uint32_t bh[2], bl[2];
+                        split_tf32(h ? yv[2 * u].y : yv[2 * u].x, bh[0], bl[0]);
+                        split_tf32(h ? yv[2 * u + 1].y : yv[2 * u + 1].x, bh[1], bl[1]);
+                        mma_tf32(acc[h], al, bh);
+                        mma_tf32(acc[h], ah, bl);
+                        mma_tf32(acc[h], ah, bh);
+                    }
+                }
+            }
+            __syncwarp();
+#pragma unroll
+            for (int h = 0; h < 2; ++h)
+#pragma unroll
+                for (int q = 0; q < 4; ++q) {
+                    sum_add(sum[h][q], acc[h][q]);
+                    acc[h][q] = 0.f;
+                }
+        }
+        // rows 2gq and 2gq + 1 of the block, columns 4tq to 4tq + 3
+        float4* o = (float4*)(out + (size_t)tp_out[p] * 256) + 8 * gq + tq;
+        o[0] = make_float4(sum_value(sum[0][0]), sum_value(sum[1][0]), sum_value(sum[0][1]), sum_value(sum[1][1]));
+        o[4] = make_float4(sum_value(sum[0][2]), sum_value(sum[1][2]), sum_value(sum[0][3]), sum_value(sum[1][3]));
+        if (nb == 0) r = lane < nb_next ? y_row[(size_t)b_next * capY + lane] : -1;
+        b = b_next;
+        nb = nb_next;
+        b_next = b_after;
+    }
 }
 
 // diag(F) per MO from the diagonal tile pairs
@@ -975,10 +1003,6 @@ static cudaError_t set_attrs() {
     cudaError_t e;
     e = cudaFuncSetAttribute(k_xc<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024);
     if (e != cudaSuccess) return e;
-    e = cudaFuncSetAttribute(k_transform<T, 1>, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024);
-    if (e != cudaSuccess) return e;
-    e = cudaFuncSetAttribute(k_transform<T, 4>, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024);
-    if (e != cudaSuccess) return e;
     e = cudaFuncSetAttribute(k_density<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024);
     return e;
 }
@@ -989,6 +1013,12 @@ static cudaError_t ensure_attrs() {
     if (e != cudaSuccess) return e;
     if (dev >= 0 && dev < 64 && g_attr_done[dev]) return cudaSuccess;
     e = cudaFuncSetAttribute(k_ci_small, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kCiSmallSmem);
+    if (e != cudaSuccess) return e;
+    e = cudaFuncSetAttribute(k_transform<1>, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024);
+    if (e != cudaSuccess) return e;
+    e = cudaFuncSetAttribute(k_transform<4>, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024);
+    if (e != cudaSuccess) return e;
+    e = cudaFuncSetAttribute(k_transform_tc, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024);
     if (e != cudaSuccess) return e;
     e = set_attrs<double>();
     if (e != cudaSuccess) return e;
@@ -1029,24 +1059,35 @@ cudaError_t launch_xc_rot(Ctx* c) {
     return launch_xc(c, true, 0, c->n_tiles, c->n_occ_tiles);
 }
 
-// CTAs sharing one occupied tile's pairs: what sscf_autotune chose, or enough
-// for kTfCtas per SM, at least 8 (four for every size before: FP64 at 343
-// molecules 5.1 + 3.3 ms, with 24 3.9 + 2.2, as the SMs share the work more
-// evenly; FP32 at 997 1.58 + 1.33 ms, with 10 1.50 + 1.09, with 20 1.97 + 1.45)
-constexpr int kTfCtas = 16;
-static int transform_split(const Ctx* c) {
+// CTAs sharing one occupied tile's pairs: what sscf_autotune chose, or enough for
+// 16 (FP64) or 8 (FP32, twice the warps) per SM. FP64 at 343 molecules: four
+// 5.1 + 3.3 ms, 24 3.9 + 2.2, as the SMs share the work more evenly. FP32: 4 per SM
+// 1.39 + 0.99 ms at 997, 8 1.31 + 0.98, 16 1.33 + 0.90; the same at 4096, where
+// the lower limit decides.
+static int transform_split(const Ctx* c, bool fp64) {
     if (c->tf_split > 0) return c->tf_split;
-    return std::min(32, std::max(8, (kTfCtas * c->n_sm + c->n_occ_tiles - 1) / c->n_occ_tiles));
+    const int per_tile = ((fp64 ? 16 : 8) * c->n_sm + c->n_occ_tiles - 1) / c->n_occ_tiles;
+    return fp64 ? std::min(32, std::max(8, per_tile)) : std::min(16, std::max(4, per_tile));
 }
 
+// (the register budget of sscf_autotune is the FP64 kernel's)
 template <typename T>
 static cudaError_t transform_t(Ctx* c, const int* ptr, const int* bl, const int* outl, void* out) {
-    const size_t smem = (size_t)kTfWarps * tf_stage_vals<T>() * sizeof(T) + (size_t)c->max_cl_mol * 2;
-    auto kern = c->tf_regs == 1 ? k_transform<T, 4> : k_transform<T, 1>;
-    const int split = transform_split(c);
-    kern<<<c->n_tiles * split, kTfWarps * 32, smem, c->stream>>>(
-        split, c->max_cl_mol, c->d_tile_row0, c->cap, c->capY, ptr, bl, outl, c->d_cci_ptr, c->d_cci_row,
-        c->d_cci_slot, (const T*)c->d_c_val[c->cur], c->d_y_n, c->d_y_row, (const T*)c->d_y_val, (T*)out);
+    constexpr bool kFP64 = std::is_same<T, double>::value;
+    const int split = transform_split(c, kFP64);
+    const int grid = c->n_tiles * split;
+    if constexpr (kFP64) {
+        const size_t smem = (size_t)kTfWarps * kTfStageVals * sizeof(T) + (size_t)c->max_cl_mol * 2;
+        auto kern = c->tf_regs == 1 ? k_transform<4> : k_transform<1>;
+        kern<<<grid, kTfWarps * 32, smem, c->stream>>>(
+            split, c->max_cl_mol, c->d_tile_row0, c->cap, c->capY, ptr, bl, outl, c->d_cci_ptr, c->d_cci_row,
+            c->d_cci_slot, (const T*)c->d_c_val[c->cur], c->d_y_n, c->d_y_row, (const T*)c->d_y_val, (T*)out);
+    } else {
+        const size_t smem = (size_t)kTcWarps * 32 * sizeof(int2) + (size_t)c->max_cl_mol * 2;
+        k_transform_tc<<<grid, kTcWarps * 32, smem, c->stream>>>(
+            split, c->max_cl_mol, c->d_tile_row0, c->cap, c->capY, ptr, bl, outl, c->d_cci_ptr, c->d_cci_row,
+            c->d_cci_slot, (const T*)c->d_c_val[c->cur], c->d_y_n, c->d_y_row, (const T*)c->d_y_val, (T*)out);
+    }
     return cudaGetLastError();
 }
 
@@ -1054,8 +1095,7 @@ cudaError_t launch_transform_rot(Ctx* c) {
     c->n_launch += 3;
     cudaError_t e = ensure_attrs();
     if (e != cudaSuccess) return e;
-    if ((size_t)kTfWarps * (c->prec == SSCF_FP64 ? tf_stage_vals<double>() * 8 : tf_stage_vals<float>() * 4) +
-            (size_t)c->max_cl_mol * 2 > 200 * 1024)
+    if ((size_t)kTfWarps * kTfStageVals * 8 + (size_t)c->max_cl_mol * 2 > 200 * 1024)
         return cudaErrorInvalidValue;
     if (c->prec == SSCF_FP64) {
         e = transform_t<double>(c, c->d_rot_tp_ptr, c->d_rot_tp_b, c->d_rot_tp_out, c->d_F);
