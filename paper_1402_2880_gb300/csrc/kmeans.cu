@@ -31,8 +31,11 @@ __device__ __forceinline__ double d2_rn(const double* a, const double* b) {
     return __dadd_rn(__dadd_rn(__dmul_rn(dx, dx), __dmul_rn(dy, dy)), __dmul_rn(dz, dz));
 }
 
+// Squared distances are compared as their bits (they are not negative): a CTA's
+// warps share one FP64 pipe of two lanes per clock.
+__device__ __forceinline__ long long key(double d) { return __double_as_longlong(d); }
 // (d, i) < (e, j) lexicographically
-__device__ __forceinline__ bool lex_less(double d, int i, double e, int j) { return d < e || (d == e && i < j); }
+__device__ __forceinline__ bool lex_less(long long d, int i, long long e, int j) { return d < e || (d == e && i < j); }
 
 // Squared distances of all (molecule, centre) pairs, molecule-major.
 __global__ void k_km_dist(int n, int nc, const double* __restrict__ pos, const double* __restrict__ cen,
@@ -43,26 +46,33 @@ __global__ void k_km_dist(int n, int nc, const double* __restrict__ pos, const d
     D[i] = d2_rn(pos + 3 * (size_t)m, cen + 3 * (size_t)c);
 }
 
-// What a centre holds: its members sorted by (distance^2, molecule).
+// What a centre holds: its members sorted by (distance^2 as a key, molecule).
+// full: the last member's key with the sign bit set once there are n_link, else 0.
 struct KmCentre {
-    double d[kMaxMolPerGroup];
+    long long d[kMaxMolPerGroup];
+    long long full;
     int m[kMaxMolPerGroup];
     int n, lock;
 };
+constexpr long long kKeyBits = 0x7fffffffffffffffll;
+constexpr int kKmLoads = 8;   // distances in flight per lane
 constexpr int kKmSpin = 1 << 22;   // polls of a centre's lock before a warp gives up
 
 // The matching. A warp takes an unlinked molecule, finds its next centre (lanes
 // over the centres, a lexicographic minimum), and inserts it under the centre's
-// lock; a displaced molecule is the warp's next one and goes on after the centre
-// that let it go, so that nothing but the centres' lists is kept. A step is a
-// row of distances and a few hundred clocks in a list, and chains of steps are
-// serial: the lists sit in shared memory where they fit one CTA (IN_SMEM), in
-// global memory with many CTAs else. D = NULL: distances from the positions
-// (more pairs than are worth storing). No warp waits while it holds a lock.
-// 1000 molecules, 150 centres, 101 matchings: 34 ms; with a pair of launches and
-// a host round trip per round of proposals, each centre scanning all molecules,
-// 219-318 ms (1000 molecules of a strongly disordered liquid, 48 matchings: 21
-// against 950 ms).
+// lock, a lane per member; a displaced molecule is the warp's next one and goes on
+// after the centre that let it go, so that nothing but the centres' lists is kept.
+// A full centre's last member only ever comes closer, so a centre whose last
+// member is closer already would reject the molecule and is passed over without
+// a proposal. A step is a row of distances and a few hundred clocks in a list, and
+// chains of steps are serial: the lists sit in shared memory where they fit
+// one CTA (IN_SMEM), in global memory with many CTAs else. D = NULL: distances
+// from the positions (more pairs than are worth storing). No warp waits while it
+// holds a lock.
+// 1000 molecules, 150 centres, 101 matchings: 7 ms (34 with the distances compared
+// in FP64, whose two lanes per clock a CTA's warps shared, rejections proposed one by
+// one and one CTA for every size); with a pair of launches and a host round trip per
+// round of proposals, each centre scanning all molecules, 219-318 ms.
 template <bool IN_SMEM>
 __global__ void __launch_bounds__(1024) k_km_match(int n, int nc, int n_link, const double* __restrict__ pos,
                                                    const double* __restrict__ cen, const double* __restrict__ D,
@@ -71,84 +81,103 @@ __global__ void __launch_bounds__(1024) k_km_match(int n, int nc, int n_link, co
     extern __shared__ __align__(16) unsigned char kmraw[];
     KmCentre* const L = IN_SMEM ? (KmCentre*)kmraw : lists;
     if (IN_SMEM) {
-        for (int c = threadIdx.x; c < nc; c += blockDim.x) L[c].n = L[c].lock = 0;
+        for (int c = threadIdx.x; c < nc; c += blockDim.x) {
+            L[c].n = L[c].lock = 0;
+            L[c].full = 0;
+        }
         __syncthreads();
     }
     const int lane = threadIdx.x & 31;
+    auto fence = [] {
+        if (IN_SMEM) __threadfence_block();
+        else __threadfence();
+    };
+    const int per = (n + 31) / 32;
     for (;;) {
-        int m = 0;
-        if (lane == 0) m = atomicAdd(next, 1);
-        m = __shfl_sync(0xffffffffu, m, 0);
-        if (m >= n) break;
-        double ld = -1.0;   // the last proposal of m: everything after (ld, lc) is open
+        // (molecules that warps take at the same time lie far apart, or they would queue for one centre)
+        int t = 0;
+        if (lane == 0) t = atomicAdd(next, 1);
+        t = __shfl_sync(0xffffffffu, t, 0);
+        if (t >= 32 * per) break;
+        int m = (t & 31) * per + (t >> 5);
+        if (m >= n) continue;
+        long long ld = -1;   // the last proposal of m: everything after (ld, lc) is open
         int lc = -1;
         while (m >= 0) {
-            double bd = INFINITY;
+            long long bd = 0x7fffffffffffffffll;
             int bc = 0x7fffffff;
-            for (int c = lane; c < nc; c += 32) {
-                const double d = D ? D[(size_t)m * nc + c] : d2_rn(pos + 3 * (size_t)m, cen + 3 * (size_t)c);
-                if (lex_less(ld, lc, d, c) && lex_less(d, c, bd, bc)) {
-                    bd = d;
-                    bc = c;
+            for (int c0 = lane; c0 < nc; c0 += 32 * kKmLoads) {
+                long long dv[kKmLoads];
+#pragma unroll
+                for (int u = 0; u < kKmLoads; ++u) {
+                    const int c = min(c0 + 32 * u, nc - 1);
+                    dv[u] = key(D ? D[(size_t)m * nc + c] : d2_rn(pos + 3 * (size_t)m, cen + 3 * (size_t)c));
+                }
+#pragma unroll
+                for (int u = 0; u < kKmLoads; ++u) {
+                    const int c = c0 + 32 * u;
+                    if (c >= nc) break;
+                    const long long d = dv[u], full = *(volatile long long*)&L[c].full;
+                    if ((full == 0 || d <= (full & kKeyBits)) && lex_less(ld, lc, d, c) && lex_less(d, c, bd, bc)) {
+                        bd = d;
+                        bc = c;
+                    }
                 }
             }
 #pragma unroll
             for (int o = 16; o > 0; o >>= 1) {
-                const double od = __shfl_xor_sync(0xffffffffu, bd, o);
+                const long long od = __shfl_xor_sync(0xffffffffu, bd, o);
                 const int oc = __shfl_xor_sync(0xffffffffu, bc, o);
                 if (lex_less(od, oc, bd, bc)) {
                     bd = od;
                     bc = oc;
                 }
             }
-            int out = -1;   // the molecule to go on with, and its last proposal's distance
-            double out_d = 0.0;
+            int ok = 0;
             if (lane == 0) {
-                if (bc >= nc) {   // no centre left: cannot happen while there is room for every molecule
-                    atomicExch(failed, 1);
-                } else {
-                    volatile KmCentre& k = L[bc];
-                    int spins = 0;
-                    while (atomicCAS(&L[bc].lock, 0, 1) != 0)
-                        if (++spins > kKmSpin) break;
-                    if (spins > kKmSpin) {
-                        atomicExch(failed, 1);
-                    } else {
-                        __threadfence();
-                        const int held = k.n;
-                        int p = held;
-                        if (held == n_link) {
-                            const double wd = k.d[held - 1];
-                            const int wm = k.m[held - 1];
-                            if (lex_less(bd, m, wd, wm)) {   // the worst member is displaced
-                                out = wm;
-                                out_d = wd;
-                                p = held - 1;
-                            } else {                         // m is rejected
-                                out = m;
-                                out_d = bd;
-                                p = -1;
-                            }
-                        }
-                        if (p >= 0) {
-                            for (; p > 0; --p) {
-                                const double qd = k.d[p - 1];
-                                const int qm = k.m[p - 1];
-                                if (!lex_less(bd, m, qd, qm)) break;
-                                k.d[p] = qd;
-                                k.m[p] = qm;
-                            }
-                            k.d[p] = bd;
-                            k.m[p] = m;
-                            if (held < n_link) k.n = held + 1;
-                        }
-                        __threadfence();
-                        atomicExch(&L[bc].lock, 0);
-                    }
-                }
+                int spins = kKmSpin + 1;
+                if (bc < nc)   // (no centre left: cannot happen while there is room for every molecule)
+                    for (spins = 0; spins <= kKmSpin && atomicCAS(&L[bc].lock, 0, 1) != 0;) ++spins;
+                ok = spins <= kKmSpin;
+                if (!ok) atomicExch(failed, 1);
             }
-            m = __shfl_sync(0xffffffffu, out, 0);
-            ld = __shfl_sync(0xffffffffu, out_d, 0);
+            if (!__shfl_sync(0xffffffffu, ok, 0)) break;
+            __syncwarp();
+            fence();
+            // the centre's members, one per lane; those before m; the worst of n_link + 1 goes on
+            volatile KmCentre& k = L[bc];
+            const int held = k.n;
+            const bool mine = lane < held;
+            const long long qd = mine ? k.d[lane] : 0;
+            const int qm = mine ? k.m[lane] : 0;
+            const int p = __popc(__ballot_sync(0xffffffffu, mine && lex_less(qd, qm, bd, m)));
+            int out = -1;   // the molecule to go on with, and its last proposal's distance
+            long long out_d = 0;
+            if (held == n_link) {
+                out = __shfl_sync(0xffffffffu, qm, held - 1);
+                out_d = __shfl_sync(0xffffffffu, qd, held - 1);
+            }
+            if (p == n_link) {   // m is rejected
+                out = m;
+                out_d = bd;
+            } else {
+                if (mine && lane >= p && lane + 1 < n_link) {
+                    k.d[lane + 1] = qd;
+                    k.m[lane + 1] = qm;
+                }
+                if (lane == 0) {
+                    k.d[p] = bd;
+                    k.m[p] = m;
+                    if (held < n_link) k.n = held + 1;
+                }
+                const long long last = __shfl_sync(0xffffffffu, qd, max(n_link - 2, 0));
+                if (lane == 0 && held >= n_link - 1) k.full = (p == n_link - 1 ? bd : last) | ~kKeyBits;
+            }
+            fence();
+            __syncwarp();
+            if (lane == 0) atomicExch(&L[bc].lock, 0);
+            m = out;
+            ld = out_d;
             lc = bc;
         }
     }
@@ -161,24 +190,36 @@ __global__ void __launch_bounds__(1024) k_km_match(int n, int nc, int n_link, co
 // Every centre's members as holders, and the centroid of the members summed in
 // increasing molecule index; a centre without members keeps its place.
 __global__ void k_km_centroids(int nc, const double* __restrict__ pos, const KmCentre* __restrict__ lists,
-                               const double* __restrict__ cen, double* __restrict__ cen_new,
-                               int* __restrict__ holder) {
+                               const double* __restrict__ cen, const int* __restrict__ failed,
+                               double* __restrict__ cen_new, int* __restrict__ holder) {
     const int c = blockIdx.x * blockDim.x + threadIdx.x;
+    if (c == 0) cen_new[3 * (size_t)nc] = (double)*failed;   // to be read with the centres
     if (c >= nc) return;
     const int k = lists[c].n;
-    double s0 = 0.0, s1 = 0.0, s2 = 0.0;
-    int last = -1;
-    for (int i = 0; i < k; ++i) {
-        int m = 0x7fffffff;   // the next member by index
-        for (int j = 0; j < k; ++j) {
-            const int q = lists[c].m[j];
-            if (q > last && q < m) m = q;
+    int m[kMaxMolPerGroup];
+    double x[kMaxMolPerGroup][3];
+#pragma unroll
+    for (int i = 0; i < kMaxMolPerGroup; ++i) m[i] = i < k ? lists[c].m[i] : 0x7fffffff;
+#pragma unroll
+    for (int i = 1; i < kMaxMolPerGroup; ++i)   // by index
+#pragma unroll
+        for (int j = i; j > 0; --j) {
+            const int a = min(m[j - 1], m[j]), b = max(m[j - 1], m[j]);
+            m[j - 1] = a;
+            m[j] = b;
         }
-        last = m;
-        holder[m] = c;
-        s0 = __dadd_rn(s0, pos[3 * (size_t)m]);
-        s1 = __dadd_rn(s1, pos[3 * (size_t)m + 1]);
-        s2 = __dadd_rn(s2, pos[3 * (size_t)m + 2]);
+#pragma unroll
+    for (int i = 0; i < kMaxMolPerGroup; ++i)
+#pragma unroll
+        for (int d = 0; d < 3; ++d) x[i][d] = i < k ? pos[3 * (size_t)m[i] + d] : 0.0;
+    double s0 = 0.0, s1 = 0.0, s2 = 0.0;
+#pragma unroll
+    for (int i = 0; i < kMaxMolPerGroup; ++i) {
+        if (i >= k) break;
+        holder[m[i]] = c;
+        s0 = __dadd_rn(s0, x[i][0]);
+        s1 = __dadd_rn(s1, x[i][1]);
+        s2 = __dadd_rn(s2, x[i][2]);
     }
     cen_new[3 * c] = k == 0 ? cen[3 * c] : __ddiv_rn(s0, (double)k);
     cen_new[3 * c + 1] = k == 0 ? cen[3 * c + 1] : __ddiv_rn(s1, (double)k);
@@ -214,26 +255,29 @@ struct KmState {
 };
 constexpr long long kKmMaxPairs = 1ll << 27;           // distances stored up to here (1 GB)
 constexpr size_t kKmMaxSmem = 200 * 1024;
+// Molecules up to which one CTA with the lists in shared memory matches faster than
+// 128 with them in global memory (us per iteration, host included: 125 molecules 46
+// against 64, 343 87 against 98, 1000 116 against 79, 4096 832 against 175).
+constexpr int kKmOneCta = 512;
 
 // The links of the centres `cen` (in st.lists) and the centroids they give.
 int link_all(cudaStream_t s, const KmState& st, const double* cen, double* cen_new) {
     const int th = 256;
-    KM_CK(cudaMemsetAsync(st.next, 0, 8, s));
+    const size_t list_bytes = (size_t)st.nc * sizeof(KmCentre);
+    KM_CK(cudaMemsetAsync(st.lists, 0, list_bytes + 8, s));   // and next, which follows them
     if (st.D) {
         const long long pairs = (long long)st.n * st.nc;
         k_km_dist<<<(unsigned)((pairs + th - 1) / th), th, 0, s>>>(st.n, st.nc, st.pos, cen, st.D);
     }
-    const size_t smem = (size_t)st.nc * sizeof(KmCentre);
-    if (smem <= kKmMaxSmem) {
-        KM_CK(cudaFuncSetAttribute(k_km_match<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-        k_km_match<true><<<1, 1024, smem, s>>>(st.n, st.nc, st.n_link, st.pos, cen, st.D, st.lists, st.next,
-                                               st.next + 1);
+    if (st.n <= kKmOneCta && list_bytes <= kKmMaxSmem) {
+        KM_CK(cudaFuncSetAttribute(k_km_match<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)list_bytes));
+        k_km_match<true><<<1, 1024, list_bytes, s>>>(st.n, st.nc, st.n_link, st.pos, cen, st.D, st.lists, st.next,
+                                                     st.next + 1);
     } else {
-        KM_CK(cudaMemsetAsync(st.lists, 0, smem, s));
         k_km_match<false><<<128, th, 0, s>>>(st.n, st.nc, st.n_link, st.pos, cen, st.D, st.lists, st.next,
                                              st.next + 1);
     }
-    k_km_centroids<<<(st.nc + th - 1) / th, th, 0, s>>>(st.nc, st.pos, st.lists, cen, cen_new, st.holder);
+    k_km_centroids<<<(st.nc + 31) / 32, 32, 0, s>>>(st.nc, st.pos, st.lists, cen, st.next + 1, cen_new, st.holder);
     KM_CK(cudaGetLastError());
     return SSCF_OK;
 }
@@ -275,7 +319,7 @@ extern "C" int sscf_group_molecules(int n_atoms, const double* xyz, int n_link, 
         g[best]++;
     }
     const int nc = (int)(g[0] * g[1] * g[2]);
-    std::vector<double> cen(3 * (size_t)nc), cen_new(3 * (size_t)nc);
+    std::vector<double> cen(3 * (size_t)nc + 1), cen_new(3 * (size_t)nc + 1);   // and whether a warp gave up
     {
         size_t c = 0;
         for (long long k = 0; k < g[2]; ++k)
@@ -293,12 +337,12 @@ extern "C" int sscf_group_molecules(int n_atoms, const double* xyz, int n_link, 
     km.nc = nc;
     km.n_link = n_link;
     km.pos = buf.get<double>(3 * (size_t)n);
-    double* d_cen = buf.get<double>(3 * (size_t)nc);
-    double* d_cen_new = buf.get<double>(3 * (size_t)nc);
-    km.lists = buf.get<KmCentre>(nc);
+    double* d_cen = buf.get<double>(cen.size());
+    double* d_cen_new = buf.get<double>(cen.size());
+    km.lists = buf.get<KmCentre>((size_t)nc + 1);
     km.holder = buf.get<int>(n);
-    km.next = buf.get<int>(2);
-    if (!km.pos || !d_cen || !d_cen_new || !km.lists || !km.holder || !km.next) return SSCF_ERR_OOM;
+    km.next = (int*)(km.lists + nc);
+    if (!km.pos || !d_cen || !d_cen_new || !km.lists || !km.holder) return SSCF_ERR_OOM;
     // (without room for the distances the matching computes them as it goes)
     km.D = (long long)n * nc <= kKmMaxPairs ? buf.get<double>((size_t)n * nc) : nullptr;
     KM_CK(cudaMemcpyAsync(km.pos, pos.data(), pos.size() * 8, cudaMemcpyHostToDevice, st));
@@ -306,12 +350,13 @@ extern "C" int sscf_group_molecules(int n_atoms, const double* xyz, int n_link, 
     int s = link_all(st, km, d_cen, d_cen_new);
     if (s != SSCF_OK) return s;
     int it = 0;
-    int given_up[2] = {0, 0};
     for (it = 1; it <= max_iter; ++it) {
         KM_CK(cudaMemcpyAsync(cen_new.data(), d_cen_new, cen_new.size() * 8, cudaMemcpyDeviceToHost, st));
-        KM_CK(cudaMemcpyAsync(given_up, km.next, 8, cudaMemcpyDeviceToHost, st));
         KM_CK(cudaStreamSynchronize(st));
-        if (given_up[1]) return SSCF_ERR_TIMEOUT;
+        if (cen_new[3 * (size_t)nc] != 0.0) return SSCF_ERR_TIMEOUT;
+        std::swap(d_cen, d_cen_new);   // the links are due whether or not the centres have settled
+        s = link_all(st, km, d_cen, d_cen_new);
+        if (s != SSCF_OK) return s;
         double moved = 0.0;
         for (int c = 0; c < nc; ++c) {
             const double dx = cen_new[3 * c] - cen[3 * c], dy = cen_new[3 * c + 1] - cen[3 * c + 1],
@@ -321,17 +366,14 @@ extern "C" int sscf_group_molecules(int n_atoms, const double* xyz, int n_link, 
             moved += std::sqrt(t + zz);
         }
         std::swap(cen, cen_new);
-        std::swap(d_cen, d_cen_new);
-        s = link_all(st, km, d_cen, d_cen_new);
-        if (s != SSCF_OK) return s;
         if (moved / nc < tol) break;
     }
     if (it > max_iter) it = max_iter;
     std::vector<int> holder(n);
     KM_CK(cudaMemcpyAsync(holder.data(), km.holder, (size_t)n * 4, cudaMemcpyDeviceToHost, st));
-    KM_CK(cudaMemcpyAsync(given_up, km.next, 8, cudaMemcpyDeviceToHost, st));
+    KM_CK(cudaMemcpyAsync(cen_new.data(), d_cen_new, cen_new.size() * 8, cudaMemcpyDeviceToHost, st));
     KM_CK(cudaStreamSynchronize(st));
-    if (given_up[1]) return SSCF_ERR_TIMEOUT;
+    if (cen_new[3 * (size_t)nc] != 0.0) return SSCF_ERR_TIMEOUT;
     std::vector<int> remap(nc, -1);
     for (int m = 0; m < n; ++m) {
         if (holder[m] < 0 || holder[m] >= nc) return SSCF_ERR_STATE;

@@ -1,5 +1,6 @@
 """Grouping at the edges of the matching kernel's ranges, bit for bit against the oracle: one
-molecule, one molecule per centre, and more centres than one CTA's shared memory lists
+molecule, one molecule per centre, the last size of one CTA with its lists in shared memory and the
+first of many CTAs with them in global memory, and more centres than one CTA's shared memory lists
 (those lists are in global memory, written by many CTAs)."""
 import numpy as np
 import pytest
@@ -11,7 +12,8 @@ from synth import lattice_water
 pytestmark = pytest.mark.gpu
 
 
-@pytest.mark.parametrize("n,n_link,max_iter", [(1, 8, 100), (7, 1, 100), (130, 3, 0), (2001, 1, 2)])
+@pytest.mark.parametrize("n,n_link,max_iter", [(1, 8, 100), (7, 1, 100), (130, 3, 0), (512, 7, 3), (513, 7, 3),
+                                               (2001, 1, 2)])
 def test_groups_match_oracle(n, n_link, max_iter):
     library()
     from paper_1402_2880_gb300 import group_molecules
