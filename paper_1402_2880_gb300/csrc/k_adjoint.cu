@@ -17,6 +17,7 @@
 #include <type_traits>
 
 #include "shares.h"
+#include "block_scan.h"
 #include "sscf_internal.h"
 
 namespace sscf {
@@ -37,8 +38,7 @@ __global__ void __launch_bounds__(256) k_zlists(int n_occ_tiles, int n_groups, i
     const int gw = (n_groups + 31) >> 5;
     unsigned* pres = (unsigned*)smraw;          // gw: groups with occupied tiles in row r
     unsigned* outg = pres + gw;                 // gw: groups of Z's tiles
-    __shared__ int part[256];
-    __shared__ int s_nout;
+    __shared__ int part[33];
     const int r = blockIdx.x;
     for (int i = threadIdx.x; i < gw; i += blockDim.x) pres[i] = outg[i] = 0u;
     __syncthreads();
@@ -64,30 +64,19 @@ __global__ void __launch_bounds__(256) k_zlists(int n_occ_tiles, int n_groups, i
     int cnt = 0;
     for (int g = g0; g < g1; ++g)
         if ((outg[g >> 5] >> (g & 31)) & 1) cnt += group_not[g];
-    part[threadIdx.x] = cnt;
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        int run = 0;
-        for (int i = 0; i < (int)blockDim.x; ++i) {
-            const int v = part[i];
-            part[i] = run;
-            run += v;
-        }
-        s_nout = run;
-    }
-    __syncthreads();
-    if (s_nout > cap) {
+    int pos = block_scan(cnt, part);
+    const int n_out = part[32];
+    if (n_out > cap) {
         if (threadIdx.x == 0) {
             atomicOr(err, kErrCapacity);
             z_nt[r] = 0;
         }
         return;
     }
-    int pos = part[threadIdx.x];
     for (int g = g0; g < g1; ++g)
         if ((outg[g >> 5] >> (g & 31)) & 1)
             for (int i = 0; i < group_not[g]; ++i) z_tile[(size_t)r * cap + pos++] = group_ot0[g] + i;
-    if (threadIdx.x == 0) z_nt[r] = s_nout;
+    if (threadIdx.x == 0) z_nt[r] = n_out;
 }
 
 // first position of the sorted list with a tile >= t

@@ -45,7 +45,7 @@ __global__ void k_cluster_reduce(const int* __restrict__ cl_mol0, const int* __r
     }
 }
 
-// One CTA: fixed-order reductions (deterministic) and the mixing update.
+// One CTA of 32 to 1024 threads: fixed-order reductions (deterministic) and the mixing update.
 __global__ void k_finish(int n_atoms, int n_mol, int mix, double beta, const double* __restrict__ e_mol,
                          double* __restrict__ q, double* __restrict__ q_prev, const double* __restrict__ dq,
                          const double* __restrict__ Q, double* __restrict__ dq_in, double* __restrict__ Q_in,
@@ -61,7 +61,7 @@ __global__ void k_finish(int n_atoms, int n_mol, int mix, double beta, const dou
     s_coul[threadIdx.x] = coul;
     s_max[threadIdx.x] = mx;
     __syncthreads();
-    for (int off = blockDim.x / 2; off > 0; off >>= 1) {
+    for (int off = blockDim.x / 2; off >= 32; off >>= 1) {
         if ((int)threadIdx.x < off) {
             s_band[threadIdx.x] += s_band[threadIdx.x + off];
             s_coul[threadIdx.x] += s_coul[threadIdx.x + off];
@@ -69,11 +69,22 @@ __global__ void k_finish(int n_atoms, int n_mol, int mix, double beta, const dou
         }
         __syncthreads();
     }
+    if (threadIdx.x < 32) {
+        band = s_band[threadIdx.x];
+        coul = s_coul[threadIdx.x];
+        mx = s_max[threadIdx.x];
+#pragma unroll
+        for (int off = 16; off > 0; off >>= 1) {
+            band += __shfl_down_sync(0xffffffffu, band, off);
+            coul += __shfl_down_sync(0xffffffffu, coul, off);
+            mx = fmax(mx, __shfl_down_sync(0xffffffffu, mx, off));
+        }
+    }
     if (threadIdx.x == 0) {
-        sc->e_band = s_band[0];
-        sc->e_coul = 0.5 * s_coul[0];
-        sc->energy = s_band[0] + 0.5 * s_coul[0];
-        sc->dq_max = s_max[0];
+        sc->e_band = band;
+        sc->e_coul = 0.5 * coul;
+        sc->energy = band + 0.5 * coul;
+        sc->dq_max = mx;
         if (!isfinite(sc->energy)) atomicOr(&sc->err, kErrNonFinite);
     }
     // after a capacity error the step's MOs are the previous ones: keep the charges
@@ -129,7 +140,10 @@ cudaError_t launch_charges_finish(Ctx* c, bool mix) {
     k_cluster_reduce<<<c->n_clusters, 256, 0, c->stream>>>(c->d_cl_mol0, c->d_cl_nmol, c->d_e_mol, c->d_q, c->d_q_prev,
                                                           c->d_dq, c->d_Q, c->d_cl_E, c->d_cl_dq);
     c->n_launch += 1;
-    k_finish<<<1, 1024, 0, c->stream>>>(c->n_atoms, c->n_mol, mix ? 1 : 0, c->prm.mix_beta, c->d_e_mol, c->d_q,
+    // a thread per atom up to 1024: the sums' order is that of the atoms either way
+    int threads = 32;
+    while (threads < 1024 && threads < c->n_atoms) threads *= 2;
+    k_finish<<<1, threads, 0, c->stream>>>(c->n_atoms, c->n_mol, mix ? 1 : 0, c->prm.mix_beta, c->d_e_mol, c->d_q,
                                         c->d_q_prev, c->d_dq, c->d_Q, c->d_dq_in, c->d_Q_in, c->d_sc);
     return cudaGetLastError();
 }

@@ -14,6 +14,7 @@
 #include <algorithm>
 #include <vector>
 
+#include "block_scan.h"
 #include "sscf_internal.h"
 
 #include <type_traits>
@@ -200,13 +201,14 @@ __global__ void __launch_bounds__(1024) k_rot_select_small(int last_shift, int n
     }
     for (int i = threadIdx.x; i < 256; i += blockDim.x) s_h[i] = 0u;
     __syncthreads();
-    // every candidate key, a block per warp
+    // every candidate key, a block per warp or, of fewer blocks than warps, several warps per block
+    const int w_per = n_gnb < 32 ? 32 / n_gnb : 1, sub = warp % w_per;
     auto each = [&](auto f) {
-        for (int e = warp; e < n_gnb; e += 32) {
+        for (int e = warp / w_per; e < n_gnb; e += 32 / w_per) {
             const int no = 4 * group_nmol[gnb_row[e]], B = gnb_col[e], nv = 2 * group_nmol[B], nvt = group_nvt[B];
             const T* fe = F + (size_t)blk_tp0[e] * 256;
 #pragma unroll 4
-            for (int p = lane; p < no * 16; p += 32) {
+            for (int p = lane + 32 * sub; p < no * 16; p += 32 * w_per) {
                 const int i = p >> 4, j = p & 15;   // a block has one virtual tile: nvt = 1, nv <= 16
                 if (j >= nv) continue;
                 const double v = fabs((double)fe[(size_t)(i >> 4) * nvt * 256 + (i & 15) * 16 + j]);
@@ -674,23 +676,12 @@ __global__ void __launch_bounds__(1024) k_closure_labels(SweepArgs a, int* __res
     __syncthreads();
     for (int u = threadIdx.x; u < nu; u += blockDim.x) atomicAdd(&cnt[slab[u]], 1);
     __syncthreads();
-    __shared__ int part[1024];
+    __shared__ int part[33];
     const int per = (nu + blockDim.x - 1) / blockDim.x;
     const int lo = threadIdx.x * per, hi = min(nu, lo + per);
     int sum = 0;
     for (int i = lo; i < hi; ++i) sum += cnt[i];
-    part[threadIdx.x] = sum;
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        int run = 0;
-        for (int i = 0; i < (int)blockDim.x; ++i) {
-            const int v = part[i];
-            part[i] = run;
-            run += v;
-        }
-    }
-    __syncthreads();
-    int run = part[threadIdx.x];
+    int run = block_scan(sum, part);
     for (int i = lo; i < hi; ++i) {
         const int c = cnt[i];
         a.lab_start[2 * g0 + i] = run;
@@ -737,8 +728,7 @@ __global__ void __launch_bounds__(256) k_closure(SweepArgs a) {
     short* oslot = (short*)(oldt + a.cap);     // per new slot: its slot in the row, or -1
     __shared__ int s_big[kBigMax];
     __shared__ int s_nbig;
-    __shared__ int part[256];
-    __shared__ int s_total;
+    __shared__ int part[33];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nwarps = blockDim.x >> 5;
     const int* lab = a.unit_lab + 2 * g0;
     const int* lstart = a.lab_start + 2 * g0;
@@ -798,30 +788,16 @@ __global__ void __launch_bounds__(256) k_closure(SweepArgs a) {
     const int w0 = threadIdx.x * per, w1 = min(nw, w0 + per);
     int cnt = 0;
     for (int w = w0; w < w1; ++w) cnt += wpos[w];
-    part[threadIdx.x] = cnt;
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        int run = 0;
-        for (int i = 0; i < (int)blockDim.x; ++i) {
-            const int v = part[i];
-            part[i] = run;
-            run += v;
-        }
-        s_total = run;
-    }
-    __syncthreads();
-    const int n1 = s_total;
+    int run = block_scan(cnt, part);
+    const int n1 = part[32];
     if (n1 > a.cap) {
         if (threadIdx.x == 0) atomicOr(a.err, kErrCapacity);
         return;
     }
-    {
-        int run = part[threadIdx.x];
-        for (int w = w0; w < w1; ++w) {
-            const int c = wpos[w];
-            wpos[w] = run;
-            run += c;
-        }
+    for (int w = w0; w < w1; ++w) {
+        const int c = wpos[w];
+        wpos[w] = run;
+        run += c;
     }
     __syncthreads();
     // the new row: tile ids, the slot each had in the row (binary search of the

@@ -8,6 +8,7 @@
 // reduced over the row blocks the two columns share.
 #include <cuda_bf16.h>
 
+#include "block_scan.h"
 #include "sscf_internal.h"
 
 #include <algorithm>
@@ -32,24 +33,13 @@ __global__ void k_ci_count(int n_mol, int cap, const int* __restrict__ c_nt, con
 
 // exclusive scan of n counts into ptr (n + 1 entries); one CTA of 1024 threads
 __global__ void k_scan(int n, const int* __restrict__ cnt, int* __restrict__ ptr) {
-    __shared__ int part[1024];
+    __shared__ int part[33];
     const int per = (n + blockDim.x - 1) / blockDim.x;
     const int lo = threadIdx.x * per, hi = min(n, lo + per);
     int s = 0;
     for (int i = lo; i < hi; ++i) s += cnt[i];
-    part[threadIdx.x] = s;
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        int run = 0;
-        for (int i = 0; i < (int)blockDim.x; ++i) {
-            int v = part[i];
-            part[i] = run;
-            run += v;
-        }
-        ptr[n] = run;
-    }
-    __syncthreads();
-    int run = part[threadIdx.x];
+    int run = block_scan(s, part);
+    if (threadIdx.x == 0) ptr[n] = part[32];
     for (int i = lo; i < hi; ++i) {
         ptr[i] = run;
         run += cnt[i];
@@ -79,7 +69,7 @@ __global__ void __launch_bounds__(kSortThreads) k_ci_sort(const int* __restrict_
     extern __shared__ unsigned sbits[];               // n_rows bits, then the set bits before each word
     const int nw = (n_rows + 31) >> 5;
     int* wpre = (int*)(sbits + nw);
-    __shared__ int part[kSortThreads];
+    __shared__ int part[33];
     const int t = blockIdx.x;
     const int lo = ptr[t], n = ptr[t + 1] - lo;
     if (n <= 1) return;
@@ -107,18 +97,7 @@ __global__ void __launch_bounds__(kSortThreads) k_ci_sort(const int* __restrict_
     const int w0 = threadIdx.x * per, w1 = min(nw, w0 + per);
     int c = 0;
     for (int w = w0; w < w1; ++w) c += __popc(sbits[w]);
-    part[threadIdx.x] = c;
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        int run = 0;
-        for (int i = 0; i < (int)blockDim.x; ++i) {
-            const int v = part[i];
-            part[i] = run;
-            run += v;
-        }
-    }
-    __syncthreads();
-    int run = part[threadIdx.x];
+    int run = block_scan(c, part);
     for (int w = w0; w < w1; ++w) {
         wpre[w] = run;
         run += __popc(sbits[w]);
@@ -216,7 +195,7 @@ __global__ void k_xc(int tile_lo, int n_t, int n_share, int n_rows, int own_belo
     unsigned* bits = (unsigned*)sm;               // n_rows bits
     int* wpre = (int*)(bits + nw);                // prefix of popcounts per word
     short* rowpos = (short*)(wpre + nw);          // n_rows: index into the tile's column list or -1
-    __shared__ int s_total;
+    __shared__ int part[33];
     // tiles from own_below on (the longer ones: every reachable row) first
     const int t = tile_lo + (int)((blockIdx.x / n_share + (unsigned)max(own_below - tile_lo, 0)) % n_t);
     const int share = blockIdx.x % n_share;   // of the tile's rows of Y
@@ -246,16 +225,17 @@ __global__ void k_xc(int tile_lo, int n_t, int n_share, int n_rows, int own_belo
         }
     }
     __syncthreads();
-    if (threadIdx.x == 0) {
-        int run = 0;
-        for (int w = 0; w < nw; ++w) {
-            wpre[w] = run;
-            run += __popc(bits[w]);
-        }
-        s_total = run;
+    const int w_per = (nw + blockDim.x - 1) / blockDim.x;
+    const int w0 = threadIdx.x * w_per, w1 = min(nw, w0 + w_per);
+    int n_set = 0;
+    for (int w = w0; w < w1; ++w) n_set += __popc(bits[w]);
+    int before = block_scan(n_set, part);
+    for (int w = w0; w < w1; ++w) {
+        wpre[w] = before;
+        before += __popc(bits[w]);
     }
     __syncthreads();
-    const int ny = s_total;
+    const int ny = part[32];
     if (ny > capY) {
         if (threadIdx.x == 0) {
             atomicOr(err, kErrCapacity);
