@@ -242,12 +242,11 @@ int sscf_step(sscf_ctx* ctx, sscf_step_info* info);
 /* Launch-shape autotuner (no counterpart in the paper): on the current state
  * it builds H and Y = H C as a step would, times the occupied-virtual transform
  * (three launches after one warm-up, CUDA events on the context's stream) for
- * 1, 2, 4 and 8 CTAs sharing each occupied tile's pairs, each with two
- * register budgets of the kernel (uncut, or cut for four resident CTAs per
- * SM), and keeps the fastest for later steps. Results of later calls do not
- * depend on the choice (each pair is summed the same way). Drops a captured
- * CUDA graph. tf_split_out (host, may be NULL) receives the CTAs per tile plus
- * 16 if the cut register budget won. Errors: STATE before sscf_guess, CUDA. */
+ * 1, 2, 4 and 8 CTAs sharing each occupied tile's pairs and for the number
+ * taken by size, and keeps the fastest for later steps. Results of later
+ * calls do not depend on the choice (each pair is summed the same way). Drops a
+ * captured CUDA graph. tf_split_out (host, may be NULL) receives the fastest of
+ * the four. Errors: STATE before sscf_guess, CUDA. */
 int sscf_autotune(sscf_ctx* ctx, int* tf_split_out);
 
 /* CUDA graphs: when enabled, sscf_step captures its device work (all kernel

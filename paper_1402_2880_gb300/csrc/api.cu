@@ -1111,35 +1111,36 @@ int sscf_autotune(sscf_ctx* h, int* tf_split_out) {
     cudaEvent_t e0, e1;
     CK(cudaEventCreate(&e0));
     CK(cudaEventCreate(&e1));
-    const int cand[] = {1, 2, 4, 8};
-    int best = c.tf_split, best_regs = c.tf_regs;
-    float best_ms = 1e30f;
+    const int cand[] = {0, 1, 2, 4, 8};   // 0: by size
+    int best = 0, best_fixed = 1;
+    float best_ms = 1e30f, best_fixed_ms = 1e30f;
+    const int before = c.tf_split;
     cudaError_t err = cudaSuccess;
-    for (int regs = 0; regs < 2 && err == cudaSuccess; ++regs)
-        for (int s : cand) {
-            c.tf_split = s;
-            c.tf_regs = regs;
-            err = launch_transform_rot(&c);   // warm-up
-            if (err != cudaSuccess) break;
-            err = cudaEventRecord(e0, c.stream);
-            for (int r = 0; r < 3 && err == cudaSuccess; ++r) err = launch_transform_rot(&c);
-            if (err == cudaSuccess) err = cudaEventRecord(e1, c.stream);
-            if (err == cudaSuccess) err = cudaEventSynchronize(e1);
-            float ms = 0.f;
-            if (err == cudaSuccess) err = cudaEventElapsedTime(&ms, e0, e1);
-            if (err != cudaSuccess) break;
-            if (ms < best_ms) {
-                best_ms = ms;
-                best = s;
-                best_regs = regs;
-            }
+    for (int s : cand) {
+        c.tf_split = s;
+        err = launch_transform_rot(&c);   // warm-up
+        if (err != cudaSuccess) break;
+        err = cudaEventRecord(e0, c.stream);
+        for (int r = 0; r < 3 && err == cudaSuccess; ++r) err = launch_transform_rot(&c);
+        if (err == cudaSuccess) err = cudaEventRecord(e1, c.stream);
+        if (err == cudaSuccess) err = cudaEventSynchronize(e1);
+        float ms = 0.f;
+        if (err == cudaSuccess) err = cudaEventElapsedTime(&ms, e0, e1);
+        if (err != cudaSuccess) break;
+        if (ms < best_ms) {
+            best_ms = ms;
+            best = s;
         }
+        if (s > 0 && ms < best_fixed_ms) {
+            best_fixed_ms = ms;
+            best_fixed = s;
+        }
+    }
     cudaEventDestroy(e0);
     cudaEventDestroy(e1);
-    c.tf_split = best;
-    c.tf_regs = best_regs;
+    c.tf_split = err == cudaSuccess ? best : before;
     if (err != cudaSuccess) return SSCF_ERR_CUDA;
-    if (tf_split_out) *tf_split_out = best + 16 * best_regs;
+    if (tf_split_out) *tf_split_out = best_fixed;
     return SSCF_OK;
 }
 

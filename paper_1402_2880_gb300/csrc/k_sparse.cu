@@ -370,28 +370,31 @@ __global__ void k_xc(int tile_lo, int n_t, int n_share, int n_rows, int own_belo
 
 // ---------------------------------------------------------------------------
 // Tile-pair transform: out[p] (16x16) = C[:, a]^T Y[:, b] for every listed
-// pair (a, b). One CTA per tile a with a shared map row block -> slot of a.
-// One warp per pair: it walks b's rows (sorted), and for the rows present in
-// a it stages the two 6x16 tiles (C[r, a] and Y[r, b]) in a per-warp buffer
-// with 16-byte loads, kStage row blocks at a time; every lane then owns a 2x4
-// block of the 16x16 result and does 8 FMAs per K step from one 8-byte and
-// two 16-byte shared loads. Rows are summed in ascending order (fixed order),
-// 32 of b's rows at a time. FP64 storage; FP32 storage: k_transform_tc.
+// pair (a, b). CTAs (a, split) share tile a's pairs, each with a map row block ->
+// slot of a in shared memory. Rows are summed in ascending order (fixed order),
+// 32 of b's rows at a time. FP64 storage here; FP32 storage: k_transform_tc.
+//
+// A quarter of an SM starts one FP64 instruction of a warp every 64 clocks, busy
+// or not, so a CTA's four warps work on one pair, four columns of b each; with a
+// pair per warp, a system with fewer pairs than four per SM waited for three
+// quarters idle (32 molecules 89 us a launch, now 29; 343 3.8 + 2.1 ms, now 3.2 + 1.9). They walk b's rows (sorted) and stage the 6x16 tiles
+// C[r, a] and Y[r, b] of the rows present in a, kStage row blocks at a time, into
+// one of two buffers while the loads of the next ones are in flight; a lane
+// owns 2x1 of the result and takes a 16-byte and an 8-byte shared load for two FMAs.
 // ---------------------------------------------------------------------------
 constexpr int kTfWarps = 4;
-constexpr int kStage = 4;   // row blocks taken per warp at a time
-constexpr int kTfStageVals = kStage * 2 * kTileVals;   // staged values per warp: [kStage][2][96]
-// MINB: resident CTAs per SM the register budget is cut for (1: no cut)
-template <int MINB>
-__global__ void __launch_bounds__(kTfWarps * 32, MINB)
+constexpr int kStage = 4;   // row blocks staged at a time
+constexpr int kTfStageVals = kStage * 2 * kTileVals;   // values of a buffer: [kStage][2][96]
+
+__global__ void __launch_bounds__(kTfWarps * 32)
 k_transform(int n_split, int n_rows, const int* __restrict__ tile_row0, int cap, int capY, const int* __restrict__ tp_ptr,
-            const int* __restrict__ tp_b,
-            const int* __restrict__ tp_out, const int* __restrict__ cci_ptr, const int* __restrict__ cci_row,
-            const int* __restrict__ cci_slot, const double* __restrict__ c_val, const int* __restrict__ y_n,
-            const int* __restrict__ y_row, const double* __restrict__ y_val, double* __restrict__ out) {
+            const int* __restrict__ tp_b, const int* __restrict__ tp_out, const int* __restrict__ cci_ptr,
+            const int* __restrict__ cci_row, const int* __restrict__ cci_slot, const double* __restrict__ c_val,
+            const int* __restrict__ y_n, const int* __restrict__ y_row, const double* __restrict__ y_val,
+            double* __restrict__ out) {
     extern __shared__ __align__(16) unsigned char sraw[];
-    double* stage = (double*)sraw;                                        // [warps][kTfStageVals]
-    short* slot_of = (short*)(stage + (size_t)kTfWarps * kTfStageVals);   // n_rows (cluster-local)
+    double2* stage = (double2*)sraw;                                 // two buffers
+    short* slot_of = (short*)((double*)sraw + 2 * kTfStageVals);     // n_rows (cluster-local)
     // CTA (a, s) takes the pairs of tile a with index = s (mod n_split)
     const int a = blockIdx.x / n_split, split = blockIdx.x % n_split;
     const int p0 = tp_ptr[a], p1 = tp_ptr[a + 1];
@@ -403,86 +406,88 @@ k_transform(int n_split, int n_rows, const int* __restrict__ tile_row0, int cap,
     for (int k = threadIdx.x; k < nc; k += blockDim.x) slot_of[cci_row[lo + k] - r0] = (short)cci_slot[lo + k];
     __syncthreads();
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    double* buf = stage + (size_t)warp * kTfStageVals;
-    const int i0 = 2 * (lane >> 2), j0 = 4 * (lane & 3);
-    constexpr int kPerTile = kTileVals / 2;   // 16-byte loads per tile
-    for (int p = p0 + split + warp * n_split; p < p1; p += kTfWarps * n_split) {
+    const int i0 = 2 * (lane >> 2), j0 = 4 * warp + (lane & 3);
+    constexpr int kHalf = kTileVals / 2, kLoads = kStage * 2 * kHalf / (kTfWarps * 32);   // 16-byte pieces
+    static_assert(kLoads * kTfWarps * 32 == kStage * 2 * kHalf, "");
+    int phase = 0;
+    for (int p = p0 + split; p < p1; p += n_split) {
         const int b = tp_b[p];
         const int nb = y_n[b];
         const int* yr = y_row + (size_t)b * capY;
-        double accd[8];
-        double acc[8];
-#pragma unroll
-        for (int q = 0; q < 8; ++q) {
-            acc[q] = 0;
-            accd[q] = 0.0;
-        }
-        for (int k0 = 0; k0 < nb; k0 += 32) {
-            const int k = k0 + lane;
-            const int s = k < nb ? slot_of[yr[k] - r0] : -1;
-            unsigned m = __ballot_sync(0xffffffffu, s >= 0);
-            while (m) {
-                // stage up to kStage matched row blocks
-                int rows[kStage];
-                int nst = 0;
-#pragma unroll
-                for (int g = 0; g < kStage; ++g) {
-                    rows[g] = -1;
-                    if (m) {
-                        const int src = __ffs(m) - 1;
-                        m &= m - 1;
-                        rows[g] = src;
-                        ++nst;
-                    }
+        int k0 = -32, at = -1;   // the 32 rows being staged; a lane's tile C[r, a] among them
+        unsigned m = 0;          // those not staged yet
+        // the next up to kStage matched row blocks: their number (0: none left), and this thread's pieces
+        double2 v[kLoads];
+        auto next = [&] {
+            while (!m) {
+                k0 += 32;
+                if (k0 >= nb) return 0;
+                at = -1;
+                if (k0 + lane < nb) {
+                    const int r = yr[k0 + lane], sl = slot_of[r - r0];
+                    if (sl >= 0) at = r * cap + sl;
                 }
+                m = __ballot_sync(0xffffffffu, at >= 0);
+            }
+            int n = 0, tile[kStage], row[kStage];
 #pragma unroll
-                for (int g = 0; g < kStage; ++g) {
-                    if (g >= nst) break;
-                    const int ss = __shfl_sync(0xffffffffu, s, rows[g]);
-                    const int kk = k0 + rows[g];
-                    const int r = yr[kk];
-                    const double2* cs = (const double2*)(c_val + ((size_t)r * cap + ss) * kTileVals);
-                    const double2* ys = (const double2*)(y_val + ((size_t)b * capY + kk) * kTileVals);
-                    double2* bc = (double2*)(buf + (size_t)g * 2 * kTileVals);
-                    double2* by = (double2*)(buf + (size_t)g * 2 * kTileVals + kTileVals);
-                    for (int v = lane; v < kPerTile; v += 32) {
-                        bc[v] = cs[v];
-                        by[v] = ys[v];
-                    }
-                }
-                __syncwarp();
-                for (int g = 0; g < nst; ++g) {
-                    const double* bc = buf + (size_t)g * 2 * kTileVals;
-                    const double* by = bc + kTileVals;
-#pragma unroll
-                    for (int q = 0; q < 6; ++q) {
-                        const double c0 = bc[q * 16 + i0], c1 = bc[q * 16 + i0 + 1];
-                        const double y0 = by[q * 16 + j0], y1 = by[q * 16 + j0 + 1];
-                        const double y2 = by[q * 16 + j0 + 2], y3 = by[q * 16 + j0 + 3];
-                        acc[0] += c0 * y0;
-                        acc[1] += c0 * y1;
-                        acc[2] += c0 * y2;
-                        acc[3] += c0 * y3;
-                        acc[4] += c1 * y0;
-                        acc[5] += c1 * y1;
-                        acc[6] += c1 * y2;
-                        acc[7] += c1 * y3;
-                    }
-                }
-                __syncwarp();
+            for (int g = 0; g < kStage; ++g) {
+                const int src = m ? __ffs(m) - 1 : 0;
+                n += m != 0;
+                m &= m - 1;
+                tile[g] = __shfl_sync(0xffffffffu, at, src);
+                row[g] = k0 + src;
             }
 #pragma unroll
-            for (int q = 0; q < 8; ++q) {
-                accd[q] += acc[q];
-                acc[q] = 0;
+            for (int j = 0; j < kLoads; ++j) {
+                const int piece = threadIdx.x + j * kTfWarps * 32, g = piece / (2 * kHalf), q = piece % (2 * kHalf);
+                int t = tile[0], k = row[0];
+#pragma unroll
+                for (int h = 1; h < kStage; ++h)
+                    if (g == h) {
+                        t = tile[h];
+                        k = row[h];
+                    }
+                if (g < n)
+                    v[j] = q < kHalf ? *((const double2*)(c_val + (size_t)t * kTileVals) + q)
+                                     : *((const double2*)(y_val + ((size_t)b * capY + k) * kTileVals) + q - kHalf);
+            }
+            return n;
+        };
+        double sum0 = 0.0, sum1 = 0.0, acc0 = 0.0, acc1 = 0.0;
+        int n = next();
+        while (n) {
+            double2* buf = stage + phase * (kTfStageVals / 2);
+            phase ^= 1;
+#pragma unroll
+            for (int j = 0; j < kLoads; ++j) {
+                const int piece = threadIdx.x + j * kTfWarps * 32;
+                if (piece < n * 2 * kHalf) buf[piece] = v[j];
+            }
+            __syncthreads();   // (the other buffer's readers are past it before anyone writes there again)
+            const bool last = m == 0;   // of these 32 rows
+            const int staged = n;
+            n = next();
+            for (int g = 0; g < staged; ++g) {
+                const double* bc = (const double*)(buf + (size_t)g * 2 * kHalf);
+                const double* by = bc + kTileVals;
+#pragma unroll
+                for (int q = 0; q < 6; ++q) {
+                    const double2 c = *(const double2*)(bc + q * 16 + i0);
+                    const double y = by[q * 16 + j0];
+                    acc0 += c.x * y;
+                    acc1 += c.y * y;
+                }
+            }
+            if (last) {
+                sum0 += acc0;
+                sum1 += acc1;
+                acc0 = acc1 = 0.0;
             }
         }
         double* o = out + (size_t)tp_out[p] * 256;
-#pragma unroll
-        for (int u = 0; u < 4; ++u) {
-            o[i0 * 16 + j0 + u] = accd[u];
-            o[(i0 + 1) * 16 + j0 + u] = accd[4 + u];
-        }
+        o[i0 * 16 + j0] = sum0;
+        o[(i0 + 1) * 16 + j0] = sum1;
     }
 }
 
@@ -994,9 +999,7 @@ static cudaError_t ensure_attrs() {
     if (dev >= 0 && dev < 64 && g_attr_done[dev]) return cudaSuccess;
     e = cudaFuncSetAttribute(k_ci_small, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kCiSmallSmem);
     if (e != cudaSuccess) return e;
-    e = cudaFuncSetAttribute(k_transform<1>, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024);
-    if (e != cudaSuccess) return e;
-    e = cudaFuncSetAttribute(k_transform<4>, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024);
+    e = cudaFuncSetAttribute(k_transform, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024);
     if (e != cudaSuccess) return e;
     e = cudaFuncSetAttribute(k_transform_tc, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024);
     if (e != cudaSuccess) return e;
@@ -1039,27 +1042,24 @@ cudaError_t launch_xc_rot(Ctx* c) {
     return launch_xc(c, true, 0, c->n_tiles, c->n_occ_tiles);
 }
 
-// CTAs sharing one occupied tile's pairs: what sscf_autotune chose, or enough for
-// 16 (FP64) or 8 (FP32, twice the warps) per SM. FP64 at 343 molecules: four
-// 5.1 + 3.3 ms, 24 3.9 + 2.2, as the SMs share the work more evenly. FP32: 4 per SM
-// 1.39 + 0.99 ms at 997, 8 1.31 + 0.98, 16 1.33 + 0.90; the same at 4096, where
-// the lower limit decides.
+// CTAs sharing one tile's pairs: what sscf_autotune chose, or enough for 32 (FP64) or 8
+// (FP32) per SM. FP64 at 343 molecules: 8 per SM 3.51 + 2.43 ms, 16 3.45 + 2.07, 32
+// 3.19 + 1.95, as the SMs share the work more evenly. FP32: 4 per SM 1.39 + 0.99 ms at
+// 997, 8 1.31 + 0.98, 16 1.33 + 0.90; the same at 4096, where the lower limit decides.
 static int transform_split(const Ctx* c, bool fp64) {
     if (c->tf_split > 0) return c->tf_split;
-    const int per_tile = ((fp64 ? 16 : 8) * c->n_sm + c->n_occ_tiles - 1) / c->n_occ_tiles;
-    return fp64 ? std::min(32, std::max(8, per_tile)) : std::min(16, std::max(4, per_tile));
+    const int per_tile = ((fp64 ? 32 : 8) * c->n_sm + c->n_occ_tiles - 1) / c->n_occ_tiles;
+    return fp64 ? std::min(128, std::max(8, per_tile)) : std::min(16, std::max(4, per_tile));
 }
 
-// (the register budget of sscf_autotune is the FP64 kernel's)
 template <typename T>
 static cudaError_t transform_t(Ctx* c, const int* ptr, const int* bl, const int* outl, void* out) {
     constexpr bool kFP64 = std::is_same<T, double>::value;
     const int split = transform_split(c, kFP64);
     const int grid = c->n_tiles * split;
     if constexpr (kFP64) {
-        const size_t smem = (size_t)kTfWarps * kTfStageVals * sizeof(T) + (size_t)c->max_cl_mol * 2;
-        auto kern = c->tf_regs == 1 ? k_transform<4> : k_transform<1>;
-        kern<<<grid, kTfWarps * 32, smem, c->stream>>>(
+        const size_t smem = (size_t)2 * kTfStageVals * sizeof(T) + (size_t)c->max_cl_mol * 2;
+        k_transform<<<grid, kTfWarps * 32, smem, c->stream>>>(
             split, c->max_cl_mol, c->d_tile_row0, c->cap, c->capY, ptr, bl, outl, c->d_cci_ptr, c->d_cci_row,
             c->d_cci_slot, (const T*)c->d_c_val[c->cur], c->d_y_n, c->d_y_row, (const T*)c->d_y_val, (T*)out);
     } else {
@@ -1075,8 +1075,7 @@ cudaError_t launch_transform_rot(Ctx* c) {
     c->n_launch += 3;
     cudaError_t e = ensure_attrs();
     if (e != cudaSuccess) return e;
-    if ((size_t)kTfWarps * kTfStageVals * 8 + (size_t)c->max_cl_mol * 2 > 200 * 1024)
-        return cudaErrorInvalidValue;
+    if ((size_t)2 * kTfStageVals * 8 + (size_t)c->max_cl_mol * 2 > 200 * 1024) return cudaErrorInvalidValue;
     if (c->prec == SSCF_FP64) {
         e = transform_t<double>(c, c->d_rot_tp_ptr, c->d_rot_tp_b, c->d_rot_tp_out, c->d_F);
         if (e == cudaSuccess)

@@ -87,7 +87,6 @@ struct Ctx {
     int apply_variant = 0;   // 0 specialised sweep kernels where they apply, 1 generic only,
                              // 2 specialised with one CTA per block
     int tf_split = 0;        // CTAs sharing one occupied tile's pairs in the transform (sscf_autotune; 0: by size)
-    int tf_regs = 0;         // transform register budget: 0 uncut, 1 cut for 4 CTAs per SM (sscf_autotune)
     int n_sm = 152;          // multiprocessors of the context's device
     bool have_guess = false;
     int iteration = 0;
