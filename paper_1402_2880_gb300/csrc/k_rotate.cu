@@ -1211,7 +1211,8 @@ __global__ void __launch_bounds__(apply_threads<T>()) k_apply_colour(SweepArgs a
 //           four pairs of a level in flight. Self blocks, rotations, combination
 //           blocks with few pairs, and everything in FP64 storage, where the FP64
 //           pipe (two lanes per clock and SM) is the bound and slots without a
-//           pair are not to cost anything.
+//           pair are not to cost anything: there a CTA's warps share the panel
+//           and each level's pairs.
 // n = max(MOs of A, MOs of B) is the modulus of the in-block colour; the dense
 // loop exists for every n a pair of groups can have, so blocks of partly filled
 // groups run it as well (their missing MOs are zero columns without pairs).
@@ -1219,7 +1220,7 @@ __global__ void __launch_bounds__(apply_threads<T>()) k_apply_colour(SweepArgs a
 // side in registers, the others staged for the generic kernel): occupied pass
 // at 4096 molecules 68.9 -> 41.9 ms, at 997 9.9 -> 5.3; four passes over all
 // MOs at 512 18.6 -> 5.2; rotations at 4096 14.8 -> 9.6, at 997 3.2 -> 1.7.
-// FP64 at 343 molecules: occupied pass 14.5 -> 12.7, rotations 2.3 -> 1.4.
+// FP64 at 343 molecules: occupied pass 14.5 -> 10.4, rotations 2.3 -> 1.5.
 constexpr int kFullCH = 32;                  // row blocks per word of the bits of rows with work
 constexpr int kFullBatch = 8;                // 16-byte pieces of a tile per lane and run of 32 row pairs, all in flight
 // runs a CTA takes at least: one per warp, or two where a launch could have more than kWsManyRuns
@@ -1241,9 +1242,12 @@ template <typename T, int MODE, bool ALL> struct WarpShape {
     static constexpr int ntb = MODE == 0 ? 1 : nta;
     static constexpr int nmax = ALL ? 48 : 32;                 // largest modulus
     static constexpr int gstep = ALL ? 6 : 4;                  // MOs per molecule and side
-    // FP64 CTAs are half as large: the pipe is busy with a few warps per SM, and the smaller the
-    // pieces, the more evenly the SMs share it
-    static constexpr int warps = f32 ? 4 : 2, threads = 32 * warps;
+    // warps that share a run: FP32 one; FP64 all four of the CTA, each a quarter of a level's pairs (a
+    // quarter of an SM starts one FP64 instruction of a warp every 64 clocks, busy or not; with a run
+    // per warp a colour of few blocks left most quarters idle: occupied pass at 343 molecules 12.7 ms,
+    // now 10.4; a step's sweeps at 32 0.44 ms, now 0.19)
+    static constexpr int warps = 4, threads = 32 * warps;
+    static constexpr int team = f32 ? 1 : warps, runs = warps / team;   // runs a CTA has in hand
     // order of the CTAs: all shares of a block, then the next block (the long blocks first: the short
     // ones even out the end; FP64 occupied pass at 343 molecules 15.9 -> 12.7 ms, rotations at 4096
     // 9.7 -> 9.2), or the first share of all blocks, then the second (FP32 combinations, whose later
@@ -1263,10 +1267,10 @@ template <typename T, int MODE, bool ALL> struct WarpShape {
     static constexpr int panel = (nta + ntb) * 16 * kWsPad * (int)sizeof(T);
     static constexpr int per_warp = 2 * raw > panel ? 2 * raw : panel;
     static_assert(MODE == 0 || ALL || per_warp >= nta * 16 * 64 * 4, "");
-    static constexpr size_t smem = (size_t)table + (size_t)warps * per_warp;   // + row bits
+    static constexpr size_t smem = (size_t)table + (size_t)runs * per_warp;   // + row bits
     // resident CTAs the register budget is cut for: the dense loop holds 2 n values per row; FP64
     // runs as many as its panels leave room for
-    static constexpr int min_ctas = f32 ? (MODE == 0 ? 6 : (ALL ? 2 : 3)) : (MODE == 0 ? 6 : (ALL ? 2 : 4));
+    static constexpr int min_ctas = f32 ? (MODE == 0 ? 6 : (ALL ? 2 : 3)) : (MODE == 0 ? 6 : (ALL ? 3 : 5));
 };
 
 // 1.0 where |v| >= t, 0.0 below (and for NaN): one compare that writes the
@@ -1372,7 +1376,7 @@ k_apply_warp(SweepArgs a, int p0, int nb, int min_runs) {
     constexpr int kWsWarps = Sh::warps, kWsThreads = Sh::threads;
     constexpr int NTA = Sh::nta, NTB = Sh::ntb;
     extern __shared__ __align__(16) unsigned char smraw[];
-    __shared__ int s_wsum[kWsWarps], s_next;
+    __shared__ int s_wsum[kWsWarps], s_next, s_lvl[Sh::team > 1 ? kMaxSub + 1 : 1];
     if (*a.err & (kErrCapacity | kErrSortSize)) return;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const BlockInfo& info = ((const BlockInfo*)a.blk_info)[p0 + (Sh::by_block ? blockIdx.x / (gridDim.x / nb) : blockIdx.x % nb)];
@@ -1443,6 +1447,8 @@ k_apply_warp(SweepArgs a, int p0, int nb, int min_runs) {
     const int run_lo = share * per, run_hi = min(n_run, run_lo + per);
     if (run_lo >= run_hi) return;
     if (threadIdx.x == 0) s_next = run_lo;
+    if constexpr (Sh::team > 1)
+        for (int l = threadIdx.x; l <= kMaxSub; l += kWsThreads) s_lvl[l] = a.pr_lvl[(size_t)e * (kMaxSub + 1) + l];
     for (int w = wlo; w < whi; ++w) {
         wpre[w] = before;
         before += __popc(bits[w]);
@@ -1491,12 +1497,12 @@ k_apply_warp(SweepArgs a, int p0, int nb, int min_runs) {
         else pair2[q] = make_float2(__uint_as_float(63u << 12), 0.f);
     }
     __syncthreads();
-    T* const mem = (T*)(smraw + Sh::table + (size_t)warp * Sh::per_warp);   // the warp's
+    T* const mem = (T*)(smraw + Sh::table + (size_t)(warp / Sh::team) * Sh::per_warp);   // the run's
     T* const val = (T*)a.out_val;                                           // in place
     // the block's pairs on the panel, in schedule order (lanes hold different rows)
     auto run_list = [&](bool active) {
         // pairs of one level touch different columns: up to four of them in flight
-        if (active) {
+        {
             auto upd = [&](int q, auto width) {
                 constexpr int N = decltype(width)::value;
                 T *px[N], *py[N], xv[N], yv[N], c0[N], c1[N];
@@ -1544,6 +1550,28 @@ k_apply_warp(SweepArgs a, int p0, int nb, int min_runs) {
                 else off = __float_as_uint(pair2[q].x);
                 return off >> 12 & 63u;
             };
+            if constexpr (Sh::team > 1) {   // a level's pairs, a warp's share each
+                for (int l = 0; l < kMaxSub; ++l) {
+                    const int q0 = s_lvl[l], q1 = s_lvl[l + 1], part = (q1 - q0 + Sh::team - 1) / Sh::team;
+                    const int end = min(q1, q0 + (warp + 1) * part);
+                    if (active)
+                        for (int q = q0 + warp * part; q < end;) {
+                            if (q + 4 <= end) {
+                                upd(q, std::integral_constant<int, 4>());
+                                q += 4;
+                            } else if (q + 2 <= end) {
+                                upd(q, std::integral_constant<int, 2>());
+                                q += 2;
+                            } else {
+                                upd(q, std::integral_constant<int, 1>());
+                                q += 1;
+                            }
+                        }
+                    if (q1 > q0) __syncthreads();
+                }
+                return;
+            }
+            if (!active) return;
             for (int q = 0; q < np;) {
                 const unsigned l = level(q);
                 if (level(q + 3) == l) {
@@ -1631,17 +1659,25 @@ k_apply_warp(SweepArgs a, int p0, int nb, int min_runs) {
         return o;
     };
     auto grab = [&]() { return lane == 0 ? atomicAdd(&s_next, 1) : 0; };
-    int run = __shfl_sync(0xffffffffu, grab(), 0);
+    int run = run_lo;
+    if constexpr (Sh::team == 1) run = __shfl_sync(0xffffffffu, grab(), 0);
     if (run >= run_hi) return;
     if (MODE == 0 || !dense) {
         T* const pq = mem + kV * qp * kWsPad + qe;
-        constexpr int kTiles = F32 ? NTA + NTB : 2;   // tiles in flight
+        // tiles in flight; a team's warps move different tiles
+        constexpr int kTiles = F32 ? NTA + NTB : 1;
+        const int t_lo = Sh::team > 1 ? warp : 0;
+        auto all_wait = [] {
+            if constexpr (Sh::team > 1) __syncthreads();
+            else __syncwarp();
+        };
         while (run < run_hi) {
             const Row r = look_up(run);
-            const int grabbed = grab();
+            int grabbed = run + 1;
+            if constexpr (Sh::team == 1) grabbed = grab();
             const int take = min(32, n_ent - 32 * run);
 #pragma unroll
-            for (int t0 = 0; t0 < NTA + NTB; t0 += kTiles) {
+            for (int t0 = t_lo; t0 < NTA + NTB; t0 += kTiles * Sh::team) {
                 V v[kTiles][kTimes];
 #pragma unroll
                 for (int u = 0; u < kTimes; ++u) {
@@ -1661,15 +1697,15 @@ k_apply_warp(SweepArgs a, int p0, int nb, int min_runs) {
                         for (int w = 0; w < kV; ++w)
                             pq[((t0 + t) * 16 + w) * kWsPad + kAt * u] = ((const T*)&v[t][u])[w];
             }
-            __syncwarp();
+            all_wait();
             run_list(lane < take);
-            __syncwarp();
+            all_wait();
 #pragma unroll
             for (int u = 0; u < kTimes; ++u) {
                 const Row o = row_from(r, kAt * u + qe);
                 if (kAt * u + qe >= take) continue;
 #pragma unroll
-                for (int t = 0; t < NTA + NTB; ++t) {
+                for (int t = t_lo; t < NTA + NTB; t += Sh::team) {
                     if (!touched(t)) continue;
                     V f;
                     bool nz = false;
@@ -1684,8 +1720,8 @@ k_apply_warp(SweepArgs a, int p0, int nb, int min_runs) {
                     if (nz) raise(o, t, tile);
                 }
             }
-            __syncwarp();
-            run = __shfl_sync(0xffffffffu, grabbed, 0);
+            all_wait();
+            run = Sh::team > 1 ? grabbed : __shfl_sync(0xffffffffu, grabbed, 0);
         }
         return;
     }
@@ -2139,7 +2175,7 @@ static cudaError_t apply_warp_t(Ctx* c, SweepArgs& a, int col_lo, int col_hi) {
         const int nb = ptr[col + 1] - ptr[col];
         if (nb == 0) continue;
         const int runs = (kAoPerMol / Sh::halves * c->max_cl_mol + 31) / 32;   // at most, of a block
-        const int per = MODE == 1 && (long long)nb * runs > kWsManyRuns * full ? 2 * Sh::warps : Sh::warps;
+        const int per = MODE == 1 && (long long)nb * runs > kWsManyRuns * full ? 2 * Sh::runs : Sh::runs;
         int gx = (runs + per - 1) / per;
         if (MODE == 0) gx = std::min(gx, (kWsRotWaves * full + nb - 1) / nb);
         if (c->apply_variant == 2) gx = 1;
