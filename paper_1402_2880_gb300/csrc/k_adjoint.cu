@@ -93,17 +93,19 @@ __device__ __forceinline__ int first_at(const int* __restrict__ list, int n, int
 // Z's values. A CTA makes the 48 x 32 outputs of one MO group's molecules (48 AO
 // rows) and one out group A (two tiles), over the in groups B adjacent to A that
 // any of the rows holds: per B it stages the rows' 48 x 32 values and the 32 x 32
-// block F[B, A], so that a block of F is read once per group of molecules, and
+// block F[B, A] (loading the next B's meanwhile), so that a block of F is read once per group of molecules, and
 // each of 96 threads keeps 4 x 4 outputs. Terms are added in the order of the
 // row's tiles and of the MOs inside a tile, one product at a time; a tile that a
 // row does not hold contributes zeros. (One warp per row and out tile read a
 // block of F for six rows of work and looked it up by a binary search:
-// 27.6 ms at 2000 molecules; now 6.6.)
+// 27.6 ms at 2000 molecules; 6.6 with scalar multiply-adds, F staged value by
+// value and loads not overlapped; now 5.6.)
 constexpr int kZThreads = 96;
 constexpr int kZRows = kMaxMolPerGroup * kAoPerMol;   // 48
 constexpr int kZStride = kZRows + 4;                  // values per staged MO (16-byte aligned, bank-spread)
+constexpr int kFStride = 36;                          // values per staged MO of B
 template <typename T> __host__ __device__ constexpr size_t zmul_smem(int max_nb) {
-    return (size_t)32 * kZStride * sizeof(T) + (size_t)32 * 32 * sizeof(T) +
+    return (size_t)32 * kZStride * sizeof(T) + (size_t)32 * kFStride * sizeof(T) +
            (size_t)max_nb * kMaxMolPerGroup * sizeof(int2) + (size_t)max_nb * sizeof(int);
 }
 template <typename T>
@@ -116,8 +118,8 @@ k_zmul(int g_lo, int max_nb, int cap, const int* __restrict__ group_cl, const in
        const T* __restrict__ F, const int* __restrict__ z_nt, const int* __restrict__ z_tile, T* __restrict__ z_val) {
     extern __shared__ __align__(16) unsigned char smraw[];
     T* sc = (T*)smraw;                                // [32 MOs of B][kZStride]: the rows' values
-    T* sf = sc + 32 * kZStride;                       // [32 MOs of B][32 MOs of A]
-    int2* slot = (int2*)(sf + 32 * 32);               // [neighbour of A][molecule]: slots of B's two tiles, or -1
+    T* sf = sc + 32 * kZStride;                       // [32 MOs of B][kFStride]: F[B, A], 32 MOs of A
+    int2* slot = (int2*)(sf + 32 * kFStride);         // [neighbour of A][molecule]: slots of B's two tiles, or -1
     int* any = (int*)(slot + (size_t)max_nb * kMaxMolPerGroup);   // [neighbour of A]: some row holds a tile of B
     __shared__ int s_mol[kMaxMolPerGroup], s_z[kMaxMolPerGroup];
     const int G = g_lo + blockIdx.y, cl = group_cl[G], A = cl_g0[cl] + blockIdx.x;
@@ -162,55 +164,95 @@ k_zmul(int g_lo, int max_nb, int cap, const int* __restrict__ group_cl, const in
     for (int i = 0; i < 4; ++i)
 #pragma unroll
         for (int j = 0; j < 4; ++j) acc[i][j] = (T)0;
+    // 16-byte pieces: of the rows along the MOs, turned to [MO][row], and of F[B, A], whose tile pairs
+    // are stored for blocks (lower group, upper group), inside a group for positions a <= b; turned
+    // when stored the other way. The next neighbour's are loaded during this one's products.
     using V = typename std::conditional<sizeof(T) == 4, float4, double2>::type;
-    constexpr int kV = 16 / (int)sizeof(T);
-    for (int k = 0; k < nb; ++k) {
-        if (!any[k]) continue;
-        const int e = e0 + k, B = gnb_col[e];
-        __syncthreads();   // the buffers are free
-        // rows: 16-byte pieces along the MOs, turned to [MO][row]
-        constexpr int kPer = 16 / kV;   // pieces per tile row
-        for (int i = threadIdx.x; i < kZRows * 2 * kPer; i += kZThreads) {
+    constexpr int kV = 16 / (int)sizeof(T), kPer = 16 / kV;   // values of a piece, pieces per tile row
+    constexpr int kC = kZRows * 2 * kPer / kZThreads, kF = (4 * 16 * kPer + kZThreads - 1) / kZThreads;
+    static_assert(kC * kZThreads == kZRows * 2 * kPer, "");
+    V vc[kC], vf[kF];
+    int turned = 0;   // bit pB * 2 + pA: the tile pair is stored as [A][B]
+    auto load = [&](int k) {
+        const int e = e0 + k, B = gnb_col[e], eb = B <= A ? gnb_rev[e] : e;   // entry (min, max)
+        const int ntB = group_not[B];
+        turned = B < A ? 0 : B == A ? 4 : 15;   // (inside a group [pB][pA] is stored for pB <= pA)
+#pragma unroll
+        for (int h = 0; h < kC; ++h) {
+            const int i = threadIdx.x + h * kZThreads;
             const int row = i / (2 * kPer), rem = i - row * (2 * kPer), t = rem / kPer, p = rem - t * kPer;
             const int q = row / kAoPerMol;
             const int s = q < nm ? (t ? slot[k * kMaxMolPerGroup + q].y : slot[k * kMaxMolPerGroup + q].x) : -1;
-            T v[kV];
-#pragma unroll
-            for (int u = 0; u < kV; ++u) v[u] = (T)0;
+            vc[h] = V{};
             if (s >= 0)
-                *(V*)v = *(const V*)(c_val + ((size_t)s_mol[q] * cap + s) * kTileVals + (row - q * kAoPerMol) * kTileW +
-                                     p * kV);
-#pragma unroll
-            for (int u = 0; u < kV; ++u) sc[(t * 16 + p * kV + u) * kZStride + row] = v[u];
+                vc[h] = *(const V*)(c_val + ((size_t)s_mol[q] * cap + s) * kTileVals + (row - q * kAoPerMol) * kTileW +
+                                    p * kV);
         }
-        // F[B, A]: tile pairs are stored for blocks (lower group, upper group), inside a group for
-        // positions a <= b; transposed when stored the other way
-        const int eb = B <= A ? gnb_rev[e] : e;   // entry (min, max)
-        for (int i = threadIdx.x; i < 32 * 32; i += kZThreads) {
-            const int ib = i >> 5, ja = i & 31;           // MO of B, MO of A
-            const int pB = ib >> 4, pA = ja >> 4;
-            T v = (T)0;
-            if (pB < group_not[B] && pA < ntA) {
-                const bool straight = B < A || (B == A && pB <= pA);   // stored as [B][A]
-                const int tp = straight ? blk_tp[(size_t)eb * 9 + pB * 3 + pA] : blk_tp[(size_t)eb * 9 + pA * 3 + pB];
-                const T* f = F + (size_t)tp * 256;
-                v = straight ? f[(ib & 15) * 16 + (ja & 15)] : f[(ja & 15) * 16 + (ib & 15)];
+#pragma unroll
+        for (int h = 0; h < kF; ++h) {
+            const int i = threadIdx.x + h * kZThreads, t = i / (16 * kPer), piece = i - t * (16 * kPer);
+            const int pB = t >> 1, pA = t & 1;
+            vf[h] = V{};
+            if (t < 4 && pB < ntB && pA < ntA) {
+                const int tp = blk_tp[(size_t)eb * 9 + ((turned >> (pB * 2 + pA)) & 1 ? pA * 3 + pB : pB * 3 + pA)];
+                vf[h] = *((const V*)(F + (size_t)tp * 256) + piece);
             }
-            sf[i] = v;
+        }
+    };
+    auto next = [&](int k) {
+        while (k < nb && !any[k]) ++k;
+        return k;
+    };
+    int k = next(0);
+    if (k < nb) load(k);
+    while (k < nb) {
+        __syncthreads();   // the buffers are free
+#pragma unroll
+        for (int h = 0; h < kC; ++h) {
+            const int i = threadIdx.x + h * kZThreads;
+            const int row = i / (2 * kPer), rem = i - row * (2 * kPer), t = rem / kPer, p = rem - t * kPer;
+#pragma unroll
+            for (int u = 0; u < kV; ++u) sc[(t * 16 + p * kV + u) * kZStride + row] = ((const T*)&vc[h])[u];
+        }
+#pragma unroll
+        for (int h = 0; h < kF; ++h) {
+            const int i = threadIdx.x + h * kZThreads, t = i / (16 * kPer), piece = i - t * (16 * kPer);
+            const int r = piece / kPer, c = (piece - r * kPer) * kV, pB = t >> 1, pA = t & 1;
+            if (t >= 4) continue;
+            if ((turned >> t) & 1) {
+#pragma unroll
+                for (int u = 0; u < kV; ++u)
+                    sf[(pB * 16 + c + u) * kFStride + pA * 16 + r] = ((const T*)&vf[h])[u];
+            } else {
+                *(V*)(sf + (pB * 16 + r) * kFStride + pA * 16 + c) = vf[h];
+            }
         }
         __syncthreads();
+        k = next(k + 1);
+        if (k < nb) load(k);
 #pragma unroll 8
         for (int q = 0; q < 32; ++q) {
             T c[4], f[4];
 #pragma unroll
             for (int u = 0; u < 4; u += kV) {
                 *(V*)(c + u) = *(const V*)(sc + q * kZStride + 4 * ti + u);
-                *(V*)(f + u) = *(const V*)(sf + q * 32 + 4 * tj + u);
+                *(V*)(f + u) = *(const V*)(sf + q * kFStride + 4 * tj + u);
             }
 #pragma unroll
-            for (int i = 0; i < 4; ++i)
+            for (int i = 0; i < 4; ++i) {
+                if constexpr (sizeof(T) == 4) {
 #pragma unroll
-                for (int j = 0; j < 4; ++j) acc[i][j] += c[i] * f[j];
+                    for (int j = 0; j < 4; j += 2) {
+                        const float2 v = __ffma2_rn(make_float2(c[i], c[i]), make_float2(f[j], f[j + 1]),
+                                                    make_float2(acc[i][j], acc[i][j + 1]));
+                        acc[i][j] = v.x;
+                        acc[i][j + 1] = v.y;
+                    }
+                } else {
+#pragma unroll
+                    for (int j = 0; j < 4; ++j) acc[i][j] += c[i] * f[j];
+                }
+            }
         }
     }
 #pragma unroll
