@@ -201,6 +201,8 @@ __global__ void __launch_bounds__(1024) k_rot_select_small(int last_shift, int n
     }
     for (int i = threadIdx.x; i < 256; i += blockDim.x) s_h[i] = 0u;
     __syncthreads();
+    // tau <= |F| and 0 < |F|, compared as keys (64 clocks of an SM quarter for an FP64 compare)
+    const unsigned long long k_inf = dkey(INFINITY), k_tau = tau > 0.0 ? dkey(tau) : 1ull;
     // every candidate key, a block per warp or, of fewer blocks than warps, several warps per block
     const int w_per = n_gnb < 32 ? 32 / n_gnb : 1, sub = warp % w_per;
     auto each = [&](auto f) {
@@ -211,16 +213,15 @@ __global__ void __launch_bounds__(1024) k_rot_select_small(int last_shift, int n
             for (int p = lane + 32 * sub; p < no * 16; p += 32 * w_per) {
                 const int i = p >> 4, j = p & 15;   // a block has one virtual tile: nvt = 1, nv <= 16
                 if (j >= nv) continue;
-                const double v = fabs((double)fe[(size_t)(i >> 4) * nvt * 256 + (i & 15) * 16 + j]);
-                f(v, v >= tau && v > 0.0);
+                const unsigned long long k = dkey(fabs((double)fe[(size_t)(i >> 4) * nvt * 256 + (i & 15) * 16 + j]));
+                f(k, k >= k_tau && k <= k_inf);
             }
         }
     };
     unsigned cnt = 0;
     unsigned long long mx = 0ull;
-    each([&](double v, bool in) {
-        const unsigned long long k = dkey(v);
-        if (k > mx && v == v) mx = k;
+    each([&](unsigned long long k, bool in) {
+        if (k > mx && k <= k_inf) mx = k;
         cnt += in;
     });
     cnt = __reduce_add_sync(0xffffffffu, cnt);
@@ -236,8 +237,7 @@ __global__ void __launch_bounds__(1024) k_rot_select_small(int last_shift, int n
     unsigned long long prefix = 0ull, mask = 0ull, rank = kmax;
     if (s_cnt > kmax) {
         for (int shift = 56; shift >= last_shift; shift -= 8) {
-            each([&](double v, bool in) {
-                const unsigned long long k = dkey(v);
+            each([&](unsigned long long k, bool in) {
                 if (in && (k & mask) == prefix) atomicAdd(&s_h[k >> shift & 255ull], 1u);
             });
             __syncthreads();

@@ -5,8 +5,10 @@
 
 namespace sscf {
 
-// atoms of a share (at least, so that small clusters do not get empty warps) and shares (at most)
-constexpr int kShareAtoms = 64;
+// atoms of a share (at least) and shares (at most). A warp's FP64 instructions take 64 clocks each
+// whatever else its quarter of an SM does, so small clusters are spread thin: 96 atoms, shares of
+// 64, 32, 16: 32, 22, 12 us; 648 atoms 62, 44, 40 us with the sum of the shares (8: 43).
+constexpr int kShareAtoms = 16;
 constexpr int kMaxShares = 64;
 
 // the atoms [b0, b1) of this CTA's share of [lo, hi)
