@@ -2,7 +2,6 @@
 // the DFTB Hamiltonian of Eq. (H_dftb2) and the per-molecule initial guess.
 #include <math.h>
 
-#include "shares.h"
 #include "sscf_internal.h"
 
 namespace sscf {
@@ -148,28 +147,45 @@ k_gamma_mixed(int n, const double* __restrict__ xyz, const int* __restrict__ spe
     if (warp == 0 && a0 + lane < n) Q[a0 + lane] = acc;
 }
 
-// FP64: one warp per 32 atoms a and share y of the atoms b; the shares are
-// summed in order by k_sum_shares. The FP64 pipe (2 lanes per clock and SM)
-// bounds it: every SM has to take part, and the term is a product with
-// 1/sqrt instead of a square root and a division (648 atoms: 1.17 -> 0.04 ms).
-__global__ void __launch_bounds__(32) k_gamma_fp64(int n, const double* __restrict__ xyz,
-                                                   const int* __restrict__ species, const int* __restrict__ atom_lo,
-                                                   const int* __restrict__ atom_hi, const double* __restrict__ dq,
-                                                   double invU0, double invU1, double* __restrict__ part) {
-    const int a0 = blockIdx.x * 32, a = min(a0 + (int)threadIdx.x, n - 1);
-    const double x = xyz[3 * a], y = xyz[3 * a + 1], z = xyz[3 * a + 2];
+// FP64, summed over the same tiles in the same order. A quarter of an SM starts one
+// FP64 instruction of a warp every 64 clocks, and a term takes about 30 of them: a
+// CTA's four warps make the terms of 8 atoms with a tile, 32 at a time each,
+// and 8 lanes add them up. (A thread per atom for everything, 256 atoms per CTA:
+// 1.17 ms at 648 atoms. With the charge kernels around it 1.85 ms at 1029, now 0.15;
+// shares of the sum in any order 0.07, but an SCF that does not settle turns a
+// last bit into another result.)
+constexpr int kGamma64Atoms = 8;
+__global__ void __launch_bounds__(128) k_gamma_fp64(int n, const double* __restrict__ xyz,
+                                                    const int* __restrict__ species, const int* __restrict__ atom_lo,
+                                                    const int* __restrict__ atom_hi, const double* __restrict__ dq,
+                                                    double invU0, double invU1, double* __restrict__ Q) {
+    __shared__ double s_t[kGammaTile][kGamma64Atoms + 1];
+    const int at = threadIdx.x & (kGamma64Atoms - 1), slot = threadIdx.x / kGamma64Atoms, slots = 128 / kGamma64Atoms;
+    const int a0 = blockIdx.x * kGamma64Atoms, a = min(a0 + at, n - 1);
+    const double xa[3] = {xyz[3 * a], xyz[3 * a + 1], xyz[3 * a + 2]};
     const double ia = species[a] == 0 ? invU0 : invU1;
     const int lo = atom_lo[a], hi = atom_hi[a];
-    int b0, b1;
-    share_range(atom_lo[a0], atom_hi[min(a0 + 31, n - 1)], b0, b1);
+    const int blo = atom_lo[a0 & ~(kGammaTile - 1)], bhi = atom_hi[min(a0 + kGamma64Atoms - 1, n - 1)];
     double acc = 0.0;
-    for (int b = b0; b < b1; ++b) {
-        const double dx = xyz[3 * b] - x, dy = xyz[3 * b + 1] - y, dz = xyz[3 * b + 2] - z;
-        const double h = 0.5 * (ia + (species[b] == 0 ? invU0 : invU1));
-        const double term = dq[b] * rsqrt(dx * dx + dy * dy + dz * dz + h * h);
-        if (b >= lo && b < hi) acc += term;
+    for (int b0 = blo; b0 < bhi; b0 += kGammaTile) {
+        const int t_lo = max(0, lo - b0), t_hi = min(kGammaTile, hi - b0);
+        for (int t = slot; t < kGammaTile; t += slots) {
+            if (t < t_lo || t >= t_hi) continue;
+            const int b = b0 + t;
+            const double dx = xyz[3 * b] - xa[0], dy = xyz[3 * b + 1] - xa[1], dz = xyz[3 * b + 2] - xa[2];
+            const double d2 = dx * dx + dy * dy + dz * dz;
+            const double h = 0.5 * (ia + (species[b] == 0 ? invU0 : invU1));
+            s_t[t][at] = dq[b] / sqrt(d2 + h * h);
+        }
+        __syncthreads();
+        if (threadIdx.x < kGamma64Atoms) {
+            double part = 0.0;
+            for (int t = t_lo; t < t_hi; ++t) part += s_t[t][at];
+            acc += part;
+        }
+        __syncthreads();
     }
-    if (a0 + (int)threadIdx.x < n) part[(size_t)blockIdx.y * n + a] = acc;
+    if (threadIdx.x < kGamma64Atoms && a0 + at < n) Q[a0 + at] = acc;
 }
 
 // H = H0 + 1/2 S (Q_a + Q_b) on every molecule-pair block (Eq. H_dftb2);
@@ -420,17 +436,13 @@ cudaError_t launch_sk_blocks(Ctx* c) {
 
 cudaError_t launch_gamma(Ctx* c, const double* dq, double* Q) {
     const double i0 = 1.0 / c->prm.U[0], i1 = 1.0 / c->prm.U[1];
-    const int blocks = (c->n_atoms + 31) / 32;
-    if (c->prec == SSCF_FP64) {
-        k_gamma_fp64<<<dim3(blocks, c->n_shares), 32, 0, c->stream>>>(c->n_atoms, c->d_xyz, c->d_species, c->d_atom_lo,
-                                                                      c->d_atom_hi, dq, i0, i1, c->d_share);
-        k_sum_shares<<<(c->n_atoms + 127) / 128, 128, 0, c->stream>>>(c->n_atoms, c->n_shares, c->d_share, Q);
-        c->n_launch += 2;
-    } else {
-        k_gamma_mixed<<<blocks, 32 * kGammaWarps, 0, c->stream>>>(c->n_atoms, c->d_xyz, c->d_species, c->d_atom_lo,
-                                                                  c->d_atom_hi, dq, i0, i1, Q);
-        c->n_launch += 1;
-    }
+    c->n_launch += 1;
+    if (c->prec == SSCF_FP64)
+        k_gamma_fp64<<<(c->n_atoms + kGamma64Atoms - 1) / kGamma64Atoms, 128, 0, c->stream>>>(
+            c->n_atoms, c->d_xyz, c->d_species, c->d_atom_lo, c->d_atom_hi, dq, i0, i1, Q);
+    else
+        k_gamma_mixed<<<(c->n_atoms + 31) / 32, 32 * kGammaWarps, 0, c->stream>>>(
+            c->n_atoms, c->d_xyz, c->d_species, c->d_atom_lo, c->d_atom_hi, dq, i0, i1, Q);
     return cudaGetLastError();
 }
 

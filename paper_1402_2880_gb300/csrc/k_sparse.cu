@@ -721,12 +721,6 @@ __device__ __forceinline__ void sum_add(float2& s, float v, float& lost) {
 // The sums of a pair's 36 products over its 32 lanes: lane u sums product u (32
 // entries, from entry u on around: no bank conflicts) and four entries of one of
 // the last four products, which the eight lanes that share it then add up.
-__device__ __forceinline__ void pair_sums(const double* acc, int lane, double& p0, double& p1) {
-    const double *row0 = acc + lane * 32, *row1 = acc + (32 + (lane >> 3)) * 32 + 4 * (lane & 7);
-    p0 = p1 = 0.0;
-    for (int j = 0; j < 32; ++j) p0 += row0[(j + lane) & 31];
-    for (int j = 0; j < 4; ++j) p1 += row1[j];
-}
 __device__ __forceinline__ void pair_sums(const float2* acc, int lane, double& p0, double& p1) {
     const float2 *row0 = acc + lane * 32, *row1 = acc + (32 + (lane >> 3)) * 32 + 4 * (lane & 7);
     Sum3 s0 = {0.f, 0.f, 0.f}, s1 = {0.f, 0.f, 0.f};
@@ -872,61 +866,109 @@ k_density(int n_occ_tiles, int map_n, const int* __restrict__ mol_ot0, int cap, 
         }
         flush(acc, n_part++);
         __syncwarp();
-        double p[2];
-        pair_sums((const L*)wsum, lane, p[0], p[1]);
-        if constexpr (kSplit) {
-            unsigned any = 0;
-#pragma unroll
-            for (int u = 0; u < 18; ++u) any |= *(const unsigned*)&low[u] & 0x7fff7fffu;
-            if (__any_sync(0xffffffffu, any != 0)) {   // the third parts, in the same way
-                __syncwarp();
-                float2* f = (float2*)wsum + lane;
-#pragma unroll
-                for (int u = 0; u < 36; ++u)
-                    f[u * 32] = make_float2(u & 1 ? __high2float(low[u / 2]) : __low2float(low[u / 2]), 0.f);
-                __syncwarp();
-                double l0, l1;
-                pair_sums((const L*)wsum, lane, l0, l1);
-                p[0] += l0;
-                p[1] += l1;
-            }
-        }
-#pragma unroll
-        for (int off = 4; off > 0; off >>= 1) p[1] += __shfl_xor_sync(0xffffffffu, p[1], off);
-        __syncwarp();
-        // the products weighted by S (36) and by H0 (36) back to shared memory, then four lanes
-        // each for the sums of P o S over the atoms of m and of n (AOs: O s, p, p, p, then H1 s,
-        // H2 s) and of P o H0
-        const bool self = n == m;
-        const int er = self ? e : mp_rev[e];
-#pragma unroll
-        for (int i = 0; i < 2; ++i) {
-            if (i && (lane & 7)) break;
-            const int u = i ? 32 + (lane >> 3) : lane;
-            const double P = 2.0 * p[i];
-            if (P_out) {
-                P_out[(size_t)e * 36 + u] = P;
+        if constexpr (!kSplit) {
+            // lane u < 36 adds up product u over the 32 lanes (rotated start: no bank conflicts) and
+            // weights it by S and H0; then row sums of P o S by the atoms of m, column sums by the atoms
+            // of n (AOs: O s, p, p, p, then H1 s, H2 s), and sum P o H0 (in FP64 storage the order of the
+            // sums is kept: an SCF that does not settle turns a last bit into another result)
+            const bool self = n == m;
+            const int er = self ? e : mp_rev[e];
+            double qr[3] = {0, 0, 0}, qc[3] = {0, 0, 0}, eb = 0.0;
+            for (int u = lane; u < 36; u += 32) {
+                const double* row = wsum + u * 32;
+                double v = 0.0;
+                for (int j = 0; j < 32; ++j) v += row[(j + lane) & 31];
+                const double P = 2.0 * v;
                 const int k = u / 6, l = u - 6 * k;   // AO of m, AO of n
-                if (!self) P_out[(size_t)er * 36 + l * 6 + k] = P;
+                if (P_out) {
+                    P_out[(size_t)e * 36 + u] = P;
+                    if (!self) P_out[(size_t)er * 36 + l * 6 + k] = P;
+                }
+                const double pq = P * Sb[(size_t)e * 36 + u];
+                qr[0] += k < 4 ? pq : 0.0;
+                qr[1] += k == 4 ? pq : 0.0;
+                qr[2] += k == 5 ? pq : 0.0;
+                qc[0] += l < 4 ? pq : 0.0;
+                qc[1] += l == 4 ? pq : 0.0;
+                qc[2] += l == 5 ? pq : 0.0;
+                eb += P * H0b[(size_t)e * 36 + u];
             }
-            wsum[u] = P * Sb[(size_t)e * 36 + u];
-            wsum[36 + u] = P * H0b[(size_t)e * 36 + u];
-        }
-        __syncwarp();
-        if (lane < 28) {
-            const double* w9 = wsum + (sum_id == 6 ? 36 : 0) + 9 * (lane & 3);
-            double v = 0.0;
 #pragma unroll
-            for (int j = 0; j < 9; ++j) v += (take >> j) & 1 ? w9[j] : 0.0;
-            v += __shfl_xor_sync(0x0fffffffu, v, 1);
-            v += __shfl_xor_sync(0x0fffffffu, v, 2);
-            if ((lane & 3) == 0) {
-                double* out = (double*)dpart;   // per entry: atoms O, H1, H2 and the energy
-                if (sum_id < 3 || sum_id == 6) out[4 * (size_t)e + min(sum_id, 3)] = v;
-                if (sum_id >= 3 && !self) out[4 * (size_t)er + sum_id - 3] = v;
+            for (int off = 16; off > 0; off >>= 1) {
+#pragma unroll
+                for (int i = 0; i < 3; ++i) {
+                    qr[i] += __shfl_xor_sync(0xffffffffu, qr[i], off);
+                    qc[i] += __shfl_xor_sync(0xffffffffu, qc[i], off);
+                }
+                eb += __shfl_xor_sync(0xffffffffu, eb, off);
             }
+            __syncwarp();
+            if (lane == 0) {
+                dpart[2 * (size_t)e] = make_double2(qr[0], qr[1]);
+                dpart[2 * (size_t)e + 1] = make_double2(qr[2], eb);
+                if (!self) {
+                    dpart[2 * (size_t)er] = make_double2(qc[0], qc[1]);
+                    dpart[2 * (size_t)er + 1] = make_double2(qc[2], eb);
+                }
+            }
+            continue;
+        } else {
+            double p[2];
+            pair_sums((const float2*)wsum, lane, p[0], p[1]);
+            {
+                unsigned any = 0;
+#pragma unroll
+                for (int u = 0; u < 18; ++u) any |= *(const unsigned*)&low[u] & 0x7fff7fffu;
+                if (__any_sync(0xffffffffu, any != 0)) {   // the third parts, in the same way
+                    __syncwarp();
+                    float2* f = (float2*)wsum + lane;
+#pragma unroll
+                    for (int u = 0; u < 36; ++u)
+                        f[u * 32] = make_float2(u & 1 ? __high2float(low[u / 2]) : __low2float(low[u / 2]), 0.f);
+                    __syncwarp();
+                    double l0, l1;
+                    pair_sums((const float2*)wsum, lane, l0, l1);
+                    p[0] += l0;
+                    p[1] += l1;
+                }
+            }
+#pragma unroll
+            for (int off = 4; off > 0; off >>= 1) p[1] += __shfl_xor_sync(0xffffffffu, p[1], off);
+            __syncwarp();
+            // the products weighted by S (36) and by H0 (36) back to shared memory, then four lanes
+            // each for the sums of P o S over the atoms of m and of n (AOs: O s, p, p, p, then H1 s,
+            // H2 s) and of P o H0
+            const bool self = n == m;
+            const int er = self ? e : mp_rev[e];
+#pragma unroll
+            for (int i = 0; i < 2; ++i) {
+                if (i && (lane & 7)) break;
+                const int u = i ? 32 + (lane >> 3) : lane;
+                const double P = 2.0 * p[i];
+                if (P_out) {
+                    P_out[(size_t)e * 36 + u] = P;
+                    const int k = u / 6, l = u - 6 * k;   // AO of m, AO of n
+                    if (!self) P_out[(size_t)er * 36 + l * 6 + k] = P;
+                }
+                wsum[u] = P * Sb[(size_t)e * 36 + u];
+                wsum[36 + u] = P * H0b[(size_t)e * 36 + u];
+            }
+            __syncwarp();
+            if (lane < 28) {
+                const double* w9 = wsum + (sum_id == 6 ? 36 : 0) + 9 * (lane & 3);
+                double v = 0.0;
+#pragma unroll
+                for (int j = 0; j < 9; ++j) v += (take >> j) & 1 ? w9[j] : 0.0;
+                v += __shfl_xor_sync(0x0fffffffu, v, 1);
+                v += __shfl_xor_sync(0x0fffffffu, v, 2);
+                if ((lane & 3) == 0) {
+                    double* out = (double*)dpart;   // per entry: atoms O, H1, H2 and the energy
+                    if (sum_id < 3 || sum_id == 6) out[4 * (size_t)e + min(sum_id, 3)] = v;
+                    if (sum_id >= 3 && !self) out[4 * (size_t)er + sum_id - 3] = v;
+                }
+            }
+            __syncwarp();
         }
-        __syncwarp();
     }
 }
 

@@ -6,8 +6,8 @@
 namespace sscf {
 
 // atoms of a share (at least) and shares (at most). A warp's FP64 instructions take 64 clocks each
-// whatever else its quarter of an SM does, so small clusters are spread thin: 96 atoms, shares of
-// 64, 32, 16: 32, 22, 12 us; 648 atoms 62, 44, 40 us with the sum of the shares (8: 43).
+// whatever else its quarter of an SM does, so small clusters are spread thin (648 atoms, shares of 64
+// and of 16: 48 and 21 us)
 constexpr int kShareAtoms = 16;
 constexpr int kMaxShares = 64;
 
@@ -16,15 +16,6 @@ __device__ __forceinline__ void share_range(int lo, int hi, int& b0, int& b1) {
     const int per = (hi - lo + (int)gridDim.y - 1) / (int)gridDim.y;
     b0 = min(hi, lo + (int)blockIdx.y * per);
     b1 = min(hi, b0 + per);
-}
-
-// out[i] = sum over the shares, in order
-static __global__ void k_sum_shares(int n, int n_shares, const double* __restrict__ part, double* __restrict__ out) {
-    const int i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= n) return;
-    double s = 0.0;
-    for (int y = 0; y < n_shares; ++y) s += part[(size_t)y * n + i];
-    out[i] = s;
 }
 
 }  // namespace sscf
