@@ -1377,12 +1377,15 @@ k_apply_warp(SweepArgs a, int p0, int nb, int min_runs) {
     constexpr int NTA = Sh::nta, NTB = Sh::ntb;
     extern __shared__ __align__(16) unsigned char smraw[];
     __shared__ int s_wsum[kWsWarps], s_next, s_lvl[Sh::team > 1 ? kMaxSub + 1 : 1];
-    if (*a.err & (kErrCapacity | kErrSortSize)) return;
+    // The next colour's CTAs may start once all of these have, and wait below for these to end: what a
+    // CTA reads before that was written before the sweep's first colour.
+    asm volatile("griddepcontrol.launch_dependents;");
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const BlockInfo& info = ((const BlockInfo*)a.blk_info)[p0 + (Sh::by_block ? blockIdx.x / (gridDim.x / nb) : blockIdx.x % nb)];
     const int4 i0 = info.i0, i1 = info.i1, i2 = info.i2;
     const int e = i0.x, np = i0.y, touch = i0.z, n_rows = i0.w;
-    if (np == 0) return;
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+    if (np == 0 || (*a.err & (kErrCapacity | kErrSortSize))) return;
     const int pa = i1.x, pb = i1.y;
     if (i1.z != n_rows) {
         if (threadIdx.x == 0) atomicOr(a.err, kErrCapacity);
@@ -2171,6 +2174,15 @@ static cudaError_t apply_warp_t(Ctx* c, SweepArgs& a, int col_lo, int col_hi) {
     // CTAs per block: shares of `per` runs for as many runs as the largest cluster's rows can give
     // (variant 2: one CTA takes all runs of its block; same results)
     const int full = c->n_sm * Sh::min_ctas;
+    // A colour's CTAs start while the last of the one before run, so that the end of one launch hides the
+    // start of the next: rotations at 997 molecules 1.74 -> 1.50 ms, at 4096 9.3 -> 9.0, FP64 at 343 1.52 ->
+    // 1.40; FP32 combinations 5.28 -> 5.20 and 42.2 -> 42.0. Not FP64 combinations, whose long blocks come
+    // first and would gather on the SMs that end early (343: 10.4 -> 11.9), and not inside a captured graph.
+    cudaStreamCaptureStatus capture = cudaStreamCaptureStatusNone;
+    e = cudaStreamIsCapturing(c->stream, &capture);
+    if (e != cudaSuccess) return e;
+    const bool overlap = (Sh::f32 || MODE == 0) && capture == cudaStreamCaptureStatusNone;
+    bool after_colour = false;
     for (int col = col_lo; col < col_hi; ++col) {
         const int nb = ptr[col + 1] - ptr[col];
         if (nb == 0) continue;
@@ -2179,7 +2191,19 @@ static cudaError_t apply_warp_t(Ctx* c, SweepArgs& a, int col_lo, int col_hi) {
         int gx = (runs + per - 1) / per;
         if (MODE == 0) gx = std::min(gx, (kWsRotWaves * full + nb - 1) / nb);
         if (c->apply_variant == 2) gx = 1;
-        k_apply_warp<T, MODE, ALL><<<nb * gx, Sh::threads, smem, c->stream>>>(a, ptr[col], nb, per);
+        cudaLaunchConfig_t cfg = {};
+        cfg.gridDim = dim3(nb * gx);
+        cfg.blockDim = dim3(Sh::threads);
+        cfg.dynamicSmemBytes = smem;
+        cfg.stream = c->stream;
+        cudaLaunchAttribute early = {};
+        early.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+        early.val.programmaticStreamSerializationAllowed = 1;
+        cfg.attrs = &early;
+        cfg.numAttrs = overlap && after_colour ? 1 : 0;
+        e = cudaLaunchKernelEx(&cfg, k_apply_warp<T, MODE, ALL>, a, ptr[col], nb, per);
+        if (e != cudaSuccess) return e;
+        after_colour = true;
         c->n_launch += 1;
     }
     return cudaGetLastError();
