@@ -1230,6 +1230,13 @@ constexpr int kWsManyRuns = 32;
 // rotations: CTAs of a launch as a multiple of the resident ones (2, 4, 8, 16: 13.8, 10.8, 9.6, 9.5 ms
 // at 4096 molecules, 1.91, 1.88, 1.74, 1.74 at 997)
 constexpr int kWsRotWaves = 8;
+// combinations: the same limit. Without one a colour's CTAs grow with the square of the cluster (12,288 at
+// 4096 molecules, 3.1 million at 65,536), nearly all without a row of work, and each reads its block's flags
+// to find that out. Occupied pass, limits 2, 4, 8, 16, 32 and none: 41.8, 38.8, 38.0, 37.1, 37.1, 37.1 ms at
+// 4096 molecules; 135, 123, 119, 120, 122, 127 at 8192; 357, 349, 342, 340, 347, 502 at 32,768; 750, 750, 745,
+// 741, 744, 1503 at 65,536; FP64 at 1000 108, 98.4, 95.0, 93.0, 93.1, 93.1. Four passes over all MOs at 4096
+// 43.2, 42.9, 41.9, 43.8, 51.7, 68.0; at 65,536 714, 714, 714, 741, 771, 10593.
+constexpr int kWsCombWaves = 16;
 constexpr int kWsPad = 34;                   // floats per panel column: 16-byte pieces scatter over all banks
 // pairs from which a combination block runs dense, as a divisor of n^2: the dense loop costs
 // ~8 n^2 clocks per row whatever the number of pairs, the list ~15 per pair with more latency (3, 4,
@@ -2187,10 +2194,9 @@ static cudaError_t apply_warp_t(Ctx* c, SweepArgs& a, int col_lo, int col_hi) {
         const int nb = ptr[col + 1] - ptr[col];
         if (nb == 0) continue;
         const int runs = (kAoPerMol / Sh::halves * c->max_cl_mol + 31) / 32;   // at most, of a block
-        const int per = MODE == 1 && (long long)nb * runs > kWsManyRuns * full ? 2 * Sh::runs : Sh::runs;
-        int gx = (runs + per - 1) / per;
-        if (MODE == 0) gx = std::min(gx, (kWsRotWaves * full + nb - 1) / nb);
-        if (c->apply_variant == 2) gx = 1;
+        const SweepShape shape = sweep_shape(nb, runs, Sh::runs, full, MODE == 0 ? kWsRotWaves : kWsCombWaves,
+                                             MODE == 0 ? 0 : kWsManyRuns);
+        const int gx = c->apply_variant == 2 ? 1 : shape.shares;
         cudaLaunchConfig_t cfg = {};
         cfg.gridDim = dim3(nb * gx);
         cfg.blockDim = dim3(Sh::threads);
@@ -2201,7 +2207,7 @@ static cudaError_t apply_warp_t(Ctx* c, SweepArgs& a, int col_lo, int col_hi) {
         early.val.programmaticStreamSerializationAllowed = 1;
         cfg.attrs = &early;
         cfg.numAttrs = overlap && after_colour ? 1 : 0;
-        e = cudaLaunchKernelEx(&cfg, k_apply_warp<T, MODE, ALL>, a, ptr[col], nb, per);
+        e = cudaLaunchKernelEx(&cfg, k_apply_warp<T, MODE, ALL>, a, ptr[col], nb, shape.min_runs);
         if (e != cudaSuccess) return e;
         after_colour = true;
         c->n_launch += 1;

@@ -38,6 +38,28 @@ constexpr int kMaxSub = 48;                    // in-block colours (<= MOs per g
 constexpr int kRotCap = 32 * 16;               // pairs of one occupied-virtual block
 constexpr int kOrthoCap = 48 * 48;             // pairs of one orthonormalisation block
 
+// Shape of a sweep's launch for one colour: CTAs per block, and the runs (32 AO
+// rows or row pairs with work) that each takes at least.
+struct SweepShape {
+    int shares, min_runs;
+};
+// blocks: of the colour; runs: of a block, at most (all rows of the largest
+// cluster); warps: runs that a CTA has in hand; resident: CTAs that run at the
+// same time; waves: limit of the launch's CTAs as a multiple of those; many_runs: a
+// launch of more runs than this per resident CTA (0: none is) takes two per warp.
+// The limit keeps the launch in proportion to the work: a block's rows with work
+// are those its MOs reach, whatever the cluster's size, and blocks x runs CTAs
+// grow with its square.
+inline SweepShape sweep_shape(int blocks, int runs, int warps, int resident, int waves, int many_runs) {
+    const bool many = many_runs > 0 && (long long)blocks * runs > (long long)many_runs * resident;
+    SweepShape s;
+    s.min_runs = many ? 2 * warps : warps;
+    const int all = (runs + s.min_runs - 1) / s.min_runs;
+    const int limit = (int)(((long long)waves * resident + blocks - 1) / blocks);
+    s.shares = all < limit ? all : limit;
+    return s;
+}
+
 // Error word bits set by kernels (read back by the host after a step).
 enum : unsigned {
     kErrCapacity = 1u,       // a row of C or a column of Y ran out of slots
