@@ -497,14 +497,6 @@ __device__ __forceinline__ void two_sum(float a, float b, float& s, float& e) {
     const float t = __fsub_rn(s, a);
     e = __fadd_rn(__fsub_rn(a, __fsub_rn(s, t)), __fsub_rn(b, t));
 }
-// Sum of partial sums to be rounded to FP32: a float and what its roundings
-// dropped (exact unless the terms are 24 binary orders apart, then to 2^-48).
-__device__ __forceinline__ void sum_add(float2& s, float v) {
-    float h, e;
-    two_sum(s.x, v, h, e);
-    s = make_float2(h, __fadd_rn(s.y, e));
-}
-__device__ __forceinline__ float sum_value(float2 s) { return isfinite(s.x) ? __fadd_rn(s.x, s.y) : s.x; }
 
 // x = hi + lo with hi, lo in TF32 (10 explicit mantissa bits each): hi by
 // round-to-nearest, ties away, lo the rounded remainder, so hi + lo carries ~21
@@ -531,15 +523,16 @@ __device__ __forceinline__ void mma_tf32(float (&d)[4], const uint32_t (&a)[4], 
 // AO rows of up to four matched row blocks (24 rows, 3 k-steps of 8) at a time.
 // Each product is split into TF32 hi + lo parts and summed as hi*hi + hi*lo +
 // lo*hi (the lo*lo term is below FP32 rounding), into FP32 fragments that are
-// added up in two floats every 32 of b's rows.
+// added up in FP64 every 32 of b's rows.
 // A row of a 6x16 tile is 64 bytes, so a warp reads a fragment's four rows of two
 // columns per lane straight from memory: no staging, no shared-memory traffic, and
 // a's tiles are found in L1 by the CTA's other warps (b's pass it by). Bound by the
 // splits (48 of ~75 instructions a k-step) and the L2 latency that three CTAs'
 // 80-register warps leave uncovered (issue slots 55 % used); four CTAs spill, two
-// are 20 % slower. Staged through shared memory, with cvt.rna.tf32 and sums in
-// FP64 (a quarter of the FP64 pipe's time): 8.0 + 6.3 ms for the two
-// transforms at 4096 molecules, now 6.2 + 4.8; at 997 1.48 + 1.07, now 1.23 + 0.90.
+// are 20 % slower. Staged through shared memory, with cvt.rna.tf32: 6.45 + 3.95 ms
+// for the two transforms of an early iteration at 4096 molecules, now 5.27 + 3.17; at
+// 997 1.50 + 1.21, now 1.18 + 0.81. (The sums in two floats, 48 bits: 5.06 + 2.97
+// and 1.13 + 0.78, but they are to carry no less than FP64 does.)
 constexpr int kTcWarps = 8, kTcCtas = 3;
 __device__ __forceinline__ float2 load_stream(const float* p) {
     float2 v;
@@ -585,13 +578,13 @@ k_transform_tc(int n_split, int n_rows, const int* __restrict__ tile_row0, int c
         const int* yr = y_row + (size_t)b * capY;
         const float* yb = y_val + (size_t)b * capY * kTileVals;
         float acc[2][4];
-        float2 sum[2][4];
+        double sum[2][4];
 #pragma unroll
         for (int h = 0; h < 2; ++h)
 #pragma unroll
             for (int q = 0; q < 4; ++q) {
                 acc[h][q] = 0.f;
-                sum[h][q] = make_float2(0.f, 0.f);
+                sum[h][q] = 0.0;
             }
         for (int k0 = 0; k0 < nb; k0 += 32) {
             const int k = k0 + lane;
@@ -648,14 +641,14 @@ k_transform_tc(int n_split, int n_rows, const int* __restrict__ tile_row0, int c
             for (int h = 0; h < 2; ++h)
 #pragma unroll
                 for (int q = 0; q < 4; ++q) {
-                    sum_add(sum[h][q], acc[h][q]);
+                    sum[h][q] += (double)acc[h][q];
                     acc[h][q] = 0.f;
                 }
         }
         // rows 2gq and 2gq + 1 of the block, columns 4tq to 4tq + 3
         float4* o = (float4*)(out + (size_t)tp_out[p] * 256) + 8 * gq + tq;
-        o[0] = make_float4(sum_value(sum[0][0]), sum_value(sum[1][0]), sum_value(sum[0][1]), sum_value(sum[1][1]));
-        o[4] = make_float4(sum_value(sum[0][2]), sum_value(sum[1][2]), sum_value(sum[0][3]), sum_value(sum[1][3]));
+        o[0] = make_float4((float)sum[0][0], (float)sum[1][0], (float)sum[0][1], (float)sum[1][1]);
+        o[4] = make_float4((float)sum[0][2], (float)sum[1][2], (float)sum[0][3], (float)sum[1][3]);
         if (nb == 0) r = lane < nb_next ? y_row[(size_t)b_next * capY + lane] : -1;
         b = b_next;
         nb = nb_next;
