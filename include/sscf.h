@@ -209,7 +209,8 @@ int sscf_set_fock_blocks(sscf_ctx* ctx, const double* X);
 /* Density matrix P = 2 C_occ C_occ^T (Eq. pop) of the current MOs on the
  * molecule-pair pattern, the input of the caller's next Fock build: dense
  * 6x6 blocks (row-major) in the pair order of sscf_get_blocks, into P (host,
- * n_mp * 36 doubles), summed in FP64. Charges and mixing state are not
+ * n_mp * 36 doubles), summed with no less than FP64's precision (mixed: FP32 sums of
+ * at most 32 products are what is added up). Charges and mixing state are not
  * changed. Errors: INVALID_ARG, STATE (before sscf_guess), OOM (its device
  * buffer is allocated by the first call), CUDA. */
 int sscf_get_density_blocks(sscf_ctx* ctx, double* P);

@@ -16,9 +16,10 @@
 
 #include <type_traits>
 
-#include "shares.h"
 #include "block_scan.h"
+#include "shares.h"
 #include "sscf_internal.h"
+#include "sum3.h"
 
 namespace sscf {
 
@@ -346,46 +347,58 @@ __device__ __forceinline__ void pair_terms(const SKd& P, const double* xa, const
     }
 }
 
-// s + e = a + b exactly
-__device__ __forceinline__ void two_sum(float a, float b, float& s, float& e) {
-    s = __fadd_rn(a, b);
-    const float t = __fsub_rn(s, a);
-    e = __fadd_rn(__fsub_rn(a, __fsub_rn(s, t)), __fsub_rn(b, t));
-}
-
 // One CTA per row block m, one warp per pattern neighbour n: P_mn (n >= m only,
 // P_nm = P_mn^T) and W_mn = 2 sum_t C[m,t] Z[n,t]^T on the tiles both rows hold,
-// written as 6 x 6 blocks. Products of FP32 values are rounded to FP32 and
-// summed without further error worth the name: FP64 sums in FP64 storage, pairs
-// of floats (the running sum and what its roundings dropped, 48 bits) in FP32
-// storage. FP64 additions bounded the kernel (two lanes per clock and SM; 72 of
-// them per shared tile and lane): 34.2 ms at 2000 molecules with the pair terms; now 2.5, and 0.33 for those.
+// written as 6 x 6 blocks. Products of FP32 values are rounded to FP32 and added
+// up without further error worth the name: in FP64 in FP64 storage, in three
+// floats (no less than FP64 carries) in FP32 storage, where FP64 additions
+// bounded the kernel (two lanes per clock and SM; 72 of them per shared tile
+// and lane): 34.2 ms at 2000 molecules with the pair terms; now 3.2, and 0.33 for
+// those. (Two floats, 48 bits: 2.5.)
 constexpr int kGradWarps = 8;
 template <typename T> struct SumOf;
 template <> struct SumOf<double> {
     double v;
-    __device__ __forceinline__ void zero() { v = 0.0; }
-    __device__ __forceinline__ void add_product(double a, double b) { v += a * b; }
     __device__ __forceinline__ void add(const SumOf& o) { v += o.v; }
     __device__ __forceinline__ double value() const { return v; }
 };
 template <> struct SumOf<float> {
-    float hi, lo;
-    __device__ __forceinline__ void zero() { hi = lo = 0.f; }
-    __device__ __forceinline__ void add_product(float a, float b) {
-        float e;
-        two_sum(hi, __fmul_rn(a, b), hi, e);
-        lo = __fadd_rn(lo, e);
-    }
-    __device__ __forceinline__ void add(const SumOf& o) {
-        float e;
-        two_sum(hi, o.hi, hi, e);
-        lo = __fadd_rn(lo, __fadd_rn(e, o.lo));
-    }
-    __device__ __forceinline__ double value() const { return (double)hi + (double)lo; }
+    Sum3 v;
+    __device__ __forceinline__ void add(const SumOf& o) { v.add(o.v); }
+    __device__ __forceinline__ double value() const { return v.value(); }
 };
+// two sums of products
+template <typename T> struct SumsOf;
+template <> struct SumsOf<double> {
+    double v[2];
+    __device__ __forceinline__ void zero() { v[0] = v[1] = 0.0; }
+    __device__ __forceinline__ void add_products(double a, double b0, double b1) {
+        v[0] += a * b0;
+        v[1] += a * b1;
+    }
+    __device__ __forceinline__ SumOf<double> get(int i) const { return {v[i]}; }
+};
+template <> struct SumsOf<float> {
+    Sum3x2 v;
+    __device__ __forceinline__ void zero() { v.h = v.l = v.m = make_float2(0.f, 0.f); }
+    __device__ __forceinline__ void add_products(float a, float b0, float b1) {
+        v.add(make_float2(__fmul_rn(a, b0), __fmul_rn(a, b1)));
+    }
+    __device__ __forceinline__ SumOf<float> get(int i) const {
+        return {i ? Sum3{v.h.y, v.l.y, v.m.y} : Sum3{v.h.x, v.l.x, v.m.x}};
+    }
+};
+// What a lane of a tile's 16 columns sums: FP64 all 36 products, the halves of the
+// warp on two tiles; FP32, whose sums are three registers, 18 (three AO rows of m per
+// half), both halves on one tile. (FP32 sums one by one instead of in pairs: 4.0 ms;
+// the next tile's values loaded ahead, or three CTAs per SM: spills, 3.6 and 3.2.)
+template <typename T> struct GradShape;
+template <> struct GradShape<double> { static constexpr int tiles = 2; };
+template <> struct GradShape<float> { static constexpr int tiles = 1; };
+// the lanes' sums of one product, and the padding that spreads them over the banks
+template <typename T> __host__ __device__ constexpr int grad_lanes() { return 16 * GradShape<T>::tiles; }
 template <typename T> __host__ __device__ constexpr size_t grad_smem(int map_n) {
-    return (size_t)((map_n + 3) & ~3) * 4 + (size_t)kGradWarps * 36 * 33 * sizeof(SumOf<T>);
+    return (size_t)((map_n + 3) & ~3) * 4 + (size_t)kGradWarps * 36 * (grad_lanes<T>() + 1) * sizeof(SumOf<T>);
 }
 template <typename T>
 __global__ void __launch_bounds__(kGradWarps * 32, 2)
@@ -395,7 +408,9 @@ k_grad_blocks(int n_occ_tiles, int map_n, const int* __restrict__ mol_ot0, int c
               const int* __restrict__ mp_col, const int* __restrict__ mp_rev, double* __restrict__ Pb,
               double* __restrict__ Wb) {
     extern __shared__ __align__(16) int smap[];   // map_n: slot in C row m of each occupied tile of m's cluster, or -1
-    SumOf<T>* sums = (SumOf<T>*)(smap + ((map_n + 3) & ~3));   // [warp][36][33]: the lanes' sums
+    constexpr int kTiles = GradShape<T>::tiles, kRows = 3 * kTiles;   // tiles at a time, AO rows of m per lane
+    constexpr int kLanes = grad_lanes<T>(), kPad = kLanes + 1;
+    SumOf<T>* sums = (SumOf<T>*)(smap + ((map_n + 3) & ~3));   // [warp][36][kPad]: the lanes' sums
     const int m = blockIdx.x;
     const int t0 = mol_ot0[m];
     for (int i = threadIdx.x; i < map_n; i += blockDim.x) smap[i] = -1;
@@ -409,16 +424,18 @@ k_grad_blocks(int n_occ_tiles, int map_n, const int* __restrict__ mol_ot0, int c
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int e0 = mp_ptr[m], ne = mp_ptr[m + 1] - e0;
     const int col = lane & 15, half = lane >> 4;
-    SumOf<T>* mys = sums + (size_t)warp * 36 * 33;
+    const int row0 = kTiles == 2 ? 0 : kRows * half;   // the lane's first AO row of m
+    SumOf<T>* mys = sums + (size_t)warp * 36 * kPad;
     // 2 sum_t C[m,t] B[n,t]^T over the occupied tiles of row n's list that row m holds
     auto block = [&](int n, const int* __restrict__ b_nt, const int* __restrict__ b_tile, const T* __restrict__ b_val,
                      double* out, double* out_t) {
-        SumOf<T> acc[36];
+        SumsOf<T> acc[kRows * 3];
 #pragma unroll
-        for (int u = 0; u < 36; ++u) acc[u].zero();
+        for (int u = 0; u < kRows * 3; ++u) acc[u].zero();
         const int nt = b_nt[n];
-        // 32 of n's tiles at a time, the shared ones found with one ballot; the halves of the warp
-        // take them in turn
+        const T* cm0 = c_val + (size_t)m * cap * kTileVals + row0 * kTileW + col;
+        const T* bn0 = b_val + (size_t)n * cap * kTileVals + col;
+        // 32 of n's tiles at a time, the shared ones found with one ballot
         for (int base = 0; base < nt; base += 32) {
             const int s = base + lane;
             const int t = s < nt ? b_tile[(size_t)n * cap + s] : n_occ_tiles;
@@ -426,37 +443,35 @@ k_grad_blocks(int n_occ_tiles, int map_n, const int* __restrict__ mol_ot0, int c
             unsigned mm = __ballot_sync(0xffffffffu, sm_ >= 0);
             const bool past = __any_sync(0xffffffffu, s < nt && t >= n_occ_tiles);
             while (mm) {
-                const int b0 = __ffs(mm) - 1;
+                int src = __ffs(mm) - 1;
                 mm &= mm - 1;
-                int b1 = -1;
-                if (mm) {
-                    b1 = __ffs(mm) - 1;
+                if (kTiles == 2) {   // the second half takes the next one
+                    const int b1 = __ffs(mm) - 1;
                     mm &= mm - 1;
+                    if (half) src = b1;
                 }
-                const int src = half ? b1 : b0;
                 const int sl = __shfl_sync(0xffffffffu, sm_, src < 0 ? 0 : src);
                 if (src < 0) continue;
-                const T* cm = c_val + ((size_t)m * cap + sl) * kTileVals + col;
-                const T* bn = b_val + ((size_t)n * cap + base + src) * kTileVals + col;
-                T a6[6], b6[6];
+                const T* cm = cm0 + sl * kTileVals;
+                const T* bn = bn0 + (base + src) * kTileVals;
+                T a6[kRows], b6[6];
 #pragma unroll
-                for (int k = 0; k < 6; ++k) {
-                    a6[k] = cm[k * kTileW];
-                    b6[k] = bn[k * kTileW];
-                }
+                for (int k = 0; k < kRows; ++k) a6[k] = cm[k * kTileW];
 #pragma unroll
-                for (int k = 0; k < 6; ++k)
+                for (int k = 0; k < 6; ++k) b6[k] = bn[k * kTileW];
 #pragma unroll
-                    for (int l = 0; l < 6; ++l) acc[k * 6 + l].add_product(a6[k], b6[l]);
+                for (int k = 0; k < kRows; ++k)
+#pragma unroll
+                    for (int l = 0; l < 3; ++l) acc[k * 3 + l].add_products(a6[k], b6[2 * l], b6[2 * l + 1]);
             }
             if (past) break;   // tiles are sorted: occupied tiles first
         }
 #pragma unroll
-        for (int u = 0; u < 36; ++u) mys[u * 33 + lane] = acc[u];
+        for (int u = 0; u < kRows * 6; ++u) mys[(row0 * 6 + u) * kPad + (kTiles == 2 ? lane : col)] = acc[u / 2].get(u & 1);
         __syncwarp();
         for (int u = lane; u < 36; u += 32) {
-            SumOf<T> v = mys[u * 33];
-            for (int j = 1; j < 32; ++j) v.add(mys[u * 33 + j]);
+            SumOf<T> v = mys[u * kPad];
+            for (int j = 1; j < kLanes; ++j) v.add(mys[u * kPad + j]);
             const double x = 2.0 * v.value();
             out[u] = x;
             if (out_t) out_t[(u % 6) * 6 + u / 6] = x;

@@ -10,6 +10,7 @@
 
 #include "block_scan.h"
 #include "sscf_internal.h"
+#include "sum3.h"
 
 #include <algorithm>
 #include <type_traits>
@@ -491,13 +492,6 @@ k_transform(int n_split, int n_rows, const int* __restrict__ tile_row0, int cap,
     }
 }
 
-// s + e = a + b exactly, s the rounded sum
-__device__ __forceinline__ void two_sum(float a, float b, float& s, float& e) {
-    s = __fadd_rn(a, b);
-    const float t = __fsub_rn(s, a);
-    e = __fadd_rn(__fsub_rn(a, __fsub_rn(s, t)), __fsub_rn(b, t));
-}
-
 // x = hi + lo with hi, lo in TF32 (10 explicit mantissa bits each): hi by
 // round-to-nearest, ties away, lo the rounded remainder, so hi + lo carries ~21
 // bits. Rounded in the bits, as cvt.rna.tf32 rounds (the kernel ran 5 % longer
@@ -678,30 +672,12 @@ constexpr int kDensWarps = 8;
 constexpr int kDensFlush = 32;  // tiles per lane in one FP32 sum
 constexpr int kDensUnroll = 1;  // shared tiles per half-warp and round (2 measured no faster)
 constexpr int kDensMinBlocks = 2;   // resident CTAs per SM the register budget aims at
-// A sum of floats in three, each the roundings dropped by the one before: 70 bits.
-// FP32 storage adds its partial sums of 32 products so (where FP64 carried 53): the
-// FP64 pipe, two lanes per clock and SM, was two thirds busy with them and with
-// the sums over a warp (density at 997 and 4096 molecules 0.55 and 3.60 ms, now 0.43
-// and 2.83). A lane keeps two floats in shared memory and the third, 2^-48 of the sum,
-// as eight bits of bf16 in a register (as floats: 0.47 and 3.14 ms).
-struct Sum3 {
-    float h, l, m;
-    __device__ __forceinline__ void add(float v) {
-        float e, d;
-        two_sum(h, v, h, e);
-        two_sum(l, e, l, d);
-        m = __fadd_rn(m, d);
-    }
-    __device__ __forceinline__ void add(float2 v) {
-        float d;
-        add(v.x);
-        two_sum(l, v.y, l, d);
-        m = __fadd_rn(m, d);
-    }
-    __device__ __forceinline__ double value() const {
-        return isfinite(h) ? ((double)h + (double)l) + (double)m : (double)h;
-    }
-};
+// FP32 storage adds its partial sums of 32 products in three floats (Sum3; FP64
+// before): the FP64 pipe, two lanes per clock and SM, was two thirds busy with
+// them and with the sums over a warp (density at 997 and 4096 molecules 0.55 and
+// 3.60 ms, now 0.43 and 2.83). A lane keeps two floats in shared memory and the
+// third, 2^-48 of the sum, as eight bits of bf16 in a register (as floats: 0.47 and
+// 3.14 ms): 56 bits where FP64 carried 53.
 
 // s += v; lost: what the two floats of s drop of it
 __device__ __forceinline__ void sum_add(float2& s, float v, float& lost) {

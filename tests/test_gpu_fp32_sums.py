@@ -9,7 +9,7 @@ of the second one is 2^-48.
 import numpy as np
 import pytest
 
-from gpu_common import context, water
+from gpu_common import P, context, water
 
 pytestmark = pytest.mark.gpu
 
@@ -37,3 +37,26 @@ def test_transform_adds_its_partial_sums_in_fp64():
     F_ov, _ = ctx.get_F()
     ctx.close()
     assert F_ov[0, 0] == 2.0 ** -51
+
+
+def test_gradients_add_their_products_in_fp64():
+    """dE/dV0 (ss-sigma) of two molecules that share ten occupied tiles, one term of P in every second one:
+    both ordered pairs of the O s orbitals, P = 2 sum, times the decay at their distance (a square root,
+    a division and an exponential of about -4, a few units in the last place each)."""
+    s = water(40)
+    ctx = context(s, precision=1)
+    n_tiles = int(sum(-(-4 * k // 16) for k in np.bincount(s.group_of_mol)))
+    assert n_tiles >= 10
+    nt = np.zeros(s.n_mol, dtype=np.int32)
+    nt[:2] = 10
+    vals = np.zeros((2, 10, 6, 16))
+    vals[0, ::2, 0, 0] = 1.0
+    vals[1, ::2, 0, 0] = TERMS
+    ctx.set_C_tiles(nt, np.tile(np.arange(10, dtype=np.int32), 2), vals.reshape(-1, 6, 16))
+    _, dpar = ctx.gradients()
+    ctx.close()
+    O = s.xyz.reshape(-1, 3, 3)[:2, 0]
+    r = np.sqrt(((O[1] - O[0]) ** 2).sum())
+    assert r < P["r_cut"]
+    ref = 2.0 * 2.0 * 2.0 ** -51 * np.exp(-r / P["r_decay"])
+    assert abs(dpar[0] - ref) <= 64 * 2.0 ** -53 * ref
