@@ -212,11 +212,14 @@ __global__ void k_build_h(int n_mp, const int* __restrict__ mp_row, const int* _
 // ---- per-molecule generalised eigensolve (step II) --------------------------
 // Cholesky S = L L^T, A = L^-1 H L^-T, cyclic Jacobi on A, x = L^-T v. Every
 // index is a constant once the loops are unrolled, so that the 6x6 matrices are
-// registers. Jacobi converges quadratically: the sweep that starts with the
-// off-diagonal part below 1e-12 of the matrix ends with it below rounding and is
-// the last (running until it was below 1e-17 took most of 60 sweeps of rounding
-// noise). 5.0 ms before, with indexed matrices in local memory, for any number
-// of molecules up to the GPU's threads; now 0.43.
+// registers. The sweep that starts with the off-diagonal part below 3e-15 of the
+// matrix ends with it at the rounding of the matrix and is the last: running until
+// it was below 1e-17 took most of 60 sweeps of rounding noise. (Not earlier:
+// convergence is quadratic only above the gaps, so a cluster of eigenvalues closer
+// than 1e-12 kept that much when 1e-12 was taken for the last sweep, a residual of
+// 9e-13 where 3e-15 is due. 5.8 sweeps of a random matrix then, 6.0 now.) 5.0 ms
+// before, with indexed matrices in local memory, for any number of molecules up to
+// the GPU's threads; now 0.43.
 __device__ __forceinline__ bool small_geneig6(const double* __restrict__ Hm, const double* __restrict__ Sm, double* X) {
     double Li[36];   // L, then its inverse (lower triangles)
     {
@@ -287,8 +290,8 @@ __device__ __forceinline__ bool small_geneig6(const double* __restrict__ Hm, con
                 tot += A[i * 6 + j] * A[i * 6 + j];
                 if (i != j) off += A[i * 6 + j] * A[i * 6 + j];
             }
-        if (off == 0.0) break;
-        const bool last = off <= 1e-24 * tot;
+        if (off <= 1e-34 * tot) break;
+        const bool last = off <= 1e-29 * tot;
 #pragma unroll
         for (int p = 0; p < 5; ++p)
 #pragma unroll
