@@ -602,12 +602,12 @@ static cudaError_t adjoint_t(Ctx* c, double* d_grad, double* d_par, double* d_gm
     for (int g = 0; g < c->n_groups; ++g) max_nb = std::max(max_nb, c->h_gnb_ptr[g + 1] - c->h_gnb_ptr[g]);
     const size_t smem_z = zmul_smem<T>(max_nb), smem_g = grad_smem<T>(c->max_cl_otiles);
     if (smem_l > 200 * 1024 || smem_z > 200 * 1024 || smem_g > 200 * 1024) return cudaErrorInvalidValue;
-    cudaError_t e = cudaFuncSetAttribute(k_zlists, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem_l);
+    cudaError_t e = allow_dynamic_smem(k_zlists);
     if (e != cudaSuccess) return e;
     k_zlists<<<c->n_mol, 256, smem_l, c->stream>>>(
         c->n_occ_tiles, c->n_groups, c->cap, c->d_c_nt[in], c->d_c_tile[in], c->d_tile_group, c->d_group_ot0,
         c->d_group_not, c->d_gnb_ptr, c->d_gnb_col, c->d_c_nt[zb], c->d_c_tile[zb], &c->d_sc->err);
-    e = cudaFuncSetAttribute(k_zmul<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem_z);
+    e = allow_dynamic_smem(k_zmul<T>);
     if (e != cudaSuccess) return e;
     // groups of molecules on grid y (65535 at most), out groups of their cluster on grid x
     for (int g0 = 0; g0 < c->n_groups; g0 += 65535) {
@@ -628,7 +628,7 @@ static cudaError_t adjoint_t(Ctx* c, double* d_grad, double* d_par, double* d_gm
     double* Pb = c->d_adj;
     double* Wb = Pb + (size_t)c->n_mp * 36;
     double* pt = Wb + (size_t)c->n_mp * 36;
-    e = cudaFuncSetAttribute(k_grad_blocks<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem_g);
+    e = allow_dynamic_smem(k_grad_blocks<T>);
     if (e != cudaSuccess) return e;
     k_grad_blocks<T><<<c->n_mol, kGradWarps * 32, smem_g, c->stream>>>(
         c->n_occ_tiles, c->max_cl_otiles, c->d_mol_ot0, c->cap, c->d_c_nt[in], c->d_c_tile[in],

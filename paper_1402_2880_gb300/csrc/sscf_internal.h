@@ -38,6 +38,18 @@ constexpr int kMaxSub = 48;                    // in-block colours (<= MOs per g
 constexpr int kRotCap = 32 * 16;               // pairs of one occupied-virtual block
 constexpr int kOrthoCap = 48 * 48;             // pairs of one orthonormalisation block
 
+// Dynamic shared memory for `kernel` up to what a CTA may opt into. Always the same
+// value: the attribute belongs to the kernel, which contexts of other sizes launch
+// from other threads. A context that set its own size could lower another's between
+// that one's setting and its launch, which then failed.
+template <typename K> inline cudaError_t allow_dynamic_smem(K* kernel) {
+    cudaFuncAttributes fa;
+    cudaError_t e = cudaFuncGetAttributes(&fa, kernel);
+    if (e != cudaSuccess) return e;
+    return cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                kMaxDynSmem - (int)fa.sharedSizeBytes);
+}
+
 // Shape of a sweep's launch for one colour: CTAs per block, and the runs (32 AO
 // rows or row pairs with work) that each takes at least.
 struct SweepShape {
