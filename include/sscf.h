@@ -304,7 +304,10 @@ int sscf_set_precision(sscf_ctx* ctx, int precision);
  * through the derivatives of the Slater-Koster blocks and of gamma.
  * dE_dxyz: host, 3*n_atoms (Ha/bohr, atom-major x, y, z), or NULL.
  * dE_dparams: host, 8: dE/dV0[0..3], dE/dS0[0..3], or NULL.
- * The charges of the current MOs become the SCC input (as sscf_reset_charges). */
+ * The charges of the current MOs become the SCC input (as sscf_reset_charges).
+ * Errors: STATE before sscf_guess, OOM (nothing changed), CAPACITY, NONFINITE, CUDA.
+ * The first call allocates its working memory (1,368 bytes per molecule pair and
+ * at most 1,536 per atom), which the context keeps. */
 int sscf_gradients(sscf_ctx* ctx, double* dE_dxyz, double* dE_dparams);
 
 /* Batch mode: per-cluster results of the last charge update (sscf_step,

@@ -894,7 +894,6 @@ int sscf_create(const sscf_system* sys, const sscf_params* prm, void* cuda_strea
     AL(c.d_Q, (size_t)c.n_atoms * 8);
     AL(c.d_e_mol, (size_t)c.n_mol * 8);
     c.n_shares = std::min(kMaxShares, (3 * c.max_cl_mol + kShareAtoms - 1) / kShareAtoms);
-    AL(c.d_share, (size_t)c.n_shares * c.n_atoms * 3 * 8);
     AL(c.d_cl_E, (size_t)c.n_clusters * 8);
     AL(c.d_cl_sel, (size_t)c.n_clusters * 6 * 8);
     AL(c.d_cl_hist, (size_t)c.n_clusters * 256 * 8);
@@ -1317,7 +1316,9 @@ int sscf_gradients(sscf_ctx* h, double* dE_dxyz, double* dE_dparams) {
     if (!h) return SSCF_ERR_INVALID_ARG;
     Ctx& c = h->c;
     if (!c.have_guess) return SSCF_ERR_STATE;
+    // kept for later calls, whichever of them was got
     if (!c.d_adj) CKS(dalloc(&c, &c.d_adj, adjoint_scratch_values(&c)));
+    if (!c.d_share) CKS(dalloc(&c, &c.d_share, (size_t)c.n_shares * c.n_atoms * 3));
     CK(cudaMemsetAsync(c.d_sc, 0, offsetof(DeviceScalars, hist), c.stream));
     // charges of the current MOs (they become the SCC input), H without threshold
     CKS(density_async(c, false));

@@ -279,7 +279,7 @@ struct Ctx {
     unsigned char* d_stage = nullptr;   // staging of sscf_set_C_tiles (grown as needed)
     size_t stage_bytes = 0;
     int n_shares = 1;             // shares of a sum over the atom pairs of a cluster
-    double* d_share = nullptr;    // n_shares x 3 n_atoms: their partial sums
+    double* d_share = nullptr;    // adjoint: n_shares x 3 n_atoms partial sums (allocated by the first sscf_gradients)
     double* d_adj = nullptr;      // adjoint: P and W blocks, terms of the atom pairs (allocated by the first sscf_gradients)
     double* d_grad = nullptr;     // 3 n_atoms: dE/dxyz
     double* d_par = nullptr;      // 8: dE/d(V0, S0)
