@@ -1113,10 +1113,11 @@ int sscf_autotune(sscf_ctx* h, int* tf_split_out) {
     const int cand[] = {0, 1, 2, 4, 8};   // 0: by size
     int best = 0, best_fixed = 1;
     float best_ms = 1e30f, best_fixed_ms = 1e30f;
-    const int before = c.tf_split;
+    int& split = c.tf_split[c.prec];
+    const int before = split;
     cudaError_t err = cudaSuccess;
     for (int s : cand) {
-        c.tf_split = s;
+        split = s;
         err = launch_transform_rot(&c);   // warm-up
         if (err != cudaSuccess) break;
         err = cudaEventRecord(e0, c.stream);
@@ -1137,7 +1138,7 @@ int sscf_autotune(sscf_ctx* h, int* tf_split_out) {
     }
     cudaEventDestroy(e0);
     cudaEventDestroy(e1);
-    c.tf_split = err == cudaSuccess ? best : before;
+    split = err == cudaSuccess ? best : before;
     if (err != cudaSuccess) return SSCF_ERR_CUDA;
     if (tf_split_out) *tf_split_out = best_fixed;
     return SSCF_OK;

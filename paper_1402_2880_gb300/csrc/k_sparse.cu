@@ -1053,20 +1053,10 @@ cudaError_t launch_xc_rot(Ctx* c) {
     return launch_xc(c, true, 0, c->n_tiles, c->n_occ_tiles);
 }
 
-// CTAs sharing one tile's pairs: what sscf_autotune chose, or enough for 32 (FP64) or 8
-// (FP32) per SM. FP64 at 343 molecules: 8 per SM 3.51 + 2.43 ms, 16 3.45 + 2.07, 32
-// 3.19 + 1.95, as the SMs share the work more evenly. FP32: 4 per SM 1.39 + 0.99 ms at
-// 997, 8 1.31 + 0.98, 16 1.33 + 0.90; the same at 4096, where the lower limit decides.
-static int transform_split(const Ctx* c, bool fp64) {
-    if (c->tf_split > 0) return c->tf_split;
-    const int per_tile = ((fp64 ? 32 : 8) * c->n_sm + c->n_occ_tiles - 1) / c->n_occ_tiles;
-    return fp64 ? std::min(128, std::max(8, per_tile)) : std::min(16, std::max(4, per_tile));
-}
-
 template <typename T>
 static cudaError_t transform_t(Ctx* c, const int* ptr, const int* bl, const int* outl, void* out) {
     constexpr bool kFP64 = std::is_same<T, double>::value;
-    const int split = transform_split(c, kFP64);
+    const int split = transform_split(c);
     const int grid = c->n_tiles * split;
     if constexpr (kFP64) {
         const size_t smem = (size_t)2 * kTfStageVals * sizeof(T) + (size_t)c->max_cl_mol * 2;

@@ -120,7 +120,9 @@ struct Ctx {
     int closure_window = 0;  // colours per closure (bounded fill); 0: one closure per sweep
     int apply_variant = 0;   // 0 specialised sweep kernels where they apply, 1 generic only,
                              // 2 specialised with one CTA per block
-    int tf_split = 0;        // CTAs sharing one occupied tile's pairs in the transform (sscf_autotune; 0: by size)
+    // CTAs sharing one occupied tile's pairs in the transform (sscf_autotune; 0: by size), per storage
+    // precision: the two have kernels and ranges of their own
+    int tf_split[2] = {0, 0};
     int n_sm = 152;          // multiprocessors of the context's device
     bool have_guess = false;
     int iteration = 0;
@@ -309,6 +311,19 @@ struct Ctx {
     std::vector<double> prof_ms;
     std::vector<long long> prof_calls;
 };
+
+// CTAs sharing one tile's pairs in the transform: what sscf_autotune chose for the
+// storage precision, or enough for 32 (FP64) or 8 (FP32) per SM. FP64 at 343
+// molecules: 8 per SM 3.51 + 2.43 ms, 16 3.45 + 2.07, 32 3.19 + 1.95, as the SMs share
+// the work more evenly. FP32: 4 per SM 1.39 + 0.99 ms at 997, 8 1.31 + 0.98, 16 1.33 +
+// 0.90; the same at 4096, where the lower limit decides.
+inline int transform_split(const Ctx* c) {
+    if (c->tf_split[c->prec] > 0) return c->tf_split[c->prec];
+    const bool fp64 = c->prec == SSCF_FP64;
+    const int per_tile = ((fp64 ? 32 : 8) * c->n_sm + c->n_occ_tiles - 1) / c->n_occ_tiles;
+    const int lo = fp64 ? 8 : 4, hi = fp64 ? 128 : 16;
+    return per_tile < lo ? lo : per_tile > hi ? hi : per_tile;
+}
 
 // ---- memory -----------------------------------------------------------------
 int dev_alloc(Ctx* c, void** p, size_t bytes);
