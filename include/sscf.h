@@ -244,10 +244,12 @@ int sscf_step(sscf_ctx* ctx, sscf_step_info* info);
  * it builds H and Y = H C as a step would, times the occupied-virtual transform
  * (three launches after one warm-up, CUDA events on the context's stream) for
  * 1, 2, 4 and 8 CTAs sharing each occupied tile's pairs and for the number
- * taken by size, and keeps the fastest for later steps. Results of later
- * calls do not depend on the choice (each pair is summed the same way). Drops a
- * captured CUDA graph. tf_split_out (host, may be NULL) receives the fastest of
- * the four. Errors: STATE before sscf_guess, CUDA. */
+ * taken by size, and keeps the fastest for later steps in the context's present
+ * storage precision. Results of later calls do not depend on the choice (each pair
+ * is summed the same way). Drops a captured CUDA graph. tf_split_out (host, may be
+ * NULL) receives the fastest of the four, plus 16 times the number taken by size if
+ * that was faster still and is in force: CTAs per tile v / 16 if v > 16, else v.
+ * Errors: STATE before sscf_guess, CUDA. */
 int sscf_autotune(sscf_ctx* ctx, int* tf_split_out);
 
 /* CUDA graphs: when enabled, sscf_step captures its device work (all kernel

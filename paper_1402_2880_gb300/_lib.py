@@ -338,7 +338,8 @@ class Context:
         return out
 
     def autotune(self) -> int:
-        """Pick the transform's launch shape by timing it on the current state; returns the choice."""
+        """Pick the transform's launch shape by timing it on the current state; returns the choice
+        v: v CTAs per tile, or v // 16 (the number taken by size) if v > 16."""
         s = ctypes.c_int()
         _check(self.lib.sscf_autotune(self.h, ctypes.byref(s)), "sscf_autotune")
         return s.value

@@ -1115,6 +1115,8 @@ int sscf_autotune(sscf_ctx* h, int* tf_split_out) {
     float best_ms = 1e30f, best_fixed_ms = 1e30f;
     int& split = c.tf_split[c.prec];
     const int before = split;
+    split = 0;
+    const int by_size = transform_split(&c);
     cudaError_t err = cudaSuccess;
     for (int s : cand) {
         split = s;
@@ -1140,7 +1142,7 @@ int sscf_autotune(sscf_ctx* h, int* tf_split_out) {
     cudaEventDestroy(e1);
     split = err == cudaSuccess ? best : before;
     if (err != cudaSuccess) return SSCF_ERR_CUDA;
-    if (tf_split_out) *tf_split_out = best_fixed;
+    if (tf_split_out) *tf_split_out = best > 0 ? best : best_fixed + 16 * by_size;
     return SSCF_OK;
 }
 
