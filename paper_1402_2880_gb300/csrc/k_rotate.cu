@@ -1224,8 +1224,9 @@ __global__ void __launch_bounds__(apply_threads<T>()) k_apply_colour(SweepArgs a
 constexpr int kFullCH = 32;                  // row blocks per word of the bits of rows with work
 constexpr int kFullBatch = 8;                // 16-byte pieces of a tile per lane and run of 32 row pairs, all in flight
 // runs a CTA takes at least: one per warp, or two where a launch could have more than kWsManyRuns
-// runs per resident CTA (at 4096 molecules most shares are empty, and fewer of them are launched:
-// 43.0 -> 41.9 ms; at 997 one per warp spreads better, 5.8 -> 5.3)
+// runs per CTA that its registers leave room for (at 4096 molecules most shares are empty, and fewer of
+// them are launched: 43.0 -> 41.9 ms; at 997 one per warp spreads better, 5.8 -> 5.3; passes over all MOs
+// at 700, where the line lies near 900 molecules, 7.6 ms against 8.3 with two)
 constexpr int kWsManyRuns = 32;
 // rotations: CTAs of a launch as a multiple of the resident ones (2, 4, 8, 16: 13.8, 10.8, 9.6, 9.5 ms
 // at 4096 molecules, 1.91, 1.88, 1.74, 1.74 at 997)
@@ -1234,8 +1235,8 @@ constexpr int kWsRotWaves = 8;
 // 4096 molecules, 3.1 million at 65,536), nearly all without a row of work, and each reads its block's flags
 // to find that out. Occupied pass, limits 2, 4, 8, 16, 32 and none: 41.8, 38.8, 38.0, 37.1, 37.1, 37.1 ms at
 // 4096 molecules; 135, 123, 119, 120, 122, 127 at 8192; 357, 349, 342, 340, 347, 502 at 32,768; 750, 750, 745,
-// 741, 744, 1503 at 65,536; FP64 at 1000 108, 98.4, 95.0, 93.0, 93.1, 93.1. Four passes over all MOs at 4096
-// 43.2, 42.9, 41.9, 43.8, 51.7, 68.0; at 65,536 714, 714, 714, 741, 771, 10593.
+// 741, 744, 1503 at 65,536; FP64 at 1000 108, 98.4, 95.0, 93.0, 93.1, 93.1. Four passes over all MOs, limits 4, 8,
+// 16, 32, 64 and none: 43.2, 42.9, 41.9, 43.8, 51.7, 68.0 at 4096; 714, 714, 714, 741, 771, 10593 at 65,536.
 constexpr int kWsCombWaves = 16;
 constexpr int kWsPad = 34;                   // floats per panel column: 16-byte pieces scatter over all banks
 // pairs from which a combination block runs dense, as a divisor of n^2: the dense loop costs
@@ -1275,9 +1276,13 @@ template <typename T, int MODE, bool ALL> struct WarpShape {
     static constexpr int per_warp = 2 * raw > panel ? 2 * raw : panel;
     static_assert(MODE == 0 || ALL || per_warp >= nta * 16 * 64 * 4, "");
     static constexpr size_t smem = (size_t)table + (size_t)runs * per_warp;   // + row bits
-    // resident CTAs the register budget is cut for: the dense loop holds 2 n values per row; FP64
-    // runs as many as its panels leave room for
+    // CTAs per SM the register budget is cut for: the dense loop holds 2 n values per row; FP64 runs as
+    // many as its panels leave room for
     static constexpr int min_ctas = f32 ? (MODE == 0 ? 6 : (ALL ? 2 : 3)) : (MODE == 0 ? 6 : (ALL ? 3 : 5));
+    // resident CTAs: as many, but in FP32 passes over all MOs, whose 117 KB leave room for one (four
+    // warps, one per quarter of an SM)
+    static constexpr int fit = kSmSmem / ((int)smem + 1024), resident = fit < min_ctas ? fit : min_ctas;
+    static constexpr int many_runs = kWsManyRuns * min_ctas / resident;
 };
 
 // 1.0 where |v| >= t, 0.0 below (and for NaN): one compare that writes the
@@ -2178,7 +2183,7 @@ static cudaError_t apply_warp_t(Ctx* c, SweepArgs& a, int col_lo, int col_hi) {
     const std::vector<int>& ptr = MODE == 0 ? c->h_colour_ptr : c->h_ocolour_ptr;
     // CTAs per block: shares of `per` runs for as many runs as the largest cluster's rows can give
     // (variant 2: one CTA takes all runs of its block; same results)
-    const int full = c->n_sm * Sh::min_ctas;
+    const int full = c->n_sm * Sh::resident;
     // A colour's CTAs start while the last of the one before run, so that the end of one launch hides the
     // start of the next: rotations at 997 molecules 1.74 -> 1.50 ms, at 4096 9.3 -> 9.0, FP64 at 343 1.52 ->
     // 1.40; FP32 combinations 5.28 -> 5.20 and 42.2 -> 42.0. Not FP64 combinations, whose long blocks come
@@ -2193,7 +2198,7 @@ static cudaError_t apply_warp_t(Ctx* c, SweepArgs& a, int col_lo, int col_hi) {
         if (nb == 0) continue;
         const int runs = (kAoPerMol / Sh::halves * c->max_cl_mol + 31) / 32;   // at most, of a block
         const SweepShape shape = sweep_shape(nb, runs, Sh::runs, full, MODE == 0 ? kWsRotWaves : kWsCombWaves,
-                                             MODE == 0 ? 0 : kWsManyRuns);
+                                             MODE == 0 ? 0 : Sh::many_runs);
         const int gx = c->apply_variant == 2 ? 1 : shape.shares;
         cudaLaunchConfig_t cfg = {};
         cfg.gridDim = dim3(nb * gx);

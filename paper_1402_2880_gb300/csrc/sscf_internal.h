@@ -34,6 +34,7 @@ constexpr int kTileW = 16;
 constexpr int kTileVals = kAoPerMol * kTileW;  // 96
 constexpr int kMaxMolPerGroup = 8;
 constexpr int kMaxDynSmem = 227 * 1024;          // dynamic shared memory a CTA may opt into
+constexpr int kSmSmem = 228 * 1024;              // shared memory of an SM, of which every CTA takes 1 KB more
 constexpr int kMaxSub = 48;                    // in-block colours (<= MOs per group side)
 constexpr int kRotCap = 32 * 16;               // pairs of one occupied-virtual block
 constexpr int kOrthoCap = 48 * 48;             // pairs of one orthonormalisation block
