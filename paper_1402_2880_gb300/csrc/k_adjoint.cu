@@ -91,49 +91,17 @@ __device__ __forceinline__ int first_at(const int* __restrict__ list, int n, int
     return lo;
 }
 
-// Z's values. A CTA makes the 48 x 32 outputs of one MO group's molecules (48 AO
-// rows) and one out group A (two tiles), over the in groups B adjacent to A that
-// any of the rows holds: per B it stages the rows' 48 x 32 values and the 32 x 32
-// block F[B, A] (loading the next B's meanwhile), so that a block of F is read once per group of molecules, and
-// each of 96 threads keeps 4 x 4 outputs. Terms are added in the order of the
-// row's tiles and of the MOs inside a tile, one product at a time; a tile that a
-// row does not hold contributes zeros. (One warp per row and out tile read a
-// block of F for six rows of work and looked it up by a binary search:
-// 27.6 ms at 2000 molecules; 6.6 with scalar multiply-adds, F staged value by
-// value and loads not overlapped; now 5.6.)
-constexpr int kZThreads = 96;
-constexpr int kZRows = kMaxMolPerGroup * kAoPerMol;   // 48
-constexpr int kZStride = kZRows + 4;                  // values per staged MO (16-byte aligned, bank-spread)
-constexpr int kFStride = 36;                          // values per staged MO of B
-// Neighbours of A in one launch, whose slots are in shared memory. Where a group has more (MANY), the
-// neighbours from nb_lo on are taken and the sums go on from where the launch before left them. (One
-// kernel for both: other registers, 5.9 ms instead of 5.6 at 2000 molecules.)
-constexpr int kZNb = 128;
-template <typename T> __host__ __device__ constexpr size_t zmul_smem(int max_nb) {
-    return (size_t)32 * kZStride * sizeof(T) + (size_t)32 * kFStride * sizeof(T) +
-           (size_t)max_nb * kMaxMolPerGroup * sizeof(int2) + (size_t)max_nb * sizeof(int);
-}
-template <typename T, bool MANY>
-__global__ void __launch_bounds__(kZThreads)
-k_zmul(int g_lo, int nb_lo, int max_nb, int cap, const int* __restrict__ group_cl, const int* __restrict__ cl_g0,
-       const int* __restrict__ grp_mol_ptr, const int* __restrict__ grp_mol,
-       const int* __restrict__ c_nt, const int* __restrict__ c_tile, const T* __restrict__ c_val,
-       const int* __restrict__ group_ot0, const int* __restrict__ group_not, const int* __restrict__ gnb_ptr,
-       const int* __restrict__ gnb_col, const int* __restrict__ blk_tp, const int* __restrict__ gnb_rev,
-       const T* __restrict__ F, const int* __restrict__ z_nt, const int* __restrict__ z_tile, T* __restrict__ z_val) {
-    extern __shared__ __align__(16) unsigned char smraw[];
-    T* sc = (T*)smraw;                                // [32 MOs of B][kZStride]: the rows' values
-    T* sf = sc + 32 * kZStride;                       // [32 MOs of B][kFStride]: F[B, A], 32 MOs of A
-    int2* slot = (int2*)(sf + 32 * kFStride);         // [neighbour of A][molecule]: slots of B's two tiles, or -1
-    int* any = (int*)(slot + (size_t)max_nb * kMaxMolPerGroup);   // [neighbour of A]: some row holds a tile of B
-    __shared__ int s_mol[kMaxMolPerGroup], s_z[kMaxMolPerGroup];
-    const int G = g_lo + blockIdx.y, cl = group_cl[G], A = cl_g0[cl] + blockIdx.x;
-    if (A >= cl_g0[cl + 1]) return;
-    const int m0 = grp_mol_ptr[G], nm = grp_mol_ptr[G + 1] - m0;
-    const int e0 = gnb_ptr[A] + (MANY ? nb_lo : 0), nb = MANY ? min(max_nb, gnb_ptr[A + 1] - e0) : gnb_ptr[A + 1] - e0;
-    if (MANY && nb <= 0) return;
-    const int otA = group_ot0[A], ntA = group_not[A];
-    // the rows with tiles of A in Z, and their first slot there
+// What the kernels below start with, for one MO group's molecules (rows) and one out
+// group A: the rows, their first slot of A's tiles in Z (-1: none), and for up to
+// max_nb neighbours B of A the slots of B's two tiles in the rows (or -1) and whether
+// any row holds one. False if no row has tiles of A.
+template <int THREADS>
+__device__ __forceinline__ bool z_lookup(int m0, int nm, int otA, int e0, int nb, int cap,
+                                         const int* __restrict__ grp_mol, const int* __restrict__ c_nt,
+                                         const int* __restrict__ c_tile, const int* __restrict__ group_ot0,
+                                         const int* __restrict__ group_not, const int* __restrict__ gnb_col,
+                                         const int* __restrict__ z_nt, const int* __restrict__ z_tile, int* s_mol,
+                                         int* s_z, int2* slot, int* any) {
     bool mine = false;
     if ((int)threadIdx.x < nm) {
         const int r = grp_mol[m0 + threadIdx.x];
@@ -144,10 +112,10 @@ k_zmul(int g_lo, int nb_lo, int max_nb, int cap, const int* __restrict__ group_c
         s_mol[threadIdx.x] = r;
         s_z[threadIdx.x] = mine ? p : -1;
     }
-    if (!__syncthreads_or(mine)) return;
-    for (int i = threadIdx.x; i < nb; i += kZThreads) any[i] = 0;
+    if (!__syncthreads_or(mine)) return false;
+    for (int i = threadIdx.x; i < nb; i += THREADS) any[i] = 0;
     __syncthreads();
-    for (int i = threadIdx.x; i < nb * nm; i += kZThreads) {
+    for (int i = threadIdx.x; i < nb * nm; i += THREADS) {
         const int k = i / nm, q = i - k * nm;
         const int B = gnb_col[e0 + k], t = group_ot0[B];
         const int* ct = c_tile + (size_t)s_mol[q] * cap;
@@ -164,10 +132,59 @@ k_zmul(int g_lo, int nb_lo, int max_nb, int cap, const int* __restrict__ group_c
         if (s.x >= 0 || s.y >= 0) any[k] = 1;
     }
     __syncthreads();
+    return true;
+}
+
+// Z's values in FP32 storage. A CTA makes the 48 x 32 outputs of one MO group's molecules (48 AO
+// rows) and one out group A (two tiles), over the in groups B adjacent to A that
+// any of the rows holds: per B it stages the rows' 48 x 32 values and the 32 x 32
+// block F[B, A] (loading the next B's meanwhile), so that a block of F is read once per group of molecules, and
+// each of 96 threads keeps 4 x 4 outputs. Terms are added in the order of the
+// row's tiles and of the MOs inside a tile, one product at a time; a tile that a
+// row does not hold contributes zeros. (One warp per row and out tile read a
+// block of F for six rows of work and looked it up by a binary search:
+// 27.6 ms at 2000 molecules; 6.6 with scalar multiply-adds, F staged value by
+// value and loads not overlapped; now 5.4, with the registers cut for seven CTAs per
+// SM; 5.7 cut for six.)
+constexpr int kZThreads = 96;
+constexpr int kZRows = kMaxMolPerGroup * kAoPerMol;   // 48
+constexpr int kZStride = kZRows + 4;                  // values per staged MO (16-byte aligned, bank-spread)
+constexpr int kFStride = 36;                          // values per staged MO of B
+// Neighbours of A in one launch, whose slots are in shared memory. Where a group has more (MANY), the
+// neighbours from nb_lo on are taken and the sums go on from where the launch before left them. (One
+// kernel for both was slower: 5.9 ms instead of 5.6 at 2000 molecules.)
+constexpr int kZNb = 128;
+__host__ __device__ constexpr size_t z_lookup_smem(int max_nb) {
+    return (size_t)max_nb * (kMaxMolPerGroup * sizeof(int2) + sizeof(int));
+}
+constexpr size_t kZmulSmem = (size_t)32 * (kZStride + kFStride) * sizeof(float);   // and z_lookup_smem
+template <bool MANY>
+__global__ void __launch_bounds__(kZThreads, 7)
+k_zmul(int g_lo, int nb_lo, int max_nb, int cap, const int* __restrict__ group_cl, const int* __restrict__ cl_g0,
+       const int* __restrict__ grp_mol_ptr, const int* __restrict__ grp_mol,
+       const int* __restrict__ c_nt, const int* __restrict__ c_tile, const float* __restrict__ c_val,
+       const int* __restrict__ group_ot0, const int* __restrict__ group_not, const int* __restrict__ gnb_ptr,
+       const int* __restrict__ gnb_col, const int* __restrict__ blk_tp, const int* __restrict__ gnb_rev,
+       const float* __restrict__ F, const int* __restrict__ z_nt, const int* __restrict__ z_tile, float* __restrict__ z_val) {
+    extern __shared__ __align__(16) unsigned char smraw[];
+    float* sc = (float*)smraw;                                // [32 MOs of B][kZStride]: the rows' values
+    float* sf = sc + 32 * kZStride;                       // [32 MOs of B][kFStride]: F[B, A], 32 MOs of A
+    int2* slot = (int2*)(sf + 32 * kFStride);         // [neighbour of A][molecule]: slots of B's two tiles, or -1
+    int* any = (int*)(slot + (size_t)max_nb * kMaxMolPerGroup);   // [neighbour of A]: some row holds a tile of B
+    __shared__ int s_mol[kMaxMolPerGroup], s_z[kMaxMolPerGroup];
+    const int G = g_lo + blockIdx.y, cl = group_cl[G], A = cl_g0[cl] + blockIdx.x;
+    if (A >= cl_g0[cl + 1]) return;
+    const int m0 = grp_mol_ptr[G], nm = grp_mol_ptr[G + 1] - m0;
+    const int e0 = gnb_ptr[A] + (MANY ? nb_lo : 0), nb = MANY ? min(max_nb, gnb_ptr[A + 1] - e0) : gnb_ptr[A + 1] - e0;
+    if (MANY && nb <= 0) return;
+    const int otA = group_ot0[A], ntA = group_not[A];
+    if (!z_lookup<kZThreads>(m0, nm, otA, e0, nb, cap, grp_mol, c_nt, c_tile, group_ot0, group_not, gnb_col, z_nt, z_tile,
+                             s_mol, s_z, slot, any))
+        return;
     const int ti = threadIdx.x >> 3, tj = threadIdx.x & 7;   // rows 4 ti .. 4 ti + 3, MOs 4 tj .. 4 tj + 3 of A
-    T acc[4][4];
+    float acc[4][4];
     // output row i of the thread: where its four values go (NULL: nowhere)
-    auto out = [&](int i) -> T* {
+    auto out = [&](int i) -> float* {
         const int row = 4 * ti + i, q = row / kAoPerMol;
         if (q >= nm || s_z[q] < 0 || (tj >> 2) >= ntA) return nullptr;
         return z_val + ((size_t)s_mol[q] * cap + s_z[q] + (tj >> 2)) * kTileVals + (row - q * kAoPerMol) * kTileW +
@@ -176,16 +193,16 @@ k_zmul(int g_lo, int nb_lo, int max_nb, int cap, const int* __restrict__ group_c
 #pragma unroll
     for (int i = 0; i < 4; ++i)
 #pragma unroll
-        for (int j = 0; j < 4; ++j) acc[i][j] = (T)0;
+        for (int j = 0; j < 4; ++j) acc[i][j] = 0.f;
     if (MANY && nb_lo > 0)
         for (int i = 0; i < 4; ++i)
-            if (const T* z = out(i))
+            if (const float* z = out(i))
                 for (int j = 0; j < 4; ++j) acc[i][j] = z[j];
     // 16-byte pieces: of the rows along the MOs, turned to [MO][row], and of F[B, A], whose tile pairs
     // are stored for blocks (lower group, upper group), inside a group for positions a <= b; turned
     // when stored the other way. The next neighbour's are loaded during this one's products.
-    using V = typename std::conditional<sizeof(T) == 4, float4, double2>::type;
-    constexpr int kV = 16 / (int)sizeof(T), kPer = 16 / kV;   // values of a piece, pieces per tile row
+    using V = float4;
+    constexpr int kV = 4, kPer = 16 / kV;   // values of a piece, pieces per tile row
     constexpr int kC = kZRows * 2 * kPer / kZThreads, kF = (4 * 16 * kPer + kZThreads - 1) / kZThreads;
     static_assert(kC * kZThreads == kZRows * 2 * kPer, "");
     V vc[kC], vf[kF];
@@ -229,7 +246,7 @@ k_zmul(int g_lo, int nb_lo, int max_nb, int cap, const int* __restrict__ group_c
             const int i = threadIdx.x + h * kZThreads;
             const int row = i / (2 * kPer), rem = i - row * (2 * kPer), t = rem / kPer, p = rem - t * kPer;
 #pragma unroll
-            for (int u = 0; u < kV; ++u) sc[(t * 16 + p * kV + u) * kZStride + row] = ((const T*)&vc[h])[u];
+            for (int u = 0; u < kV; ++u) sc[(t * 16 + p * kV + u) * kZStride + row] = ((const float*)&vc[h])[u];
         }
 #pragma unroll
         for (int h = 0; h < kF; ++h) {
@@ -239,7 +256,7 @@ k_zmul(int g_lo, int nb_lo, int max_nb, int cap, const int* __restrict__ group_c
             if ((turned >> t) & 1) {
 #pragma unroll
                 for (int u = 0; u < kV; ++u)
-                    sf[(pB * 16 + c + u) * kFStride + pA * 16 + r] = ((const T*)&vf[h])[u];
+                    sf[(pB * 16 + c + u) * kFStride + pA * 16 + r] = ((const float*)&vf[h])[u];
             } else {
                 *(V*)(sf + (pB * 16 + r) * kFStride + pA * 16 + c) = vf[h];
             }
@@ -249,36 +266,154 @@ k_zmul(int g_lo, int nb_lo, int max_nb, int cap, const int* __restrict__ group_c
         if (k < nb) load(k);
 #pragma unroll 8
         for (int q = 0; q < 32; ++q) {
-            T c[4], f[4];
-#pragma unroll
-            for (int u = 0; u < 4; u += kV) {
-                *(V*)(c + u) = *(const V*)(sc + q * kZStride + 4 * ti + u);
-                *(V*)(f + u) = *(const V*)(sf + q * kFStride + 4 * tj + u);
-            }
+            float c[4], f[4];
+            *(V*)c = *(const V*)(sc + q * kZStride + 4 * ti);
+            *(V*)f = *(const V*)(sf + q * kFStride + 4 * tj);
 #pragma unroll
             for (int i = 0; i < 4; ++i) {
-                if constexpr (sizeof(T) == 4) {
 #pragma unroll
-                    for (int j = 0; j < 4; j += 2) {
-                        const float2 v = __ffma2_rn(make_float2(c[i], c[i]), make_float2(f[j], f[j + 1]),
-                                                    make_float2(acc[i][j], acc[i][j + 1]));
-                        acc[i][j] = v.x;
-                        acc[i][j + 1] = v.y;
-                    }
-                } else {
-#pragma unroll
-                    for (int j = 0; j < 4; ++j) acc[i][j] += c[i] * f[j];
+                for (int j = 0; j < 4; j += 2) {
+                    const float2 v = __ffma2_rn(make_float2(c[i], c[i]), make_float2(f[j], f[j + 1]),
+                                                make_float2(acc[i][j], acc[i][j + 1]));
+                    acc[i][j] = v.x;
+                    acc[i][j + 1] = v.y;
                 }
             }
         }
     }
 #pragma unroll
     for (int i = 0; i < 4; ++i) {
-        T* z = out(i);
-        if (!z) continue;
-#pragma unroll
-        for (int u = 0; u < 4; u += kV) *(V*)(z + u) = *(const V*)(acc[i] + u);
+        if (float* z = out(i)) *(V*)z = *(const V*)acc[i];
     }
+}
+
+// The same in FP64 storage, whose pipe (two lanes per clock and SM) bounds it: no product may be
+// spent on a tile that a row does not hold, and those are many in a large cluster (in the kernel
+// above 1.3 times the products that are there at 1000 molecules, 1.8 at 2000). A CTA takes the
+// same rows and out group, a warp one molecule, and walks the tiles that its own row holds; a
+// lane keeps rows kh, kh + 2, kh + 4 of column j of A's tiles. Terms in the same
+// order. (With absent tiles as zeros 40.4 ms at 1000 molecules, one warp per row and
+// out tile 37.9; now 30.9, of which the products take 29.9. The adjoint at 2000:
+// 178, 139, now 106 ms.)
+constexpr int kZ64Threads = 32 * kMaxMolPerGroup;
+constexpr int kF64Stride = 34;   // values per staged MO of B (16-byte aligned)
+constexpr size_t kZmul64Smem =
+    (size_t)2 * (32 * kF64Stride + kMaxMolPerGroup * 2 * kTileVals) * sizeof(double);   // and z_lookup_smem
+template <bool MANY>
+__global__ void __launch_bounds__(kZ64Threads)
+k_zmul64(int g_lo, int nb_lo, int max_nb, int cap, const int* __restrict__ group_cl, const int* __restrict__ cl_g0,
+         const int* __restrict__ grp_mol_ptr, const int* __restrict__ grp_mol,
+         const int* __restrict__ c_nt, const int* __restrict__ c_tile, const double* __restrict__ c_val,
+         const int* __restrict__ group_ot0, const int* __restrict__ group_not, const int* __restrict__ gnb_ptr,
+         const int* __restrict__ gnb_col, const int* __restrict__ blk_tp, const int* __restrict__ gnb_rev,
+         const double* __restrict__ F, const int* __restrict__ z_nt, const int* __restrict__ z_tile,
+         double* __restrict__ z_val) {
+    extern __shared__ __align__(16) unsigned char smraw[];
+    double* sf = (double*)smraw;                      // two buffers: [32 MOs of B][kF64Stride]: F[B, A]
+    double* sc = sf + 2 * 32 * kF64Stride;            // two buffers: [molecule][B's two tiles]
+    int2* slot = (int2*)(sc + 2 * kMaxMolPerGroup * 2 * kTileVals);   // as above
+    int* any = (int*)(slot + (size_t)max_nb * kMaxMolPerGroup);
+    __shared__ int s_mol[kMaxMolPerGroup], s_z[kMaxMolPerGroup];
+    const int G = g_lo + blockIdx.y, cl = group_cl[G], A = cl_g0[cl] + blockIdx.x;
+    if (A >= cl_g0[cl + 1]) return;
+    const int m0 = grp_mol_ptr[G], nm = grp_mol_ptr[G + 1] - m0;
+    const int e0 = gnb_ptr[A] + (MANY ? nb_lo : 0), nb = MANY ? min(max_nb, gnb_ptr[A + 1] - e0) : gnb_ptr[A + 1] - e0;
+    if (MANY && nb <= 0) return;
+    const int otA = group_ot0[A], ntA = group_not[A];
+    if (!z_lookup<kZ64Threads>(m0, nm, otA, e0, nb, cap, grp_mol, c_nt, c_tile, group_ot0, group_not, gnb_col, z_nt,
+                               z_tile, s_mol, s_z, slot, any))
+        return;
+    const int lane = threadIdx.x & 31, q = threadIdx.x >> 5;   // q: the warp's molecule
+    const int j = lane & 15, kh = lane >> 4;
+    const bool mine = q < nm && s_z[q] >= 0;
+    // row kh of the warp's first tile of A in Z (only where mine)
+    double* const z = z_val + (mine ? ((size_t)s_mol[q] * cap + s_z[q]) * kTileVals + kh * kTileW + j : 0);
+    double acc[2][3];
+#pragma unroll
+    for (int a = 0; a < 2; ++a)
+#pragma unroll
+        for (int u = 0; u < 3; ++u)
+            acc[a][u] = MANY && nb_lo > 0 && mine && a < ntA ? z[a * kTileVals + 2 * u * kTileW] : 0.0;
+    double2 vc[3] = {}, vf[2] = {};
+    int turned = 0;   // as above
+    auto load = [&](int k) {
+        const int e = e0 + k, B = gnb_col[e], eb = B <= A ? gnb_rev[e] : e;   // entry (min, max)
+        const int ntB = group_not[B];
+        turned = B < A ? 0 : B == A ? 4 : 15;
+#pragma unroll
+        for (int h = 0; h < 3; ++h) {
+            const int i = lane + 32 * h, t = i / (kTileVals / 2), p = i - t * (kTileVals / 2);
+            const int s = q < nm ? (t ? slot[k * kMaxMolPerGroup + q].y : slot[k * kMaxMolPerGroup + q].x) : -1;
+            if (s >= 0) vc[h] = *((const double2*)(c_val + ((size_t)s_mol[q] * cap + s) * kTileVals) + p);
+        }
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {
+            const int i = threadIdx.x + h * kZ64Threads, t = i >> 7, pB = t >> 1, pA = t & 1;
+            if (pB < ntB && pA < ntA) {
+                const int tp = blk_tp[(size_t)eb * 9 + ((turned >> t) & 1 ? pA * 3 + pB : pB * 3 + pA)];
+                vf[h] = *((const double2*)(F + (size_t)tp * 256) + (i & 127));
+            }
+        }
+    };
+    auto next = [&](int k) {
+        while (k < nb && !any[k]) ++k;
+        return k;
+    };
+    int phase = 0, k = next(0);
+    if (k < nb) load(k);
+    while (k < nb) {
+        // (a buffer is written again after the barrier that all threads reach past its products)
+        double* const f = sf + phase * 32 * kF64Stride;
+        double* const c = sc + (phase * kMaxMolPerGroup + q) * 2 * kTileVals;
+        phase ^= 1;
+#pragma unroll
+        for (int h = 0; h < 3; ++h) ((double2*)c)[lane + 32 * h] = vc[h];
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {
+            const int i = threadIdx.x + h * kZ64Threads, t = i >> 7, pB = t >> 1, pA = t & 1;
+            const int r = (i & 127) >> 3, col = 2 * (i & 7);
+            if ((turned >> t) & 1) {
+                f[(pB * 16 + col) * kF64Stride + pA * 16 + r] = vf[h].x;
+                f[(pB * 16 + col + 1) * kF64Stride + pA * 16 + r] = vf[h].y;
+            } else {
+                *(double2*)(f + (pB * 16 + r) * kF64Stride + pA * 16 + col) = vf[h];
+            }
+        }
+        __syncthreads();
+        const int2 held = q < nm ? slot[k * kMaxMolPerGroup + q] : make_int2(-1, -1);
+        k = next(k + 1);
+        if (k < nb) load(k);
+        auto products = [&](auto two) {
+#pragma unroll
+            for (int t = 0; t < 2; ++t) {
+                if ((t ? held.y : held.x) < 0) continue;
+                const double *ct = c + t * kTileVals + kh * kTileW, *ft = f + t * 16 * kF64Stride + j;
+#pragma unroll 4
+                for (int i = 0; i < 16; i += 2) {
+                    double2 x[3];
+#pragma unroll
+                    for (int u = 0; u < 3; ++u) x[u] = *(const double2*)(ct + 2 * u * kTileW + i);
+#pragma unroll
+                    for (int a = 0; a < (decltype(two)::value ? 2 : 1); ++a) {
+                        const double f0 = ft[i * kF64Stride + 16 * a], f1 = ft[(i + 1) * kF64Stride + 16 * a];
+#pragma unroll
+                        for (int u = 0; u < 3; ++u) {
+                            acc[a][u] += x[u].x * f0;
+                            acc[a][u] += x[u].y * f1;
+                        }
+                    }
+                }
+            }
+        };
+        if (ntA > 1) products(std::true_type());
+        else products(std::false_type());
+    }
+    if (mine)
+#pragma unroll
+        for (int a = 0; a < 2; ++a)
+#pragma unroll
+            for (int u = 0; u < 3; ++u)
+                if (a < ntA) z[a * kTileVals + 2 * u * kTileW] = acc[a][u];
 }
 
 struct SKd {
@@ -615,21 +750,26 @@ static cudaError_t adjoint_t(Ctx* c, double* d_grad, double* d_par, double* d_gm
     int max_nb = 1;
     for (int g = 0; g < c->n_groups; ++g) max_nb = std::max(max_nb, c->h_gnb_ptr[g + 1] - c->h_gnb_ptr[g]);
     const int per = std::min(max_nb, kZNb);
-    const size_t smem_z = zmul_smem<T>(per), smem_g = grad_smem<T>(c->max_cl_otiles);
+    constexpr bool kFP64 = std::is_same<T, double>::value;
+    const size_t smem_z = (kFP64 ? kZmul64Smem : kZmulSmem) + z_lookup_smem(per), smem_g = grad_smem<T>(c->max_cl_otiles);
     if (smem_l > (size_t)kMaxDynSmem || smem_g > (size_t)kMaxDynSmem) return cudaErrorInvalidValue;
     cudaError_t e = allow_dynamic_smem(k_zlists);
     if (e != cudaSuccess) return e;
     k_zlists<<<c->n_mol, 256, smem_l, c->stream>>>(
         c->n_occ_tiles, c->n_groups, c->cap, c->d_c_nt[in], c->d_c_tile[in], c->d_tile_group, c->d_group_ot0,
         c->d_group_not, c->d_gnb_ptr, c->d_gnb_col, c->d_c_nt[zb], c->d_c_tile[zb], &c->d_sc->err);
-    auto zmul = max_nb > kZNb ? k_zmul<T, true> : k_zmul<T, false>;
+    const bool many = max_nb > kZNb;
+    auto zmul = [&] {
+        if constexpr (kFP64) return many ? k_zmul64<true> : k_zmul64<false>;
+        else return many ? k_zmul<true> : k_zmul<false>;
+    }();
     e = allow_dynamic_smem(zmul);
     if (e != cudaSuccess) return e;
     // groups of molecules on grid y (65535 at most), out groups of their cluster on grid x
     for (int nb_lo = 0; nb_lo < max_nb; nb_lo += per)
         for (int g0 = 0; g0 < c->n_groups; g0 += 65535) {
             const int ng = std::min(65535, c->n_groups - g0);
-            zmul<<<dim3(c->max_cl_groups, ng), kZThreads, smem_z, c->stream>>>(
+            zmul<<<dim3(c->max_cl_groups, ng), kFP64 ? kZ64Threads : kZThreads, smem_z, c->stream>>>(
                 g0, nb_lo, per, c->cap, c->d_group_cl, c->d_cl_g0, c->d_grp_mol_ptr, c->d_grp_mol, c->d_c_nt[in], c->d_c_tile[in],
                 (const T*)c->d_c_val[in], c->d_group_ot0, c->d_group_not, c->d_gnb_ptr, c->d_gnb_col, c->d_ort_blk_tp[1],
                 c->d_gnb_rev, (const T*)c->d_sig, c->d_c_nt[zb], c->d_c_tile[zb], (T*)c->d_c_val[zb]);
