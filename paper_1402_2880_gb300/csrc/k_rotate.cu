@@ -180,9 +180,13 @@ __global__ void k_rot_pick(int shift, int last_shift, int n_clusters, ClSel* cl,
 
 // The whole selection (k_rot_stats, the radix passes) in one CTA, for a single
 // cluster of few blocks (kSelSmallBlocks): the launches between the passes cost
-// more than the passes (11 of them, 17 in FP64, ~4 us each; now one of 14 us at 8
-// molecules, 56 in FP64 at 32).
-constexpr int kSelSmallBlocks = 512;
+// more than the passes (11 of them, 17 in FP64, ~4 us each), until one CTA has too
+// many keys to read. With the pair lists, without and with more candidates than the
+// cap, us in one CTA against the launches: FP32 at 16 blocks 22 and 37 against 52 and
+// 72, at 64 (45 and 64 molecules) 28 and 62 against 54 and 66, 36 and 80 against 58 and
+// 68, at 308 191 to 279 against 76 to 81; FP64 at 64 30 and 91 against 76 and 95, 32 and
+// 116 against 80 and 102, at 308 291 to 433 against 107.
+constexpr int kSelSmallBlocks = 64;
 template <typename T>
 __global__ void __launch_bounds__(1024) k_rot_select_small(int last_shift, int n_gnb, const int* __restrict__ gnb_row,
                                                            const int* __restrict__ gnb_col,
