@@ -182,6 +182,9 @@ __global__ void __launch_bounds__(1024) k_ci_small(int n_mol, int n_tiles, int c
 // ---------------------------------------------------------------------------
 // CTAs per SM that a launch aims at (FP32, one CTA per tile: 4.4 ms at 4096 molecules, 1.18 at 997;
 // 8: 4.4 and 0.73; 32: 3.7 and 0.68; FP64 at 343: 1.86 -> 0.99)
+// clusters of a few rows in a batch, H and S, us, so many CTAs against four rows per warp: 1000 of 3
+// molecules, FP32 56 + 49, 28 + 25, FP64 59 + 51, 45 + 29; 300 of 30, FP32 264 + 229, 210 + 162, FP64
+// 1475 + 984, 1417 + 963
 constexpr int kXcCtas = 32;
 constexpr int kXcBatch = 4;   // matched neighbours whose loads are in flight together
 template <typename T>
@@ -1031,8 +1034,10 @@ cudaError_t launch_xc(Ctx* c, bool use_h, int tile_lo, int tile_hi, int own_belo
     const int nr = c->max_cl_mol;
     const size_t smem = (size_t)((nr + 31) / 32) * 8 + (size_t)nr * 2 + 64;
     if (smem > 200 * 1024) return cudaErrorInvalidValue;
-    // CTAs per tile: enough for kXcCtas per SM
-    const int sh = std::min(8, std::max(1, (kXcCtas * c->n_sm + n - 1) / n));
+    // CTAs per tile: enough for kXcCtas per SM, but a warp gets four rows unless that leaves the SMs with
+    // fewer than eight (each CTA of a tile builds the tile's maps anew)
+    const int fill = (8 * c->n_sm + n - 1) / n, most = (kXcCtas * c->n_sm + n - 1) / n;
+    const int sh = std::min({8, most, std::max(fill, (nr + 31) / 32)});
     if (c->prec == SSCF_FP64)
         k_xc<double><<<n * sh, 256, smem, c->stream>>>(tile_lo, n, sh, nr, own_below, c->cap, c->capY, c->d_tile_row0, c->d_cci_ptr, c->d_cci_row,
                                                   c->d_cci_slot, (const double*)c->d_c_val[b], c->d_mp_ptr,
