@@ -695,7 +695,9 @@ __global__ void k_pair_sum(int n_mol, int n_mp, const int* __restrict__ mp_ptr, 
 // dE/dx_a of dq^T gamma dq / 2: -dq_a sum_b dq_b gamma_ab^3 (x_a - x_b), one
 // warp per 32 atoms a and share of the atoms b (the FP64 pipe bounds it: one
 // thread per atom over all b kept a third of the SMs busy, 7.3 ms at 6000
-// atoms; now 1.3).
+// atoms; now 1.3). rsqrt is nearer to the exact value than a division by a square
+// root: 1.01 and 1.50 units of 2^-53 at most over 4 million arguments from 0.01 to
+// 10^6, 0.36 and 0.50 on average.
 __global__ void __launch_bounds__(32) k_gamma_force(int n, const double* __restrict__ xyz,
                                                     const int* __restrict__ species, const int* __restrict__ atom_lo,
                                                     const int* __restrict__ atom_hi, const double* __restrict__ dq,

@@ -6,9 +6,9 @@
 // after the other. Here the labels are the colours of a greedy edge colouring
 // of the MO-group graph, and inside a block pairs go by the in-block colour
 // (i_loc + j_loc) mod n. Every 2x2 update uses coefficients fixed at the start
-// of the sweep, so the whole sweep acts on each AO row of C independently:
-// the apply kernel gives one CTA to one AO row, walks the colours in order
-// and reads and writes C once.
+// of the sweep, so the whole sweep acts on each AO row of C independently. A
+// colour is one launch: every block's rows with work are shared by its CTAs, which
+// read and write the tiles of the block's two sides in place.
 #include <math.h>
 
 #include <algorithm>
