@@ -755,17 +755,21 @@ static cudaError_t adjoint_t(Ctx* c, double* d_grad, double* d_par, double* d_gm
     constexpr bool kFP64 = std::is_same<T, double>::value;
     const size_t smem_z = (kFP64 ? kZmul64Smem : kZmulSmem) + z_lookup_smem(per), smem_g = grad_smem<T>(c->max_cl_otiles);
     if (smem_l > (size_t)kMaxDynSmem || smem_g > (size_t)kMaxDynSmem) return cudaErrorInvalidValue;
-    cudaError_t e = allow_dynamic_smem(k_zlists);
+    cudaError_t e = allow_dynamic_smem<k_zlists>();
     if (e != cudaSuccess) return e;
     k_zlists<<<c->n_mol, 256, smem_l, c->stream>>>(
         c->n_occ_tiles, c->n_groups, c->cap, c->d_c_nt[in], c->d_c_tile[in], c->d_tile_group, c->d_group_ot0,
         c->d_group_not, c->d_gnb_ptr, c->d_gnb_col, c->d_c_nt[zb], c->d_c_tile[zb], &c->d_sc->err);
     const bool many = max_nb > kZNb;
     auto zmul = [&] {
-        if constexpr (kFP64) return many ? k_zmul64<true> : k_zmul64<false>;
-        else return many ? k_zmul<true> : k_zmul<false>;
+        if constexpr (kFP64) {
+            e = many ? allow_dynamic_smem<k_zmul64<true>>() : allow_dynamic_smem<k_zmul64<false>>();
+            return many ? k_zmul64<true> : k_zmul64<false>;
+        } else {
+            e = many ? allow_dynamic_smem<k_zmul<true>>() : allow_dynamic_smem<k_zmul<false>>();
+            return many ? k_zmul<true> : k_zmul<false>;
+        }
     }();
-    e = allow_dynamic_smem(zmul);
     if (e != cudaSuccess) return e;
     // groups of molecules on grid y (65535 at most), out groups of their cluster on grid x
     for (int nb_lo = 0; nb_lo < max_nb; nb_lo += per)
@@ -787,7 +791,7 @@ static cudaError_t adjoint_t(Ctx* c, double* d_grad, double* d_par, double* d_gm
     double* Pb = c->d_adj;
     double* Wb = Pb + (size_t)c->n_mp * 36;
     double* pt = Wb + (size_t)c->n_mp * 36;
-    e = allow_dynamic_smem(k_grad_blocks<T>);
+    e = allow_dynamic_smem<k_grad_blocks<T>>();
     if (e != cudaSuccess) return e;
     k_grad_blocks<T><<<c->n_mol, kGradWarps * 32, smem_g, c->stream>>>(
         c->n_occ_tiles, c->max_cl_otiles, c->d_mol_ot0, c->cap, c->d_c_nt[in], c->d_c_tile[in],

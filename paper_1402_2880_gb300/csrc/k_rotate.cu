@@ -2137,14 +2137,14 @@ static cudaError_t closure_t(Ctx* c, int mode, int which, int col_lo, int col_hi
     a.col_hi = col_hi;
     const size_t smem = closure_smem_bytes(c);
     if (smem > (size_t)kMaxDynSmem) return cudaErrorInvalidValue;
-    cudaError_t e = allow_dynamic_smem(k_closure<T>);
+    cudaError_t e = allow_dynamic_smem<k_closure<T>>();
     if (e != cudaSuccess) return e;
     a.lab_start = c->d_lab_start;
     a.lab_cnt = c->d_lab_cnt;
     a.lab_mem = c->d_lab_mem;
     const size_t lsmem = closure_labels_smem_bytes(c);
     if (lsmem > (size_t)kMaxDynSmem) return cudaErrorInvalidValue;
-    e = allow_dynamic_smem(k_closure_labels);
+    e = allow_dynamic_smem<k_closure_labels>();
     if (e != cudaSuccess) return e;
     k_closure_labels<<<c->n_clusters, 1024, lsmem, c->stream>>>(a, c->d_unit_lab);
     k_closure<T><<<c->n_mol, 256, smem, c->stream>>>(a);
@@ -2156,7 +2156,7 @@ static cudaError_t closure_t(Ctx* c, int mode, int which, int col_lo, int col_hi
 template <typename T, int MODE, int NT, int PCAP>
 static cudaError_t apply_generic_t(Ctx* c, const SweepArgs& a, int col_lo, int col_hi) {
     const size_t smem = (size_t)NT * 16 * apply_nrp<T>() * sizeof(T) + (size_t)2 * PCAP * sizeof(T) + (size_t)PCAP * 4;
-    cudaError_t e = allow_dynamic_smem(k_apply_colour<T, MODE, NT, PCAP>);
+    cudaError_t e = allow_dynamic_smem<k_apply_colour<T, MODE, NT, PCAP>>();
     if (e != cudaSuccess) return e;
     const std::vector<int>& ptr = MODE == 0 ? c->h_colour_ptr : c->h_ocolour_ptr;
     constexpr int CH = ApplyShape<T>::chunk;
@@ -2178,7 +2178,7 @@ static cudaError_t apply_warp_t(Ctx* c, SweepArgs& a, int col_lo, int col_hi) {
     const int chunks = (c->n_mol + kFullCH - 1) / kFullCH;
     const size_t smem = Sh::smem + (size_t)std::min(chunks, (c->max_cl_mol + kFullCH - 1) / kFullCH) * 8;
     if (smem > (size_t)kMaxDynSmem) return cudaErrorInvalidValue;
-    cudaError_t e = allow_dynamic_smem(k_apply_warp<T, MODE, ALL>);
+    cudaError_t e = allow_dynamic_smem<k_apply_warp<T, MODE, ALL>>();
     if (e != cudaSuccess) return e;
     if (a.n_blk == 0) return cudaSuccess;
     a.blk_info = c->d_blk_info;

@@ -270,7 +270,7 @@ int link_all(cudaStream_t s, const KmState& st, const double* cen, double* cen_n
         k_km_dist<<<(unsigned)((pairs + th - 1) / th), th, 0, s>>>(st.n, st.nc, st.pos, cen, st.D);
     }
     if (st.n <= kKmOneCta && list_bytes <= kKmMaxSmem) {
-        KM_CK(allow_dynamic_smem(k_km_match<true>));
+        KM_CK(allow_dynamic_smem<k_km_match<true>>());
         k_km_match<true><<<1, 1024, list_bytes, s>>>(st.n, st.nc, st.n_link, st.pos, cen, st.D, st.lists, st.next,
                                                      st.next + 1);
     } else {

@@ -22,6 +22,7 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include <atomic>
 #include <string>
 #include <vector>
 
@@ -39,16 +40,21 @@ constexpr int kMaxSub = 48;                    // in-block colours (<= MOs per g
 constexpr int kRotCap = 32 * 16;               // pairs of one occupied-virtual block
 constexpr int kOrthoCap = 48 * 48;             // pairs of one orthonormalisation block
 
-// Dynamic shared memory for `kernel` up to what a CTA may opt into. Always the same
+// Dynamic shared memory for a kernel up to what a CTA may opt into. Always the same
 // value: the attribute belongs to the kernel, which contexts of other sizes launch
 // from other threads. A context that set its own size could lower another's between
 // that one's setting and its launch, which then failed.
-template <typename K> inline cudaError_t allow_dynamic_smem(K* kernel) {
-    cudaFuncAttributes fa;
-    cudaError_t e = cudaFuncGetAttributes(&fa, kernel);
-    if (e != cudaSuccess) return e;
-    return cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                kMaxDynSmem - (int)fa.sharedSizeBytes);
+template <auto Kernel> inline cudaError_t allow_dynamic_smem() {
+    static std::atomic<int> fixed{-1};   // the kernel's static shared memory, asked for once (1 us)
+    int bytes = fixed.load(std::memory_order_relaxed);
+    if (bytes < 0) {
+        cudaFuncAttributes fa;
+        const cudaError_t e = cudaFuncGetAttributes(&fa, Kernel);
+        if (e != cudaSuccess) return e;
+        bytes = (int)fa.sharedSizeBytes;
+        fixed.store(bytes, std::memory_order_relaxed);
+    }
+    return cudaFuncSetAttribute(Kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kMaxDynSmem - bytes);
 }
 
 // Shape of a sweep's launch for one colour: CTAs per block, and the runs (32 AO
