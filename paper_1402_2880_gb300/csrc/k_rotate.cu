@@ -1209,7 +1209,9 @@ __global__ void __launch_bounds__(apply_threads<T>()) k_apply_colour(SweepArgs a
 //           they are. Per slot two FMAs, a compare and a multiply per value, and
 //           half a coefficient load: 7.6 clocks of an SM quarter per slot and row
 //           packed, 8.2 unpacked, in a loop of its own; the FMA and ALU pipes
-//           would take 4, the operand reads of the register file bound it.
+//           would take 4, the operand reads of the register file bound it. (In passes over
+//           all MOs one warp per quarter of an SM waits for instructions of the unrolled
+//           loops, results and barriers instead: 15 to 27 % of the issue slots used.)
 //   list    the block's pairs one after the other in schedule order, both sides
 //           in a shared-memory panel [column][lane], one AO row per lane, up to
 //           four pairs of a level in flight. Self blocks, rotations, combination
@@ -2185,13 +2187,14 @@ static cudaError_t apply_warp_t(Ctx* c, SweepArgs& a, int col_lo, int col_hi) {
     k_block_info<MODE, ALL><<<(a.n_blk + 127) / 128, 128, 0, c->stream>>>(a, a.n_blk, (BlockInfo*)c->d_blk_info);
     c->n_launch += 1;
     const std::vector<int>& ptr = MODE == 0 ? c->h_colour_ptr : c->h_ocolour_ptr;
-    // CTAs per block: shares of `per` runs for as many runs as the largest cluster's rows can give
-    // (variant 2: one CTA takes all runs of its block; same results)
+    // CTAs per block: sweep_shape, for as many runs as the largest cluster's rows can give (variant 2: one CTA
+    // takes all runs of its block; same results)
     const int full = c->n_sm * Sh::resident;
     // A colour's CTAs start while the last of the one before run, so that the end of one launch hides the
     // start of the next: rotations at 997 molecules 1.74 -> 1.50 ms, at 4096 9.3 -> 9.0, FP64 at 343 1.52 ->
     // 1.40; FP32 combinations 5.28 -> 5.20 and 42.2 -> 42.0. Not FP64 combinations, whose long blocks come
-    // first and would gather on the SMs that end early (343: 10.4 -> 11.9), and not inside a captured graph.
+    // first and would gather on the SMs that end early (343: 10.4 -> 11.9), and not inside a captured graph, where
+    // it has not been tried.
     cudaStreamCaptureStatus capture = cudaStreamCaptureStatusNone;
     e = cudaStreamIsCapturing(c->stream, &capture);
     if (e != cudaSuccess) return e;
