@@ -520,7 +520,7 @@ __device__ __forceinline__ void mma_tf32(float (&d)[4], const uint32_t (&a)[4], 
 // AO rows of up to four matched row blocks (24 rows, 3 k-steps of 8) at a time.
 // Each product is split into TF32 hi + lo parts and summed as hi*hi + hi*lo +
 // lo*hi (the lo*lo term is below FP32 rounding), into FP32 fragments that are
-// added up in FP64 every 32 of b's rows.
+// added up in FP64 every 32 of b's rows (one alone, in a small system, is taken as it is: 2 us of a launch's 19).
 // A row of a 6x16 tile is 64 bytes, so a warp reads a fragment's four rows of two
 // columns per lane straight from memory: no staging, no shared-memory traffic, and
 // a's tiles are found in L1 by the CTA's other warps (b's pass it by). Bound by the
@@ -576,13 +576,11 @@ k_transform_tc(int n_split, int n_rows, const int* __restrict__ tile_row0, int c
         const float* yb = y_val + (size_t)b * capY * kTileVals;
         float acc[2][4];
         double sum[2][4];
+        bool added = false;
 #pragma unroll
         for (int h = 0; h < 2; ++h)
 #pragma unroll
-            for (int q = 0; q < 4; ++q) {
-                acc[h][q] = 0.f;
-                sum[h][q] = 0.0;
-            }
+            for (int q = 0; q < 4; ++q) acc[h][q] = 0.f;
         for (int k0 = 0; k0 < nb; k0 += 32) {
             const int k = k0 + lane;
             int at = -1;   // index of the tile C[r, a]
@@ -634,18 +632,33 @@ k_transform_tc(int n_split, int n_rows, const int* __restrict__ tile_row0, int c
                 }
             }
             __syncwarp();
+            if (!added && k0 + 32 >= nb) break;   // the only partial sums: as they are
+            if (added) {
+#pragma unroll
+                for (int h = 0; h < 2; ++h)
+#pragma unroll
+                    for (int q = 0; q < 4; ++q) sum[h][q] += (double)acc[h][q];
+            } else {
+#pragma unroll
+                for (int h = 0; h < 2; ++h)
+#pragma unroll
+                    for (int q = 0; q < 4; ++q) sum[h][q] = (double)acc[h][q];
+            }
 #pragma unroll
             for (int h = 0; h < 2; ++h)
 #pragma unroll
-                for (int q = 0; q < 4; ++q) {
-                    sum[h][q] += (double)acc[h][q];
-                    acc[h][q] = 0.f;
-                }
+                for (int q = 0; q < 4; ++q) acc[h][q] = 0.f;
+            added = true;
         }
+        if (added)
+#pragma unroll
+            for (int h = 0; h < 2; ++h)
+#pragma unroll
+                for (int q = 0; q < 4; ++q) acc[h][q] = (float)sum[h][q];
         // rows 2gq and 2gq + 1 of the block, columns 4tq to 4tq + 3
         float4* o = (float4*)(out + (size_t)tp_out[p] * 256) + 8 * gq + tq;
-        o[0] = make_float4((float)sum[0][0], (float)sum[1][0], (float)sum[0][1], (float)sum[1][1]);
-        o[4] = make_float4((float)sum[0][2], (float)sum[1][2], (float)sum[0][3], (float)sum[1][3]);
+        o[0] = make_float4(acc[0][0], acc[1][0], acc[0][1], acc[1][1]);
+        o[4] = make_float4(acc[0][2], acc[1][2], acc[0][3], acc[1][3]);
         if (nb == 0) r = lane < nb_next ? y_row[(size_t)b_next * capY + lane] : -1;
         b = b_next;
         nb = nb_next;
